@@ -43,9 +43,9 @@ struct BatchLayout {
         DW = I.dc == 4 ? 8 : 12;
         C = (I.R + K - 1) / K;
         ngroups = threads / I.group_threads;
-        chain_stride = (int)(up16((size_t)I.slot_stride) + up16((size_t)I.P));
+        chain_stride = (int)up16((size_t)I.slot_stride);
         nbufs = I.resident ? C : ngroups;
-        thr_words = (int)(up16((size_t)I.nL3 * 4) / 4);
+        thr_words = (int)(up16((size_t)IndexRule(I.Lmax).row_words() * 4) / 4);
         size_t o = 0;
         sdesc = o;  o += (size_t)I.N * DW * 4;
         items = o;  o += up16((size_t)2 * I.N * 4);
@@ -74,7 +74,9 @@ __device__ __forceinline__ void group_sync(int bar, int gsize) {
         named_barrier(bar, gsize);
 }
 
-template <int DC>
+// W: 4-copy words of an update unit (2 when P % 16 == 0: the rows' halves are then whole
+// 8-byte words, and one descriptor, one address and one wide load per neighbour serve 8 copies).
+template <int DC, int W, bool WIDE>
 __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* s_keys, cg::cluster_group& cluster,
                             int rank, int K) {
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -94,6 +96,8 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
     const int N = I.N, P = I.P, R = I.R, C = L.C;
     const int c_begin = rank * C;
     const int c_count = max(0, min(C, R - c_begin));
+    const IndexRule index(I.Lmax);
+    const UnitRule<WIDE> rule(I.Lmax);
     const int gsize = I.group_threads, ngroups = L.ngroups;
     const int grp = tid / gsize, gtid = tid - grp * gsize;
 
@@ -115,14 +119,13 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
             s_E[x] = I.E[c_begin + x];
             s_M[x] = I.M[c_begin + x];
         }
-        if (I.thr_resident)  // every rung's row, so a chain never reloads one after a swap
-            for (int x = tid; x < I.R * L.thr_words; x += nt) {
-                const int r = x / L.thr_words, c = x - r * L.thr_words;
-                s_thr[x] = c < I.nL3 ? I.thr[(size_t)r * I.nL3 + c] : 0u;
+        if (I.thr_resident) {  // every rung's row, so a chain never reloads one after a swap
+            const int nL = 2 * I.Lmax + 1;
+            for (int x = tid; x < R * nL; x += nt) {
+                const int r = x / nL, l = x - r * nL;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) s_thr[(size_t)r * L.thr_words + c * index.S + l] = I.thr[3 * x + c];
             }
-        for (int b = 0; b < L.nbufs; ++b) {
-            int8_t* ones = reinterpret_cast<int8_t*>(s_chains + (size_t)b * L.chain_stride + I.slot_stride);
-            for (int x = tid; x < P; x += nt) ones[x] = 1;
         }
         if (I.resident) {
             for (int lc = 0; lc < c_count; ++lc)
@@ -138,8 +141,9 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
     const uint32_t ginv = chunk_ginv(G);
     const bool p16 = (P & 15) == 0;  // streamed chains move 16 copies per load and store
     const uint32_t hinv = chunk_ginv(P >> 4);
+    const int U = G / W;  // units of a row and parity
     int lg = 0;
-    while ((1 << lg) < G) ++lg;
+    while ((1 << lg) < U) ++lg;
     const int gmask = (1 << lg) - 1;
     const int bar = 1 + grp;
     uint32_t* thr_g = s_thr + (size_t)grp * L.thr_words;
@@ -147,6 +151,8 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
     const int lane = tid & 31, gwarp = gtid >> 5;
     const bool g_fixed = (gsize & gmask) == 0;
     const int g_own = gtid & gmask, q_lane = gtid >> lg, q_step = gsize >> lg;
+    const uint32_t half = (uint32_t)P >> 1;
+    const UnitOffsets off_own = row_offsets<W>((uint32_t)g_own, half);
 
     for (int s = 0; s < I.n_sweeps; ++s) {
         const uint32_t t = (uint32_t)(I.t0 + s);
@@ -160,41 +166,52 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
                     load_split(buf, I.spins + (size_t)rho * I.slot_stride, N, P, G, ginv, gtid, gsize);
             }
             const int rung = s_rung[rho];
-            const uint32_t* thr_c;
+            const uint32_t thr_c = thr_base<WIDE>(
+                (uint32_t)L.thr + 4u * (uint32_t)L.thr_words * (uint32_t)(I.thr_resident ? rung : grp), I.Lmax);
             if (I.thr_resident) {
-                thr_c = s_thr + (size_t)rung * L.thr_words + 3 * I.Lmax;
                 if (!I.resident) group_sync(bar, gsize);  // the streamed chain is in place
             } else {
-                for (int x = gtid; x < I.nL3; x += gsize) thr_g[x] = I.thr[(size_t)rung * I.nL3 + x];
+                for (int l = gtid; l <= 2 * I.Lmax; l += gsize)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) thr_g[c * index.S + l] = I.thr[(size_t)rung * I.nL3 + 3 * l + c];
                 group_sync(bar, gsize);
-                thr_c = thr_g + 3 * I.Lmax;
             }
-            int sumL = 0, sumC = 0, nf = 0;  // sumC and nf count twice (see unit_commit)
+            FlipSums sums;
+            sums.clear();
             for (int lev = 0; lev < I.n_levels; ++lev) {
                 const int base = s_loff[lev];
                 if (g_fixed) {
-                    // this thread's column g never changes (see the single-problem kernel)
-                    if (g_own < G) {
+                    // this thread's column never changes (see the single-problem kernel)
+                    if (g_own < U) {
                         const int end = s_loff[lev + 1];
-                        for (int q = base + q_lane; q < end; q += q_step)
-                            packed_unit<DC, false>(buf, s_sdesc, s_items[q], nullptr, q, g_own, G, P, t,
-                                                   (uint32_t)rho, skey, thr_c, sumL, sumC, nf);
+                        for (int q = base + q_lane; q < end; q += q_step) {
+                            const UnitEval<W> e =
+                                unit_eval<DC, W, false, WIDE>(buf, s_sdesc, s_items[q], off_own, nullptr, t, (uint32_t)rho,
+                                                        (uint32_t)(W * g_own), rule, skey);
+                            uint32_t F[W];
+                            unit_flips<W, false, WIDE>(e, smem, rule, thr_c, F);
+                            unit_commit<W>(e, F, sums);
+                        }
                     }
                 } else {
                     const int units = (s_loff[lev + 1] - base) << lg;
                     for (int u = gtid; u < units; u += gsize) {
                         const int g = u & gmask;
-                        if (g >= G) continue;
-                        const int q = base + (u >> lg);
-                        packed_unit<DC, false>(buf, s_sdesc, s_items[q], nullptr, q, g, G, P, t, (uint32_t)rho, skey,
-                                               thr_c, sumL, sumC, nf);
+                        if (g >= U) continue;
+                        const UnitEval<W> e =
+                            unit_eval<DC, W, false, WIDE>(buf, s_sdesc, s_items[base + (u >> lg)],
+                                                    row_offsets<W>((uint32_t)g, half), nullptr, t, (uint32_t)rho,
+                                                    (uint32_t)(W * g), rule, skey);
+                        uint32_t F[W];
+                        unit_flips<W, false, WIDE>(e, smem, rule, thr_c, F);
+                        unit_commit<W>(e, F, sums);
                     }
                 }
                 group_sync(bar, gsize);
             }
-            const int dE = __reduce_add_sync(0xFFFFFFFFu, -2 * sumL);
-            const int dM = __reduce_add_sync(0xFFFFFFFFu, -2 * (sumC - nf));  // both counted twice
-            nf = __reduce_add_sync(0xFFFFFFFFu, nf) >> 1;
+            const int dE = __reduce_add_sync(0xFFFFFFFFu, sums.dE(rule));
+            const int dM = __reduce_add_sync(0xFFFFFFFFu, sums.dM(rule));
+            const int nf = __reduce_add_sync(0xFFFFFFFFu, sums.flips());
             if (lane == 0) {
                 red_g[gwarp * 3 + 0] = dE;
                 red_g[gwarp * 3 + 1] = dM;
@@ -277,6 +294,30 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
     }
 }
 
+__device__ __forceinline__ void run_any(const BatchInstance& I, unsigned char* smem, uint4* s_keys,
+                                        cg::cluster_group& cluster, int rank, int K) {
+    if (IndexRule(I.Lmax).wide) {  // large couplings: one instantiation a class
+        if (I.dc == 4)
+            run_problem<4, 1, true>(I, smem, s_keys, cluster, rank, K);
+        else
+            run_problem<8, 1, true>(I, smem, s_keys, cluster, rank, K);
+    } else if (I.dc == 4) {
+        if (I.unit_words == 4)
+            run_problem<4, 4, false>(I, smem, s_keys, cluster, rank, K);
+        else if (I.unit_words == 2)
+            run_problem<4, 2, false>(I, smem, s_keys, cluster, rank, K);
+        else
+            run_problem<4, 1, false>(I, smem, s_keys, cluster, rank, K);
+    } else {
+        if (I.unit_words == 4)
+            run_problem<8, 4, false>(I, smem, s_keys, cluster, rank, K);
+        else if (I.unit_words == 2)
+            run_problem<8, 2, false>(I, smem, s_keys, cluster, rank, K);
+        else
+            run_problem<8, 1, false>(I, smem, s_keys, cluster, rank, K);
+    }
+}
+
 __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_job;
@@ -286,10 +327,7 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
     const int K = (int)cluster.num_blocks();
     if (bp.single) {
         // one problem on this one cluster; the host keeps its counters
-        if (bp.one.dc == 4)
-            run_problem<4>(bp.one, smem, s_keys, cluster, rank, K);
-        else
-            run_problem<8>(bp.one, smem, s_keys, cluster, rank, K);
+        run_any(bp.one, smem, s_keys, cluster, rank, K);
         if (K > 1) cluster.sync();  // peers are done reading this CTA's published (E, M)
         return;
     }
@@ -300,10 +338,7 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
         cluster.sync();  // every CTA has read the job before rank 0 may reuse or release s_job
         if (job >= bp.count) break;
         const BatchInstance I = bp.inst[bp.order[job]];
-        if (I.dc == 4)
-            run_problem<4>(I, smem, s_keys, cluster, rank, K);
-        else
-            run_problem<8>(I, smem, s_keys, cluster, rank, K);
+        run_any(I, smem, s_keys, cluster, rank, K);
         cluster.sync();  // peers are done reading this CTA's published (E, M)
         if (rank == 0 && threadIdx.x == 0) {
             // a finished problem's counters advance on the device, so the same launch can be
@@ -345,22 +380,26 @@ __global__ void batch_init_kernel(const BatchInstance* inst, const int2* map) {
         I.slot_of_rung[rho] = rho;
     }
     __syncthreads();
-    // E from the site descriptors: each edge once (neighbour row > own row), h once (the
-    // slot whose row is the constant +1 row)
-    const int DW = I.dc == 4 ? 8 : 12;
-    const uint32_t np = (uint32_t)I.N * (uint32_t)I.P;
+    // E from the site descriptors: each edge once (neighbour row > own row), h once. The
+    // couplings come back out of the multipliers, h out of the constant word (see SiteDesc).
+    const int DW = I.dc == 4 ? 8 : 12, NS = I.dc - 1;
+    const int zero = IndexRule(I.Lmax).zero();
     long long e = 0, mm = 0;
     for (int x = threadIdx.x; x < I.N * I.P; x += blockDim.x) {
         const int i = x / I.P, k = x - i * I.P;
         const uint32_t* d = I.sdesc + (size_t)i * DW;
+        const uint32_t row = I.dc == 4 ? d[7] : d[3];
         const int si = sp[x];
-        int f = 0;
-        for (int sl = 0; sl < I.dc; ++sl) {
-            const uint32_t row = d[4 + sl];
-            if (row <= d[0]) continue;
-            const int J = (int)(int8_t)((d[2 + (sl >> 2)] >> (8 * (sl & 3))) & 0xFFu);
-            f += J * (row >= np ? 1 : (int)sp[row + k]);
+        int f = 0, sumJ = 0;
+        for (int sl = 0; sl < NS; ++sl) {
+            const int J = I.dc == 4 ? -(int)(d[4 + sl] * 127u)
+                                    : (int)(int8_t)((d[1 + (sl >> 2)] >> (8 * (sl & 3))) & 0xFFu);
+            const uint32_t off = I.dc == 4 ? d[1 + sl] : d[4 + sl];
+            sumJ += J;
+            if (off > row) f += J * (int)sp[off + k];
         }
+        const uint32_t c = (d[0] - kInv127 * (uint32_t)sumJ * 0x01010101u) & 0xFFu;  // h + sum J + zero
+        f += (int)c - sumJ - zero;
         e += (long long)si * f;
         mm += (long long)si * sp[(size_t)i * I.P + ((k + 1 == I.P) ? 0 : k + 1)];
     }
@@ -625,7 +664,7 @@ int ptq::prepare_request(const pt_request& r, Prepared& pr, char* why, size_t wh
     if (pr.coef.size() < 2) pr.coef.assign(2, 0.0);
     level_schedule(N, adj, pr.items, pr.level_off, per_round, P / 4);  // rows of P bytes (int8 packed)
     pr.n_levels = (int)pr.level_off.size() - 1;
-    build_site_desc(N, P, pr.dc, adj, adjJ, inst->h, pr.sdesc);
+    build_site_desc(N, P, pr.dc, Lmax, adj, adjJ, inst->h, pr.sdesc);
     return PT_OK;
 }
 
@@ -684,6 +723,31 @@ void ptq::fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base
     I.swap_stats = (unsigned long long*)(base + p.off_sw);
 }
 
+// A wider unit costs less per copy (one descriptor, address and wide load per neighbour for
+// more copies; measured in isolation at 186, 166 and 146 cycles per four copies and warp for
+// 1, 2 and 4 words) but gives a level fewer units to spread over the group, so the width is
+// the one with the least rounds x cost on a level of average size. Rows' halves have to be
+// whole units.
+int ptq::choose_unit_words(const BatchInstance& I, int group_threads) {
+    if (IndexRule(I.Lmax).wide) return 1;
+    static const int kCost[3] = {186, 332, 584};
+    const double items = 2.0 * I.N / std::max(1, I.n_levels);
+    int best = 1;
+    double best_cost = 0.0;
+    for (int k = 0; k < 3; ++k) {
+        const int W = 1 << k;
+        if (I.P % (8 * W)) break;
+        int cols = 1;
+        while (cols < I.P / (8 * W)) cols <<= 1;
+        const double cost = std::ceil(items * cols / group_threads) * kCost[k];
+        if (k == 0 || cost < best_cost) {
+            best = W;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen) {
     // threads per chain: about one 4-copy unit per thread in an average level, at least two
     // warps, and no more groups than a CTA has chains; chains stay resident when they fit.
@@ -707,7 +771,7 @@ void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_
     while (g > 32 && up_ok(g) && threads / g > 15) g <<= 1;  // named barriers 1..15 (0: the CTA's)
     // every rung's threshold row in shared memory when the rows take at most 48 KB and the
     // chains still fit; resident chains come first
-    const int thr_words = (int)(up16((size_t)I.nL3 * 4) / 4);
+    const int thr_words = (int)(up16((size_t)IndexRule(I.Lmax).row_words() * 4) / 4);
     const int thr_ok = (size_t)I.R * thr_words * 4 <= 49152 ? 1 : 0;
     for (;;) {
         I.group_threads = g;
@@ -724,6 +788,7 @@ void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_
         g <<= 1;  // one streaming buffer per group: fewer, larger groups
         while (up_ok(g) && threads / g > 15) g <<= 1;
     }
+    I.unit_words = choose_unit_words(I, I.group_threads);
 }
 
 // Groups per request, the CTA's shared memory and the persistent grid for one layout.

@@ -342,349 +342,571 @@ __device__ __forceinline__ void store_split16(int8_t* dst, const int8_t* src, in
     }
 }
 
-// One 4-copy unit of the packed path: copies k = 8g + par + 2w (w = 0..3) of site i, which
-// are bytes 4g..4g+3 of the row's parity-par half.
-// Site descriptor (DW words): row offset i*P, i, packed J bytes (two words), then the row
-// offsets of the DC neighbour slots (the slot after the last neighbour holds h against the
-// constant +1 row; the remaining slots have J = 0).
-// Each neighbour slot contributes one word (its 4 copies) to field_times_spin, which forms
-// L = s (h + sum_j J_ij s_j) of the four copies. The Trotter column
-// m/2+1 = 2 - [left differs] - [right differs] comes from the opposite-parity word and one
-// edge byte with byte XORs.
+// ------------------------------------------------------------------------- update unit
+// A unit is the W * 4 copies of one parity of one site that one thread updates together:
+// bytes 4 W u .. 4 W (u + 1) - 1 of that parity's half of the site's row, one +-1 byte a copy.
+//
+// All of a unit's arithmetic up to the table lookup is done on four copies at once, as plain
+// 32-bit integer multiply-adds on the words of +-1 bytes. A word V of +-1 bytes is
+// 0x01010101 + 254 B with B the word of 0 / 1 bytes "spin is -1", so with k = -J / 127 modulo
+// 2^32 (127 is odd) k V = k 0x01010101 - 2 J B: a sum of such products over the neighbours,
+// plus a constant word, is exactly the word whose four bytes are h + sum_j J_j s_j + Lmax,
+// because each byte of the result is in [0, 2 Lmax] and everything is exact modulo 2^32. One
+// multiply-add per neighbour word replaces the byte transposes and dp4a a per-copy field takes.
+// The product with the own spin mirrors the byte where the spin is -1 (x -> 2 Lmax - x): an
+// exclusive-or with the spin's sign mask and one multiply-add. The Trotter term enters as
+// D = [left differs] + [right differs] per byte (doubled). What bounds the packed kernels is
+// the ALU pipe (logic, permute, compare: half the issue width); the multiply-adds run on the
+// FMA pipe beside it.
+//
+// Site descriptor of a class of NS = DC - 1 neighbour slots (unused slots: J = 0, own row),
+// row offsets in bytes:
+//   DC = 4:  C4, off0..2 | k0..2, own row offset                        (8 words)
+//   DC = 8:  C4, J0..3 and J4..6 as bytes, own row offset | off0..3 | off4..6, 0   (12 words)
+// C4 carries h + sum J + Lmax + the index bias in every byte, less the 0x01010101 terms. With
+// seven slots the products are taken with J itself and the sum is scaled by -1/127 once.
 template <int DC>
 struct SiteDesc {
     static constexpr int DW = (DC == 4) ? 8 : 12;
+    static constexpr int NS = DC - 1;
 };
 
-// L_w = s_w (h + sum_j J_j s_j,w) for the four copies w of a unit, from the DC neighbour
-// words a[d] (4 copies of slot d as +-1 bytes), the own word S and the J bytes. A 4x4 byte
-// transpose per four slots feeds dp4a. With four slots the neighbour bytes are first
-// multiplied by the own spins ((a ^ s) | 1 is the product of two +-1 bytes), so dp4a gives
-// L directly; with eight the field is formed first and multiplied by the spin after, which
-// takes fewer ALU operations.
 template <int DC>
-__device__ __forceinline__ void field_times_spin(const uint32_t* a, uint32_t S, const uint32_t* jpack, int* L) {
-    int f[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int b = 0; b < DC / 4; ++b) {
-        uint32_t a0 = a[4 * b + 0], a1 = a[4 * b + 1], a2 = a[4 * b + 2], a3 = a[4 * b + 3];
-        if (DC == 4) {
-            a0 = (a0 ^ S) | 0x01010101u;
-            a1 = (a1 ^ S) | 0x01010101u;
-            a2 = (a2 ^ S) | 0x01010101u;
-            a3 = (a3 ^ S) | 0x01010101u;
-        }
-        const uint32_t t0 = __byte_perm(a0, a1, 0x5140u), t1 = __byte_perm(a0, a1, 0x7362u);
-        const uint32_t t2 = __byte_perm(a2, a3, 0x5140u), t3 = __byte_perm(a2, a3, 0x7362u);
-        f[0] = __dp4a((int)__byte_perm(t0, t2, 0x5410u), (int)jpack[b], f[0]);
-        f[1] = __dp4a((int)__byte_perm(t0, t2, 0x7632u), (int)jpack[b], f[1]);
-        f[2] = __dp4a((int)__byte_perm(t1, t3, 0x5410u), (int)jpack[b], f[2]);
-        f[3] = __dp4a((int)__byte_perm(t1, t3, 0x7632u), (int)jpack[b], f[3]);
-    }
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        if (DC == 4) {
-            L[w] = f[w];
-        } else {
-            const int sw = (int)(int8_t)((S >> (8 * w)) & 0xFFu);  // +1 or -1
-            L[w] = sw * f[w];
-        }
-    }
-}
-
-// All ones when the attempt with random word u is accepted against threshold th, else zero:
-// u < th, read off the borrow of u - th (one subtract with carry out, one subtract of the
-// carry), so that the flip mask and the sums below are formed by multiply-adds on the FMA
-// pipe instead of compares and selects on the ALU pipe. Inline words (PRE = false) are first
-// capped at 2^32 - 2, which folds in the "accept always" entry 0xFFFFFFFF exactly.
-template <bool PRE>
-__device__ __forceinline__ uint32_t accept_mask(uint32_t u, uint32_t th) {
-    if (!PRE) u = min(u, 0xFFFFFFFEu);
-    uint32_t d, m;
-    asm("sub.cc.u32 %0, %2, %3;\n\tsubc.u32 %1, 0, 0;" : "=r"(d), "=r"(m) : "r"(u), "r"(th));
-    return m;
-}
-
-// Threshold entry thr_c[3 L + col] of copy w, col = byte w of Z: the byte offset
-// 4 (3 L + col) comes out of one dp4a (Z's byte w times 4, plus 12 L), keeping the byte
-// extraction and the index arithmetic off the ALU pipe.
-__device__ __forceinline__ uint32_t thr_entry(const uint32_t* thr_c, uint32_t Z, int L, int w) {
-    const int off = __dp4a((int)Z, 4 << (8 * w), 12 * L);
-    return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(thr_c) + off);
-}
-
-// The packed unit in three steps, so that a unit can be evaluated before the threshold row
-// it needs is known: evaluate (loads, fields, Trotter columns, random words), decide the
-// flips against one threshold row, commit (flip store and the sweep's sums).
-struct UnitEval {
-    uint32_t* own;  // the unit's word in shared memory
-    uint32_t S;     // its 4 copies as +-1 bytes
-    uint32_t Z;     // Trotter column m/2+1 per copy
-    int L[4];       // L = s (h + sum_j J s_j) per copy
-    uint32_t u[4];  // random words
+struct SiteTerms {
+    uint32_t off[DC - 1];
+    uint32_t k[DC - 1];
+    uint32_t c4, row;
 };
 
-template <int DC, bool PRE, typename Key = PhiloxKey>
-__device__ __forceinline__ UnitEval packed_unit_eval(int8_t* sp, const uint32_t* s_sdesc, uint32_t item,
-                                                     const uint4* rb, int q, int g, int G, int P, uint32_t t,
-                                                     uint32_t slot, const Key& key) {
-    UnitEval e;
-    const uint32_t par = item & 1u;
-    const uint32_t* desc = s_sdesc + (item >> 1) * SiteDesc<DC>::DW;
-    const uint4 d0 = *reinterpret_cast<const uint4*>(desc);
-    const uint32_t half = (uint32_t)P >> 1;
-    const uint32_t w4 = 4u * (uint32_t)g;
-    const uint32_t own_off = par * half + w4;  // this parity's word in every row
-    uint32_t nrow[DC];
-    uint32_t jpack[DC / 4];
-    {
-        const uint4 d1 = *reinterpret_cast<const uint4*>(desc + 4);
-        nrow[0] = d1.x;
-        nrow[1] = d1.y;
-        nrow[2] = d1.z;
-        nrow[3] = d1.w;
-        jpack[0] = d0.z;
-        if (DC == 8) {
-            const uint4 d2 = *reinterpret_cast<const uint4*>(desc + 8);
-            nrow[DC > 4 ? 4 : 0] = d2.x;
-            nrow[DC > 5 ? 5 : 0] = d2.y;
-            nrow[DC > 6 ? 6 : 0] = d2.z;
-            nrow[DC > 7 ? 7 : 0] = d2.w;
-            jpack[DC > 4 ? 1 : 0] = d0.w;
-        }
-    }
-    const uint32_t row = d0.x;
-    e.own = reinterpret_cast<uint32_t*>(sp + row + own_off);
-    const uint32_t S = *e.own;
-    const uint32_t O = *reinterpret_cast<const uint32_t*>(sp + row + (half - par * half) + w4);
-    // the one Trotter neighbour outside the word: odd copy 8g-1 for even copies, even copy
-    // 8g+8 for odd ones (periodic); parity selects by multiply-add, not by select
-    const uint32_t e_even = half + (g == 0 ? half - 1u : w4 - 1u);
-    const uint32_t e_odd = (w4 + 4u == half) ? 0u : w4 + 4u;
-    const uint32_t edge = (uint8_t)sp[row + e_even + par * (e_odd - e_even)];
-    uint32_t a[DC];
-#pragma unroll
-    for (int d = 0; d < DC; ++d) a[d] = *reinterpret_cast<const uint32_t*>(sp + nrow[d] + own_off);
-    uint4 r4;
-    if (PRE) {
-        r4 = rb[q * G + g];
-    } else {
-        r4 = philox(make_uint4(t, d0.y, slot, (par << 24) | (uint32_t)g), key);
-    }
-    e.u[0] = r4.x;
-    e.u[1] = r4.y;
-    e.u[2] = r4.z;
-    e.u[3] = r4.w;
-
-    // left / right Trotter neighbours: the opposite-parity word itself or shifted by one byte
-    // with the edge copy (selectors 0x3210 = itself, 0x2104 = up, 0x4321 = down)
-    const uint32_t Ln = __byte_perm(O, edge, 0x2104u + par * (0x3210u - 0x2104u));
-    const uint32_t Rn = __byte_perm(O, edge, 0x3210u + par * (0x4321u - 0x3210u));
-    const uint32_t X = (S ^ Ln) & 0x02020202u;
-    const uint32_t Y = (S ^ Rn) & 0x02020202u;
-    e.Z = 0x02020202u - ((X + Y) >> 1);
-    e.S = S;
-    field_times_spin<DC>(a, S, jpack, e.L);
-    return e;
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
 }
 
-// 0xFE in byte w when copy w flips under the threshold row thr_c (offset to L = 0, m = -2).
-// Produced words (PRE) are already min(u, 2^32 - 2), which folds in the "always" entry.
+template <int DC>
+__device__ __forceinline__ SiteTerms<DC> load_site(const uint32_t* desc) {
+    SiteTerms<DC> s;
+    const uint4 d0 = *reinterpret_cast<const uint4*>(desc);
+    const uint4 d1 = *reinterpret_cast<const uint4*>(desc + 4);
+    if constexpr (DC == 4) {
+        s.c4 = d0.x;
+        s.off[0] = d0.y;
+        s.off[1] = d0.z;
+        s.off[2] = d0.w;
+        s.k[0] = d1.x;
+        s.k[1] = d1.y;
+        s.k[2] = d1.z;
+        s.row = d1.w;
+    } else {
+        const uint4 d2 = *reinterpret_cast<const uint4*>(desc + 8);
+        s.c4 = d0.x;
+        s.row = d0.w;
+        s.off[0] = d1.x;
+        s.off[1] = d1.y;
+        s.off[2] = d1.z;
+        s.off[3] = d1.w;
+        s.off[4] = d2.x;
+        s.off[5] = d2.y;
+        s.off[6] = d2.z;
+        // byte b of a J word, sign-extended (a selector nibble with its top bit set repeats the sign)
+        s.k[0] = prmt(d0.y, 0u, 0x8880u);
+        s.k[1] = prmt(d0.y, 0u, 0x9991u);
+        s.k[2] = prmt(d0.y, 0u, 0xAAA2u);
+        s.k[3] = prmt(d0.y, 0u, 0xBBB3u);
+        s.k[4] = prmt(d0.z, 0u, 0x8880u);
+        s.k[5] = prmt(d0.z, 0u, 0x9991u);
+        s.k[6] = prmt(d0.z, 0u, 0xAAA2u);
+    }
+    return s;
+}
+
+// Bytes L + Lmax + bias of four copies from their neighbour words a[], own word V and its
+// sign mask (0xFF in the bytes of -1 spins).
+template <int DC>
+__device__ __forceinline__ uint32_t site_index(const SiteTerms<DC>& s, const uint32_t* a, uint32_t V, uint32_t kM) {
+    uint32_t f;
+    if constexpr (DC == 4) {
+        f = s.c4;
+#pragma unroll
+        for (int d = 0; d < DC - 1; ++d) f += s.k[d] * a[d];
+    } else {
+        uint32_t g = s.k[0] * a[0];
+#pragma unroll
+        for (int d = 1; d < DC - 1; ++d) g += s.k[d] * a[d];
+        f = s.c4 + (0u - kInv127) * g;
+    }
+    const uint32_t m = prmt(V, 0u, 0xBA98u);  // every byte's sign, repeated
+    return (f ^ m) + kM * m;
+}
+
+// u.s8 x s.s8 dot product of four bytes: the flip masks' bytes are 0xFE, -2 as signed.
+__device__ __forceinline__ int dp4a_us(uint32_t a, uint32_t b, int c) {
+    int d;
+    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+// The attempt with random word u is accepted against threshold th: u < th, and always for
+// the entry 0xFFFFFFFF, for which inline words (PRE = false) are first capped at 2^32 - 2
+// (produced words already are).
 template <bool PRE>
-__device__ __forceinline__ uint32_t unit_flips(const UnitEval& e, const uint32_t* thr_c) {
-    uint32_t F = 0;
+__device__ __forceinline__ bool accepts(uint32_t u, uint32_t th) {
+    if (!PRE) u = min(u, 0xFFFFFFFEu);
+    return u < th;
+}
+
+// How one launch or problem finds its table entries (see IndexRule). The Trotter differences
+// are taken at the mask's bit, so D counts kUnit per neighbour that differs.
+template <bool WIDE>
+struct UnitRule {
+    static constexpr uint32_t kMask = WIDE ? 0x40404040u : 0x02020202u;
+    static constexpr int kUnit = WIDE ? 64 : 2;
+    uint32_t kM;  // site_index's mirror multiplier
+    uint32_t sD;  // entries (narrow) or bytes (wide) of a column's stride, per unit of D
+    int zero;     // the index byte of L = 0
+    __device__ __forceinline__ explicit UnitRule(int Lmax) {
+        const IndexRule r(Lmax);
+        kM = r.kM;
+        zero = r.zero();
+        sD = WIDE ? (uint32_t)r.S / 16u : (uint32_t)r.S / 2u;
+    }
+};
+
+// 0xFE in byte w when copy w flips: L = biased L bytes, D = Trotter differences, thr = byte
+// offset in shared memory of the threshold row (wide: of its last column).
+template <bool PRE, bool WIDE>
+__device__ __forceinline__ uint32_t flips4(const unsigned char* smem, const UnitRule<WIDE>& rule, uint32_t L,
+                                           uint32_t D, const uint32_t* u, uint32_t thr) {
+    uint32_t off[4];
+    if constexpr (!WIDE) {
+        const uint32_t idx = L - rule.sD * D;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) off[w] = __dp4a(idx, 4u << (8 * w), thr);
+    } else {
+        const uint32_t m = 0u - rule.sD;  // -S / 16 as a signed byte
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+            off[w] = __dp4a(L, 4u << (8 * w), (uint32_t)dp4a_us(D, (m & 0xFFu) << (8 * w), (int)thr));
+    }
+    uint32_t F = 0u;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-        F -= accept_mask<PRE>(e.u[w], thr_entry(thr_c, e.Z, e.L[w], w)) * (0xFEu << (8 * w));
+        const uint32_t th = *reinterpret_cast<const uint32_t*>(smem + off[w]);
+        if (accepts<PRE>(u[w], th)) F |= 0xFEu << (8 * w);
     }
     return F;
 }
-
-// sumC2 and nflip2 count twice the Trotter columns and the flips: the flip mask bytes
-// (F & 0x02020202 = 2 per flip) feed dp4a directly.
-__device__ __forceinline__ void unit_commit(const UnitEval& e, uint32_t F, int& sumL, int& sumC2, int& nflip2) {
-#pragma unroll
-    for (int w = 0; w < 4; ++w) sumL += ((F >> (8 * w)) & 0x2u) ? e.L[w] : 0;
-    const uint32_t Fm = F & 0x02020202u;
-    nflip2 = __dp4a((int)Fm, 0x01010101, nflip2);
-    sumC2 = __dp4a((int)e.Z, (int)Fm, sumC2);
-    if (F) *e.own = e.S ^ F;
+// The row offset flips4 takes for a row that starts at byte `row`.
+template <bool WIDE>
+__device__ __forceinline__ uint32_t thr_base(uint32_t row, int Lmax) {
+    return WIDE ? row + 8u * (uint32_t)IndexRule(Lmax).S : row;
 }
 
-template <int DC, bool PRE, typename Key = PhiloxKey>
-__device__ __forceinline__ void packed_unit(int8_t* sp, const uint32_t* s_sdesc, uint32_t item, const uint4* rb,
-                                            int q, int g, int G, int P, uint32_t t, uint32_t slot,
-                                            const Key& key, const uint32_t* thr_c, int& sumL, int& sumC2,
-                                            int& nflip2) {
-    const UnitEval e = packed_unit_eval<DC, PRE, Key>(sp, s_sdesc, item, rb, q, g, G, P, t, slot, key);
-    // flips and sums in one pass (the acceptance predicate feeds both)
-    uint32_t F = 0;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        const uint32_t m = accept_mask<PRE>(e.u[w], thr_entry(thr_c, e.Z, e.L[w], w));
-        F -= m * (0xFEu << (8 * w));
-        sumL -= (int)m * e.L[w];
+// Sums of a sweep over the flipped copies, each times -2: flips, biased L bytes, D.
+struct FlipSums {
+    int n, L, D;
+    __device__ __forceinline__ void clear() { n = L = D = 0; }
+    __device__ __forceinline__ void add4(uint32_t F, uint32_t Lb, uint32_t Db) {
+        n = dp4a_us(0x01010101u, F, n);
+        L = dp4a_us(Lb, F, L);
+        D = dp4a_us(Db, F, D);
     }
-    const uint32_t Fm = F & 0x02020202u;
-    nflip2 = __dp4a((int)Fm, 0x01010101, nflip2);
-    sumC2 = __dp4a((int)e.Z, (int)Fm, sumC2);
-    if (F) *e.own = e.S ^ F;
-}
-
-// Byte offsets, within a shared-memory row, of what a unit of one fixed column reads: its
-// own word, the opposite-parity word at the same copies, and the one Trotter neighbour
-// outside that word. [0] for an even-copy unit, [1] for an odd one. Used by the split
-// kernel, whose rows also hold copies of the neighbouring CTA.
-struct UnitOffsets {
-    uint32_t own[2], opp[2], edge[2];
+    __device__ __forceinline__ void add(const FlipSums& o) {
+        n += o.n;
+        L += o.L;
+        D += o.D;
+    }
+    // the changes the flips make: E by -2 sum L, M by -2 sum m with m = 2 - (neighbours that differ) * 2
+    template <bool WIDE>
+    __device__ __forceinline__ int dE(const UnitRule<WIDE>& r) const { return L - r.zero * n; }
+    template <bool WIDE>
+    __device__ __forceinline__ int dM(const UnitRule<WIDE>&) const { return 2 * n - D / (UnitRule<WIDE>::kUnit / 2); }
+    __device__ __forceinline__ int flips() const { return -n / 2; }
 };
 
-// The packed unit evaluated from precomputed row offsets (the split kernel's rows). PRE: the
-// random words are read from *rbq; else word w of philox((t, i, slot, p<<24 | gg)), gg the
-// unit's 8-copy chunk in the whole chain.
-template <int DC, bool PRE>
-__device__ __forceinline__ UnitEval split_unit_eval(int8_t* sp, const uint32_t* s_sdesc, uint32_t item,
-                                                    const uint4* rbq, const UnitOffsets& o, uint32_t t,
-                                                    uint32_t slot, uint32_t gg, const PhiloxKey& key) {
-    UnitEval e;
-    const uint32_t par = item & 1u;
-    const uint32_t* desc = s_sdesc + (item >> 1) * SiteDesc<DC>::DW;
-    const uint4 d0 = *reinterpret_cast<const uint4*>(desc);
-    uint32_t nrow[DC];
-    uint32_t jpack[DC / 4];
-    {
-        const uint4 d1 = *reinterpret_cast<const uint4*>(desc + 4);
-        nrow[0] = d1.x;
-        nrow[1] = d1.y;
-        nrow[2] = d1.z;
-        nrow[3] = d1.w;
-        jpack[0] = d0.z;
-        if (DC == 8) {
-            const uint4 d2 = *reinterpret_cast<const uint4*>(desc + 8);
-            nrow[DC > 4 ? 4 : 0] = d2.x;
-            nrow[DC > 5 ? 5 : 0] = d2.y;
-            nrow[DC > 6 ? 6 : 0] = d2.z;
-            nrow[DC > 7 ? 7 : 0] = d2.w;
-            jpack[DC > 4 ? 1 : 0] = d0.w;
-        }
+// Byte offsets, within a shared-memory row, of what a unit of one fixed column reads: its
+// own words, the opposite-parity words at the same copies, and the one Trotter neighbour
+// outside those. [0] for an even-copy unit, [1] for an odd one.
+struct UnitOffsets {
+    uint32_t own[2], opp[2], edge[2];
+    __device__ __forceinline__ uint32_t own_of(uint32_t par) const { return own[0] + par * (own[1] - own[0]); }
+    __device__ __forceinline__ uint32_t opp_of(uint32_t par) const { return opp[0] + par * (opp[1] - opp[0]); }
+    __device__ __forceinline__ uint32_t edge_of(uint32_t par) const { return edge[0] + par * (edge[1] - edge[0]); }
+};
+
+// W consecutive words at an address aligned to 4 W bytes, in one access.
+template <int W>
+__device__ __forceinline__ void load_words(const int8_t* p, uint32_t* v) {
+    if constexpr (W == 1) {
+        v[0] = *reinterpret_cast<const uint32_t*>(p);
+    } else if constexpr (W == 2) {
+        const uint2 x = *reinterpret_cast<const uint2*>(p);
+        v[0] = x.x;
+        v[1] = x.y;
+    } else {
+        const uint4 x = *reinterpret_cast<const uint4*>(p);
+        v[0] = x.x;
+        v[1] = x.y;
+        v[2] = x.z;
+        v[3] = x.w;
     }
-    const uint32_t row = d0.x;
-    const uint32_t own_off = o.own[0] + par * (o.own[1] - o.own[0]);
-    e.own = reinterpret_cast<uint32_t*>(sp + row + own_off);
-    const uint32_t S = *e.own;
-    const uint32_t O = *reinterpret_cast<const uint32_t*>(sp + row + o.opp[0] + par * (o.opp[1] - o.opp[0]));
-    const uint32_t edge = (uint8_t)sp[row + o.edge[0] + par * (o.edge[1] - o.edge[0])];
-    uint32_t a[DC];
+}
+template <int W>
+__device__ __forceinline__ void store_words(int8_t* p, const uint32_t* v) {
+    if constexpr (W == 1)
+        *reinterpret_cast<uint32_t*>(p) = v[0];
+    else if constexpr (W == 2)
+        *reinterpret_cast<uint2*>(p) = make_uint2(v[0], v[1]);
+    else
+        *reinterpret_cast<uint4*>(p) = make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+// The unit in three steps, so that a unit can be evaluated before the threshold row it needs
+// is known: evaluate (loads, index bytes, random words), decide the flips against one
+// threshold row, commit (flip store and the sweep's sums).
+template <int W>
+struct UnitEval {
+    int8_t* own;        // the unit's words in shared memory
+    uint32_t V[W];      // its copies as +-1 bytes
+    uint32_t L[W];      // biased L bytes
+    uint32_t D[W];      // Trotter differences
+    uint32_t u[4 * W];  // random words
+};
+
+// The Trotter differences of a unit's words V with opposite-parity words O: their left and
+// right neighbours are O itself and O shifted by one copy with the edge copy coming in (at
+// the low end for even copies, at the high end for odd ones).
+template <int W, bool WIDE>
+__device__ __forceinline__ void trotter_differences(const uint32_t* V, const uint32_t* O, uint32_t edge, uint32_t par,
+                                                    uint32_t* D, uint32_t last_odd_sel = 0x4321u) {
+    constexpr uint32_t mask = UnitRule<WIDE>::kMask;
 #pragma unroll
-    for (int d = 0; d < DC; ++d) a[d] = *reinterpret_cast<const uint32_t*>(sp + nrow[d] + own_off);
-    const uint4 r4 = PRE ? *rbq : philox(make_uint4(t, d0.y, slot, (par << 24) | gg), key);
-    e.u[0] = r4.x;
-    e.u[1] = r4.y;
-    e.u[2] = r4.z;
-    e.u[3] = r4.w;
-    const uint32_t Ln = __byte_perm(O, edge, 0x2104u + par * (0x3210u - 0x2104u));
-    const uint32_t Rn = __byte_perm(O, edge, 0x3210u + par * (0x4321u - 0x3210u));
-    const uint32_t X = (S ^ Ln) & 0x02020202u;
-    const uint32_t Y = (S ^ Rn) & 0x02020202u;
-    e.Z = 0x02020202u - ((X + Y) >> 1);
-    e.S = S;
-    field_times_spin<DC>(a, S, jpack, e.L);
+    for (int x = 0; x < W; ++x) {
+        const uint32_t lo = x == 0 ? edge : O[x > 0 ? x - 1 : 0], hi = x == W - 1 ? edge : O[x < W - 1 ? x + 1 : x];
+        const uint32_t even_sel = x == 0 ? 0x2104u : 0x2107u;
+        const uint32_t odd_sel = x == W - 1 ? last_odd_sel : 0x4321u;
+        const uint32_t in = (W == 1) ? edge : (par ? hi : lo);
+        const uint32_t sh = prmt(O[x], in, even_sel + par * (odd_sel - even_sel));
+        D[x] = ((V[x] ^ O[x]) & mask) + ((V[x] ^ sh) & mask);
+    }
+}
+
+// Random words of a unit: read from rbq[0 .. W-1] (PRE), else word w of philox((t, i, slot,
+// par<<24 | gg + x)) for word x, gg the unit's first 8-copy chunk in the whole chain.
+template <int W, bool PRE, typename Key>
+__device__ __forceinline__ void unit_words(uint32_t* u, uint32_t item, const uint4* rbq, uint32_t t, uint32_t slot,
+                                           uint32_t gg, const Key& key) {
+#pragma unroll
+    for (int x = 0; x < W; ++x) {
+        const uint4 r =
+            PRE ? rbq[x] : philox(make_uint4(t, item >> 1, slot, ((item & 1u) << 24) | (gg + (uint32_t)x)), key);
+        u[4 * x + 0] = r.x;
+        u[4 * x + 1] = r.y;
+        u[4 * x + 2] = r.z;
+        u[4 * x + 3] = r.w;
+    }
+}
+
+// The unit's spins, index bytes and Trotter differences, from its site's terms.
+template <int DC, int W, bool WIDE>
+__device__ __forceinline__ void unit_eval_site(UnitEval<W>& e, int8_t* sp, const SiteTerms<DC>& s, uint32_t par,
+                                               const UnitOffsets& o, const UnitRule<WIDE>& rule) {
+    const uint32_t own_off = o.own_of(par);
+    const uint32_t edge = (uint8_t)sp[s.row + o.edge_of(par)];
+    e.own = sp + s.row + own_off;
+    uint32_t O[W], a[DC - 1][W];
+    load_words<W>(e.own, e.V);
+    load_words<W>(sp + s.row + o.opp_of(par), O);
+#pragma unroll
+    for (int d = 0; d < DC - 1; ++d) load_words<W>(sp + s.off[d] + own_off, a[d]);
+    trotter_differences<W, WIDE>(e.V, O, edge, par, e.D);
+#pragma unroll
+    for (int x = 0; x < W; ++x) {
+        uint32_t ax[DC - 1];
+#pragma unroll
+        for (int d = 0; d < DC - 1; ++d) ax[d] = a[d][x];
+        e.L[x] = site_index<DC>(s, ax, e.V[x], rule.kM);
+    }
+}
+
+template <int DC, int W, bool PRE, bool WIDE, typename Key = PhiloxKey>
+__device__ __forceinline__ UnitEval<W> unit_eval(int8_t* sp, const uint32_t* s_sdesc, uint32_t item,
+                                                 const UnitOffsets& o, const uint4* rbq, uint32_t t, uint32_t slot,
+                                                 uint32_t gg, const UnitRule<WIDE>& rule, const Key& key) {
+    UnitEval<W> e;
+    const SiteTerms<DC> s = load_site<DC>(s_sdesc + (item >> 1) * SiteDesc<DC>::DW);
+    unit_words<W, PRE>(e.u, item, rbq, t, slot, gg, key);
+    unit_eval_site<DC, W, WIDE>(e, sp, s, item & 1u, o, rule);
     return e;
 }
 
-// Decide and commit in one pass (PRE: produced words, u < thr alone is the rule).
-template <bool PRE>
-__device__ __forceinline__ void unit_decide_commit(const UnitEval& e, const uint32_t* thr_c, int& sumL, int& sumC2,
-                                                   int& nflip2) {
-    uint32_t F = 0;
+template <int W, bool PRE, bool WIDE>
+__device__ __forceinline__ void unit_flips(const UnitEval<W>& e, const unsigned char* smem, const UnitRule<WIDE>& rule,
+                                           uint32_t thr, uint32_t* F) {
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        const uint32_t m = accept_mask<PRE>(e.u[w], thr_entry(thr_c, e.Z, e.L[w], w));
-        F -= m * (0xFEu << (8 * w));
-        sumL -= (int)m * e.L[w];
-    }
-    const uint32_t Fm = F & 0x02020202u;
-    nflip2 = __dp4a((int)Fm, 0x01010101, nflip2);
-    sumC2 = __dp4a((int)e.Z, (int)Fm, sumC2);
-    if (F) *e.own = e.S ^ F;
+    for (int x = 0; x < W; ++x) F[x] = flips4<PRE, WIDE>(smem, rule, e.L[x], e.D[x], e.u + 4 * x, thr);
 }
 
-}  // namespace ptq
+template <int W>
+__device__ __forceinline__ void unit_commit(const UnitEval<W>& e, const uint32_t* F, FlipSums& sums) {
+    uint32_t any = 0u, v[W];
+#pragma unroll
+    for (int x = 0; x < W; ++x) {
+        sums.add4(F[x], e.L[x], e.D[x]);
+        any |= F[x];
+        v[x] = e.V[x] ^ F[x];  // a +-1 byte flips by an exclusive-or with 0xFE
+    }
+    if (any) store_words<W>(e.own, v);
+}
 
-namespace ptq {
+// Row offsets of column u of a one-CTA chain (half = P / 2 bytes a parity).
+template <int W>
+__device__ __forceinline__ UnitOffsets row_offsets(uint32_t u, uint32_t half) {
+    const uint32_t b = 4u * W * u;
+    UnitOffsets o;
+    o.own[0] = b;
+    o.own[1] = half + b;
+    o.opp[0] = half + b;
+    o.opp[1] = b;
+    o.edge[0] = half + (u == 0 ? half - 1u : b - 1u);
+    o.edge[1] = b + 4u * W == half ? 0u : b + 4u * W;
+    return o;
+}
 
-// Bit-packed chains (shared memory only): row i is P/8 bytes, bit k of byte g is copy 8g+k,
+// ------------------------------------------------------------------------- any even P, any degree
+// The same unit (W = 1) for the shapes the classes above leave out: P not a multiple of 8, or
+// more than seven neighbours. Each parity's half of a row is padded to whole words (G words;
+// pad bytes hold +1 and never flip) and a site lists its neighbours' (row offset, multiplier)
+// pairs, padded to a multiple of four, so the neighbour loop runs to the site's own degree.
+// Descriptor of a site: C4, own row offset, neighbour slots in use, 0 | off, k, off, k | ...
+__host__ __device__ inline int rows_desc_words(int slots) { return 4 + 2 * slots; }
+
+struct RowsColumn {
+    UnitOffsets o;
+    uint32_t odd_sel;  // where the edge copy enters an odd unit's last word
+    uint32_t live;     // mask of the bytes that are copies
+};
+__device__ __forceinline__ RowsColumn rows_column(uint32_t g, uint32_t G, uint32_t n_par) {
+    RowsColumn c;
+    const uint32_t half = 4u * G, b = 4u * g;
+    c.o.own[0] = b;
+    c.o.own[1] = half + b;
+    c.o.opp[0] = half + b;
+    c.o.opp[1] = b;
+    c.o.edge[0] = half + (g == 0 ? n_par - 1u : b - 1u);
+    c.o.edge[1] = g + 1u == G ? 0u : b + 4u;
+    const uint32_t r = g + 1u == G ? n_par - 4u * (G - 1u) : 4u;  // copies in this word, 1..4
+    c.odd_sel = r == 4u ? 0x4321u : (r == 3u ? 0x4421u : (r == 2u ? 0x4441u : 0x4444u));
+    c.live = 0xFFFFFFFFu >> (8u * (4u - r));
+    return c;
+}
+
+// What a unit of that form needs of its site: the header, the first four neighbours, and
+// where the others are listed.
+struct RowsTerms {
+    uint4 head, n0, n1;
+    const uint32_t* rest;
+};
+__device__ __forceinline__ RowsTerms load_rows_site(const uint32_t* desc) {
+    RowsTerms s;
+    s.head = *reinterpret_cast<const uint4*>(desc);
+    s.n0 = *reinterpret_cast<const uint4*>(desc + 4);
+    s.n1 = *reinterpret_cast<const uint4*>(desc + 8);
+    s.rest = desc + 12;
+    return s;
+}
+
+template <bool WIDE>
+__device__ __forceinline__ void rows_eval_site(UnitEval<1>& e, int8_t* sp, const RowsTerms& s, uint32_t par,
+                                               const RowsColumn& c, const UnitRule<WIDE>& rule) {
+    const uint32_t own_off = c.o.own_of(par);
+    const uint32_t edge = (uint8_t)sp[s.head.y + c.o.edge_of(par)];
+    e.own = sp + s.head.y + own_off;
+    uint32_t O[1], a[4], f = s.head.x;
+    load_words<1>(e.own, e.V);
+    load_words<1>(sp + s.head.y + c.o.opp_of(par), O);
+    load_words<1>(sp + s.n0.x + own_off, a);
+    load_words<1>(sp + s.n0.z + own_off, a + 1);
+    load_words<1>(sp + s.n1.x + own_off, a + 2);
+    load_words<1>(sp + s.n1.z + own_off, a + 3);
+    f += s.n0.y * a[0] + s.n0.w * a[1] + s.n1.y * a[2] + s.n1.w * a[3];
+#pragma unroll 2
+    for (uint32_t d = 4; d < s.head.z; d += 4) {
+        const uint4 p0 = *reinterpret_cast<const uint4*>(s.rest + 2 * d - 8);
+        const uint4 p1 = *reinterpret_cast<const uint4*>(s.rest + 2 * d - 4);
+        load_words<1>(sp + p0.x + own_off, a);
+        load_words<1>(sp + p0.z + own_off, a + 1);
+        load_words<1>(sp + p1.x + own_off, a + 2);
+        load_words<1>(sp + p1.z + own_off, a + 3);
+        f += p0.y * a[0] + p0.w * a[1] + p1.y * a[2] + p1.w * a[3];
+    }
+    trotter_differences<1, WIDE>(e.V, O, edge, par, e.D, c.odd_sel);
+    const uint32_t m = prmt(e.V[0], 0u, 0xBA98u);
+    e.L[0] = (f ^ m) + rule.kM * m;
+}
+
+// ------------------------------------------------------------------------- one copy a thread
+// For chains whose levels hold no more copies than a CTA has threads: a level then costs the
+// latency of one update, about 4.7 cycles per instruction of the thread that runs it, so a
+// thread takes one copy (about 40 instructions against about 95 for the four-copy unit).
+// Rows and descriptors are those of the word-wise form above, with J and h themselves.
+struct CopyEval {
+    int8_t* own;
+    int s, L, m;  // spin, s (h + sum_j J_j s_j), s (left + right)
+    uint32_t u;   // random word
+};
+struct CopySums {
+    int n, L, M;  // over flipped copies: count, sum of L, sum of m
+};
+__device__ __forceinline__ UnitOffsets copy_offsets(uint32_t h, uint32_t half, uint32_t n_par) {
+    UnitOffsets o;
+    o.own[0] = h;
+    o.own[1] = half + h;
+    o.opp[0] = half + h;
+    o.opp[1] = h;
+    o.edge[0] = half + (h == 0u ? n_par - 1u : h - 1u);
+    o.edge[1] = h + 1u == n_par ? 0u : h + 1u;
+    return o;
+}
+__device__ __forceinline__ CopyEval copy_eval(int8_t* sp, const uint32_t* desc, uint32_t par, const UnitOffsets& o,
+                                              uint32_t word) {
+    CopyEval e;
+    const RowsTerms t = load_rows_site(desc);
+    const uint32_t own_off = o.own_of(par);
+    e.own = sp + t.head.y + own_off;
+    e.s = *e.own;
+    const int nn = sp[t.head.y + o.opp_of(par)] + sp[t.head.y + o.edge_of(par)];
+    int f = (int)t.head.x;
+    f += (int)t.n0.y * sp[t.n0.x + own_off] + (int)t.n0.w * sp[t.n0.z + own_off];
+    f += (int)t.n1.y * sp[t.n1.x + own_off] + (int)t.n1.w * sp[t.n1.z + own_off];
+#pragma unroll 2
+    for (uint32_t d = 4; d < t.head.z; d += 4) {
+        const uint4 p0 = *reinterpret_cast<const uint4*>(t.rest + 2 * d - 8);
+        const uint4 p1 = *reinterpret_cast<const uint4*>(t.rest + 2 * d - 4);
+        f += (int)p0.y * sp[p0.x + own_off] + (int)p0.w * sp[p0.z + own_off];
+        f += (int)p1.y * sp[p1.x + own_off] + (int)p1.w * sp[p1.z + own_off];
+    }
+    e.L = e.s * f;
+    e.m = e.s * nn;
+    e.u = word;
+    return e;
+}
+// thr: byte offset of the entry L = 0, m = 0; S: entries of a column.
+__device__ __forceinline__ bool copy_flips(const CopyEval& e, const unsigned char* smem, int thr, int S) {
+    return e.u < *reinterpret_cast<const uint32_t*>(smem + (thr + 4 * e.L + 2 * S * e.m));
+}
+__device__ __forceinline__ void copy_commit(const CopyEval& e, bool flip, CopySums& sums) {
+    if (flip) {
+        *e.own = (int8_t)(-e.s);
+        sums.n += 1;
+        sums.L += e.L;
+        sums.M += e.m;
+    }
+}
+
+// Bit-packed chains (shared memory only), one bit a copy: row i is P/8 bytes, bit k of byte g is copy 8g+k,
 // set = spin -1. lut[p*256 + b] spreads the four parity-p bits (p, p+2, p+4, p+6) of byte b
 // into four +1/-1 bytes, so each neighbour contributes one byte load and one table load and
-// the field / Trotter logic of packed_unit is reused unchanged.
-template <int DC, bool PRE>
+// the index arithmetic of the int8 unit is reused unchanged.
+template <int DC, bool WIDE>
 __device__ __forceinline__ void packed_unit_bits(uint8_t* bp, const uint32_t* s_sdesc, uint32_t item,
-                                                 const uint4* rb, int q, int g, int G, const uint32_t* lut,
+                                                 int g, int G, const uint32_t* lut,
                                                  uint32_t t, uint32_t slot, const PhiloxKey& key,
-                                                 const uint32_t* thr_c, int& sumL, int& sumC2, int& nflip2) {
+                                                 const unsigned char* smem, const UnitRule<WIDE>& rule, uint32_t thr,
+                                                 FlipSums& sums) {
     const uint32_t par = item & 1u;
-    const uint32_t* desc = s_sdesc + (item >> 1) * SiteDesc<DC>::DW;
-    const uint4 d0 = *reinterpret_cast<const uint4*>(desc);
-    const uint32_t row = d0.x;
-    uint32_t nrow[DC];
-    uint32_t jpack[DC / 4];
-    {
-        const uint4 d1 = *reinterpret_cast<const uint4*>(desc + 4);
-        nrow[0] = d1.x;
-        nrow[1] = d1.y;
-        nrow[2] = d1.z;
-        nrow[3] = d1.w;
-        jpack[0] = d0.z;
-        if (DC == 8) {
-            const uint4 d2 = *reinterpret_cast<const uint4*>(desc + 8);
-            nrow[DC > 4 ? 4 : 0] = d2.x;
-            nrow[DC > 5 ? 5 : 0] = d2.y;
-            nrow[DC > 6 ? 6 : 0] = d2.z;
-            nrow[DC > 7 ? 7 : 0] = d2.w;
-            jpack[DC > 4 ? 1 : 0] = d0.w;
-        }
-    }
+    const SiteTerms<DC> s = load_site<DC>(s_sdesc + (item >> 1) * SiteDesc<DC>::DW);
     const uint32_t ug = (uint32_t)g, last = (uint32_t)G - 1u;
-    const uint32_t own = bp[row + ug];
+    const uint32_t own = bp[s.row + ug];
     // the one Trotter neighbour outside the byte: copy 8g-1 (bit 7 of byte g-1) for even
     // copies, copy 8g+8 (bit 0 of byte g+1) for odd ones, periodic in the row
-    const uint32_t eb = par ? (bp[row + (ug == last ? 0u : ug + 1u)] & 1u)
-                            : ((uint32_t)bp[row + (ug == 0 ? last : ug - 1u)] >> 7);
+    const uint32_t eb = par ? (bp[s.row + (ug == last ? 0u : ug + 1u)] & 1u)
+                            : ((uint32_t)bp[s.row + (ug == 0 ? last : ug - 1u)] >> 7);
     const uint32_t* lut_p = lut + (par << 8);
-    uint32_t nbyte[DC];
+    uint32_t nbyte[DC - 1];
 #pragma unroll
-    for (int d = 0; d < DC; ++d) nbyte[d] = bp[nrow[d] + ug];
-    uint4 r4;
-    if (PRE) {
-        r4 = rb[q * G + g];
-    } else {
-        r4 = philox(make_uint4(t, d0.y, slot, (par << 24) | (uint32_t)g), key);
-    }
-    const uint32_t u[4] = {r4.x, r4.y, r4.z, r4.w};
-    const uint32_t S = lut_p[own];
+    for (int d = 0; d < DC - 1; ++d) nbyte[d] = bp[s.off[d] + ug];
+    uint32_t u[4];
+    unit_words<1, false>(u, item, nullptr, t, slot, ug, key);
+    const uint32_t V = lut_p[own];
     const uint32_t Rn = par ? lut[256 + (((own >> 1) | (eb << 7)) & 0xFFu)] : lut[256 + own];
     const uint32_t Ln = par ? lut[own] : lut[((own << 1) | eb) & 0xFFu];
-    const uint32_t X = (S ^ Ln) & 0x02020202u;
-    const uint32_t Y = (S ^ Rn) & 0x02020202u;
-    const uint32_t Z = 0x02020202u - ((X + Y) >> 1);
+    const uint32_t D = ((V ^ Ln) & UnitRule<WIDE>::kMask) + ((V ^ Rn) & UnitRule<WIDE>::kMask);
+    uint32_t a[DC - 1];
+#pragma unroll
+    for (int d = 0; d < DC - 1; ++d) a[d] = lut_p[nbyte[d]];
+    const uint32_t L = site_index<DC>(s, a, V, rule.kM);
+    const uint32_t F = flips4<false, WIDE>(smem, rule, L, D, u, thr);
+    sums.add4(F, L, D);
+    // bits 0, 2, 4, 6 from bytes 0..3
+    const uint32_t f1 = (F >> 1) & 0x01010101u, fb = f1 | (f1 >> 6);
+    if (F) bp[s.row + ug] = (uint8_t)(own ^ (((fb | (fb >> 12)) & 0x55u) << par));
+}
 
-    uint32_t a[DC];
+// Bit-packed chains, one nibble of every byte: a word holds 16 copies of one parity of a site,
+// unit k (of four) as bit k of its four bytes, so that copy 16 c + 4 k + w of that parity is
+// bit 8 w + k of word c; a row is P/32 even words, then P/32 odd ones. A thread takes a whole
+// word: one load per neighbour, one descriptor and one address serve 16 copies, and no other
+// thread writes its word. The one-bit form above costs a byte load and a table load per
+// neighbour and four copies; this one an AND and a multiply-add. The arithmetic is the int8
+// unit's with 0 / 1 bytes: sum_j J_j B_j of unit k comes from the words masked at bit k, that
+// is scaled by 2^k, and is shifted down once the sum is formed. Every byte has to hold
+// 2^k 2 Lmax until then: k <= 2 for Lmax <= 31 (kNibbleLmax), and unit 3 starts from words
+// shifted by 3. Descriptors hold J itself and C4 = h + sum J + Lmax in every byte ("plain").
+// With the Trotter column taken as the count of equal neighbours no index bias is needed.
+struct NibbleSums {
+    int n, L, C;  // minus the sums over flipped copies of 1, L + Lmax and the Trotter column
+};
+template <int DC, int NS>
+__device__ __forceinline__ void nibble_unit(int8_t* sp, const uint32_t* s_sdesc, uint32_t item, uint32_t c,
+                                            uint32_t cols, uint32_t t, uint32_t slot, const PhiloxKey& key,
+                                            const unsigned char* smem, uint32_t S, uint32_t kM, uint32_t thr,
+                                            NibbleSums& sums) {
+    const uint32_t par = item & 1u;
+    const SiteTerms<DC> s = load_site<DC>(s_sdesc + (item >> 1) * SiteDesc<DC>::DW);
+    const uint32_t own_off = 4u * (par * cols + c), opp = s.row + 4u * (cols - par * cols);
+    // the word the opposite parity's edge copy is in: the one before for even copies, after for odd
+    const uint32_t ce = par ? (c + 1u == cols ? 0u : c + 1u) : (c == 0u ? cols - 1u : c - 1u);
+    uint32_t* own = reinterpret_cast<uint32_t*>(sp + s.row + own_off);
+    const uint32_t V = *own;
+    const uint32_t O = *reinterpret_cast<const uint32_t*>(sp + opp + 4u * c);
+    const uint32_t E = *reinterpret_cast<const uint32_t*>(sp + opp + 4u * ce);
+    uint32_t W[NS];
 #pragma unroll
-    for (int d = 0; d < DC; ++d) a[d] = lut_p[nbyte[d]];
-    int L[4];
-    field_times_spin<DC>(a, S, jpack, L);
-    uint32_t F = 0, flipbits = 0;
+    for (int d = 0; d < NS; ++d) W[d] = *reinterpret_cast<const uint32_t*>(sp + s.off[d] + own_off);
+    uint32_t u[16];
+    unit_words<4, false>(u, item, nullptr, t, slot, 4u * c, key);
+    // the opposite parity shifted by one copy: bytes up (even copies) or down (odd copies) by
+    // one, and the byte that comes in from the next unit, its top one from the edge word
+    // (bits above the nibble are never looked at)
+    const uint32_t in = par ? (O >> 1) | (E << 3) : (O >> 23) | (E >> 27);
+    const uint32_t sh = prmt(O, in, 0x2104u + par * (0x4321u - 0x2104u));
+    uint32_t flip = 0u;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        const uint32_t m = accept_mask<PRE>(u[w], thr_entry(thr_c, Z, L[w], w));
-        F -= m * (0xFEu << (8 * w));
-        flipbits -= m * (1u << (2 * w));
-        sumL -= (int)m * L[w];
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t mk = 0x01010101u << k;
+        const int ks = k == 3 ? 0 : k;  // the scale of this unit's sum
+        uint32_t g = 0u;
+#pragma unroll
+        for (int d = 0; d < NS; ++d) g += s.k[d] * ((k == 3 ? W[d] >> 3 : W[d]) & (0x01010101u << ks));
+        const uint32_t f = ((s.c4 << ks) - 2u * g) >> ks;
+        const uint32_t m = (uint32_t)((int)((V & mk) * 255u) >> k);  // 0xFF where the spin is -1
+        const uint32_t L = (f ^ m) + kM * m;
+        const uint32_t C = ((~(V ^ O) & mk) + (~(V ^ sh) & mk)) >> k;
+        const uint32_t idx = L + S * C;
+        uint32_t F = 0u;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const uint32_t th = *reinterpret_cast<const uint32_t*>(smem + __dp4a(idx, 4u << (8 * w), thr));
+            if (accepts<false>(u[4 * k + w], th)) F |= 0xFFu << (8 * w);
+        }
+        sums.n = dp4a_us(0x01010101u, F, sums.n);
+        sums.L = dp4a_us(L, F, sums.L);
+        sums.C = dp4a_us(C, F, sums.C);
+        flip |= F & mk;
     }
-    const uint32_t Fm = F & 0x02020202u;
-    nflip2 = __dp4a((int)Fm, 0x01010101, nflip2);
-    sumC2 = __dp4a((int)Z, (int)Fm, sumC2);
-    if (flipbits) bp[row + ug] = (uint8_t)(own ^ (flipbits << par));
+    if (flip) *own = V ^ flip;
 }
 
 }  // namespace ptq

@@ -56,6 +56,7 @@ struct PlanKey {
 struct PlanChoice {
     int path, threads, producers;
     int cluster, group_threads, thr_resident;  // path 7
+    int copy;
 };
 static std::mutex g_plan_mutex;
 static std::map<PlanKey, PlanChoice> g_plan_cache;
@@ -277,32 +278,33 @@ static void drop_odd_updates(std::vector<uint32_t>& items, std::vector<int32_t>&
 }
 
 // ---------------------------------------------------------------------------------
-// Packed-path site descriptors (see SiteDesc in pt_kernels.cu).
+// Packed-path site descriptors (see SiteDesc in pt_device.cuh).
 // P = bytes per chain row: the copy count for int8 chains, copies / 8 for bit-packed ones.
-void ptq::build_site_desc(int N, int P, int dclass, const std::vector<std::vector<int>>& adj,
-                            const std::vector<std::vector<int>>& adjJ, const int32_t* h, std::vector<uint32_t>& desc) {
-    const int DW = dclass == 4 ? 8 : 12;
-    const uint32_t ones_row = (uint32_t)(((size_t)N * P + 15) & ~(size_t)15);
+void ptq::build_site_desc(int N, int P, int dclass, int Lmax, const std::vector<std::vector<int>>& adj,
+                            const std::vector<std::vector<int>>& adjJ, const int32_t* h, std::vector<uint32_t>& desc,
+                            bool plain) {
+    const int DW = dclass == 4 ? 8 : 12, NS = dclass - 1;
+    const uint32_t zero = plain ? (uint32_t)Lmax : (uint32_t)IndexRule(Lmax).zero();
     desc.assign((size_t)N * DW, 0u);
     for (int i = 0; i < N; ++i) {
         uint32_t* d = &desc[(size_t)i * DW];
-        d[0] = (uint32_t)i * (uint32_t)P;
-        d[1] = (uint32_t)i;
-        uint32_t jp[2] = {0u, 0u};
-        for (int s8 = 0; s8 < dclass; ++s8) {
-            int J = 0;
-            uint32_t r = ones_row;
-            if (s8 < (int)adj[i].size()) {
-                J = adjJ[i][s8];
-                r = (uint32_t)adj[i][s8] * (uint32_t)P;
-            } else if (s8 == (int)adj[i].size()) {
-                J = h[i];
+        const uint32_t row = (uint32_t)i * (uint32_t)P;
+        uint32_t sumJ = 0u;
+        for (int s = 0; s < NS; ++s) {
+            const bool used = s < (int)adj[i].size();
+            const int J = used ? adjJ[i][s] : 0;
+            const uint32_t off = used ? (uint32_t)adj[i][s] * (uint32_t)P : row;
+            sumJ += (uint32_t)J;
+            if (dclass == 4) {
+                d[1 + s] = off;
+                d[4 + s] = plain ? (uint32_t)J : (uint32_t)J * (0u - kInv127);
+            } else {
+                d[4 + s] = off;
+                d[1 + (s >> 2)] |= (uint32_t)(uint8_t)(int8_t)J << (8 * (s & 3));
             }
-            d[4 + s8] = r;
-            jp[s8 / 4] |= (uint32_t)(uint8_t)(int8_t)J << (8 * (s8 % 4));
         }
-        d[2] = jp[0];
-        d[3] = jp[1];
+        d[0] = ((uint32_t)h[i] + sumJ + zero + (plain ? 0u : kInv127 * sumJ)) * 0x01010101u;
+        d[dclass == 4 ? 7 : 3] = row;
     }
 }
 
@@ -379,6 +381,7 @@ static BatchInstance chains_instance(const DevProblem& p, const LaunchPlan& plan
     I.group_threads = plan.group_threads;
     I.resident = 1;
     I.thr_resident = plan.thr_resident;
+    I.unit_words = plan.unit_words;
     I.key0 = p.key0;
     I.key1 = p.key1;
     I.t0 = t0;
@@ -411,7 +414,7 @@ static bool chains_plan(const DevProblem& p, int dclass, int cluster, int widen,
         I.group_threads = force_group;
         I.resident = 1;
         I.thr_resident = 1;
-        if (batch_smem_bytes(I, cluster, 512) > cap || (size_t)I.R * ((I.nL3 * 4 + 15) / 16 * 16) > 49152)
+        if (batch_smem_bytes(I, cluster, 512) > cap || (size_t)I.R * ((IndexRule(I.Lmax).row_words() * 4 + 15) / 16 * 16) > 49152)
             I.thr_resident = 0;
     }
     if (!I.resident) return false;
@@ -430,6 +433,7 @@ static bool chains_plan(const DevProblem& p, int dclass, int cluster, int widen,
     pl.cluster = cluster;
     pl.group_threads = I.group_threads;
     pl.thr_resident = I.thr_resident;
+    pl.unit_words = choose_unit_words(I, I.group_threads);
     return true;
 }
 
@@ -604,6 +608,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                            "kernel_path 9 needs R <= 16, threads_per_block 0 or 64..384 and producer_threads a "
                            "multiple of 32 below it (0 = random words inline)");
     }
+    p.slots = rows_slots(p, dmax, (size_t)max_smem);
     int path = want_chains ? kPathPackedInline : want_path;
     const int want_threads = opt ? opt->threads_per_block : 0;
     // path 10's shape for a cluster of about K CTAs: C = the power of two at or above R / K
@@ -628,6 +633,20 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         long long t = (per_level * C + unit - 1) / unit * unit;
         t = std::max<long long>(t, std::max(64, unit));
         return (int)std::min<long long>(t, 512 / unit * unit);
+    };
+    // One copy a thread: consumer threads for the copies of an average level, one thread each,
+    // and producer threads that make a sweep's random words (a quarter as many calls) in its
+    // time. 0 threads when a level is too large for that: beyond 384 copies a thread's second
+    // round costs what the four-copy unit's longer instruction chain does.
+    auto copy_threads = [&](int* producers) {
+        int ccols = 1;
+        while (ccols < P / 2) ccols <<= 1;
+        const long long copies = ((long long)items.size() * ccols + p.n_levels - 1) / p.n_levels;
+        if (P < 2 || p.slots == 0 || copies > 384 || ccols > 256) return 0;
+        const int unit = std::max(32, ccols);
+        const int consumers = std::max(64, (int)((copies + unit - 1) / unit) * unit);
+        *producers = std::min(128, std::max(32, (int)(copies / 3 + 31) / 32 * 32));
+        return consumers + *producers <= 512 ? consumers + *producers : 0;
     };
     // a layout fits if it does with the threshold rows and / or the statistics moved out
     auto fits = [&](int pth) {
@@ -697,7 +716,18 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                 path = kPathBits;
         }
     }
+    if (path == kPathBits) {
+        // the nibble form (twice the shared memory of one bit a copy) when it holds whole words,
+        // its sums fit, and its layout does (with the tables in global memory if need be)
+        DevProblem q = p;
+        q.nibble = 1;
+        q.tables_in_smem = q.acc_in_smem = 0;
+        p.nibble = P % 32 == 0 && Lmax <= kNibbleLmax && want_threads <= 512 &&
+                   sweep_smem_bytes(q, kPathBits, packed_dc) <= (size_t)max_smem;
+        c->plan.nibble = !p.nibble ? 0 : (packed_dc == 4 ? 3 : (dmax <= 6 ? 6 : 7));
+    }
     c->plan.path = path;
+    c->plan.rows = path == kPathGeneric && p.slots > 0;
     c->plan.dclass = (path == kPathGeneric || path == kPathClassical) ? dclass : packed_dc;
     if (path == kPathClassical) {
         // every rung's row and this launch's statistics live in each CTA's shared memory
@@ -713,11 +743,25 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         }
     }
     const bool cl_pre = path == kPathCluster && opt->producer_threads > 0;
+    int copy_producers = 0;
+    if (path == kPathGeneric && want_threads == 0 && copy_threads(&copy_producers) > 0) {
+        // one copy a thread, when its random-word buffers fit too
+        DevProblem q = p;
+        if (copy_smem_bytes(q, false) > (size_t)max_smem) q.tables_in_smem = 0;
+        if (copy_smem_bytes(q, false) > (size_t)max_smem) q.acc_in_smem = 0;
+        if (copy_smem_bytes(q, false) <= (size_t)max_smem) {
+            c->plan.copy = 1;
+            p = q;
+        }
+    }
     if (p.tables_in_smem && sweep_smem_bytes(p, path, c->plan.dclass, cl_pre) > (size_t)max_smem)
         p.tables_in_smem = 0;
     if (p.acc_in_smem && sweep_smem_bytes(p, path, c->plan.dclass, cl_pre) > (size_t)max_smem) p.acc_in_smem = 0;
-    c->plan.smem_bytes = path == kPathClassical ? classical_smem_bytes(p, c->plan.chains_per_cta)
-                                                : sweep_smem_bytes(p, path, c->plan.dclass, cl_pre);
+    auto plan_smem = [&] {
+        if (path == kPathClassical) return classical_smem_bytes(p, c->plan.chains_per_cta);
+        return c->plan.copy ? copy_smem_bytes(p, false) : sweep_smem_bytes(p, path, c->plan.dclass, cl_pre);
+    };
+    c->plan.smem_bytes = plan_smem();
     if ((long long)c->plan.smem_bytes > (long long)max_smem) {
         free_ctx(c);
         return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
@@ -737,9 +781,11 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         c->plan.threads = 128;
     } else if (path == kPathClassical) {
         c->plan.threads = classical_threads(c->plan.chains_per_cta);
+    } else if (path == kPathGeneric && c->plan.copy) {
+        c->plan.threads = copy_threads(&copy_producers);
     } else {
         // enough threads for the average level (units = items * padded groups per parity)
-        int G = ((P / 2) + 3) / 4, Gp = 1;
+        int G = path == kPathBits && p.nibble ? P / 32 : ((P / 2) + 3) / 4, Gp = 1;
         while (Gp < G) Gp <<= 1;
         const long long units = (long long)items.size() * Gp;
         long long avg = (units + p.n_levels - 1) / p.n_levels;
@@ -747,6 +793,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         c->plan.threads = (int)std::min<long long>(512, std::max<long long>(128, avg));
     }
     c->plan.n_consumer = c->plan.threads;
+    if (c->plan.copy) c->plan.n_consumer -= copy_producers;
     if (path == kPathCluster) c->plan.n_consumer = c->plan.threads - opt->producer_threads;
     if (path == kPathPacked || path == kPathSplit) {
         int prod = (opt && opt->producer_threads > 0) ? opt->producer_threads
@@ -776,8 +823,8 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         if (path == kPathSplit || path == kPathSplitInline) {
             cols = P / 16 + 1;
         } else {
-            const int G = (path == kPathGeneric) ? ((P / 2) + 3) / 4 : P / 8;
-            while (cols < G) cols <<= 1;
+            const int G = (path == kPathGeneric) ? ((P / 2) + 3) / 4 : (path == kPathBits && p.nibble ? P / 32 : P / 8);
+            while (cols < (c->plan.copy ? P / 2 : G)) cols <<= 1;
         }
         const int per_round = path == kPathClassical ? c->plan.threads / c->plan.chains_per_cta
                                                      : c->plan.n_consumer / cols;
@@ -785,8 +832,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         if (P == 1) drop_odd_updates(items, level_off);
         p.n_levels = (int)level_off.size() - 1;
         // the level offsets live in shared memory: size it for this schedule's level count
-        c->plan.smem_bytes = path == kPathClassical ? classical_smem_bytes(p, c->plan.chains_per_cta)
-                                                    : sweep_smem_bytes(p, path, c->plan.dclass, cl_pre);
+        c->plan.smem_bytes = plan_smem();
         if ((long long)c->plan.smem_bytes > (long long)max_smem) {
             free_ctx(c);
             return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
@@ -794,12 +840,12 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         }
     }
 
-    // packed-path site descriptors: row offset i*P, i, packed J bytes (two words), then the
-    // row offsets of the neighbour slots; the slot after the last neighbour carries h
-    // against a constant row of +1 copies, the remaining slots have J = 0.
+    // packed-path site descriptors: the field's constant word, the neighbours' multipliers and
+    // row offsets, and the site's own row offset
     std::vector<uint32_t> desc;
-    if (path != kPathGeneric)
-        build_site_desc(N, path == kPathBits ? P / 8 : P, c->plan.dclass, adj, adjJ, inst->h, desc);
+    if (path != kPathGeneric && path != kPathClassical)
+        build_site_desc(N, path == kPathBits ? (p.nibble ? P / 4 : P / 8) : P, c->plan.dclass, Lmax, adj, adjJ, inst->h,
+                        desc, path == kPathBits && p.nibble);
 
     // overflow guard: |E| <= P * (sum|J| + sum|h|), |M| <= N*P; sum of squares stays in int64
     {
@@ -956,6 +1002,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         struct Cand {
             int path, threads, producers;
             int cluster = 1, group_threads = 0;  // path 7; path 10: CTAs and chains per CTA
+            int copy = 0;
         };
         const PlanKey key{N, P, R, packed_dc, p.n_levels, nE};
         std::vector<Cand> cands;
@@ -964,7 +1011,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             auto it = g_plan_cache.find(key);
             if (it != g_plan_cache.end())
                 cands.push_back({it->second.path, it->second.threads, it->second.producers, it->second.cluster,
-                                 it->second.group_threads});
+                                 it->second.group_threads, it->second.copy});
         }
         const bool cached = !cands.empty();
         if (!cached && P == 1) {
@@ -979,7 +1026,13 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                 if (!dup) cands.push_back({kPathClassical, classical_threads(C), 0, ctas, C});
             }
         } else if (!cached) {
-            if (fits(kPathPacked)) cands.push_back({kPathPacked, 512, 128});
+            // small levels: one copy a thread takes the places of the producer-warp plans
+            int cprod = 0;
+            const int cth = copy_threads(&cprod);
+            if (cth > 0)
+                cands.push_back({kPathPacked, cth, cprod, 1, 0, 1});
+            else if (fits(kPathPacked))
+                cands.push_back({kPathPacked, 512, 128});
             if (split_fits()) cands.push_back({kPathSplit, 512, 128});
             if (split_fits(kPathSplitInline))
                 for (int th : {384, 512})
@@ -993,7 +1046,10 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             if (R <= 16)
                 for (int th : {128, 256}) {
                     cands.push_back({kPathCluster, th, 0});
-                    cands.push_back({kPathCluster, th, th / 4});
+                    if (cth > 0 && th == 128)
+                        cands.push_back({kPathCluster, cth, cprod, 1, 0, 1});
+                    else
+                        cands.push_back({kPathCluster, th, th / 4});
                 }
             // every chain resident on one cluster (small problems: swaps never leave the
             // cluster), at the narrowest chain groups that fit and two wider ones
@@ -1036,6 +1092,22 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             }
             pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
             pc.tables_in_smem = (size_t)R * p.nL3 * 4 <= 49152 ? 1 : 0;
+            if (cd.copy) {
+                const bool cl = cd.path == kPathCluster;
+                pl.path = cd.path;
+                pl.dclass = packed_dc;
+                pl.copy = 1;
+                pl.threads = cd.threads;
+                pl.n_consumer = cd.threads - cd.producers;
+                int cols = 1;
+                while (cols < P / 2) cols <<= 1;
+                level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / cols));
+                pc.n_levels = (int)off_c.size() - 1;
+                if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.tables_in_smem = 0;
+                if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.acc_in_smem = 0;
+                pl.smem_bytes = copy_smem_bytes(pc, cl);
+                return pl.smem_bytes <= (size_t)max_smem;
+            }
             const bool cpre = cd.path == kPathCluster && cd.producers > 0;
             if (pc.tables_in_smem && sweep_smem_bytes(pc, cd.path, packed_dc, cpre) > (size_t)max_smem)
                 pc.tables_in_smem = 0;
@@ -1160,7 +1232,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                         std::lock_guard<std::mutex> lock(g_plan_mutex);
                         const Cand& cb = cands[best];
                         g_plan_cache[key] = PlanChoice{cb.path, cb.threads, cb.producers, cb.cluster, cb.group_threads,
-                                                       pl.thr_resident};
+                                                       pl.thr_resident, cb.copy};
                     }
                 }
                 (void)cudaGetLastError();

@@ -29,6 +29,38 @@ struct alignas(16) Mailbox {
 constexpr long long kTagPeriod = 16777215ll;
 constexpr int kClusterMailPasses = 4;  // path 9: swap passes whose mailboxes each CTA holds at once
 
+// Multiplicative inverses modulo 2^32 (Newton's iteration doubles the correct low bits).
+constexpr uint32_t inverse32(uint32_t a) {
+    uint32_t x = a;  // 3 correct bits for odd a
+    for (int k = 0; k < 4; ++k) x *= 2u - a * x;
+    return x;
+}
+constexpr uint32_t kInv127 = inverse32(127u), kInv255 = inverse32(255u);
+static_assert(kInv127 * 127u == 1u && kInv255 * 255u == 1u, "inverses modulo 2^32");
+
+// How the packed kernels index their threshold rows. A row in shared memory holds three
+// columns of S entries, entry col S + (L + Lmax) with col = m/2 + 1 (the public layout
+// [L + Lmax][col] is rearranged when a row is loaded). For Lmax <= 41 the whole entry index
+// fits one byte per copy (at most 6 Lmax + 4 = 250) and is formed for four copies at once;
+// S = 2 Lmax + 2 is even then, because the Trotter differences come doubled. Larger Lmax
+// ("wide") combine L and the column per copy, with S a multiple of 16 so that a column's
+// stride is a byte multiplier.
+struct IndexRule {
+    int Lmax, S, bias;   // bias: added to every byte L + Lmax, so that no column makes it negative
+    bool wide;
+    uint32_t kM;         // x -> 2 Lmax + 2 bias - x for the bytes under a sign mask m: (x ^ m) + kM m
+    __host__ __device__ explicit IndexRule(int Lmax_) : Lmax(Lmax_) {
+        wide = Lmax > 41;
+        S = wide ? (2 * Lmax + 16) / 16 * 16 : 2 * Lmax + 2;
+        bias = wide ? 0 : 2 * S;
+        kM = (uint32_t)(2 * Lmax + 2 * bias - 255) * kInv255;
+    }
+    __host__ __device__ int zero() const { return Lmax + bias; }  // the byte of L = 0
+    __host__ __device__ int row_words() const { return 3 * S; }
+};
+
+constexpr int kNibbleLmax = 31;  // path 4's nibble form: 4 (2 Lmax) fits a byte
+
 // Per-rung statistics, in this order, as unsigned 64-bit two's-complement sums.
 enum { kAccN = 0, kAccE, kAccE2, kAccM, kAccM2, kAccFlip, kAccCount };
 
@@ -58,6 +90,9 @@ struct DevProblem {
     int withhold_rung;         // test hook: rung whose chain never publishes (-1 = off)
     int acc_in_smem;           // 1: per-rung statistics gathered in shared memory per launch
     int tables_in_smem;        // 1: every rung's threshold row resident in shared memory
+    int slots;                 // path 1: neighbour slots of a site descriptor (a multiple of 4) when the
+                               // word-wise kernel runs, 0: the byte-wise one
+    int nibble;                // path 4: 1 = the nibble form of the bit-packed chain
     int exact_swaps;           // test hook: 1 = always take the FP64 swap decision
     uint32_t key0, key1;
 };
@@ -89,12 +124,21 @@ struct LaunchPlan {
     int cluster = 1;     // path 7: CTAs in the one cluster
     int group_threads = 0;  // path 7: threads sweeping one chain
     int thr_resident = 0;   // path 7: every rung's threshold row in shared memory
+    int unit_words = 1;     // path 7: words of an update unit
+    int copy = 0;           // paths 1, 3 and 9: one copy a thread (sweep_copy_kernel)
+    int nibble = 0;         // path 4: neighbour slots of the nibble form, 0 = one bit a copy
+    int rows = 0;           // path 1: the word-wise kernel (DevProblem::slots > 0)
     int chains_per_cta = 1; // path 10: chains packed on one CTA (cluster = ceil(R / chains_per_cta))
 };
 
 // Sizes of the dynamic shared-memory carve-up of the sweep kernel for a path.
 // cluster_pre: path 9 with producer warps (its plan's n_consumer < threads)
 size_t sweep_smem_bytes(const DevProblem& p, int path, int dclass, bool cluster_pre = false);
+// Path 1: neighbour slots of the word-wise kernel's descriptors when its layout fits max_smem
+// (with threshold rows and statistics in global memory if need be), else 0: byte-wise.
+int rows_slots(const DevProblem& p, int max_degree, size_t max_smem);
+// Shared memory of the one-copy-a-thread kernels (cluster: path 9).
+size_t copy_smem_bytes(const DevProblem& p, bool cluster);
 // path 10: the shared memory of a CTA holding `chains` classical chains
 size_t classical_smem_bytes(const DevProblem& p, int chains);
 
@@ -118,6 +162,7 @@ struct BatchInstance {
     int group_threads;         // threads sweeping one chain (a divisor of the CTA size)
     int resident;              // 1: a CTA keeps all its chains in shared memory for the run
     int thr_resident;          // 1: every rung's threshold row stays in shared memory for the run
+    int unit_words;            // 4-copy words of an update unit: 1, 2 or 4 (choose_unit_words)
     uint32_t key0, key1;
     long long t0, q0;          // counters before this run
     int n_sweeps, sweeps_per_swap;
@@ -171,8 +216,9 @@ void build_tables(int R, int P, int Lmax, const pt_rung* ladder, std::vector<uin
 // 4-byte words (see level_schedule); 0: in site order.
 void level_schedule(int N, const std::vector<std::vector<int>>& adj, std::vector<uint32_t>& items,
                     std::vector<int32_t>& level_off, int per_round = 0, int row_words = 0);
-void build_site_desc(int N, int row_bytes, int dclass, const std::vector<std::vector<int>>& adj,
-                     const std::vector<std::vector<int>>& adjJ, const int32_t* h, std::vector<uint32_t>& desc);
+void build_site_desc(int N, int row_bytes, int dclass, int Lmax, const std::vector<std::vector<int>>& adj,
+                     const std::vector<std::vector<int>>& adjJ, const int32_t* h, std::vector<uint32_t>& desc,
+                     bool plain = false);  // plain: J itself and an unbiased constant (path 4's nibble form)
 
 // Host-side preparation of one batched request (pt_batch.cu).
 struct Prepared {
@@ -192,6 +238,9 @@ void fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base, con
 // which the autotuner picks on the batched size mix.
 constexpr int kGroupWidenDefault = -4;
 void choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen = kGroupWidenDefault);
+
+// Words of an update unit for groups of group_threads threads.
+int choose_unit_words(const BatchInstance& I, int group_threads);
 
 // Batched launchers (pt_batch.cu).
 size_t batch_smem_bytes(const BatchInstance& I, int cluster, int threads);

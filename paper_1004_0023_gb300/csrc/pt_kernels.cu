@@ -18,6 +18,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "pt.h"
 #include "pt_device.cuh"
 #include "pt_internal.h"
@@ -28,9 +31,9 @@ namespace cg = cooperative_groups;
 
 // ------------------------------------------------------------------------- smem layouts
 
-// Threshold rows and per-rung statistics in shared memory (when they fit).
-__host__ __device__ inline size_t thr_bytes(const DevProblem& p) {
-    return up16((size_t)(p.tables_in_smem ? p.R : 1) * p.nL3 * 4);
+// Threshold rows (of row_words entries) and per-rung statistics in shared memory (when they fit).
+__host__ __device__ inline size_t thr_bytes(const DevProblem& p, int row_words) {
+    return up16((size_t)(p.tables_in_smem ? p.R : 1) * row_words * 4);
 }
 __host__ __device__ inline size_t acc_bytes(const DevProblem& p) {
     return p.acc_in_smem ? (size_t)p.R * kAccCount * 8 : 0;
@@ -47,7 +50,7 @@ struct GenericLayout {
         h = o;     o += up16((size_t)N);
         items = o; o += up16((size_t)2 * N * 4);
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
-        thr = o;   o += thr_bytes(p);
+        thr = o;   o += thr_bytes(p, p.nL3);
         acc = o;   o += acc_bytes(p);
         red = o;   o += 32 * 3 * 8;
         ctl = o;   o += 16;
@@ -55,27 +58,49 @@ struct GenericLayout {
     }
 };
 
-// Packed path (P % 8 == 0, degree + 1 <= 8): spins, one row of +1 copies (the field's h
-// slot points at it), per-site descriptors, the schedule, level offsets, the threshold
-// row(s), statistics, reduction scratch, control words and, when
+// Path 1's word-wise kernel (any even P, any degree up to 32): rows whose parity halves are
+// padded to whole words, and descriptors built in shared memory from the neighbour table.
+// With pre and cswap as FastLayout has them, for the one-copy-a-thread kernels.
+struct RowsLayout {
+    size_t spins, desc, items, loff, thr, acc, red, ctl, cmb, rbuf, total;
+    __host__ __device__ explicit RowsLayout(const DevProblem& p, bool pre = false, bool cswap = false) {
+        const size_t N = p.N, G = ((size_t)p.P / 2 + 3) / 4;
+        size_t o = 0;
+        spins = o; o += up16(N * 8 * G);
+        desc = o;  o += N * rows_desc_words(p.slots) * 4;
+        items = o; o += up16(2 * N * 4);
+        loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
+        thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
+        acc = o;   o += acc_bytes(p);
+        red = o;   o += 32 * 3 * 8;
+        ctl = o;   o += 32;
+        cmb = o;   o += cswap ? (size_t)kClusterMailPasses * p.R * 16 : 0;
+        rbuf = o;  o += pre ? 2 * (2 * N) * G * 16 : 0;
+        total = o;
+    }
+};
+
+size_t copy_smem_bytes(const DevProblem& p, bool cluster) { return RowsLayout(p, true, cluster).total; }
+
+// Packed path (P % 8 == 0, degree <= 7): spins, per-site descriptors, the schedule, level
+// offsets, the threshold row(s), statistics, reduction scratch, control words and, when
 // the random words are produced ahead, two buffers of one sweep's words each.
-// With bits, the chain is P/8 bytes per site, the constant row holds +1 copies as zero bits,
-// and two 256-entry tables spread parity bits into +1/-1 bytes.
+// With bits, the chain is P/8 bytes per site and two 256-entry tables spread parity bits
+// into +1/-1 bytes.
 // With cswap (path 9), each CTA also holds the swap mailboxes of the cluster's chains: four
 // passes of R (E, M) words each (see eos_decide_cluster).
 struct FastLayout {
-    size_t spins, ones, lut, desc, items, loff, thr, acc, red, ctl, cmb, rbuf, total;
+    size_t spins, lut, desc, items, loff, thr, acc, red, ctl, cmb, rbuf, total;
     __host__ __device__ FastLayout(const DevProblem& p, int dc, bool pre, bool bits = false, bool cswap = false) {
         const int N = p.N, P = p.P;
-        const size_t row = bits ? (size_t)P / 8 : (size_t)P;
+        const size_t row = bits ? (size_t)P / (p.nibble ? 4 : 8) : (size_t)P;
         size_t o = 0;
         spins = o; o += up16((size_t)N * row);
-        ones = o;  o += up16(row);
-        lut = o;   o += bits ? 2048 : 0;
+        lut = o;   o += bits && !p.nibble ? 2048 : 0;
         desc = o;  o += (size_t)N * (dc == 4 ? 32 : 48);
         items = o; o += up16((size_t)2 * N * 4);
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
-        thr = o;   o += thr_bytes(p);
+        thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
         acc = o;   o += acc_bytes(p);
         red = o;   o += 32 * 3 * 8;
         ctl = o;   o += 32;
@@ -88,8 +113,17 @@ struct FastLayout {
 
 size_t split_smem_bytes(const DevProblem& p, int dclass, bool pre);
 
+int rows_slots(const DevProblem& p, int max_degree, size_t max_smem) {
+    if (p.P < 2) return 0;
+    DevProblem q = p;
+    q.slots = std::max(4, (max_degree + 3) / 4 * 4);
+    q.tables_in_smem = q.acc_in_smem = 0;
+    q.n_levels = std::max(p.n_levels, 1);
+    return RowsLayout(q).total <= max_smem ? q.slots : 0;
+}
+
 size_t sweep_smem_bytes(const DevProblem& p, int path, int dclass, bool cluster_pre) {
-    if (path == kPathGeneric) return GenericLayout(p).total;
+    if (path == kPathGeneric) return p.slots > 0 ? RowsLayout(p).total : GenericLayout(p).total;
     if (path == kPathCluster) return FastLayout(p, dclass, cluster_pre, false, true).total;
     if (path == kPathPeer) return FastLayout(p, dclass, true, false).total;
     if (path == kPathSplit || path == kPathSplitInline) return split_smem_bytes(p, dclass, path == kPathSplit);
@@ -277,7 +311,8 @@ __device__ int end_of_sweep(const DevProblem& p, unsigned long long* acc, int ru
     return eos_decide(p, w, rung, E, M, timeout_ns, key, abort);
 }
 
-// Shared-memory threshold rows: every rung's row when they fit, else the current one.
+// Shared-memory threshold rows: every rung's row when they fit, else the current one. The
+// byte-wise kernels keep the public layout ...
 __device__ __forceinline__ void load_thr(const DevProblem& p, uint32_t* s_thr, int rung, int tid, int nt) {
     if (p.tables_in_smem) {
         for (int x = tid; x < p.R * p.nL3; x += nt) s_thr[x] = p.thr[x];
@@ -287,6 +322,18 @@ __device__ __forceinline__ void load_thr(const DevProblem& p, uint32_t* s_thr, i
 }
 __device__ __forceinline__ const uint32_t* thr_row(const DevProblem& p, const uint32_t* s_thr, int rung) {
     return p.tables_in_smem ? s_thr + (size_t)rung * p.nL3 : s_thr;
+}
+// ... and the packed ones rearrange it into columns (see IndexRule).
+__device__ __forceinline__ void load_thr_columns(const DevProblem& p, uint32_t* s_thr, int rung, int tid, int nt) {
+    const IndexRule rule(p.Lmax);
+    const uint32_t* src = p.tables_in_smem ? p.thr : p.thr + (size_t)rung * p.nL3;
+    const int rows = p.tables_in_smem ? p.R : 1, nL = 2 * p.Lmax + 1;
+    for (int x = tid; x < rows * nL; x += nt) {
+        const int r = x / nL, l = x - r * nL;
+        uint32_t* dst = s_thr + (size_t)r * rule.row_words() + l;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dst[c * rule.S] = src[3 * x + c];
+    }
 }
 
 // Per-launch statistics gathered in shared memory are added to the global rows once.
@@ -671,30 +718,102 @@ __device__ __forceinline__ void produce_words(uint4* buf, uint32_t t, const uint
 // CSWAP (path 9): the CTAs of all R chains form one cluster (slot = rank) and the swap
 // mailboxes live in every CTA's shared memory (eos_decide_cluster); the CTAs meet at a
 // cluster barrier only after the mailboxes are cleared and before they leave.
-template <int DC, bool PRE, bool BITS = false, bool SPEC = true, bool PEER = false, bool CSWAP = false>
+// DC = 0: path 1's word-wise kernel (RowsLayout, rows_unit_eval) on the same loop.
+// COPY (with DC = 0 and PRE): one copy a thread.
+// NIB > 0: the nibble form of the bit-packed chain with NIB neighbour slots in use.
+template <int DC, bool PRE, bool WIDE, bool BITS = false, bool SPEC = true, bool PEER = false, bool CSWAP = false,
+          int NIB = 0, bool COPY = false>
 __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot, long long t0, long long q0,
                                                   int n_sweeps, int sweeps_per_swap, long long timeout_ns,
                                                   int n_consumer, unsigned char* smem) {
     const int N = p.N, P = p.P;
     const int tid = threadIdx.x, nt = blockDim.x;
-    const FastLayout L(p, DC, PRE, BITS, CSWAP);
+    constexpr bool ROWS = DC == 0;
+    struct PackedLayout : FastLayout {
+        __device__ explicit PackedLayout(const DevProblem& q) : FastLayout(q, DC, PRE, BITS, CSWAP) {}
+    };
+    struct WordsLayout : RowsLayout {
+        __device__ explicit WordsLayout(const DevProblem& q) : RowsLayout(q, PRE, CSWAP) {}
+    };
+    const std::conditional_t<ROWS, WordsLayout, PackedLayout> L(p);
     int8_t* sp = reinterpret_cast<int8_t*>(smem + L.spins);
-    uint8_t* bp = reinterpret_cast<uint8_t*>(smem + L.spins);
-    uint32_t* s_lut = reinterpret_cast<uint32_t*>(smem + L.lut);
     uint32_t* s_desc = reinterpret_cast<uint32_t*>(smem + L.desc);
     uint32_t* s_items = reinterpret_cast<uint32_t*>(smem + L.items);
     int32_t* s_loff = reinterpret_cast<int32_t*>(smem + L.loff);
     uint32_t* s_thr = reinterpret_cast<uint32_t*>(smem + L.thr);
     long long* s_red = reinterpret_cast<long long*>(smem + L.red);
     int* s_ctl = reinterpret_cast<int*>(smem + L.ctl);
-    uint4* rbuf = reinterpret_cast<uint4*>(smem + L.rbuf);
     unsigned long long* s_acc = reinterpret_cast<unsigned long long*>(smem + L.acc);
+    uint4* rbuf = reinterpret_cast<uint4*>(smem + L.rbuf);
     unsigned long long* s_cmb = reinterpret_cast<unsigned long long*>(smem + L.cmb);
+    uint8_t* bp = nullptr;
+    uint32_t* s_lut = nullptr;
+    if constexpr (!ROWS) {
+        bp = reinterpret_cast<uint8_t*>(smem + L.spins);
+        s_lut = reinterpret_cast<uint32_t*>(smem + L.lut);
+    }
     const int NC = PRE ? n_consumer : nt;
     const bool consumer = tid < NC;
-    const int DW = SiteDesc<DC>::DW;
+    // columns of a parity of a row: words of 4 copies, or nibble words of 16
+    const int G = NIB ? P >> 5 : ((P >> 1) + 3) >> 2;
+    const uint32_t half = 4u * (uint32_t)G;
+    const int desc_words = ROWS ? rows_desc_words(p.slots) : SiteDesc<ROWS ? 4 : DC>::DW;
 
-    if (BITS) {
+    if constexpr (ROWS) {
+        const int8_t* src = p.spins + (size_t)slot * p.slot_stride;
+        const int RB = 2 * (int)half, n_par = P >> 1;
+        for (int x = tid; x < N * RB; x += nt) {
+            const int i = x / RB, c = x - i * RB;
+            const int par = c >= (int)half, h = c - par * (int)half;
+            sp[x] = h < n_par ? src[(size_t)i * P + 2 * h + par] : (int8_t)1;
+        }
+        // descriptors from the neighbour table: the sites with J = 0 are padding
+        const uint32_t zero = (uint32_t)IndexRule(p.Lmax).zero();
+        for (int i = tid; i < N; i += nt) {
+            uint32_t* d = s_desc + (size_t)i * desc_words;
+            uint32_t sumJ = 0u, n = 0u;
+            for (int k = 0; k < p.dmax; ++k) {
+                const uint32_t e = p.nbr[(size_t)i * p.dmax + k];
+                const uint32_t J = (uint32_t)(int)(int8_t)(e & 0xFFu);
+                if (J == 0u) continue;
+                d[4 + 2 * n] = (e >> 8) * (uint32_t)RB;
+                d[5 + 2 * n] = COPY ? J : J * (0u - kInv127);
+                sumJ += J;
+                ++n;
+            }
+            for (; n == 0u || (n & 3u); ++n) {  // at least the four slots every unit reads
+                d[4 + 2 * n] = (uint32_t)i * (uint32_t)RB;
+                d[5 + 2 * n] = 0u;
+            }
+            d[0] = COPY ? (uint32_t)(int)p.h[i]
+                        : ((uint32_t)(int)p.h[i] + sumJ + zero + kInv127 * sumJ) * 0x01010101u;
+            d[1] = (uint32_t)i * (uint32_t)RB;
+            d[2] = n;
+            d[3] = 0u;
+        }
+    } else if constexpr (NIB > 0) {
+        // int8 chain in global memory -> nibble words: copy 2 h + par of a site is bit
+        // 8 (h % 4) + (h / 4) % 4 of word h / 16 of its parity
+        uint32_t* words = reinterpret_cast<uint32_t*>(sp);
+        const uint4* src = reinterpret_cast<const uint4*>(p.spins + (size_t)slot * p.slot_stride);
+        for (int x = tid; x < N * G; x += nt) {  // 32 copies: one word of each parity
+            const int i = x / G, c = x - i * G;
+            uint32_t even = 0u, odd = 0u;
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const uint4 v = src[2 * x + y];
+                uint32_t e, o;
+                split_chunk(make_uint2(v.x, v.y), e, o);
+                even |= ((e >> 7) & 0x01010101u) << (2 * y);
+                odd |= ((o >> 7) & 0x01010101u) << (2 * y);
+                split_chunk(make_uint2(v.z, v.w), e, o);
+                even |= ((e >> 7) & 0x01010101u) << (2 * y + 1);
+                odd |= ((o >> 7) & 0x01010101u) << (2 * y + 1);
+            }
+            words[(2 * i) * G + c] = even;
+            words[(2 * i + 1) * G + c] = odd;
+        }
+    } else if constexpr (BITS) {
         // int8 chain in global memory -> one bit per copy in shared memory
         const uint2* src = reinterpret_cast<const uint2*>(p.spins + (size_t)slot * p.slot_stride);
         for (int x = tid; x < N * (P / 8); x += nt) {
@@ -707,8 +826,6 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             }
             bp[x] = (uint8_t)b;
         }
-        uint8_t* zeros = reinterpret_cast<uint8_t*>(smem + L.ones);
-        for (int x = tid; x < P / 8; x += nt) zeros[x] = 0;
         for (int x = tid; x < 512; x += nt) {
             const uint32_t par = (uint32_t)x >> 8, byte = (uint32_t)x & 0xFFu;
             uint32_t v = 0;
@@ -719,28 +836,36 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     } else {
         // interleaved int8 chain in global memory -> parity-split rows in shared memory
         load_split(sp, p.spins + (size_t)slot * p.slot_stride, N, P, P >> 3, chunk_ginv(P >> 3), tid, nt);
-        int8_t* ones = reinterpret_cast<int8_t*>(smem + L.ones);
-        for (int x = tid; x < P; x += nt) ones[x] = 1;
     }
     {
-        const int4* dsrc = reinterpret_cast<const int4*>(p.desc);
-        int4* ddst = reinterpret_cast<int4*>(s_desc);
-        for (int x = tid; x < N * DW / 4; x += nt) ddst[x] = dsrc[x];
+        if constexpr (!ROWS) {
+            const int4* dsrc = reinterpret_cast<const int4*>(p.desc);
+            int4* ddst = reinterpret_cast<int4*>(s_desc);
+            for (int x = tid; x < N * desc_words / 4; x += nt) ddst[x] = dsrc[x];
+        }
         for (int x = tid; x < 2 * N; x += nt) s_items[x] = p.items[x];
         for (int x = tid; x <= p.n_levels; x += nt) s_loff[x] = p.level_off[x];
     }
     int rung = p.rung_of_slot[slot];
-    load_thr(p, s_thr, rung, tid, nt);
+    load_thr_columns(p, s_thr, rung, tid, nt);
     if (p.acc_in_smem)
         for (int x = tid; x < p.R * kAccCount; x += nt) s_acc[x] = 0ull;
     long long E = p.E[slot], M = p.M[slot];  // meaningful in thread 0 only
 
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
-    const int G = P >> 3;  // 8-copy chunks per row = 4-copy units per parity
+    int lgw = 0;
+    while ((1 << lgw) < G) ++lgw;
+    const int cols = COPY ? P >> 1 : G;  // units of an item
     int lg = 0;
-    while ((1 << lg) < G) ++lg;
+    while ((1 << lg) < cols) ++lg;
     const int gmask = (1 << lg) - 1;
-    const uint32_t* thr_c = thr_row(p, s_thr, rung) + 3 * p.Lmax;
+    const UnitRule<WIDE> rule(p.Lmax);
+    // byte offset in shared memory at which the current rung's threshold row is looked up
+    const int S = IndexRule(p.Lmax).S;
+    const uint32_t thr0 =
+        COPY ? (uint32_t)L.thr + 4u * (uint32_t)(p.Lmax + S) : thr_base<WIDE>((uint32_t)L.thr, p.Lmax);
+    const uint32_t thr_step = p.tables_in_smem ? 12u * (uint32_t)S : 0u;
+    uint32_t thr_c = thr0 + thr_step * (uint32_t)rung;
     const int n_items = 2 * N;
     const int lane = tid & 31;
     if (tid == 0) {
@@ -754,7 +879,8 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     __syncthreads();
     if (CSWAP) cluster_barrier();  // every CTA's mailboxes are clear before anyone publishes
     if (PRE && !PEER && !consumer)
-        produce_words(rbuf, (uint32_t)t0, s_items, n_items, G, lg, gmask, tid - NC, nt - NC, (uint32_t)slot, key);
+        produce_words(rbuf, (uint32_t)t0, s_items, n_items, G, lgw, (1 << lgw) - 1, tid - NC, nt - NC, (uint32_t)slot,
+                      key);
     if (PEER) {
         // the peer CTA has written the first sweep's words (its arrival releases them); this
         // CTA's arrival orders nothing of its own, so it is relaxed
@@ -776,7 +902,54 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     // multiple of 2^lg: the thread then walks items q = base + (tid >> lg) + k (NC >> lg)
     const bool g_fixed = (NC & gmask) == 0;
     const int g_own = tid & gmask, q_lane = tid >> lg, q_step = NC >> lg;
-    int sumL = 0, sumC = 0, nf = 0;  // sumC and nf count twice (see unit_commit)
+    FlipSums sums;
+    sums.clear();
+    NibbleSums nib_sums = {0, 0, 0};
+    CopySums copy_sums = {0, 0, 0};
+    // A unit of item q and column g up to its index and random words, its flips against the
+    // threshold row at thr, and the commit.
+    using Column = std::conditional_t<COPY, UnitOffsets, RowsColumn>;
+    using Eval = std::conditional_t<COPY, CopyEval, UnitEval<1>>;
+    auto column = [&](int g) -> Column {
+        if constexpr (COPY)
+            return copy_offsets((uint32_t)g, half, (uint32_t)P >> 1);
+        else if constexpr (ROWS)
+            return rows_column((uint32_t)g, (uint32_t)G, (uint32_t)P >> 1);
+        else
+            return RowsColumn{row_offsets<1>((uint32_t)g, half), 0u, 0u};
+    };
+    const Column col_own = column(min(g_own, cols - 1));  // this thread's fixed one
+    auto eval = [&](int q, int g, const Column& c, const uint4* rb, uint32_t t) -> Eval {
+        const uint32_t item = s_items[q];
+        const uint32_t* desc = s_desc + (item >> 1) * (uint32_t)desc_words;
+        if constexpr (COPY) {
+            // word h % 4 of call h / 4: the words of an item's copies are consecutive
+            return copy_eval(sp, desc, item & 1u, c, reinterpret_cast<const uint32_t*>(rb + q * G)[g]);
+        } else {
+            UnitEval<1> e;
+            unit_words<1, PRE>(e.u, item, rb + q * G + g, t, (uint32_t)slot, (uint32_t)g, key);
+            if constexpr (ROWS)
+                rows_eval_site<WIDE>(e, sp, load_rows_site(desc), item & 1u, c, rule);
+            else
+                unit_eval_site<DC, 1, WIDE>(e, sp, load_site<DC>(desc), item & 1u, c.o, rule);
+            return e;
+        }
+    };
+    auto flips = [&](const Eval& e, const Column& c, uint32_t thr) -> uint32_t {
+        if constexpr (COPY) {
+            return copy_flips(e, smem, (int)thr, S);
+        } else {
+            uint32_t F[1];
+            unit_flips<1, PRE, WIDE>(e, smem, rule, thr, F);
+            return ROWS ? F[0] & c.live : F[0];
+        }
+    };
+    auto commit = [&](const Eval& e, uint32_t F) {
+        if constexpr (COPY)
+            copy_commit(e, F != 0u, copy_sums);
+        else
+            unit_commit<1>(e, &F, sums);
+    };
     SwapSide side;  // thread 0
     side.active = 0;
     const uint32_t qmod0 = (uint32_t)(q0 % kTagPeriod);
@@ -786,43 +959,69 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         const uint32_t t = (uint32_t)(t0 + s);
         if (consumer && !s_ctl[5]) {
             const uint4* rb = rbuf + (size_t)(s & 1) * n_items * G;
-            if (!spec_done) sumL = sumC = nf = 0;
-            for (int lev = spec_done ? 1 : 0; lev < p.n_levels; ++lev) {
-                const int base = s_loff[lev];
-                if (g_fixed) {
-                    // this thread's column g never changes: its row offsets are loop invariants
-                    if (g_own < G) {
-                        const int end = s_loff[lev + 1];
-                        for (int q = base + q_lane; q < end; q += q_step) {
-                            if (BITS)
-                                packed_unit_bits<DC, PRE>(bp, s_desc, s_items[q], rb, q, g_own, G, s_lut, t,
-                                                          (uint32_t)slot, key, thr_c, sumL, sumC, nf);
-                            else
-                                packed_unit<DC, PRE>(sp, s_desc, s_items[q], rb, q, g_own, G, P, t, (uint32_t)slot,
-                                                     key, thr_c, sumL, sumC, nf);
-                        }
-                    }
-                } else {
+            if (!spec_done) {
+                sums.clear();
+                copy_sums = CopySums{0, 0, 0};
+            }
+            if constexpr (NIB > 0) {
+                const IndexRule index(p.Lmax);
+                nib_sums = NibbleSums{0, 0, 0};
+                for (int lev = 0; lev < p.n_levels; ++lev) {
+                    const int base = s_loff[lev];
                     const int units = (s_loff[lev + 1] - base) << lg;
                     for (int u = tid; u < units; u += NC) {
                         const int g = u & gmask;
-                        if (g >= G) continue;
-                        const int q = base + (u >> lg);
-                        if (BITS)
-                            packed_unit_bits<DC, PRE>(bp, s_desc, s_items[q], rb, q, g, G, s_lut, t, (uint32_t)slot,
-                                                      key, thr_c, sumL, sumC, nf);
-                        else
-                            packed_unit<DC, PRE>(sp, s_desc, s_items[q], rb, q, g, G, P, t, (uint32_t)slot, key,
-                                                 thr_c, sumL, sumC, nf);
+                        if (g >= cols) continue;
+                        nibble_unit<DC, NIB>(sp, s_desc, s_items[base + (u >> lg)], (uint32_t)g, (uint32_t)G, t,
+                                             (uint32_t)slot, key, smem, (uint32_t)index.S,
+                                             (uint32_t)(2 * p.Lmax - 255) * kInv255, thr_c, nib_sums);
                     }
+                    __syncthreads();
                 }
-                if (PRE) named_barrier(1, NC); else __syncthreads();
+            } else {
+                for (int lev = spec_done ? 1 : 0; lev < p.n_levels; ++lev) {
+                    const int base = s_loff[lev];
+                    auto unit = [&](int q, int g, const Column& c) {
+                        if constexpr (BITS) {
+                            packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot, key,
+                                                       smem, rule, thr_c, sums);
+                        } else {
+                            const Eval e = eval(q, g, c, rb, t);
+                            commit(e, flips(e, c, thr_c));
+                        }
+                    };
+                    if (g_fixed) {
+                        // this thread's column never changes: its row offsets are loop invariants
+                        if (g_own < cols) {
+                            const int end = s_loff[lev + 1];
+                            for (int q = base + q_lane; q < end; q += q_step) unit(q, g_own, col_own);
+                        }
+                    } else {
+                        const int units = (s_loff[lev + 1] - base) << lg;
+                        for (int u = tid; u < units; u += NC) {
+                            const int g = u & gmask;
+                            if (g < cols) unit(base + (u >> lg), g, column(g));
+                        }
+                    }
+                    if (PRE) named_barrier(1, NC); else __syncthreads();
+                }
             }
             // a chain's per-sweep changes fit in 32 bits: each warp adds its sums to three
             // shared counters, which thread 0 reads and clears
-            const int dE = __reduce_add_sync(0xFFFFFFFFu, -2 * sumL);
-            const int dM = __reduce_add_sync(0xFFFFFFFFu, -2 * (sumC - nf));  // both counted twice
-            const int dF = __reduce_add_sync(0xFFFFFFFFu, nf) >> 1;
+            int dE = sums.dE(rule), dM = sums.dM(rule), dF = sums.flips();
+            if (COPY) {
+                dE = -2 * copy_sums.L;
+                dM = -2 * copy_sums.M;
+                dF = copy_sums.n;
+            }
+            if (NIB > 0) {
+                dE = 2 * (nib_sums.L - p.Lmax * nib_sums.n);
+                dM = 4 * (nib_sums.C - nib_sums.n);
+                dF = -nib_sums.n;
+            }
+            dE = __reduce_add_sync(0xFFFFFFFFu, dE);
+            dM = __reduce_add_sync(0xFFFFFFFFu, dM);
+            dF = __reduce_add_sync(0xFFFFFFFFu, dF);
             int* s_sum = reinterpret_cast<int*>(s_red);
             if (lane == 0) {
                 atomicAdd(s_sum + 0, dE);
@@ -854,8 +1053,8 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             }
         } else if (PRE && !consumer && s + 1 < n_sweeps) {
             // producer warps only: a consumer whose swap wait gave up skips to the barrier below
-            produce_words(rbuf + (size_t)((s + 1) & 1) * n_items * G, t + 1u, s_items, n_items, G, lg, gmask,
-                          tid - NC, nt - NC, (uint32_t)slot, key);
+            produce_words(rbuf + (size_t)((s + 1) & 1) * n_items * G, t + 1u, s_items, n_items, G, lgw,
+                          (1 << lgw) - 1, tid - NC, nt - NC, (uint32_t)slot, key);
         }
         // the next sweep's random words are complete and every consumer has finished sweep s;
         // a wait that gave up in the previous sweep ends the launch here, for every thread
@@ -883,23 +1082,23 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         // level 0 of sweep s + 1 under both candidate rungs
         const bool spec = spec_ok && s + 1 < n_sweeps;
         const int prung = s_ctl[4];
-        UnitEval ev[2];
+        Eval ev[2];
         uint32_t Fa[2] = {0u, 0u}, Fb[2] = {0u, 0u};
         bool valid[2] = {false, false};
         if (spec) {
             const uint4* rb1 = rbuf + (size_t)((s + 1) & 1) * n_items * G;
-            const uint32_t* thr_b = prung >= 0 ? thr_row(p, s_thr, prung) + 3 * p.Lmax : thr_c;
+            const uint32_t thr_b = prung >= 0 ? thr0 + thr_step * (uint32_t)prung : thr_c;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const int u = (tid - 32) + k * (NC - 32);
                 const int g = u & gmask;
-                valid[k] = tid >= 32 && u < units0 && g < G;
+                valid[k] = tid >= 32 && u < units0 && g < cols;
                 if (valid[k]) {
                     const int q = s_loff[0] + (u >> lg);
-                    ev[k] = packed_unit_eval<DC, PRE>(sp, s_desc, s_items[q], rb1, q, g, G, P, t + 1u, (uint32_t)slot,
-                                                      key);
-                    Fa[k] = unit_flips<PRE>(ev[k], thr_c);
-                    Fb[k] = prung >= 0 ? unit_flips<PRE>(ev[k], thr_b) : Fa[k];
+                    const Column c = column(g);
+                    ev[k] = eval(q, g, c, rb1, t + 1u);
+                    Fa[k] = flips(ev[k], c, thr_c);
+                    Fb[k] = prung >= 0 ? flips(ev[k], c, thr_b) : Fa[k];
                 }
             }
         }
@@ -918,15 +1117,16 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         const bool moved = nr != rung;
         if (moved) {
             rung = nr;
-            if (!p.tables_in_smem) load_thr(p, s_thr, rung, tid, NC);
-            thr_c = thr_row(p, s_thr, rung) + 3 * p.Lmax;
+            if (!p.tables_in_smem) load_thr_columns(p, s_thr, rung, tid, NC);
+            thr_c = thr0 + thr_step * (uint32_t)rung;
         }
         spec_done = spec;
         if (spec) {
-            sumL = sumC = nf = 0;
+            sums.clear();
+            copy_sums = CopySums{0, 0, 0};
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                if (valid[k]) unit_commit(ev[k], moved ? Fb[k] : Fa[k], sumL, sumC, nf);
+                if (valid[k]) commit(ev[k], moved ? Fb[k] : Fa[k]);
         }
         // the next sweep's reads of shared memory (level 1, or a reloaded threshold row) follow
         if (PRE) named_barrier(1, NC); else __syncthreads();
@@ -938,7 +1138,26 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     if (s_ctl[5]) return;  // the last sweep's wait gave up
     flush_acc(p, s_acc, tid, nt);
 
-    if (BITS) {
+    if constexpr (NIB > 0) {
+        const uint32_t* words = reinterpret_cast<const uint32_t*>(sp);
+        uint4* dst = reinterpret_cast<uint4*>(p.spins + (size_t)slot * p.slot_stride);
+        for (int x = tid; x < N * G; x += nt) {
+            const int i = x / G, c = x - i * G;
+            const uint32_t even = words[(2 * i) * G + c], odd = words[(2 * i + 1) * G + c];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                uint2 v[2];
+#pragma unroll
+                for (int z = 0; z < 2; ++z) {
+                    const int k = 2 * y + z;
+                    // +-1 bytes: 1 + 0xFE where the bit is set
+                    v[z] = join_chunk(0x01010101u + 0xFEu * ((even >> k) & 0x01010101u),
+                                      0x01010101u + 0xFEu * ((odd >> k) & 0x01010101u));
+                }
+                dst[2 * x + y] = make_uint4(v[0].x, v[0].y, v[1].x, v[1].y);
+            }
+        }
+    } else if constexpr (BITS) {
         uint2* dst = reinterpret_cast<uint2*>(p.spins + (size_t)slot * p.slot_stride);
         for (int x = tid; x < N * (P / 8); x += nt) {
             const uint32_t b = bp[x];
@@ -949,6 +1168,12 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                 v.y |= (((b >> (k + 4)) & 1u) ? 0xFFu : 0x01u) << (8 * k);
             }
             dst[x] = v;
+        }
+    } else if constexpr (ROWS) {
+        int8_t* dst = p.spins + (size_t)slot * p.slot_stride;
+        for (int x = tid; x < N * P; x += nt) {
+            const int i = x / P, k = x - i * P;
+            dst[x] = sp[(size_t)i * 2 * half + (k & 1 ? half : 0u) + (k >> 1)];
         }
     } else {
         store_split(p.spins + (size_t)slot * p.slot_stride, sp, N, P, P >> 3, chunk_ginv(P >> 3), tid, nt);
@@ -1007,10 +1232,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
         return;
     }
     const int slot = (int)(blockIdx.x >> 1);
-    if (cluster.block_rank() == 0)
-        sweep_packed_body<DC, true, false, true, true>(p, slot, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns,
-                                                       blockDim.x, smem);
-    else
+    if (cluster.block_rank() == 0) {
+        if (IndexRule(p.Lmax).wide)
+            sweep_packed_body<DC, true, true, false, true, true>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
+                                                                 timeout_ns, blockDim.x, smem);
+        else
+            sweep_packed_body<DC, true, false, false, true, true>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
+                                                                  timeout_ns, blockDim.x, smem);
+    } else
         peer_producer<DC>(p, slot, t0, n_sweeps, smem);
 }
 
@@ -1020,8 +1249,59 @@ sweep_packed_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int 
                     long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
     // the held level-0 units do not fit the 64 registers of a 1024-thread block
-    sweep_packed_body<DC, PRE, BITS, (MAXT <= 512)>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns,
-                                                    n_consumer, smem);
+    if (IndexRule(p.Lmax).wide)
+        sweep_packed_body<DC, PRE, true, BITS, (MAXT <= 512)>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap,
+                                                              timeout_ns, n_consumer, smem);
+    else
+        sweep_packed_body<DC, PRE, false, BITS, (MAXT <= 512)>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap,
+                                                               timeout_ns, n_consumer, smem);
+}
+
+// Path 4's nibble form (P % 32 == 0, Lmax <= kNibbleLmax).
+template <int DC, int NIB>
+__global__ void __launch_bounds__(512, 1)
+    sweep_nibble_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
+                        long long timeout_ns, int n_consumer) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    sweep_packed_body<DC, false, false, true, false, false, false, NIB>(p, blockIdx.x, t0, q0, n_sweeps,
+                                                                        sweeps_per_swap, timeout_ns, n_consumer, smem);
+}
+
+// One copy a thread (DevProblem::slots > 0): a CTA per chain, or (path 9) all of them in one
+// cluster, checked on entry as sweep_cluster_kernel does.
+__global__ void __launch_bounds__(512, 1)
+    sweep_copy_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
+                      long long timeout_ns, int n_consumer) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    sweep_packed_body<0, true, false, false, true, false, false, 0, true>(p, blockIdx.x, t0, q0, n_sweeps,
+                                                                          sweeps_per_swap, timeout_ns, n_consumer,
+                                                                          smem);
+}
+__global__ void __launch_bounds__(512, 1)
+    sweep_copy_cluster_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
+                              long long timeout_ns, int n_consumer) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    cg::cluster_group cluster = cg::this_cluster();
+    if (cluster.num_blocks() != (unsigned)p.R || gridDim.x != (unsigned)p.R) {
+        if (threadIdx.x == 0) atomicCAS(p.status, 0, PT_ECUDA);
+        return;
+    }
+    sweep_packed_body<0, true, false, false, true, false, true, 0, true>(p, (int)cluster.block_rank(), t0, q0,
+                                                                         n_sweeps, sweeps_per_swap, timeout_ns,
+                                                                         n_consumer, smem);
+}
+
+// Path 1's word-wise kernel: any even P and any degree up to 32 whose descriptors fit.
+__global__ void __launch_bounds__(512, 1)
+    sweep_rows_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
+                      long long timeout_ns, int n_consumer) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (IndexRule(p.Lmax).wide)
+        sweep_packed_body<0, false, true>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer,
+                                          smem);
+    else
+        sweep_packed_body<0, false, false>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer,
+                                           smem);
 }
 
 // Path 9: one cluster of R CTAs, CTA r sweeping chain r as paths 2 (PRE = false) and 3 do,
@@ -1038,8 +1318,12 @@ __global__ void __launch_bounds__(384, 1)
         if (threadIdx.x == 0) atomicCAS(p.status, 0, PT_ECUDA);
         return;
     }
-    sweep_packed_body<DC, PRE, false, true, false, true>(p, (int)cluster.block_rank(), t0, q0, n_sweeps,
-                                                         sweeps_per_swap, timeout_ns, n_consumer, smem);
+    if (IndexRule(p.Lmax).wide)
+        sweep_packed_body<DC, PRE, true, false, true, false, true>(p, (int)cluster.block_rank(), t0, q0, n_sweeps,
+                                                                   sweeps_per_swap, timeout_ns, n_consumer, smem);
+    else
+        sweep_packed_body<DC, PRE, false, false, true, false, true>(p, (int)cluster.block_rank(), t0, q0, n_sweeps,
+                                                                    sweeps_per_swap, timeout_ns, n_consumer, smem);
 }
 
 // Several problems in one cooperative launch (all chains resident at once): block b sweeps
@@ -1049,12 +1333,19 @@ __global__ void __launch_bounds__(512, 1) sweep_packed_multi_kernel(const MultiP
     extern __shared__ __align__(16) unsigned char smem[];
     const int2 m = map[blockIdx.x];
     const MultiProblem mp = probs[m.x];
-    if (mp.dc == 4)
-        sweep_packed_body<4, false>(mp.p, m.y, mp.t0, mp.q0, mp.n_sweeps, mp.sweeps_per_swap, mp.timeout_ns,
-                                    blockDim.x, smem);
+    const bool wide = IndexRule(mp.p.Lmax).wide;
+    if (mp.dc == 4 && !wide)
+        sweep_packed_body<4, false, false>(mp.p, m.y, mp.t0, mp.q0, mp.n_sweeps, mp.sweeps_per_swap, mp.timeout_ns,
+                                           blockDim.x, smem);
+    else if (mp.dc == 4)
+        sweep_packed_body<4, false, true>(mp.p, m.y, mp.t0, mp.q0, mp.n_sweeps, mp.sweeps_per_swap, mp.timeout_ns,
+                                          blockDim.x, smem);
+    else if (!wide)
+        sweep_packed_body<8, false, false>(mp.p, m.y, mp.t0, mp.q0, mp.n_sweeps, mp.sweeps_per_swap, mp.timeout_ns,
+                                           blockDim.x, smem);
     else
-        sweep_packed_body<8, false>(mp.p, m.y, mp.t0, mp.q0, mp.n_sweeps, mp.sweeps_per_swap, mp.timeout_ns,
-                                    blockDim.x, smem);
+        sweep_packed_body<8, false, true>(mp.p, m.y, mp.t0, mp.q0, mp.n_sweeps, mp.sweeps_per_swap, mp.timeout_ns,
+                                          blockDim.x, smem);
 }
 
 size_t multi_smem_bytes(const DevProblem& p, int dc) { return FastLayout(p, dc, false).total; }
@@ -1096,7 +1387,6 @@ cudaError_t launch_multi(const MultiProblem* probs, const int2* map, int n_block
 //   [4W+4, 8W+4)      odd words 0..W-1 (own)
 //   [8W+4, 8W+12)     the peer's first odd word, previous sweep, buffers 0 and 1
 //   [8W+12, 8W+14)    the peer's last odd copy, previous sweep, buffers 0 and 1
-// and one row of +1 copies after the last site (the field's h slot).
 struct SplitLayout {
     size_t spins, desc, items, loff, thr, acc, red, ctl, xch, rbuf, total;
     int W, RB, Gc;
@@ -1106,11 +1396,11 @@ struct SplitLayout {
         RB = 8 * W + 16;
         Gc = W + 1;  // word columns of an even item; odd items use W of them
         size_t o = 0;
-        spins = o; o += up16((size_t)(N + 1) * RB);
+        spins = o; o += up16((size_t)N * RB);
         desc = o;  o += (size_t)N * (dc == 4 ? 32 : 48);
         items = o; o += up16((size_t)2 * N * 4);
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
-        thr = o;   o += thr_bytes(p);
+        thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
         acc = o;   o += acc_bytes(p);
         red = o;   o += 32 * 3 * 8;
         ctl = o;   o += 32;
@@ -1147,18 +1437,10 @@ __device__ __forceinline__ UnitOffsets split_offsets(int g, int W, int b) {
     return o;
 }
 
-template <int DC, bool PRE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
-sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
-                   long long timeout_ns, int n_consumer) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    cg::cluster_group cluster = cg::this_cluster();
-    // the cluster shape is compiled in; should a launch ever run without it, no CTA touches
-    // a peer's shared memory or waits at a cluster barrier
-    if (cluster.num_blocks() != 2) {
-        if (threadIdx.x == 0) atomicCAS(p.status, 0, PT_ECUDA);
-        return;
-    }
+template <int DC, bool PRE, bool WIDE>
+__device__ __forceinline__ void split_body(const DevProblem& p, long long t0, long long q0, int n_sweeps,
+                                           int sweeps_per_swap, long long timeout_ns, int n_consumer,
+                                           unsigned char* smem, cg::cluster_group& cluster) {
     const int h = (int)cluster.block_rank();
     const bool lead = h == 0;
     const int slot = blockIdx.x >> 1;
@@ -1190,13 +1472,12 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
             const int k = split_copy(c, W, h, P);
             sp[x] = k >= 0 ? src[(size_t)i * P + k] : (int8_t)0;
         }
-        for (int x = tid; x < RB; x += nt) sp[(size_t)N * RB + x] = 1;
         // descriptors with the row offsets rescaled from P to RB bytes per row
-        const uint32_t NP = (uint32_t)N * (uint32_t)P;
         for (int x = tid; x < N * DW; x += nt) {
             const int f = x % DW;
             uint32_t v = p.desc[x];
-            if (f == 0 || f >= 4) v = v >= NP ? (uint32_t)N * RB : (v / (uint32_t)P) * (uint32_t)RB;
+            const bool is_row = DC == 4 ? ((f >= 1 && f <= 3) || f == 7) : (f == 3 || (f >= 4 && f <= 10));
+            if (is_row) v = (v / (uint32_t)P) * (uint32_t)RB;
             s_desc[x] = v;
         }
         for (int x = tid; x < 2 * N; x += nt) s_items[x] = p.items[x];
@@ -1204,13 +1485,16 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
         for (int x = tid; x < 16; x += nt) s_xch[x] = 0;
     }
     int rung = p.rung_of_slot[slot];
-    load_thr(p, s_thr, rung, tid, nt);
+    load_thr_columns(p, s_thr, rung, tid, nt);
     if (p.acc_in_smem)
         for (int x = tid; x < p.R * kAccCount; x += nt) s_acc[x] = 0ull;
     long long E = p.E[slot], M = p.M[slot];  // meaningful in thread 0 only
 
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
-    const uint32_t* thr_c = thr_row(p, s_thr, rung) + 3 * p.Lmax;
+    const UnitRule<WIDE> rule(p.Lmax);
+    const uint32_t thr0 = thr_base<WIDE>((uint32_t)L.thr, p.Lmax);
+    const uint32_t thr_step = p.tables_in_smem ? 4u * (uint32_t)IndexRule(p.Lmax).row_words() : 0u;
+    uint32_t thr_c = thr0 + thr_step * (uint32_t)rung;
     const int n_items = 2 * N;
     const int lane = tid & 31;
     if (tid == 0) {
@@ -1257,8 +1541,9 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
         sq[k] = (tid >= 32 && consumer && u < units0) ? s_loff[0] + u / Gc : -1;
     }
     bool spec_done = false;
-    int lL = 0, lC = 0, lF = 0;  // this sweep's own units in the levels (counts twice, see unit_commit)
-    int pL = 0, pC = 0, pF = 0;  // the level-0 units applied early
+    FlipSums lev_sums, pre_sums;  // this sweep's own units in the levels; the level-0 units applied early
+    lev_sums.clear();
+    pre_sums.clear();
     SwapSide side;
     side.active = 0;
     const uint32_t qmod0 = (uint32_t)(q0 % kTagPeriod);
@@ -1273,26 +1558,29 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
             if (!dead) {
                 const uint4* rb = rbuf + (size_t)b * n_items * Gc;
                 const UnitOffsets off = split_offsets(g_own, W, b);
-                if (!spec_done) pL = pC = pF = 0;
-                lL = lC = lF = 0;
+                if (!spec_done) pre_sums.clear();
+                lev_sums.clear();
                 for (int lev = spec_done ? 1 : 0; lev < p.n_levels; ++lev) {
                     if (lane_ok) {
                         const int end = s_loff[lev + 1];
                         for (int q = s_loff[lev] + q_lane; q < end; q += q_step) {
                             const uint32_t it = s_items[q];
                             if (ghost_col && (it & 1u)) continue;
-                            const UnitEval e = split_unit_eval<DC, PRE>(sp, s_desc, it, rb + q * Gc + g_own, off, t,
-                                                                        (uint32_t)slot, gg_own, key);
-                            unit_decide_commit<PRE>(e, thr_c, lL, lC, lF);
+                            const UnitEval<1> e = unit_eval<DC, 1, PRE, WIDE>(sp, s_desc, it, off, rb + q * Gc + g_own, t,
+                                                                        (uint32_t)slot, gg_own, rule, key);
+                            uint32_t F[1];
+                            unit_flips<1, PRE, WIDE>(e, smem, rule, thr_c, F);
+                            unit_commit<1>(e, F, lev_sums);
                         }
                     }
                     named_barrier(1, NC);
                 }
-                if (ghost_col) lL = lC = lF = 0;
-                const int mL = lL + pL, mC = lC + pC, mF = lF + pF;
-                const int dE = __reduce_add_sync(0xFFFFFFFFu, -2 * mL);
-                const int dM = __reduce_add_sync(0xFFFFFFFFu, -2 * (mC - mF));
-                const int dF = __reduce_add_sync(0xFFFFFFFFu, mF) >> 1;
+                if (ghost_col) lev_sums.clear();
+                FlipSums m = lev_sums;
+                m.add(pre_sums);
+                const int dE = __reduce_add_sync(0xFFFFFFFFu, m.dE(rule));
+                const int dM = __reduce_add_sync(0xFFFFFFFFu, m.dM(rule));
+                const int dF = __reduce_add_sync(0xFFFFFFFFu, m.flips());
                 int* s_sum = reinterpret_cast<int*>(s_red);
                 if (lane == 0) {
                     atomicAdd(s_sum + 0, dE);
@@ -1347,23 +1635,26 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
         // level 0 of sweep s + 1 under both candidate rungs
         const bool spec = spec_ok && s + 1 < n_sweeps;
         const int prung = s_ctl[4];
-        UnitEval ev[2];
+        UnitEval<1> ev[2];
         uint32_t Fa[2] = {0u, 0u}, Fb[2] = {0u, 0u};
         bool valid[2] = {false, false};
         if (spec) {
             const uint4* rb1 = rbuf + (size_t)(b ^ 1) * n_items * Gc;
-            const uint32_t* thr_b = prung >= 0 ? thr_row(p, s_thr, prung) + 3 * p.Lmax : thr_c;
+            const uint32_t thr_b = prung >= 0 ? thr0 + thr_step * (uint32_t)prung : thr_c;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (sq[k] < 0) continue;
                 const uint32_t it = s_items[sq[k]];
                 valid[k] = !((it & 1u) && sg[k] == W);
                 if (valid[k]) {
-                    ev[k] = split_unit_eval<DC, PRE>(sp, s_desc, it, rb1 + sq[k] * Gc + sg[k],
-                                                     split_offsets(sg[k], W, b ^ 1), t + 1u, (uint32_t)slot,
-                                                     (uint32_t)((h * W + sg[k]) % (2 * W)), key);
-                    Fa[k] = unit_flips<PRE>(ev[k], thr_c);
-                    Fb[k] = prung >= 0 ? unit_flips<PRE>(ev[k], thr_b) : Fa[k];
+                    ev[k] = unit_eval<DC, 1, PRE, WIDE>(sp, s_desc, it, split_offsets(sg[k], W, b ^ 1),
+                                                  rb1 + sq[k] * Gc + sg[k], t + 1u, (uint32_t)slot,
+                                                  (uint32_t)((h * W + sg[k]) % (2 * W)), rule, key);
+                    unit_flips<1, PRE, WIDE>(ev[k], smem, rule, thr_c, Fa + k);
+                    if (prung >= 0)
+                        unit_flips<1, PRE, WIDE>(ev[k], smem, rule, thr_b, Fb + k);
+                    else
+                        Fb[k] = Fa[k];
                 }
             }
         }
@@ -1379,22 +1670,20 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
         const bool moved = nr != rung;
         if (moved) {
             rung = nr;
-            if (!p.tables_in_smem) load_thr(p, s_thr, rung, tid, NC);
-            thr_c = thr_row(p, s_thr, rung) + 3 * p.Lmax;
+            if (!p.tables_in_smem) load_thr_columns(p, s_thr, rung, tid, NC);
+            thr_c = thr0 + thr_step * (uint32_t)rung;
         }
         spec_done = spec;
         if (spec) {
-            pL = pC = pF = 0;
+            pre_sums.clear();
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (!valid[k]) continue;
-                int jL = 0, jC = 0, jF = 0;
-                unit_commit(ev[k], moved ? Fb[k] : Fa[k], jL, jC, jF);
-                if (sg[k] != W) {
-                    pL += jL;
-                    pC += jC;
-                    pF += jF;
-                }
+                const uint32_t F[1] = {moved ? Fb[k] : Fa[k]};
+                FlipSums unit;
+                unit.clear();
+                unit_commit<1>(ev[k], F, unit);
+                if (sg[k] != W) pre_sums.add(unit);
             }
         }
         named_barrier(1, NC);
@@ -1419,6 +1708,24 @@ sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int s
         p.rung_of_slot[slot] = rung;
         p.slot_of_rung[rung] = slot;
     }
+}
+
+template <int DC, bool PRE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
+    sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
+                       long long timeout_ns, int n_consumer) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    cg::cluster_group cluster = cg::this_cluster();
+    // the cluster shape is compiled in; should a launch ever run without it, no CTA touches
+    // a peer's shared memory or waits at a cluster barrier
+    if (cluster.num_blocks() != 2) {
+        if (threadIdx.x == 0) atomicCAS(p.status, 0, PT_ECUDA);
+        return;
+    }
+    if (IndexRule(p.Lmax).wide)
+        split_body<DC, PRE, true>(p, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem, cluster);
+    else
+        split_body<DC, PRE, false>(p, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem, cluster);
 }
 
 // ------------------------------------------------------------------------- init / energy
@@ -1528,6 +1835,8 @@ __global__ void scatter_kernel(DevProblem p, const int8_t* in) {
 
 // ------------------------------------------------------------------------- launchers
 static const void* sweep_fn(const LaunchPlan& plan) {
+    if (plan.copy)
+        return plan.path == kPathCluster ? (const void*)sweep_copy_cluster_kernel : (const void*)sweep_copy_kernel;
     if (plan.path == kPathClassical) {
         switch (plan.dclass) {
             case 4: return (const void*)sweep_classical_kernel<4>;
@@ -1535,6 +1844,7 @@ static const void* sweep_fn(const LaunchPlan& plan) {
             default: return (const void*)sweep_classical_kernel<32>;
         }
     }
+    if (plan.path == kPathGeneric && plan.rows) return (const void*)sweep_rows_kernel;
     if (plan.path == kPathGeneric) {
         switch (plan.dclass) {
             case 4: return (const void*)sweep_kernel<4>;
@@ -1554,6 +1864,10 @@ static const void* sweep_fn(const LaunchPlan& plan) {
         return plan.dclass == 4 ? (const void*)sweep_split_kernel<4, true> : (const void*)sweep_split_kernel<8, true>;
     if (plan.path == kPathSplitInline)
         return plan.dclass == 4 ? (const void*)sweep_split_kernel<4, false> : (const void*)sweep_split_kernel<8, false>;
+    if (plan.path == kPathBits && plan.nibble) {
+        if (plan.dclass == 4) return (const void*)sweep_nibble_kernel<4, 3>;
+        return plan.nibble == 6 ? (const void*)sweep_nibble_kernel<8, 6> : (const void*)sweep_nibble_kernel<8, 7>;
+    }
     if (plan.path == kPathBits) {
         if (plan.threads > 512)
             return plan.dclass == 4 ? (const void*)sweep_packed_kernel<4, false, 1024, true>
@@ -1567,10 +1881,6 @@ static const void* sweep_fn(const LaunchPlan& plan) {
             return pre ? (const void*)sweep_packed_kernel<4, true, 1024> : (const void*)sweep_packed_kernel<4, false, 1024>;
         return pre ? (const void*)sweep_packed_kernel<8, true, 1024> : (const void*)sweep_packed_kernel<8, false, 1024>;
     }
-    if (!pre && plan.threads <= 384)
-        // blocks of at most 384 threads may use up to 168 registers per thread
-        return plan.dclass == 4 ? (const void*)sweep_packed_kernel<4, false, 384>
-                                : (const void*)sweep_packed_kernel<8, false, 384>;
     if (plan.dclass == 4)
         return pre ? (const void*)sweep_packed_kernel<4, true, 512> : (const void*)sweep_packed_kernel<4, false, 512>;
     return pre ? (const void*)sweep_packed_kernel<8, true, 512> : (const void*)sweep_packed_kernel<8, false, 512>;

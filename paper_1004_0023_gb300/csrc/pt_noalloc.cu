@@ -122,8 +122,10 @@ extern "C" int pt_run_noalloc(const pt_device_problem* q, int64_t n_sweeps, int3
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     p.acc_in_smem = (size_t)q->R * kAccCount * 8 <= 16384 ? 1 : 0;
     p.tables_in_smem = (size_t)q->R * p.nL3 * 4 <= 49152 ? 1 : 0;
+    p.slots = rows_slots(p, q->row_stride, (size_t)max_smem);
     LaunchPlan plan;
     plan.path = kPathGeneric;
+    plan.rows = p.slots > 0;
     plan.dclass = q->row_stride;
     if (p.tables_in_smem && sweep_smem_bytes(p, kPathGeneric, plan.dclass) > (size_t)max_smem) p.tables_in_smem = 0;
     if (p.acc_in_smem && sweep_smem_bytes(p, kPathGeneric, plan.dclass) > (size_t)max_smem) p.acc_in_smem = 0;

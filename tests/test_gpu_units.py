@@ -1,0 +1,86 @@
+"""The update units' edges against the oracle, bit for bit: the table-index bytes at the
+largest Lmax of each form, copies that do not fill a unit, sites without and with many
+neighbours, and every unit width. Tolerance zero, as in the other parity tests."""
+import os
+
+import numpy as np
+import pytest
+
+from oracle import Oracle
+from paper_1004_0023_gb300 import instances
+from paper_1004_0023_gb300 import pt
+
+pytestmark = pytest.mark.gpu
+
+THREADS = os.cpu_count() or 1
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib(libpt):
+    return libpt
+
+
+def _problem(n, degree, P, R, lmax, seed):
+    """Random graph of at most `degree` neighbours a site (site 0 has none); couplings as large
+    as |h| + sum |J| = lmax allows at one site of each sign."""
+    rng = np.random.default_rng(seed)
+    deg = [0] * n
+    ei, ej = [], []
+    a, b = np.triu_indices(n, 1)
+    for k in rng.permutation(a.size).tolist():
+        i, j = int(a[k]), int(b[k])
+        if i > 0 and deg[i] < degree and deg[j] < degree:
+            deg[i] += 1
+            deg[j] += 1
+            ei.append(i)
+            ej.append(j)
+    top = max(1, (lmax - 1) // max(degree, 1))
+    J = rng.integers(1, top + 1, len(ei)) * rng.choice([-1, 1], len(ei))
+    load = np.zeros(n, np.int64)
+    np.add.at(load, ei, np.abs(J))
+    np.add.at(load, ej, np.abs(J))
+    h = np.asarray([rng.integers(-1, 2) if load[i] < lmax else 0 for i in range(n)])
+    h[0], h[1] = lmax, -(lmax - load[1])
+    beta = 8.0 / lmax  # thresholds spread over the whole table
+    T = np.linspace(1.0, 2.0, R) * P / beta / 4
+    gamma = np.linspace(0.4, 1.5, R) * T
+    return instances.Problem(n, np.asarray(ei, np.int32), np.asarray(ej, np.int32), J.astype(np.int32),
+                             h.astype(np.int32), P, T, gamma, 0xABC0 + seed)
+
+
+CASES = [
+    # one copy a thread (path 1, and path 9 for a short ladder)
+    (9, 4, 2, 3, 9, {}), (9, 4, 6, 3, 41, {}), (12, 5, 10, 4, 42, {}), (20, 9, 18, 3, 60, {}), (34, 32, 34, 2, 127, {}),
+    (12, 3, 32, 4, 7, {}), (16, 7, 24, 5, 127, {}), (3, 0, 64, 3, 5, {}), (10, 3, 300, 2, 6, {}),
+    # path 1, a word of four copies a thread
+    (9, 4, 2, 3, 9, dict(kernel_path=1, threads_per_block=96)), (11, 5, 14, 3, 41, dict(kernel_path=1, threads_per_block=64)),
+    (20, 9, 12, 3, 42, dict(kernel_path=1, threads_per_block=96)), (34, 32, 34, 2, 127, dict(kernel_path=1, threads_per_block=128)),
+    (16, 3, 16, 3, 31, dict(kernel_path=1, threads_per_block=32)),
+    # paths 2, 3, 5, 6, 8: largest narrow and smallest wide index, both neighbour classes
+    *[(14, d, 16, 4, lmax, dict(kernel_path=path)) for path in (2, 3, 5, 6, 8) for d, lmax in
+      ((3, 41), (3, 42), (7, 41), (7, 127))],
+    # path 4: nibble words (P % 32 == 0, Lmax <= 31) and one bit a copy
+    *[(14, d, P, 3, lmax, dict(kernel_path=4)) for d in (3, 6, 7) for P, lmax in
+      ((32, 31), (96, 13), (32, 32), (40, 31), (64, 42))],
+    # path 7: units of one, two and four words
+    *[(40, d, P, 3, lmax, dict(kernel_path=7, group_threads=32)) for d, lmax in ((3, 41), (7, 41), (3, 42), (7, 42))
+      for P in (8, 16, 48, 128)],
+]
+
+
+@pytest.mark.parametrize("k", range(len(CASES)))
+def test_unit_edges_match_the_oracle(k):
+    n, degree, P, R, lmax, kw = CASES[k]
+    prob = _problem(n, degree, P, R, lmax, k)
+    g, o = pt.PT.from_problem(prob, **kw), Oracle.from_problem(prob, threads=THREADS)
+    assert g.info.lmax == lmax
+    moved = 0
+    for sweeps in (1, 1, 2, 30):
+        g.run(sweeps, 1)
+        o.run(sweeps, 1)
+        assert np.array_equal(g.read_state(), o.read_state()), (CASES[k], sweeps)
+        og, oo = g.obs(), o.obs()
+        for key in oo:
+            assert np.array_equal(np.asarray(og[key]), np.asarray(oo[key])), (CASES[k], sweeps, key)
+        moved = int(np.sum(og["flip_acc"]))
+    assert moved > 0
