@@ -4,13 +4,18 @@
 // work, largest first) and owns it until every sweep is done: CTA r of the cluster sweeps
 // chains [r*C, (r+1)*C), C = ceil(R / cluster). Within a CTA the chains are "packed" onto
 // groups of threads (the paper's chain packing, Sec. 5): a group sweeps one chain at a time
-// with the same level schedule, random-number counters and 4-copy update unit as the
-// single-problem kernel, so every problem gets exactly the bits it would get alone. For a
-// swap pass the CTAs publish (E, M) of their chains in shared memory, meet at one cluster
-// barrier, and each CTA evaluates every pair's decision from the peers' shared memory
-// (the same inputs everywhere give the same rung permutation everywhere). No CTA ever waits
-// for another cluster, so the persistent launch needs no co-residency guarantee beyond
-// the cluster's own.
+// with the same level schedule, random-number counters and update arithmetic as the
+// single-problem kernel, so every problem gets exactly the bits it would get alone.
+//
+// Nothing waits for a whole sweep of the problem. A CTA's work is the sequence of tasks
+// (sweep, chain), sweep by sweep; its groups take the next task as they come free (or, with
+// no more chains than groups, each group keeps its chain). A task needs its chain's previous
+// sweep, and the swap decision that follows it: the chain's (E, M) and its partner's, which
+// every chain publishes after its sweep in mailboxes that all CTAs of the cluster hold (as
+// path 9 does), so partners evaluate the same decision and no barrier orders the passes. A
+// task waits only for tasks of an earlier sweep, and those are taken first, so some task can
+// always run; the waits have a time limit all the same. Only the CTAs of one cluster wait
+// for one another, and those are resident together.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdarg.h>
@@ -35,31 +40,44 @@ namespace cg = cooperative_groups;
 
 namespace ptq {
 
+// Swap mailboxes of a problem: kClusterMailPasses passes of R entries.
+constexpr long long kBatchWaitNs = 20000000000ll;  // limit of every wait inside the kernel
+
 // Shared memory of one CTA while it owns problem I.
 struct BatchLayout {
-    size_t sdesc, items, loff, rung, slot, E, M, pub, thr, red, chains, total;
+    size_t sdesc, items, loff, rung, seq, E, M, mail, thr, red, ctl, chains, total;
     int C, ngroups, chain_stride, nbufs, DW, thr_words;
     __host__ __device__ BatchLayout(const BatchInstance& I, int K, int threads) {
         DW = I.dc == 4 ? 8 : 12;
         C = (I.R + K - 1) / K;
-        ngroups = threads / I.group_threads;
-        chain_stride = (int)up16((size_t)I.slot_stride);
+        ngroups = I.n_groups;
+        chain_stride = (int)up16((size_t)I.N * form_row_bytes(I.form, I.P));
         nbufs = I.resident ? C : ngroups;
         thr_words = (int)(up16((size_t)IndexRule(I.Lmax).row_words() * 4) / 4);
         size_t o = 0;
         sdesc = o;  o += (size_t)I.N * DW * 4;
         items = o;  o += up16((size_t)2 * I.N * 4);
         loff = o;   o += up16((size_t)(I.n_levels + 1) * 4);
-        rung = o;   o += up16((size_t)I.R * 4);
-        slot = o;   o += up16((size_t)I.R * 4);
+        rung = o;   o += up16((size_t)C * 4);
+        seq = o;    o += up16((size_t)C * 4);
         E = o;      o += up16((size_t)C * 8);
         M = o;      o += up16((size_t)C * 8);
-        pub = o;    o += (size_t)2 * C * 16;
+        mail = o;   o += I.mail_smem ? (size_t)kClusterMailPasses * I.R * 16 : 0;
         thr = o;    o += (size_t)(I.thr_resident ? I.R : ngroups) * thr_words * 4;
-        red = o;    o += up16((size_t)ngroups * (I.group_threads / 32) * 3 * 8);
+        red = o;    o += up16((size_t)ngroups * (I.group_threads / 32) * 3 * 4);
+        ctl = o;    o += up16((size_t)ngroups * 16);
         chains = o; o += (size_t)nbufs * chain_stride;
         total = o;
     }
+};
+
+// Shared memory of the persistent kernel that outlives a problem.
+struct BatchShared {
+    unsigned long long mbar[16];  // per group: arrival of a streamed chain
+    uint32_t phase[16];           // its parity of the next arrival
+    int next;                     // next task of this CTA
+    int abort;                    // a wait gave up
+    int job;
 };
 
 size_t batch_smem_bytes(const BatchInstance& I, int cluster, int threads) {
@@ -74,51 +92,222 @@ __device__ __forceinline__ void group_sync(int bar, int gsize) {
         named_barrier(bar, gsize);
 }
 
-// W: 4-copy words of an update unit (2 when P % 16 == 0: the rows' halves are then whole
-// 8-byte words, and one descriptor, one address and one wide load per neighbour serve 8 copies).
+// ---- asynchronous copies of whole chains between global and shared memory
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(unsigned long long* m) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(m)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait(unsigned long long* m, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(m)), "r"(parity)
+        : "memory");
+    return ok != 0u;
+}
+// One thread: `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory,
+// completing on m ...
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* m) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(m)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(m))
+                 : "memory");
+}
+// ... and out of it, as one bulk group of that thread.
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(dst),
+                 "r"(smem_u32(src)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_stores_done() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// Polls ready() until it holds, with a time limit (then status and sh.abort say so) and back-off;
+// false when some wait of this CTA gave up. The whole warp, converged.
+template <typename Ready>
+__device__ __forceinline__ bool wait_for(BatchShared& sh, int* status, Ready ready) {
+    const unsigned long long start = globaltimer_ns();
+    unsigned int nap = 0;
+    for (int polls = 0;; ++polls) {
+        if (__all_sync(0xFFFFFFFFu, ready())) return true;
+        if (polls >= 32) {
+            nap = nap ? min(2u * nap, 256u) : 16u;
+            __nanosleep(nap);
+            if (*(volatile int*)&sh.abort) return false;
+            if ((long long)(globaltimer_ns() - start) > kBatchWaitNs) {
+                if ((threadIdx.x & 31) == 0) {
+                    if (status) atomicCAS(status, 0, PT_ETIMEDOUT);
+                    *(volatile int*)&sh.abort = 1;
+                }
+                return false;
+            }
+        }
+    }
+}
+
+// One sweep of one chain by one group. A function of its own, so that its registers are the
+// unit loop's alone and not the task loop's as well (which the call saves once a sweep): with
+// both in one body the loop took 117 instructions a unit on N=512, P=64 against 88 in isolation.
+struct ChainSweep {
+    uint32_t sdesc, items, loff, thr;  // byte offsets in shared memory
+    uint32_t buf;
+    uint32_t key0, key1, t, rho;
+    int n_levels, Lmax, P, gsize, gtid, bar;
+};
+struct ChainChange {
+    int dE, dM, flips;  // this thread's share
+};
+// The levels of one sweep: unit(item, column) for every item and column g < cols of the
+// group's rows, a barrier of the group after each level.
+template <typename Offsets, typename Unit>
+__device__ __forceinline__ void run_levels(const ChainSweep& c, const uint32_t* s_items, const int32_t* s_loff,
+                                           int cols, Offsets offsets, Unit unit) {
+    int lg = 0;
+    while ((1 << lg) < cols) ++lg;
+    const int gmask = (1 << lg) - 1;
+    if ((c.gsize & gmask) == 0) {
+        // this thread's column never changes: its row offsets are loop invariants
+        const int g = c.gtid & gmask, q_lane = c.gtid >> lg, q_step = c.gsize >> lg;
+        const UnitOffsets off = offsets((uint32_t)min(g, cols - 1));
+        int base = s_loff[0];
+        for (int lev = 0; lev < c.n_levels; ++lev) {
+            const int end = s_loff[lev + 1];
+            if (g < cols)
+                for (int q = base + q_lane; q < end; q += q_step) unit(s_items[q], (uint32_t)g, off);
+            base = end;
+            group_sync(c.bar, c.gsize);
+        }
+    } else {
+        for (int lev = 0; lev < c.n_levels; ++lev) {
+            const int base = s_loff[lev], units = (s_loff[lev + 1] - base) << lg;
+            for (int u = c.gtid; u < units; u += c.gsize) {
+                const int g = u & gmask;
+                if (g < cols) unit(s_items[base + (u >> lg)], (uint32_t)g, offsets((uint32_t)g));
+            }
+            group_sync(c.bar, c.gsize);
+        }
+    }
+}
+// int8 rows, units of W words of four copies.
 template <int DC, int W, bool WIDE>
-__device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* s_keys, cg::cluster_group& cluster,
-                            int rank, int K) {
+__device__ __noinline__ ChainChange sweep_chain(const ChainSweep c) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    int8_t* buf = reinterpret_cast<int8_t*>(smem + c.buf);
+    const uint32_t* s_sdesc = reinterpret_cast<const uint32_t*>(smem + c.sdesc);
+    const UnitRule<WIDE> rule(c.Lmax);
+    const PhiloxKey key = philox_schedule(c.key0, c.key1);
+    const uint32_t half = (uint32_t)c.P >> 1, thr = thr_base<WIDE>(c.thr, c.Lmax);
+    FlipSums sums;
+    sums.clear();
+    run_levels(
+        c, reinterpret_cast<const uint32_t*>(smem + c.items), reinterpret_cast<const int32_t*>(smem + c.loff),
+        c.P / (8 * W), [&](uint32_t g) { return row_offsets<W>(g, half); },
+        [&](uint32_t item, uint32_t g, const UnitOffsets& off) {
+            const UnitEval<W> e =
+                unit_eval<DC, W, false, WIDE>(buf, s_sdesc, item, off, nullptr, c.t, c.rho, W * g, rule, key);
+            uint32_t F[W];
+            unit_flips<W, false, WIDE>(e, smem, rule, thr, F);
+            unit_commit<W>(e, F, sums);
+        });
+    return ChainChange{sums.dE(rule), sums.dM(rule), sums.flips()};
+}
+// Bit words of U units.
+template <int DC, int U>
+__device__ __noinline__ ChainChange sweep_chain_bits(const ChainSweep c) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    int8_t* buf = reinterpret_cast<int8_t*>(smem + c.buf);
+    const uint32_t* s_sdesc = reinterpret_cast<const uint32_t*>(smem + c.sdesc);
+    const PhiloxKey key = philox_schedule(c.key0, c.key1);
+    const uint32_t S = (uint32_t)IndexRule(c.Lmax).S, kM = (uint32_t)(2 * c.Lmax - 255) * kInv255;
+    const uint32_t cols = (uint32_t)c.P / (8 * U);
+    BitSums sums;
+    sums.clear();
+    run_levels(
+        c, reinterpret_cast<const uint32_t*>(smem + c.items), reinterpret_cast<const int32_t*>(smem + c.loff),
+        (int)cols, [&](uint32_t g) { return word_offsets(g, cols); },
+        [&](uint32_t item, uint32_t g, const UnitOffsets& off) {
+            bits_unit<DC, DC - 1, U>(buf, s_sdesc, item, off, g, c.t, c.rho, key, smem, S, kM, c.thr, sums);
+        });
+    return ChainChange{sums.dE(c.Lmax), sums.dM(), sums.flips()};
+}
+template <int DC>
+__device__ __forceinline__ ChainChange sweep_form(const ChainSweep& c, int form, bool wide) {
+    if (wide) return sweep_chain<DC, 1, true>(c);
+    switch (form) {
+        case kFormBits: return sweep_chain_bits<DC, 8>(c);
+        case kFormNibbles: return sweep_chain_bits<DC, 4>(c);
+        case kFormBytes4: return sweep_chain<DC, 4, false>(c);
+        case kFormBytes2: return sweep_chain<DC, 2, false>(c);
+        default: return sweep_chain<DC, 1, false>(c);
+    }
+}
+
+// A chain between its interleaved +-1 bytes in global memory and its form in shared memory.
+__device__ void load_chain(const BatchInstance& I, int8_t* buf, const int8_t* src, int tid0, int nthr) {
+    if (I.form == kFormBits)
+        load_bits<8>(reinterpret_cast<uint32_t*>(buf), src, I.N, I.P >> 6, tid0, nthr);
+    else if (I.form == kFormNibbles)
+        load_bits<4>(reinterpret_cast<uint32_t*>(buf), src, I.N, I.P >> 5, tid0, nthr);
+    else if ((I.P & 15) == 0)
+        load_split16(buf, src, I.N, I.P, I.P >> 4, chunk_ginv(I.P >> 4), tid0, nthr);
+    else
+        load_split(buf, src, I.N, I.P, I.P >> 3, chunk_ginv(I.P >> 3), tid0, nthr);
+}
+__device__ void store_chain(const BatchInstance& I, int8_t* dst, const int8_t* buf, int tid0, int nthr) {
+    if (I.form == kFormBits)
+        store_bits<8>(dst, reinterpret_cast<const uint32_t*>(buf), I.N, I.P >> 6, tid0, nthr);
+    else if (I.form == kFormNibbles)
+        store_bits<4>(dst, reinterpret_cast<const uint32_t*>(buf), I.N, I.P >> 5, tid0, nthr);
+    else if ((I.P & 15) == 0)
+        store_split16(dst, buf, I.N, I.P, I.P >> 4, chunk_ginv(I.P >> 4), tid0, nthr);
+    else
+        store_split(dst, buf, I.N, I.P, I.P >> 3, chunk_ginv(I.P >> 3), tid0, nthr);
+}
+
+__device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchShared& sh, cg::cluster_group& cluster,
+                            int rank, int K, int* status) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const BatchLayout L(I, K, nt);
     uint32_t* s_sdesc = reinterpret_cast<uint32_t*>(smem + L.sdesc);
     uint32_t* s_items = reinterpret_cast<uint32_t*>(smem + L.items);
     int32_t* s_loff = reinterpret_cast<int32_t*>(smem + L.loff);
     int32_t* s_rung = reinterpret_cast<int32_t*>(smem + L.rung);
-    int32_t* s_slot = reinterpret_cast<int32_t*>(smem + L.slot);
+    int32_t* s_seq = reinterpret_cast<int32_t*>(smem + L.seq);  // sweeps of this run a chain has finished
     long long* s_E = reinterpret_cast<long long*>(smem + L.E);
     long long* s_M = reinterpret_cast<long long*>(smem + L.M);
-    longlong2* s_pub = reinterpret_cast<longlong2*>(smem + L.pub);
     uint32_t* s_thr = reinterpret_cast<uint32_t*>(smem + L.thr);
-    long long* s_red = reinterpret_cast<long long*>(smem + L.red);
     unsigned char* s_chains = smem + L.chains;
+    // [pass mod 4][rung]: (E, M) of the chain on that rung; every CTA's own copy, or one in global memory
+    unsigned long long* mail =
+        I.mail_smem ? reinterpret_cast<unsigned long long*>(smem + L.mail) : reinterpret_cast<unsigned long long*>(I.mail);
 
     const int N = I.N, P = I.P, R = I.R, C = L.C;
     const int c_begin = rank * C;
     const int c_count = max(0, min(C, R - c_begin));
     const IndexRule index(I.Lmax);
-    const UnitRule<WIDE> rule(I.Lmax);
     const int gsize = I.group_threads, ngroups = L.ngroups;
     const int grp = tid / gsize, gtid = tid - grp * gsize;
 
-    // ---- the problem's schedule, descriptors, round keys and rung permutation; this CTA's chains
+    // ---- the problem's schedule and descriptors; this CTA's chains
     {
-        if (tid < 10)
-            reinterpret_cast<uint2*>(s_keys)[tid] =
-                make_uint2(I.key0 + (uint32_t)tid * 0x9E3779B9u, I.key1 + (uint32_t)tid * 0xBB67AE85u);
-        const int4* src = reinterpret_cast<const int4*>(I.sdesc);
+        const int4* src = reinterpret_cast<const int4*>(I.form >= kFormNibbles ? I.wdesc : I.sdesc);
         int4* dst = reinterpret_cast<int4*>(s_sdesc);
         for (int x = tid; x < N * L.DW / 4; x += nt) dst[x] = src[x];
-        for (int x = tid; x < 2 * N; x += nt) s_items[x] = I.items[x];
-        for (int x = tid; x <= I.n_levels; x += nt) s_loff[x] = I.level_off[x];
-        for (int x = tid; x < R; x += nt) {
-            s_rung[x] = I.rung_of_slot[x];
-            s_slot[x] = I.slot_of_rung[x];
-        }
+        const uint32_t* g_items = I.form == I.form_t ? I.titems : I.items;
+        const int32_t* g_loff = I.form == I.form_t ? I.tlevel_off : I.level_off;
+        for (int x = tid; x < 2 * N; x += nt) s_items[x] = g_items[x];
+        for (int x = tid; x <= I.n_levels; x += nt) s_loff[x] = g_loff[x];
         for (int x = tid; x < c_count; x += nt) {
+            s_rung[x] = I.rung_of_slot[c_begin + x];
+            s_seq[x] = 0;
             s_E[x] = I.E[c_begin + x];
             s_M[x] = I.M[c_begin + x];
         }
+        if (I.mail_smem || rank == 0)
+            for (int x = tid; x < kClusterMailPasses * R * 2; x += nt) mail[x] = 0ull;
         if (I.thr_resident) {  // every rung's row, so a chain never reloads one after a swap
             const int nL = 2 * I.Lmax + 1;
             for (int x = tid; x < R * nL; x += nt) {
@@ -127,218 +316,280 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, uint4* 
                 for (int c = 0; c < 3; ++c) s_thr[(size_t)r * L.thr_words + c * index.S + l] = I.thr[3 * x + c];
             }
         }
-        if (I.resident) {
+        if (I.resident)
             for (int lc = 0; lc < c_count; ++lc)
-                load_split(reinterpret_cast<int8_t*>(s_chains + (size_t)lc * L.chain_stride),
-                           I.spins + (size_t)(c_begin + lc) * I.slot_stride, N, P, P >> 3, chunk_ginv(P >> 3), tid,
-                           nt);
-        }
+                load_chain(I, reinterpret_cast<int8_t*>(s_chains + (size_t)lc * L.chain_stride),
+                           I.spins + (size_t)(c_begin + lc) * I.slot_stride, tid, nt);
+        if (tid == 0) sh.next = 0;
     }
     __syncthreads();
+    if (K > 1) cluster_barrier();  // every mailbox is clear before anyone publishes
 
-    const PhiloxKeyShared skey{s_keys};  // update units and swap decisions: round keys in shared memory
-    const int G = P >> 3;
-    const uint32_t ginv = chunk_ginv(G);
-    const bool p16 = (P & 15) == 0;  // streamed chains move 16 copies per load and store
-    const uint32_t hinv = chunk_ginv(P >> 4);
-    const int U = G / W;  // units of a row and parity
-    int lg = 0;
-    while ((1 << lg) < U) ++lg;
-    const int gmask = (1 << lg) - 1;
     const int bar = 1 + grp;
     uint32_t* thr_g = s_thr + (size_t)grp * L.thr_words;
-    long long* red_g = s_red + (size_t)grp * (gsize / 32) * 3;
+    int* red_g = reinterpret_cast<int*>(smem + L.red) + (size_t)grp * (gsize / 32) * 3;
+    int* ctl_g = reinterpret_cast<int*>(smem + L.ctl) + 4 * grp;
     const int lane = tid & 31, gwarp = gtid >> 5;
-    const bool g_fixed = (gsize & gmask) == 0;
-    const int g_own = gtid & gmask, q_lane = gtid >> lg, q_step = gsize >> lg;
-    const uint32_t half = (uint32_t)P >> 1;
-    const UnitOffsets off_own = row_offsets<W>((uint32_t)g_own, half);
+    const bool one_warp = gsize == 32, lead = gwarp == 0;
+    const int sps = I.sweeps_per_swap;
+    const bool keep = c_count <= ngroups;  // each group keeps one chain
+    const uint32_t qmod0 = (uint32_t)(I.q0 % kTagPeriod);
+    uint32_t phase = grp < 16 ? sh.phase[grp] : 0u;
+    bool stored = false;  // lead: a bulk store of chain `stored_lc` is in flight
+    int stored_lc = 0, stored_seq = 0;
+    int kept_s = 0;
 
-    for (int s = 0; s < I.n_sweeps; ++s) {
-        const uint32_t t = (uint32_t)(I.t0 + s);
-        for (int lc = grp < ngroups ? grp : c_count; lc < c_count; lc += ngroups) {  // threads past the last group idle
-            const int rho = c_begin + lc;
-            int8_t* buf = reinterpret_cast<int8_t*>(s_chains + (size_t)(I.resident ? lc : grp) * L.chain_stride);
-            if (!I.resident) {
-                if (p16)
-                    load_split16(buf, I.spins + (size_t)rho * I.slot_stride, N, P, P >> 4, hinv, gtid, gsize);
-                else
-                    load_split(buf, I.spins + (size_t)rho * I.slot_stride, N, P, G, ginv, gtid, gsize);
-            }
-            const int rung = s_rung[rho];
-            const uint32_t thr_c = thr_base<WIDE>(
-                (uint32_t)L.thr + 4u * (uint32_t)L.thr_words * (uint32_t)(I.thr_resident ? rung : grp), I.Lmax);
-            if (I.thr_resident) {
-                if (!I.resident) group_sync(bar, gsize);  // the streamed chain is in place
+    for (;;) {
+        // ---- the next task, its chain's last sweep and that sweep's swap decision
+        int s = 0, lc = grp, rung = 0, stop = 0;
+        if (grp >= ngroups || c_count == 0 || (keep && grp >= c_count)) break;
+        if (lead) {
+            if (keep) {
+                s = kept_s++;
+                stop = s > I.n_sweeps;
             } else {
-                for (int l = gtid; l <= 2 * I.Lmax; l += gsize)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) thr_g[c * index.S + l] = I.thr[(size_t)rung * I.nL3 + 3 * l + c];
-                group_sync(bar, gsize);
-            }
-            FlipSums sums;
-            sums.clear();
-            for (int lev = 0; lev < I.n_levels; ++lev) {
-                const int base = s_loff[lev];
-                if (g_fixed) {
-                    // this thread's column never changes (see the single-problem kernel)
-                    if (g_own < U) {
-                        const int end = s_loff[lev + 1];
-                        for (int q = base + q_lane; q < end; q += q_step) {
-                            const UnitEval<W> e =
-                                unit_eval<DC, W, false, WIDE>(buf, s_sdesc, s_items[q], off_own, nullptr, t, (uint32_t)rho,
-                                                        (uint32_t)(W * g_own), rule, skey);
-                            uint32_t F[W];
-                            unit_flips<W, false, WIDE>(e, smem, rule, thr_c, F);
-                            unit_commit<W>(e, F, sums);
-                        }
+                if (stored) {
+                    // the chain is back in global memory before its next task may load it
+                    if (lane == 0) {
+                        bulk_stores_done();
+                        fence_async();
+                        __threadfence_block();
+                        *(volatile int*)&s_seq[stored_lc] = stored_seq;
                     }
-                } else {
-                    const int units = (s_loff[lev + 1] - base) << lg;
-                    for (int u = gtid; u < units; u += gsize) {
-                        const int g = u & gmask;
-                        if (g >= U) continue;
-                        const UnitEval<W> e =
-                            unit_eval<DC, W, false, WIDE>(buf, s_sdesc, s_items[base + (u >> lg)],
-                                                    row_offsets<W>((uint32_t)g, half), nullptr, t, (uint32_t)rho,
-                                                    (uint32_t)(W * g), rule, skey);
-                        uint32_t F[W];
-                        unit_flips<W, false, WIDE>(e, smem, rule, thr_c, F);
-                        unit_commit<W>(e, F, sums);
+                    stored = false;
+                }
+                int task = 0;
+                if (lane == 0) task = atomicAdd(&sh.next, 1);
+                task = __shfl_sync(0xFFFFFFFFu, task, 0);
+                s = task / c_count;
+                lc = task - s * c_count;
+                stop = s > I.n_sweeps;
+                if (!stop && s > 0) {
+                    volatile int* seq = s_seq + lc;
+                    stop = !wait_for(sh, status, [&] { return *seq >= s; });
+                    __threadfence_block();
+                }
+            }
+            if (!stop) {
+                rung = s_rung[lc];
+                if (s > 0 && sps > 0 && s % sps == 0) {
+                    // the pass after sweep s - 1
+                    const int pass = s / sps - 1;
+                    const long long q = I.q0 + pass;
+                    const int rl = (rung & 1) == (int)(q & 1) ? rung : rung - 1;
+                    const bool lower = rl == rung;
+                    const int partner = lower ? rung + 1 : rl;
+                    if (rl >= 0 && rl + 1 < R) {
+                        const unsigned long long tag = mbox_tag(qmod0, pass);
+                        const unsigned long long* mb =
+                            mail + ((size_t)(pass & (kClusterMailPasses - 1)) * R + partner) * 2;
+                        unsigned long long wa = 0, wb = 0;
+                        stop = !wait_for(sh, status, [&] {
+                            if (I.mail_smem) {
+                                wa = ld_cluster_local_u64(mb);
+                                wb = ld_cluster_local_u64(mb + 1);
+                            } else {
+                                wa = ld_relaxed_u64(mb);
+                                wb = ld_relaxed_u64(mb + 1);
+                            }
+                            return (wa & 0xFFFFFFull) == tag && (wb & 0xFFFFFFull) == tag;
+                        });
+                        const long long E = s_E[lc], M = s_M[lc];
+                        const long long pE = (long long)wa >> 24, pM = (long long)(int32_t)(uint32_t)(wb >> 32);
+                        const bool acc = swap_accept_fast(lower ? E : pE, lower ? pE : E, lower ? M : pM,
+                                                          lower ? pM : M, I.coef[rl], I.coef[(R - 1) + rl],
+                                                          (uint32_t)q, (uint32_t)rl,
+                                                          philox_schedule(I.key0, I.key1), false);
+                        if (!stop) {
+                            if (lower && lane < (acc ? 2 : 1)) atomicAdd(I.swap_stats + 2 * rl + lane, 1ull);
+                            if (acc) rung = partner;
+                        }
+                        __syncwarp();
+                        if (lane == 0) s_rung[lc] = rung;
                     }
                 }
-                group_sync(bar, gsize);
             }
-            const int dE = __reduce_add_sync(0xFFFFFFFFu, sums.dE(rule));
-            const int dM = __reduce_add_sync(0xFFFFFFFFu, sums.dM(rule));
-            const int nf = __reduce_add_sync(0xFFFFFFFFu, sums.flips());
+        }
+        if (!one_warp) {
+            if (lead && lane == 0) {
+                ctl_g[0] = s;
+                ctl_g[1] = lc;
+                ctl_g[2] = rung;
+                ctl_g[3] = stop;
+            }
+            group_sync(bar, gsize);
+            s = ctl_g[0];
+            lc = ctl_g[1];
+            rung = ctl_g[2];
+            stop = ctl_g[3];
+        } else {
+            __syncwarp();
+        }
+        if (stop) break;
+        if (s == I.n_sweeps) {  // only the last pass's decision was left
+            if (!one_warp) group_sync(bar, gsize);  // everyone has read the group's control words
+            continue;
+        }
+
+        // ---- the chain, and its rung's thresholds
+        const int rho = c_begin + lc;
+        int8_t* g_chain = I.spins + (size_t)rho * I.slot_stride;
+        int8_t* buf = reinterpret_cast<int8_t*>(s_chains + (size_t)(I.resident ? lc : grp) * L.chain_stride);
+        const bool bulk_in = !I.resident && s > 0;
+        if (bulk_in) {
+                // the chain in its shared-memory form, as an earlier sweep's bulk store left it
+            if (lead && lane == 0) {
+                fence_async();
+                bulk_load(buf, g_chain, (uint32_t)L.chain_stride, &sh.mbar[grp]);
+            }
+        } else if (!I.resident) {
+            load_chain(I, buf, g_chain, gtid, gsize);
+        }
+        const uint32_t thr_c = (uint32_t)L.thr + 4u * (uint32_t)L.thr_words * (uint32_t)(I.thr_resident ? rung : grp);
+        if (!I.thr_resident)
+            for (int l = gtid; l <= 2 * I.Lmax; l += gsize)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) thr_g[c * index.S + l] = I.thr[(size_t)rung * I.nL3 + 3 * l + c];
+        if (bulk_in) {
+            // (the copy completes by itself; the limit only bounds the wait)
+            const unsigned long long start = globaltimer_ns();
+            while (!mbar_try_wait(&sh.mbar[grp], phase)) {
+                if ((long long)(globaltimer_ns() - start) > kBatchWaitNs) {
+                    if (status) atomicCAS(status, 0, PT_ETIMEDOUT);
+                    *(volatile int*)&sh.abort = 1;
+                    break;
+                }
+            }
+            phase ^= 1u;
+        }
+        group_sync(bar, gsize);
+
+        // ---- sweep s
+        const ChainSweep job = {(uint32_t)L.sdesc, (uint32_t)L.items, (uint32_t)L.loff, thr_c,
+                                (uint32_t)(L.chains + (size_t)(I.resident ? lc : grp) * L.chain_stride),
+                                I.key0, I.key1, (uint32_t)(I.t0 + s), (uint32_t)rho, I.n_levels, I.Lmax, P, gsize,
+                                gtid, bar};
+        const ChainChange ch =
+            I.dc == 4 ? sweep_form<4>(job, I.form, index.wide) : sweep_form<8>(job, I.form, index.wide);
+
+        // ---- the chain back (a bulk store takes it in its shared-memory form; the last sweep's
+        // is converted again), and the sweep's statistics and publication
+        const bool last = s + 1 == I.n_sweeps;
+        if (!I.resident) {
+            if (!last) {
+                fence_async();  // this thread's flips, for the copy the lead starts
+            } else {
+                store_chain(I, g_chain, buf, gtid, gsize);
+            }
+        }
+        int dE = __reduce_add_sync(0xFFFFFFFFu, ch.dE);
+        int dM = __reduce_add_sync(0xFFFFFFFFu, ch.dM);
+        int nf = __reduce_add_sync(0xFFFFFFFFu, ch.flips);
+        if (!one_warp) {
             if (lane == 0) {
                 red_g[gwarp * 3 + 0] = dE;
                 red_g[gwarp * 3 + 1] = dM;
                 red_g[gwarp * 3 + 2] = nf;
             }
-            if (!I.resident) {
-                if (p16)
-                    store_split16(I.spins + (size_t)rho * I.slot_stride, buf, N, P, P >> 4, hinv, gtid, gsize);
-                else
-                    store_split(I.spins + (size_t)rho * I.slot_stride, buf, N, P, G, ginv, gtid, gsize);
-            }
             group_sync(bar, gsize);
-            if (gtid == 0) {
-                long long sE = 0, sM = 0, sF = 0;
+        } else {
+            __syncwarp();
+        }
+        if (lead) {
+            if (!I.resident && !last) {
+                if (lane == 0) bulk_store(g_chain, buf, (uint32_t)L.chain_stride);
+                stored = true;
+                stored_lc = lc;
+                stored_seq = s + 1;
+            }
+            if (!one_warp) {
+                dE = dM = nf = 0;
                 for (int w = 0; w < gsize / 32; ++w) {
-                    sE += red_g[w * 3 + 0];
-                    sM += red_g[w * 3 + 1];
-                    sF += red_g[w * 3 + 2];
+                    dE += red_g[w * 3 + 0];
+                    dM += red_g[w * 3 + 1];
+                    nf += red_g[w * 3 + 2];
                 }
-                const long long E = s_E[lc] + sE, M = s_M[lc] + sM;
+            }
+            const long long E = s_E[lc] + dE, M = s_M[lc] + dM;
+            __syncwarp();
+            if (lane == 0) {
                 s_E[lc] = E;
                 s_M[lc] = M;
-                unsigned long long* a = I.acc + (size_t)rung * kAccCount;
-                atomicAdd(a + kAccN, 1ull);
-                atomicAdd(a + kAccE, (unsigned long long)E);
-                atomicAdd(a + kAccE2, (unsigned long long)(E * E));
-                atomicAdd(a + kAccM, (unsigned long long)M);
-                atomicAdd(a + kAccM2, (unsigned long long)(M * M));
-                atomicAdd(a + kAccFlip, (unsigned long long)sF);
             }
-            group_sync(bar, gsize);
-        }
-        __syncthreads();
-        if (I.sweeps_per_swap > 0 && (s + 1) % I.sweeps_per_swap == 0) {
-            const int pass = (s + 1) / I.sweeps_per_swap - 1;
-            const long long q = I.q0 + pass;
-            const int pb = pass & 1;
-            for (int lc = tid; lc < c_count; lc += nt) s_pub[pb * C + lc] = make_longlong2(s_E[lc], s_M[lc]);
-            if (K == 1)
-                __syncthreads();
-            else
-                cluster.sync();
-            for (int rl = (int)(q & 1) + 2 * tid; rl + 1 < R; rl += 2 * nt) {
-                const int X = s_slot[rl], Y = s_slot[rl + 1];
-                const longlong2 px = K == 1 ? s_pub[pb * C + X] : cluster.map_shared_rank(s_pub, X / C)[pb * C + X % C];
-                const longlong2 py = K == 1 ? s_pub[pb * C + Y] : cluster.map_shared_rank(s_pub, Y / C)[pb * C + Y % C];
-                const bool acc = swap_accept_fast(px.x, py.x, px.y, py.y, I.coef[rl], I.coef[(R - 1) + rl],
-                                                  (uint32_t)q, (uint32_t)rl, skey, false);
-                if (rank == 0) {
-                    atomicAdd(I.swap_stats + 2 * rl, 1ull);
-                    if (acc) atomicAdd(I.swap_stats + 2 * rl + 1, 1ull);
-                }
-                if (acc) {
-                    s_slot[rl] = Y;
-                    s_slot[rl + 1] = X;
-                    s_rung[X] = rl + 1;
-                    s_rung[Y] = rl;
+            if (sps > 0 && (s + 1) % sps == 0) {
+                const int pass = (s + 1) / sps - 1;
+                const unsigned long long tag = mbox_tag(qmod0, pass);
+                const unsigned long long wa = ((unsigned long long)E << 24) | tag;
+                const unsigned long long wb = ((unsigned long long)(uint32_t)(int32_t)M << 32) | tag;
+                unsigned long long* slot = mail + ((size_t)(pass & (kClusterMailPasses - 1)) * R + rung) * 2;
+                if (I.mail_smem) {
+                    if (lane < K) st_cluster_u64x2(slot, (unsigned)lane, wa, wb);
+                } else if (lane < 2) {
+                    st_relaxed_u64(slot + lane, lane == 0 ? wa : wb);
                 }
             }
-            __syncthreads();
+            if (lane < kAccCount) {
+                unsigned long long v = 1ull;
+                if (lane == kAccE) v = (unsigned long long)E;
+                if (lane == kAccE2) v = (unsigned long long)(E * E);
+                if (lane == kAccM) v = (unsigned long long)M;
+                if (lane == kAccM2) v = (unsigned long long)(M * M);
+                if (lane == kAccFlip) v = (unsigned long long)(long long)nf;
+                atomicAdd(I.acc + (size_t)rung * kAccCount + lane, v);
+            }
+            __syncwarp();
+            if (!keep && !stored && lane == 0) {  // (a chain being stored is marked when it has arrived)
+                __threadfence_block();
+                *(volatile int*)&s_seq[lc] = s + 1;
+            }
         }
     }
+    if (lead && stored && lane == 0) bulk_stores_done();  // only after a wait that gave up
+    __syncthreads();
+    if (gtid == 0 && grp < ngroups && grp < 16) sh.phase[grp] = phase;
 
     // ---- write the problem back
     for (int x = tid; x < c_count; x += nt) {
         I.E[c_begin + x] = s_E[x];
         I.M[c_begin + x] = s_M[x];
+        I.rung_of_slot[c_begin + x] = s_rung[x];
+        I.slot_of_rung[s_rung[x]] = c_begin + x;
     }
-    if (I.resident) {
+    if (I.resident)
         for (int lc = 0; lc < c_count; ++lc)
-            store_split(I.spins + (size_t)(c_begin + lc) * I.slot_stride,
-                        reinterpret_cast<const int8_t*>(s_chains + (size_t)lc * L.chain_stride), N, P, G, ginv, tid,
-                        nt);
-    }
-    if (rank == 0) {
-        for (int x = tid; x < R; x += nt) {
-            I.rung_of_slot[x] = s_rung[x];
-            I.slot_of_rung[x] = s_slot[x];
-        }
-    }
-}
-
-__device__ __forceinline__ void run_any(const BatchInstance& I, unsigned char* smem, uint4* s_keys,
-                                        cg::cluster_group& cluster, int rank, int K) {
-    if (IndexRule(I.Lmax).wide) {  // large couplings: one instantiation a class
-        if (I.dc == 4)
-            run_problem<4, 1, true>(I, smem, s_keys, cluster, rank, K);
-        else
-            run_problem<8, 1, true>(I, smem, s_keys, cluster, rank, K);
-    } else if (I.dc == 4) {
-        if (I.unit_words == 4)
-            run_problem<4, 4, false>(I, smem, s_keys, cluster, rank, K);
-        else if (I.unit_words == 2)
-            run_problem<4, 2, false>(I, smem, s_keys, cluster, rank, K);
-        else
-            run_problem<4, 1, false>(I, smem, s_keys, cluster, rank, K);
-    } else {
-        if (I.unit_words == 4)
-            run_problem<8, 4, false>(I, smem, s_keys, cluster, rank, K);
-        else if (I.unit_words == 2)
-            run_problem<8, 2, false>(I, smem, s_keys, cluster, rank, K);
-        else
-            run_problem<8, 1, false>(I, smem, s_keys, cluster, rank, K);
-    }
+            store_chain(I, I.spins + (size_t)(c_begin + lc) * I.slot_stride,
+                        reinterpret_cast<const int8_t*>(s_chains + (size_t)lc * L.chain_stride), tid, nt);
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_job;
-    __shared__ uint4 s_keys[5];  // round keys, two rounds per word
+    __shared__ BatchShared sh;
+    if (threadIdx.x < 16) {
+        mbar_init(&sh.mbar[threadIdx.x]);
+        sh.phase[threadIdx.x] = 0u;
+    }
+    if (threadIdx.x == 0) sh.abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async();
+    __syncthreads();
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int K = (int)cluster.num_blocks();
     if (bp.single) {
         // one problem on this one cluster; the host keeps its counters
-        run_any(bp.one, smem, s_keys, cluster, rank, K);
+        run_problem(bp.one, smem, sh, cluster, rank, K, bp.status);
         if (K > 1) cluster.sync();  // peers are done reading this CTA's published (E, M)
         return;
     }
     for (;;) {
-        if (rank == 0 && threadIdx.x == 0) s_job = atomicAdd(bp.next_job, 1);
+        if (rank == 0 && threadIdx.x == 0) sh.job = atomicAdd(bp.next_job, 1);
         cluster.sync();
-        const int job = *cluster.map_shared_rank(&s_job, 0);
-        cluster.sync();  // every CTA has read the job before rank 0 may reuse or release s_job
+        const int job = *cluster.map_shared_rank(&sh.job, 0);
+        cluster.sync();  // every CTA has read the job before rank 0 may reuse or release sh.job
         if (job >= bp.count) break;
         const BatchInstance I = bp.inst[bp.order[job]];
-        run_any(I, smem, s_keys, cluster, rank, K);
+        run_problem(I, smem, sh, cluster, rank, K, bp.status);
         cluster.sync();  // peers are done reading this CTA's published (E, M)
         if (rank == 0 && threadIdx.x == 0) {
             // a finished problem's counters advance on the device, so the same launch can be
@@ -474,13 +725,14 @@ size_t batch_smem_cap() {
     return (size_t)max_smem - 1024;  // room for the kernel's static shared memory
 }
 
-cudaError_t launch_batch_single(const BatchInstance& I, int cluster, int threads, size_t smem, cudaStream_t s) {
+cudaError_t launch_batch_single(const BatchInstance& I, int cluster, int threads, size_t smem, int* status,
+                                cudaStream_t s) {
     BatchParams bp;
     bp.inst = nullptr;
     bp.order = nullptr;
     bp.count = 1;
     bp.next_job = nullptr;
-    bp.status = nullptr;
+    bp.status = status;
     bp.single = 1;
     bp.one = I;
     return launch_batch(bp, cluster, 1, threads, smem, s);
@@ -581,6 +833,68 @@ static cudaError_t balloc(pt_batch* b, T** ptr, size_t bytes) {
     return cudaSuccess;
 }
 
+// Instructions of a unit, by class of neighbour slots and form (measured whole, per unit-warp).
+static const int kFormInstr[2][kFormCount] = {{118, 200, 352, 384, 704}, {134, 228, 400, 448, 816}};
+
+// The form with the least work for a chain that a warp sweeps, and the level schedule balanced
+// for it. A wider unit costs less per copy (one descriptor, one address and one load per
+// neighbour for more copies), and bit words are a quarter or an eighth of the bytes, so that
+// more chains are resident and every warp gets a chain of its own; but a level gives fewer
+// units to spread over a warp's lanes. So: the least warp rounds x instructions of a unit,
+// times what fewer or wider groups cost when 16 one-warp groups' chains do not fit (measured:
+// 1.8 cycles an instruction with 16 one-warp groups, 2.2 with groups of four or eight warps).
+static void choose_form(Prepared& pr, const std::vector<std::vector<int>>& adj, int per_round) {
+    const int P = pr.P;
+    double best = 0.0;
+    pr.form = -1;
+    int best_round = 1;
+    for (int form = 0; form < kFormCount; ++form) {
+        const int copies = form_unit_copies(form);
+        if (P % (2 * copies)) continue;
+        if (form >= kFormNibbles && pr.Lmax > kWordBitsLmax) continue;
+        if (form > kFormBytes1 && form < kFormNibbles && IndexRule(pr.Lmax).wide) continue;
+        int cols = 1;
+        while (cols < P / (2 * copies)) cols <<= 1;
+        // balanced levels fill whole rounds, but for the last of about every third level
+        const double rounds = std::max<double>(pr.n_levels, 2.0 * pr.N * cols / 32.0 + 0.35 * pr.n_levels);
+        const size_t chain = (size_t)pr.N * form_row_bytes(form, P);
+        const size_t fixed = (size_t)pr.N * (pr.dc == 4 ? 40 : 56) + 16384;
+        const size_t fit = fixed < 230000 ? (230000 - fixed) / std::max<size_t>(chain, 16) : 0;
+        const double spread = fit >= 16 ? 1.0 : (fit >= 10 ? 1.05 : (fit >= 2 ? 1.25 : 1.4));
+        const double cost = rounds * kFormInstr[pr.dc == 4 ? 0 : 1][form] * spread;
+        if (pr.form < 0 || cost < best) {
+            best = cost;
+            pr.form = form;
+            best_round = std::max(1, 32 / cols);
+        }
+    }
+    if (pr.form == kFormBytes1 && best_round == per_round) {
+        pr.titems = pr.items;
+        pr.tlevel_off = pr.level_off;
+    } else {
+        level_schedule(pr.N, adj, pr.titems, pr.tlevel_off, best_round, (int)(form_row_bytes(pr.form, P) / 4));
+    }
+}
+
+// Cycles a CTA takes for one sweep of its C chains in a form, by this model: a level of average
+// size takes rounds of units on the group; a round takes a warp's latency, 5.5 cycles an
+// instruction, or the issue of all the warps at work on a scheduler, 1.65 each; plus 150 cycles
+// a level for its loop and barrier, and 4000 a chain and sweep for the task, its statistics
+// and the swap decision. (Against 24 measured runs, N = 64 to 512 on clusters of 1 to 8, it is
+// off by at most 20 %, and names the faster of the two forms but for near ties.)
+static double sweep_cycles(const BatchInstance& I, int C) {
+    const int instr = kFormInstr[I.dc == 4 ? 0 : 1][I.form];
+    int cols = 1;
+    while (cols < I.P / (2 * form_unit_copies(I.form))) cols <<= 1;
+    const double g = I.group_threads;
+    const double units = 2.0 * I.N / std::max(1, I.n_levels) * cols;
+    const double full = std::floor(units / g), rest = std::ceil((units - full * g) / 32.0);
+    const int groups = std::min(C, I.n_groups);
+    auto round = [&](double warps) { return instr * std::max(5.5, 1.65 * groups * warps / 4.0); };
+    const double level = full * round(g / 32.0) + (rest > 0.0 ? round(rest) : 0.0) + 150.0;
+    return (I.n_levels * level + 4000.0) * std::max(1.0, (double)C / I.n_groups);
+}
+
 int ptq::prepare_request(const pt_request& r, Prepared& pr, char* why, size_t why_len, int per_round) {
     const pt_instance* inst = &r.inst;
     const int N = inst->n, nE = inst->n_edges, P = r.P, R = r.R;
@@ -664,7 +978,10 @@ int ptq::prepare_request(const pt_request& r, Prepared& pr, char* why, size_t wh
     if (pr.coef.size() < 2) pr.coef.assign(2, 0.0);
     level_schedule(N, adj, pr.items, pr.level_off, per_round, P / 4);  // rows of P bytes (int8 packed)
     pr.n_levels = (int)pr.level_off.size() - 1;
+    choose_form(pr, adj, per_round);
     build_site_desc(N, P, pr.dc, Lmax, adj, adjJ, inst->h, pr.sdesc);
+    if (pr.form >= kFormNibbles)
+        build_site_desc(N, (int)form_row_bytes(pr.form, P), pr.dc, Lmax, adj, adjJ, inst->h, pr.wdesc, true);
     return PT_OK;
 }
 
@@ -677,8 +994,11 @@ size_t ptq::request_block_layout(Prepared& p, size_t mailbox_entries) {
         return o;
     };
     p.off_sdesc = take(p.sdesc.size() * 4);
+    p.off_wdesc = take(p.wdesc.size() * 4);
     p.off_items = take(p.items.size() * 4);
     p.off_loff = take(p.level_off.size() * 4);
+    p.off_titems = take(p.titems.size() * 4);
+    p.off_tloff = take(p.tlevel_off.size() * 4);
     p.off_thr = take(p.thr.size() * 4);
     p.off_coef = take(p.coef.size() * 8);
     p.off_spins = take((size_t)p.R * p.slot_stride);
@@ -704,14 +1024,18 @@ void ptq::fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base
     I.nL3 = (2 * p.Lmax + 1) * 3;
     I.n_levels = p.n_levels;
     I.dc = p.dc;
+    I.form = I.form_t = p.form;
     I.slot_stride = p.slot_stride;
     I.key0 = (uint32_t)(r.seed & 0xFFFFFFFFu);
     I.key1 = (uint32_t)(r.seed >> 32);
     I.n_sweeps = (int)r.n_sweeps;
     I.sweeps_per_swap = r.sweeps_per_swap;
     I.sdesc = (const uint32_t*)(base + p.off_sdesc);
+    I.wdesc = (const uint32_t*)(base + p.off_wdesc);
     I.items = (const uint32_t*)(base + p.off_items);
     I.level_off = (const int32_t*)(base + p.off_loff);
+    I.titems = (const uint32_t*)(base + p.off_titems);
+    I.tlevel_off = (const int32_t*)(base + p.off_tloff);
     I.thr = (const uint32_t*)(base + p.off_thr);
     I.coef = (const double*)(base + p.off_coef);
     I.spins = (int8_t*)(base + p.off_spins);
@@ -721,34 +1045,10 @@ void ptq::fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base
     I.slot_of_rung = (int32_t*)(base + p.off_slot);
     I.acc = (unsigned long long*)(base + p.off_acc);
     I.swap_stats = (unsigned long long*)(base + p.off_sw);
+    I.mail = (Mailbox*)(base + p.off_mbox);
 }
 
-// A wider unit costs less per copy (one descriptor, address and wide load per neighbour for
-// more copies; measured in isolation at 186, 166 and 146 cycles per four copies and warp for
-// 1, 2 and 4 words) but gives a level fewer units to spread over the group, so the width is
-// the one with the least rounds x cost on a level of average size. Rows' halves have to be
-// whole units.
-int ptq::choose_unit_words(const BatchInstance& I, int group_threads) {
-    if (IndexRule(I.Lmax).wide) return 1;
-    static const int kCost[3] = {186, 332, 584};
-    const double items = 2.0 * I.N / std::max(1, I.n_levels);
-    int best = 1;
-    double best_cost = 0.0;
-    for (int k = 0; k < 3; ++k) {
-        const int W = 1 << k;
-        if (I.P % (8 * W)) break;
-        int cols = 1;
-        while (cols < I.P / (8 * W)) cols <<= 1;
-        const double cost = std::ceil(items * cols / group_threads) * kCost[k];
-        if (k == 0 || cost < best_cost) {
-            best = W;
-            best_cost = cost;
-        }
-    }
-    return best;
-}
-
-void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen) {
+static void groups_of_form(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen) {
     // threads per chain: about one 4-copy unit per thread in an average level, at least two
     // warps, and no more groups than a CTA has chains; chains stay resident when they fit.
     // widen > 0 doubles the group that many times (fewer chains at once, shorter levels);
@@ -773,22 +1073,40 @@ void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_
     // chains still fit; resident chains come first
     const int thr_words = (int)(up16((size_t)IndexRule(I.Lmax).row_words() * 4) / 4);
     const int thr_ok = (size_t)I.R * thr_words * 4 <= 49152 ? 1 : 0;
-    for (;;) {
+    for (bool ok = false; !ok;) {
+        // resident chains come first, then threshold rows, then the swap mailboxes; with chains
+        // streamed through one buffer a group, a few groups less than the CTA's warps could
+        // form are better than wider ones (at least five eighths of the warps at work)
         I.group_threads = g;
-        I.resident = 1;
-        I.thr_resident = thr_ok;
-        if (batch_smem_bytes(I, cluster, threads) <= smem_cap) break;
-        I.thr_resident = 0;
-        if (batch_smem_bytes(I, cluster, threads) <= smem_cap) break;
-        I.resident = 0;
-        I.thr_resident = thr_ok;
-        if (batch_smem_bytes(I, cluster, threads) <= smem_cap) break;
-        I.thr_resident = 0;
-        if (batch_smem_bytes(I, cluster, threads) <= smem_cap || !up_ok(g)) break;
-        g <<= 1;  // one streaming buffer per group: fewer, larger groups
+        const int most = threads / g, least = std::max(1, (5 * most + 7) / 8);
+        for (int n = most; n >= least && !ok; --n) {
+            I.n_groups = n;
+            for (int k = n == most ? 0 : 4; k < 8 && !ok; ++k) {
+                I.resident = k < 4 ? 1 : 0;
+                I.thr_resident = (k & 2) ? 0 : thr_ok;
+                I.mail_smem = (k & 1) ? 0 : 1;
+                ok = batch_smem_bytes(I, cluster, threads) <= smem_cap;
+            }
+        }
+        if (ok || !up_ok(g)) break;
+        g <<= 1;
         while (up_ok(g) && threads / g > 15) g <<= 1;
     }
-    I.unit_words = choose_unit_words(I, I.group_threads);
+}
+
+void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen) {
+    // the form for one-warp groups, or four-copy units where a CTA has few chains and wide
+    // groups sweep them
+    const int C = (I.R + cluster - 1) / cluster;
+    I.form = I.form_t;
+    groups_of_form(I, cluster, threads, smem_cap, widen);
+    if (I.form_t == kFormBytes1) return;
+    BatchInstance F = I;
+    F.form = kFormBytes1;
+    groups_of_form(F, cluster, threads, smem_cap, widen);
+    const bool fits_t = batch_smem_bytes(I, cluster, threads) <= smem_cap;
+    const bool fits_f = batch_smem_bytes(F, cluster, threads) <= smem_cap;
+    if (fits_f && (!fits_t || sweep_cycles(F, C) < sweep_cycles(I, C))) I = F;
 }
 
 // Groups per request, the CTA's shared memory and the persistent grid for one layout.
@@ -850,7 +1168,7 @@ static cudaError_t enqueue_run(pt_batch* b) {
     return launch_batch(bp, b->cluster, b->n_clusters, b->threads, b->smem, b->stream);
 }
 
-// Layout autotuner: times a short run (1 % of every request's sweeps, at least one) for
+// Layout autotuner: times a short run (1 % of every request's sweeps, at least two) for
 // each cluster size and group width that fits and keeps the fastest. The layout changes
 // which CTA sweeps which chain and when, never the arithmetic or the random counters, so
 // the choice cannot change any result; the state is reset afterwards.
@@ -859,7 +1177,7 @@ static int autotune(pt_batch* b) {
     std::vector<int> full(b->count);
     for (int k = 0; k < b->count; ++k) {
         full[k] = b->h_inst[k].n_sweeps;
-        b->h_inst[k].n_sweeps = std::max(1, full[k] / 100);
+        b->h_inst[k].n_sweeps = std::min(full[k], std::max(2, full[k] / 100));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
@@ -867,9 +1185,18 @@ static int autotune(pt_batch* b) {
     float best_ms = 0.f;
     int best_c = 0, best_w = 0, timed = 0;
     char why[200];
-    for (int ci = 0; ci < 4 && e == cudaSuccess; ++ci) {
+    std::vector<int> shape, seen;
+    // wider groups, then wider clusters, are tried while they are not clearly losing
+    bool wider = true;
+    for (int ci = 0; ci < 4 && e == cudaSuccess && wider; ++ci) {
+        seen.clear();
+        float cluster_ms = 0.f;
         for (int w = -4; w < 2 && e == cudaSuccess; ++w) {
             if (plan_layout(b, kClusters[ci], w, why, sizeof(why)) != PT_OK) continue;
+            shape.clear();
+            for (const BatchInstance& I : b->h_inst) shape.push_back(I.group_threads);
+            if (shape == seen) continue;  // the groups of the width before
+            seen = shape;
             for (int rep = 0; rep < (timed == 0 ? 2 : 1) && e == cudaSuccess; ++rep) {  // first: one warm-up
                 for (BatchInstance& I : b->h_inst) I.t0 = I.q0 = 0;
                 if ((e = cudaMemcpyAsync(b->d_inst, b->h_inst.data(), sizeof(BatchInstance) * b->count,
@@ -888,7 +1215,10 @@ static int autotune(pt_batch* b) {
                 best_w = w;
             }
             ++timed;
+            if (cluster_ms > 0.f && ms > 1.25f * cluster_ms) break;
+            cluster_ms = cluster_ms > 0.f ? std::min(cluster_ms, ms) : ms;
         }
+        wider = cluster_ms <= 0.f || cluster_ms <= 1.5f * best_ms;
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
@@ -915,8 +1245,7 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
     {
         // Requests are prepared independently (checks, tables, level schedule, descriptors),
         // on up to 16 host threads; the first failing request in index order is reported.
-        // Levels are balanced for one-warp chain groups (the default and the usual autotuned
-        // width): 32 threads over the power-of-two word columns of an item.
+        // Levels are balanced for one-warp chain groups (the default and the usual autotuned width).
         std::vector<int> rcs(count, PT_OK);
         std::vector<std::string> whys(count);
         auto work = [&](int first, int step) {
@@ -985,8 +1314,11 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
     for (int k = 0; k < count; ++k) {
         Prepared& p = pr[k];
         p.off_sdesc = take(p.sdesc.size() * 4);
+        p.off_wdesc = take(p.wdesc.size() * 4);
         p.off_items = take(p.items.size() * 4);
         p.off_loff = take(p.level_off.size() * 4);
+        p.off_titems = take(p.titems.size() * 4);
+        p.off_tloff = take(p.tlevel_off.size() * 4);
         p.off_thr = take(p.thr.size() * 4);
         p.off_coef = take(p.coef.size() * 8);
     }
@@ -1000,6 +1332,7 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
         p.off_slot = take((size_t)p.R * 4);
         p.off_acc = take((size_t)p.R * kAccCount * 8);
         p.off_sw = take((size_t)p.R * 16);
+        p.off_mbox = take((size_t)kClusterMailPasses * p.R * sizeof(Mailbox));
         max_state = std::max(max_state, (size_t)p.R * p.N * p.P);
         BatchInstance& I = b->h_inst[k];
         memset(&I, 0, sizeof(I));
@@ -1010,6 +1343,7 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
         I.nL3 = (2 * p.Lmax + 1) * 3;
         I.n_levels = p.n_levels;
         I.dc = p.dc;
+        I.form = I.form_t = p.form;
         I.slot_stride = p.slot_stride;
         I.key0 = (uint32_t)(reqs[k].seed & 0xFFFFFFFFu);
         I.key1 = (uint32_t)(reqs[k].seed >> 32);
@@ -1056,14 +1390,20 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
     for (int k = 0; k < count; ++k) {
         Prepared& p = pr[k];
         memcpy(&host_const[p.off_sdesc], p.sdesc.data(), p.sdesc.size() * 4);
+        if (!p.wdesc.empty()) memcpy(&host_const[p.off_wdesc], p.wdesc.data(), p.wdesc.size() * 4);
         memcpy(&host_const[p.off_items], p.items.data(), p.items.size() * 4);
         memcpy(&host_const[p.off_loff], p.level_off.data(), p.level_off.size() * 4);
+        memcpy(&host_const[p.off_titems], p.titems.data(), p.titems.size() * 4);
+        memcpy(&host_const[p.off_tloff], p.tlevel_off.data(), p.tlevel_off.size() * 4);
         memcpy(&host_const[p.off_thr], p.thr.data(), p.thr.size() * 4);
         memcpy(&host_const[p.off_coef], p.coef.data(), p.coef.size() * 8);
         BatchInstance& I = b->h_inst[k];
         I.sdesc = (const uint32_t*)(arena + p.off_sdesc);
+        I.wdesc = (const uint32_t*)(arena + p.off_wdesc);
         I.items = (const uint32_t*)(arena + p.off_items);
         I.level_off = (const int32_t*)(arena + p.off_loff);
+        I.titems = (const uint32_t*)(arena + p.off_titems);
+        I.tlevel_off = (const int32_t*)(arena + p.off_tloff);
         I.thr = (const uint32_t*)(arena + p.off_thr);
         I.coef = (const double*)(arena + p.off_coef);
         I.spins = (int8_t*)(arena + p.off_spins);
@@ -1073,6 +1413,7 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
         I.slot_of_rung = (int32_t*)(arena + p.off_slot);
         I.acc = (unsigned long long*)(arena + p.off_acc);
         I.swap_stats = (unsigned long long*)(arena + p.off_sw);
+        I.mail = (Mailbox*)(arena + p.off_mbox);
         for (int rho = 0; rho < p.R; ++rho) map.push_back(make_int2(k, rho));
     }
     // requests with the most work first, so the last ones to finish are small
@@ -1106,6 +1447,15 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
             if (it != g_layout_cache.end()) cached = it->second;
         }
         if (cached.cluster > 0 && plan_layout(b, cached.cluster, cached.widen, why, sizeof(why)) == PT_OK) {
+            // the device records carry the layout too (groups, what is resident): the launch's
+            // shared memory is sized for this one
+            if ((e = cudaMemcpyAsync(b->d_inst, b->h_inst.data(), sizeof(BatchInstance) * count,
+                                     cudaMemcpyHostToDevice, s)) != cudaSuccess ||
+                (e = cudaStreamSynchronize(s)) != cudaSuccess) {
+                free_batch(b);
+                return bfail(nullptr, PT_ECUDA, "batch setup: %s", cudaGetErrorString(e));
+            }
+            b->h2d_bytes += (int64_t)(sizeof(BatchInstance) * count);
             *out = b;
             return PT_OK;
         }
@@ -1138,6 +1488,7 @@ static int bcheck(pt_batch* b) {
     cudaError_t e = cudaMemcpyAsync(st, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(b, PT_ECUDA, "CUDA error: %s", cudaGetErrorString(e));
+    if (*st == PT_ETIMEDOUT) return bfail(b, PT_ETIMEDOUT, "a wait inside the batched kernel timed out");
     if (*st) return bfail(b, PT_ECUDA, "device status %d", *st);
     return PT_OK;
 }

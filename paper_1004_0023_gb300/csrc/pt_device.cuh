@@ -181,6 +181,12 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// Tag of pass q0 + pass, from qmod0 = q0 mod kTagPeriod (taken once per launch): a 32-bit
+// remainder by a constant instead of a 64-bit one on the path to the partner.
+__device__ __forceinline__ unsigned long long mbox_tag(uint32_t qmod0, int pass) {
+    return (unsigned long long)((qmod0 + (uint32_t)pass) % (uint32_t)kTagPeriod) + 1ull;
+}
+
 // ------------------------------------------------------------------------- misc
 __host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
@@ -844,62 +850,81 @@ __device__ __forceinline__ void packed_unit_bits(uint8_t* bp, const uint32_t* s_
     if (F) bp[s.row + ug] = (uint8_t)(own ^ (((fb | (fb >> 12)) & 0x55u) << par));
 }
 
-// Bit-packed chains, one nibble of every byte: a word holds 16 copies of one parity of a site,
-// unit k (of four) as bit k of its four bytes, so that copy 16 c + 4 k + w of that parity is
-// bit 8 w + k of word c; a row is P/32 even words, then P/32 odd ones. A thread takes a whole
-// word: one load per neighbour, one descriptor and one address serve 16 copies, and no other
-// thread writes its word. The one-bit form above costs a byte load and a table load per
-// neighbour and four copies; this one an AND and a multiply-add. The arithmetic is the int8
-// unit's with 0 / 1 bytes: sum_j J_j B_j of unit k comes from the words masked at bit k, that
-// is scaled by 2^k, and is shifted down once the sum is formed. Every byte has to hold
-// 2^k 2 Lmax until then: k <= 2 for Lmax <= 31 (kNibbleLmax), and unit 3 starts from words
-// shifted by 3. Descriptors hold J itself and C4 = h + sum J + Lmax in every byte ("plain").
-// With the Trotter column taken as the count of equal neighbours no index bias is needed.
-struct NibbleSums {
+// Bit-packed chains, whole words: a word holds 4 U copies of one parity of a site (U = 8, or
+// U = 4 with the upper nibbles empty when the copies don't fill words of 32), unit k as bit k
+// of its four bytes: copy 4 U c + 4 k + w of that parity is bit 8 w + k of word c. A row is
+// its even words, then its odd ones. A thread takes a whole word: one load per neighbour, one
+// descriptor and one address serve 4 U copies, and no other thread writes its word. The
+// one-bit form above costs a byte load and a table load per neighbour and four copies; this
+// one an AND and a multiply-add. The arithmetic is the int8 unit's with 0 / 1 bytes:
+// sum_j J_j B_j of unit k comes from the words masked at bit k, that is scaled by 2^k, and is
+// shifted down once the sum is formed. Every byte has to hold 2^k 2 Lmax until then: k <= 2
+// for Lmax <= 31 (kWordBitsLmax), so the units go in threes, each from words shifted by 3
+// more. Descriptors hold J itself and C4 = h + sum J + Lmax in every byte ("plain"). With the
+// Trotter column taken as the count of equal neighbours no index bias is needed.
+struct BitSums {
     int n, L, C;  // minus the sums over flipped copies of 1, L + Lmax and the Trotter column
+    __device__ __forceinline__ void clear() { n = L = C = 0; }
+    __device__ __forceinline__ int dE(int Lmax) const { return 2 * (L - Lmax * n); }
+    __device__ __forceinline__ int dM() const { return 4 * (C - n); }
+    __device__ __forceinline__ int flips() const { return -n; }
 };
-template <int DC, int NS>
-__device__ __forceinline__ void nibble_unit(int8_t* sp, const uint32_t* s_sdesc, uint32_t item, uint32_t c,
-                                            uint32_t cols, uint32_t t, uint32_t slot, const PhiloxKey& key,
-                                            const unsigned char* smem, uint32_t S, uint32_t kM, uint32_t thr,
-                                            NibbleSums& sums) {
+// Row offsets of word c of `cols`: own word, the opposite parity's, and the one its edge copy is
+// in (the word before for even copies, after for odd ones).
+__device__ __forceinline__ UnitOffsets word_offsets(uint32_t c, uint32_t cols) {
+    UnitOffsets o;
+    o.own[0] = 4u * c;
+    o.own[1] = 4u * (cols + c);
+    o.opp[0] = o.own[1];
+    o.opp[1] = o.own[0];
+    o.edge[0] = 4u * (cols + (c == 0u ? cols - 1u : c - 1u));
+    o.edge[1] = 4u * (c + 1u == cols ? 0u : c + 1u);
+    return o;
+}
+template <int DC, int NS, int U>
+__device__ __forceinline__ void bits_unit(int8_t* sp, const uint32_t* s_sdesc, uint32_t item, const UnitOffsets& o,
+                                          uint32_t c, uint32_t t, uint32_t slot, const PhiloxKey& key,
+                                          const unsigned char* smem, uint32_t S, uint32_t kM, uint32_t thr,
+                                          BitSums& sums) {
     const uint32_t par = item & 1u;
     const SiteTerms<DC> s = load_site<DC>(s_sdesc + (item >> 1) * SiteDesc<DC>::DW);
-    const uint32_t own_off = 4u * (par * cols + c), opp = s.row + 4u * (cols - par * cols);
-    // the word the opposite parity's edge copy is in: the one before for even copies, after for odd
-    const uint32_t ce = par ? (c + 1u == cols ? 0u : c + 1u) : (c == 0u ? cols - 1u : c - 1u);
+    const uint32_t own_off = o.own_of(par);
     uint32_t* own = reinterpret_cast<uint32_t*>(sp + s.row + own_off);
     const uint32_t V = *own;
-    const uint32_t O = *reinterpret_cast<const uint32_t*>(sp + opp + 4u * c);
-    const uint32_t E = *reinterpret_cast<const uint32_t*>(sp + opp + 4u * ce);
+    const uint32_t O = *reinterpret_cast<const uint32_t*>(sp + s.row + o.opp_of(par));
+    const uint32_t E = *reinterpret_cast<const uint32_t*>(sp + s.row + o.edge_of(par));
     uint32_t W[NS];
 #pragma unroll
     for (int d = 0; d < NS; ++d) W[d] = *reinterpret_cast<const uint32_t*>(sp + s.off[d] + own_off);
-    uint32_t u[16];
-    unit_words<4, false>(u, item, nullptr, t, slot, 4u * c, key);
     // the opposite parity shifted by one copy: bytes up (even copies) or down (odd copies) by
-    // one, and the byte that comes in from the next unit, its top one from the edge word
-    // (bits above the nibble are never looked at)
-    const uint32_t in = par ? (O >> 1) | (E << 3) : (O >> 23) | (E >> 27);
+    // one, and the byte that comes in from the next unit, its last unit's from the edge word
+    // (with U = 4, bits above the nibble are never looked at)
+    const uint32_t in = par ? ((O >> 1) & (U == 8 ? 0x7Fu : ~0u)) | (E << (U - 1))
+                            : ((O >> 23) & (U == 8 ? ~1u : ~0u)) | (E >> (23 + U));
     const uint32_t sh = prmt(O, in, 0x2104u + par * (0x4321u - 0x2104u));
     uint32_t flip = 0u;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < U; ++k) {
+        uint32_t u[4];
+        unit_words<1, false>(u, item, nullptr, t, slot, (uint32_t)U * c + (uint32_t)k, key);
         const uint32_t mk = 0x01010101u << k;
-        const int ks = k == 3 ? 0 : k;  // the scale of this unit's sum
+        constexpr int kGroup = 3;
+        const int ks = k % kGroup, kb = k - ks;  // the scale of this unit's sum, the words' shift
         uint32_t g = 0u;
 #pragma unroll
-        for (int d = 0; d < NS; ++d) g += s.k[d] * ((k == 3 ? W[d] >> 3 : W[d]) & (0x01010101u << ks));
+        for (int d = 0; d < NS; ++d) g += s.k[d] * ((W[d] >> kb) & (0x01010101u << ks));
         const uint32_t f = ((s.c4 << ks) - 2u * g) >> ks;
-        const uint32_t m = (uint32_t)((int)((V & mk) * 255u) >> k);  // 0xFF where the spin is -1
+        const uint32_t m = prmt(V << (7 - k), 0u, 0xBA98u);  // 0xFF where the spin is -1
         const uint32_t L = (f ^ m) + kM * m;
-        const uint32_t C = ((~(V ^ O) & mk) + (~(V ^ sh) & mk)) >> k;
+        // neighbours equal to the spin; at k = 7 a byte cannot hold both
+        const uint32_t C = k < 7 ? ((~(V ^ O) & mk) + (~(V ^ sh) & mk)) >> k
+                                 : ((~(V ^ O) >> 7) & 0x01010101u) + ((~(V ^ sh) >> 7) & 0x01010101u);
         const uint32_t idx = L + S * C;
         uint32_t F = 0u;
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
             const uint32_t th = *reinterpret_cast<const uint32_t*>(smem + __dp4a(idx, 4u << (8 * w), thr));
-            if (accepts<false>(u[4 * k + w], th)) F |= 0xFFu << (8 * w);
+            if (accepts<false>(u[w], th)) F |= 0xFFu << (8 * w);
         }
         sums.n = dp4a_us(0x01010101u, F, sums.n);
         sums.L = dp4a_us(L, F, sums.L);
@@ -907,6 +932,51 @@ __device__ __forceinline__ void nibble_unit(int8_t* sp, const uint32_t* s_sdesc,
         flip |= F & mk;
     }
     if (flip) *own = V ^ flip;
+}
+
+// Chains between global memory (interleaved +-1 bytes) and bit words, threads tid0, tid0 + nthr, ...
+// taking whole words of both parities: 8 U copies.
+template <int U>
+__device__ __forceinline__ void load_bits(uint32_t* words, const int8_t* chain, int N, int cols, int tid0, int nthr) {
+    const uint4* src = reinterpret_cast<const uint4*>(chain);
+    for (int x = tid0; x < N * cols; x += nthr) {
+        const int i = x / cols, c = x - i * cols;
+        uint4 v[U / 2];
+#pragma unroll
+        for (int y = 0; y < U / 2; ++y) v[y] = src[(U / 2) * x + y];
+        uint32_t even = 0u, odd = 0u;
+#pragma unroll
+        for (int y = 0; y < U / 2; ++y) {
+            uint32_t e, d;
+            split_chunk(make_uint2(v[y].x, v[y].y), e, d);
+            even |= ((e >> 7) & 0x01010101u) << (2 * y);
+            odd |= ((d >> 7) & 0x01010101u) << (2 * y);
+            split_chunk(make_uint2(v[y].z, v[y].w), e, d);
+            even |= ((e >> 7) & 0x01010101u) << (2 * y + 1);
+            odd |= ((d >> 7) & 0x01010101u) << (2 * y + 1);
+        }
+        words[2 * i * cols + c] = even;
+        words[(2 * i + 1) * cols + c] = odd;
+    }
+}
+template <int U>
+__device__ __forceinline__ void store_bits(int8_t* chain, const uint32_t* words, int N, int cols, int tid0, int nthr) {
+    uint4* dst = reinterpret_cast<uint4*>(chain);
+    for (int x = tid0; x < N * cols; x += nthr) {
+        const int i = x / cols, c = x - i * cols;
+        const uint32_t even = words[2 * i * cols + c], odd = words[(2 * i + 1) * cols + c];
+#pragma unroll
+        for (int y = 0; y < U / 2; ++y) {
+            uint2 v[2];
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                const int k = 2 * y + z;  // +-1 bytes: 1 + 0xFE where the bit is set
+                v[z] = join_chunk(0x01010101u + 0xFEu * ((even >> k) & 0x01010101u),
+                                  0x01010101u + 0xFEu * ((odd >> k) & 0x01010101u));
+            }
+            dst[(U / 2) * x + y] = make_uint4(v[0].x, v[0].y, v[1].x, v[1].y);
+        }
+    }
 }
 
 }  // namespace ptq

@@ -381,7 +381,13 @@ static BatchInstance chains_instance(const DevProblem& p, const LaunchPlan& plan
     I.group_threads = plan.group_threads;
     I.resident = 1;
     I.thr_resident = plan.thr_resident;
-    I.unit_words = plan.unit_words;
+    I.form = plan.form;
+    I.form_t = plan.form_t;
+    I.titems = p.items;
+    I.tlevel_off = p.level_off;
+    I.n_groups = plan.n_groups;
+    I.mail_smem = plan.mail_smem;
+    I.mail = p.mbox;
     I.key0 = p.key0;
     I.key1 = p.key1;
     I.t0 = t0;
@@ -396,7 +402,7 @@ static cudaError_t launch_plan_sweeps(const DevProblem& p, const LaunchPlan& pla
                                       int sps, long long timeout_ns, bool cooperative, cudaStream_t s) {
     if (plan.path == kPathPackedChains)
         return launch_batch_single(chains_instance(p, plan, t0, q0, n, sps), plan.cluster, plan.threads,
-                                   plan.smem_bytes, s);
+                                   plan.smem_bytes, p.status, s);
     return launch_sweeps(p, plan, t0, q0, n, sps, timeout_ns, cooperative, s);
 }
 
@@ -407,13 +413,18 @@ static bool chains_plan(const DevProblem& p, int dclass, int cluster, int widen,
                         int force_group = 0) {
     BatchInstance I = chains_instance(p, pl, 0, 0, 0, 0);
     I.dc = dclass;
+    // byte rows, in units as wide as P allows or of four copies (choose_groups takes one)
+    I.form_t = IndexRule(p.Lmax).wide || p.P % 16 ? kFormBytes1 : (p.P % 32 ? kFormBytes2 : kFormBytes4);
     const size_t cap = batch_smem_cap();
     choose_groups(I, cluster, 512, cap, widen);
     if (force_group > 0) {
         // the given width, with every rung's threshold row resident if that still fits
         I.group_threads = force_group;
+        I.n_groups = 512 / force_group;
         I.resident = 1;
         I.thr_resident = 1;
+        I.mail_smem = 1;
+        if (batch_smem_bytes(I, cluster, 512) > cap) I.mail_smem = 0;
         if (batch_smem_bytes(I, cluster, 512) > cap || (size_t)I.R * ((IndexRule(I.Lmax).row_words() * 4 + 15) / 16 * 16) > 49152)
             I.thr_resident = 0;
     }
@@ -433,7 +444,10 @@ static bool chains_plan(const DevProblem& p, int dclass, int cluster, int widen,
     pl.cluster = cluster;
     pl.group_threads = I.group_threads;
     pl.thr_resident = I.thr_resident;
-    pl.unit_words = choose_unit_words(I, I.group_threads);
+    pl.mail_smem = I.mail_smem;
+    pl.form = I.form;
+    pl.form_t = I.form_t;
+    pl.n_groups = I.n_groups;
     return true;
 }
 
@@ -722,7 +736,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         DevProblem q = p;
         q.nibble = 1;
         q.tables_in_smem = q.acc_in_smem = 0;
-        p.nibble = P % 32 == 0 && Lmax <= kNibbleLmax && want_threads <= 512 &&
+        p.nibble = P % 32 == 0 && Lmax <= kWordBitsLmax && want_threads <= 512 &&
                    sweep_smem_bytes(q, kPathBits, packed_dc) <= (size_t)max_smem;
         c->plan.nibble = !p.nibble ? 0 : (packed_dc == 4 ? 3 : (dmax <= 6 ? 6 : 7));
     }
@@ -1296,7 +1310,7 @@ static int enqueue_sweeps(pt_ctx* c, long long n, int sps) {
             long long chunk = n - done;
             chunk = std::min<long long>(chunk, sps > 0 ? ((1ll << 30) / sps) * sps : (1ll << 30));
             CUDA_OR_FAIL(c, launch_batch_single(chains_instance(c->dp, c->plan, c->t, c->q, (int)chunk, sps),
-                                                c->plan.cluster, c->plan.threads, c->plan.smem_bytes, c->stream));
+                                                c->plan.cluster, c->plan.threads, c->plan.smem_bytes, c->dp.status, c->stream));
             c->launches += 1;
             c->t += chunk;
             if (sps > 0) c->q += chunk / sps;

@@ -59,7 +59,7 @@ struct IndexRule {
     __host__ __device__ int row_words() const { return 3 * S; }
 };
 
-constexpr int kNibbleLmax = 31;  // path 4's nibble form: 4 (2 Lmax) fits a byte
+constexpr int kWordBitsLmax = 31;  // bit words: 4 (2 Lmax) fits a byte
 
 // Per-rung statistics, in this order, as unsigned 64-bit two's-complement sums.
 enum { kAccN = 0, kAccE, kAccE2, kAccM, kAccM2, kAccFlip, kAccCount };
@@ -123,8 +123,10 @@ struct LaunchPlan {
     size_t smem_bytes;   // dynamic shared memory per CTA
     int cluster = 1;     // path 7: CTAs in the one cluster
     int group_threads = 0;  // path 7: threads sweeping one chain
+    int mail_smem = 1;      // path 7: the swap mailboxes in shared memory
     int thr_resident = 0;   // path 7: every rung's threshold row in shared memory
-    int unit_words = 1;     // path 7: words of an update unit
+    int form = 0, form_t = 0;  // path 7: kForm* of a chain
+    int n_groups = 0;       // path 7: chain groups of a CTA
     int copy = 0;           // paths 1, 3 and 9: one copy a thread (sweep_copy_kernel)
     int nibble = 0;         // path 4: neighbour slots of the nibble form, 0 = one bit a copy
     int rows = 0;           // path 1: the word-wise kernel (DevProblem::slots > 0)
@@ -142,13 +144,24 @@ size_t copy_smem_bytes(const DevProblem& p, bool cluster);
 // path 10: the shared memory of a CTA holding `chains` classical chains
 size_t classical_smem_bytes(const DevProblem& p, int chains);
 
+// Forms of a batched chain in shared memory: int8 rows with update units of 1, 2 or 4 words of
+// four copies, or bit words of 16 (nibbles) or 32 copies (bits_unit).
+enum { kFormBytes1 = 0, kFormBytes2, kFormBytes4, kFormNibbles, kFormBits, kFormCount };
+__host__ __device__ inline size_t form_row_bytes(int form, int P) {
+    return form == kFormBits ? P / 8 : (form == kFormNibbles ? P / 4 : P);
+}
+__host__ __device__ inline int form_unit_copies(int form) { return 4 << (form == kFormNibbles ? 2 : form == kFormBits ? 3 : form); }
+
 // One request of a batched launch (device view). Every chain of the request is swept by
 // one CTA of the thread-block cluster that takes the request; the cluster's CTAs split the
 // chains and exchange (E, M) through distributed shared memory for the swap passes.
 struct BatchInstance {
-    const uint32_t* sdesc;     // [N][DW] packed-path site descriptors
+    const uint32_t* sdesc;     // [N][DW] packed-path site descriptors (int8 rows)
+    const uint32_t* wdesc;     // the same for bit words ("plain"), null for byte forms
     const uint32_t* items;     // [2N] schedule, grouped by level
     const int32_t* level_off;  // [n_levels + 1]
+    const uint32_t* titems;    // the same levels balanced for form_t on one-warp groups
+    const int32_t* tlevel_off;
     const uint32_t* thr;       // [R][nL3]
     const double* coef;        // [2(R-1)] (at least 2 entries)
     int8_t* spins;             // [R][slot_stride]
@@ -158,11 +171,15 @@ struct BatchInstance {
     int32_t* slot_of_rung;     // [R]
     unsigned long long* acc;   // [R][kAccCount] by rung
     unsigned long long* swap_stats;  // [R][2] by pair
+    Mailbox* mail;             // [kClusterMailPasses][R], used when the swap mailboxes are not in shared memory
     int N, P, R, Lmax, nL3, n_levels, dc, slot_stride;
     int group_threads;         // threads sweeping one chain (a divisor of the CTA size)
     int resident;              // 1: a CTA keeps all its chains in shared memory for the run
     int thr_resident;          // 1: every rung's threshold row stays in shared memory for the run
-    int unit_words;            // 4-copy words of an update unit: 1, 2 or 4 (choose_unit_words)
+    int mail_smem;             // 1: the swap mailboxes in every CTA's shared memory
+    int form;                  // kForm*: how a chain lies in shared memory (form_t, or kFormBytes1)
+    int form_t;                // the form with the least instructions for the chain on one-warp groups
+    int n_groups;              // groups of group_threads threads at work in a CTA
     uint32_t key0, key1;
     long long t0, q0;          // counters before this run
     int n_sweeps, sweeps_per_swap;
@@ -222,11 +239,11 @@ void build_site_desc(int N, int row_bytes, int dclass, int Lmax, const std::vect
 
 // Host-side preparation of one batched request (pt_batch.cu).
 struct Prepared {
-    int N, P, R, Lmax, dc, n_levels, slot_stride;
-    std::vector<uint32_t> sdesc, items, thr;
-    std::vector<int32_t> level_off;
+    int N, P, R, Lmax, dc, n_levels, slot_stride, form;
+    std::vector<uint32_t> sdesc, wdesc, items, titems, thr;
+    std::vector<int32_t> level_off, tlevel_off;
     std::vector<double> coef;
-    size_t off_sdesc, off_items, off_loff, off_thr, off_coef, off_spins, off_E, off_M, off_rung, off_slot, off_acc,
+    size_t off_sdesc, off_wdesc, off_items, off_loff, off_titems, off_tloff, off_thr, off_coef, off_spins, off_E, off_M, off_rung, off_slot, off_acc,
         off_sw, off_mbox = 0, off_inst = 0, off_map = 0, off_status = 0;
     long long sweep_limit;
 };
@@ -239,9 +256,6 @@ void fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base, con
 constexpr int kGroupWidenDefault = -4;
 void choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen = kGroupWidenDefault);
 
-// Words of an update unit for groups of group_threads threads.
-int choose_unit_words(const BatchInstance& I, int group_threads);
-
 // Batched launchers (pt_batch.cu).
 size_t batch_smem_bytes(const BatchInstance& I, int cluster, int threads);
 cudaError_t launch_batch(const BatchParams& bp, int cluster, int n_clusters, int threads, size_t smem,
@@ -249,7 +263,8 @@ cudaError_t launch_batch(const BatchParams& bp, int cluster, int n_clusters, int
 cudaError_t batch_max_clusters(int cluster, int threads, size_t smem, int* n_clusters);
 cudaError_t launch_batch_init(const BatchInstance* inst, const int2* map, int n_chains, cudaStream_t s);
 // One problem on one cluster of `cluster` CTAs (path 7); I carries t0, q0, n_sweeps, sweeps_per_swap.
-cudaError_t launch_batch_single(const BatchInstance& I, int cluster, int threads, size_t smem, cudaStream_t s);
+cudaError_t launch_batch_single(const BatchInstance& I, int cluster, int threads, size_t smem, int* status,
+                                cudaStream_t s);
 // The largest shared-memory need of the batched kernel: the device's opt-in maximum less
 // the kernel's static shared memory.
 size_t batch_smem_cap();

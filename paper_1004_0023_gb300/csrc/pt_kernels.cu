@@ -132,12 +132,6 @@ size_t sweep_smem_bytes(const DevProblem& p, int path, int dclass, bool cluster_
 
 
 // ------------------------------------------------------------------------- end of a sweep
-// Tag of pass q0 + pass, from qmod0 = q0 mod kTagPeriod (taken once per launch): a 32-bit
-// remainder by a constant instead of a 64-bit one on the path to the partner.
-__device__ __forceinline__ unsigned long long mbox_tag(uint32_t qmod0, int pass) {
-    return (unsigned long long)((qmod0 + (uint32_t)pass) % (uint32_t)kTagPeriod) + 1ull;
-}
-
 // A chain's side of the swap pass that follows a sweep: rl is the lower rung of its pair,
 // partner the other rung; active = 0 when no pass follows or the chain has no partner.
 struct SwapSide {
@@ -792,27 +786,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             d[3] = 0u;
         }
     } else if constexpr (NIB > 0) {
-        // int8 chain in global memory -> nibble words: copy 2 h + par of a site is bit
-        // 8 (h % 4) + (h / 4) % 4 of word h / 16 of its parity
-        uint32_t* words = reinterpret_cast<uint32_t*>(sp);
-        const uint4* src = reinterpret_cast<const uint4*>(p.spins + (size_t)slot * p.slot_stride);
-        for (int x = tid; x < N * G; x += nt) {  // 32 copies: one word of each parity
-            const int i = x / G, c = x - i * G;
-            uint32_t even = 0u, odd = 0u;
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                const uint4 v = src[2 * x + y];
-                uint32_t e, o;
-                split_chunk(make_uint2(v.x, v.y), e, o);
-                even |= ((e >> 7) & 0x01010101u) << (2 * y);
-                odd |= ((o >> 7) & 0x01010101u) << (2 * y);
-                split_chunk(make_uint2(v.z, v.w), e, o);
-                even |= ((e >> 7) & 0x01010101u) << (2 * y + 1);
-                odd |= ((o >> 7) & 0x01010101u) << (2 * y + 1);
-            }
-            words[(2 * i) * G + c] = even;
-            words[(2 * i + 1) * G + c] = odd;
-        }
+        load_bits<4>(reinterpret_cast<uint32_t*>(sp), p.spins + (size_t)slot * p.slot_stride, N, G, tid, nt);
     } else if constexpr (BITS) {
         // int8 chain in global memory -> one bit per copy in shared memory
         const uint2* src = reinterpret_cast<const uint2*>(p.spins + (size_t)slot * p.slot_stride);
@@ -904,7 +878,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     const int g_own = tid & gmask, q_lane = tid >> lg, q_step = NC >> lg;
     FlipSums sums;
     sums.clear();
-    NibbleSums nib_sums = {0, 0, 0};
+    BitSums nib_sums = {0, 0, 0};
     CopySums copy_sums = {0, 0, 0};
     // A unit of item q and column g up to its index and random words, its flips against the
     // threshold row at thr, and the commit.
@@ -965,16 +939,17 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             }
             if constexpr (NIB > 0) {
                 const IndexRule index(p.Lmax);
-                nib_sums = NibbleSums{0, 0, 0};
+                nib_sums.clear();
                 for (int lev = 0; lev < p.n_levels; ++lev) {
                     const int base = s_loff[lev];
                     const int units = (s_loff[lev + 1] - base) << lg;
                     for (int u = tid; u < units; u += NC) {
                         const int g = u & gmask;
                         if (g >= cols) continue;
-                        nibble_unit<DC, NIB>(sp, s_desc, s_items[base + (u >> lg)], (uint32_t)g, (uint32_t)G, t,
-                                             (uint32_t)slot, key, smem, (uint32_t)index.S,
-                                             (uint32_t)(2 * p.Lmax - 255) * kInv255, thr_c, nib_sums);
+                        bits_unit<DC, NIB, 4>(sp, s_desc, s_items[base + (u >> lg)],
+                                              word_offsets((uint32_t)g, (uint32_t)G), (uint32_t)g, t, (uint32_t)slot,
+                                              key, smem, (uint32_t)index.S, (uint32_t)(2 * p.Lmax - 255) * kInv255,
+                                              thr_c, nib_sums);
                     }
                     __syncthreads();
                 }
@@ -1015,9 +990,9 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                 dF = copy_sums.n;
             }
             if (NIB > 0) {
-                dE = 2 * (nib_sums.L - p.Lmax * nib_sums.n);
-                dM = 4 * (nib_sums.C - nib_sums.n);
-                dF = -nib_sums.n;
+                dE = nib_sums.dE(p.Lmax);
+                dM = nib_sums.dM();
+                dF = nib_sums.flips();
             }
             dE = __reduce_add_sync(0xFFFFFFFFu, dE);
             dM = __reduce_add_sync(0xFFFFFFFFu, dM);
@@ -1139,24 +1114,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     flush_acc(p, s_acc, tid, nt);
 
     if constexpr (NIB > 0) {
-        const uint32_t* words = reinterpret_cast<const uint32_t*>(sp);
-        uint4* dst = reinterpret_cast<uint4*>(p.spins + (size_t)slot * p.slot_stride);
-        for (int x = tid; x < N * G; x += nt) {
-            const int i = x / G, c = x - i * G;
-            const uint32_t even = words[(2 * i) * G + c], odd = words[(2 * i + 1) * G + c];
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                uint2 v[2];
-#pragma unroll
-                for (int z = 0; z < 2; ++z) {
-                    const int k = 2 * y + z;
-                    // +-1 bytes: 1 + 0xFE where the bit is set
-                    v[z] = join_chunk(0x01010101u + 0xFEu * ((even >> k) & 0x01010101u),
-                                      0x01010101u + 0xFEu * ((odd >> k) & 0x01010101u));
-                }
-                dst[2 * x + y] = make_uint4(v[0].x, v[0].y, v[1].x, v[1].y);
-            }
-        }
+        store_bits<4>(p.spins + (size_t)slot * p.slot_stride, reinterpret_cast<const uint32_t*>(sp), N, G, tid, nt);
     } else if constexpr (BITS) {
         uint2* dst = reinterpret_cast<uint2*>(p.spins + (size_t)slot * p.slot_stride);
         for (int x = tid; x < N * (P / 8); x += nt) {
@@ -1257,7 +1215,7 @@ sweep_packed_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int 
                                                                timeout_ns, n_consumer, smem);
 }
 
-// Path 4's nibble form (P % 32 == 0, Lmax <= kNibbleLmax).
+// Path 4's nibble form (P % 32 == 0, Lmax <= kWordBitsLmax).
 template <int DC, int NIB>
 __global__ void __launch_bounds__(512, 1)
     sweep_nibble_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,

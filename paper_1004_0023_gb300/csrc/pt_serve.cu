@@ -350,6 +350,16 @@ extern "C" int pt_server_submit(pt_server* s, const pt_request* r, int64_t* id) 
     return PT_OK;
 }
 
+// The layout choose_groups picked, onto a record filled anew.
+static void keep_layout(BatchInstance& to, const BatchInstance& planned) {
+    to.form = planned.form;
+    to.group_threads = planned.group_threads;
+    to.n_groups = planned.n_groups;
+    to.resident = planned.resident;
+    to.thr_resident = planned.thr_resident;
+    to.mail_smem = planned.mail_smem;
+}
+
 // Admit queued requests in arrival order while a slot and arena room are free.
 static int admit(pt_server* s) {
     std::vector<ServeReq*> fresh;
@@ -360,15 +370,16 @@ static int admit(pt_server* s) {
         q->block_off = off;
         unsigned char* base = s->arena + off;
         const Prepared& p = q->prep;
-        const int gthreads = q->inst.group_threads, resident = q->inst.resident, thr_res = q->inst.thr_resident;
+        const BatchInstance planned = q->inst;
         fill_instance(q->inst, p, base, q->req);
-        q->inst.group_threads = gthreads;
-        q->inst.resident = resident;
-        q->inst.thr_resident = thr_res;
+        keep_layout(q->inst, planned);
         std::vector<unsigned char> host(p.off_spins, 0);
         memcpy(&host[p.off_sdesc], p.sdesc.data(), p.sdesc.size() * 4);
+        if (!p.wdesc.empty()) memcpy(&host[p.off_wdesc], p.wdesc.data(), p.wdesc.size() * 4);
         memcpy(&host[p.off_items], p.items.data(), p.items.size() * 4);
         memcpy(&host[p.off_loff], p.level_off.data(), p.level_off.size() * 4);
+        memcpy(&host[p.off_titems], p.titems.data(), p.titems.size() * 4);
+        memcpy(&host[p.off_tloff], p.tlevel_off.data(), p.tlevel_off.size() * 4);
         memcpy(&host[p.off_thr], p.thr.data(), p.thr.size() * 4);
         memcpy(&host[p.off_coef], p.coef.data(), p.coef.size() * 8);
         cudaError_t e;
@@ -408,15 +419,16 @@ static int admit(pt_server* s) {
 static int upload_request(pt_server* s, ServeReq* q, cudaStream_t st) {
     unsigned char* base = s->arena + q->block_off;
     const Prepared& pr = q->prep;
-    const int gthreads = q->inst.group_threads, resident = q->inst.resident, thr_res = q->inst.thr_resident;
+    const BatchInstance planned = q->inst;
     fill_instance(q->inst, pr, base, q->req);
-    q->inst.group_threads = gthreads;
-    q->inst.resident = resident;
-    q->inst.thr_resident = thr_res;
+    keep_layout(q->inst, planned);
     std::vector<unsigned char> host(pr.off_spins, 0);
     memcpy(&host[pr.off_sdesc], pr.sdesc.data(), pr.sdesc.size() * 4);
+    if (!pr.wdesc.empty()) memcpy(&host[pr.off_wdesc], pr.wdesc.data(), pr.wdesc.size() * 4);
     memcpy(&host[pr.off_items], pr.items.data(), pr.items.size() * 4);
     memcpy(&host[pr.off_loff], pr.level_off.data(), pr.level_off.size() * 4);
+    memcpy(&host[pr.off_titems], pr.titems.data(), pr.titems.size() * 4);
+    memcpy(&host[pr.off_tloff], pr.tlevel_off.data(), pr.tlevel_off.size() * 4);
     memcpy(&host[pr.off_thr], pr.thr.data(), pr.thr.size() * 4);
     memcpy(&host[pr.off_coef], pr.coef.data(), pr.coef.size() * 8);
     std::vector<int2> map(pr.R);

@@ -84,3 +84,32 @@ def test_unit_edges_match_the_oracle(k):
             assert np.array_equal(np.asarray(og[key]), np.asarray(oo[key])), (CASES[k], sweeps, key)
         moved = int(np.sum(og["flip_acc"]))
     assert moved > 0
+
+
+BATCH = [(n, d, P, R, lmax) for n, d, lmax in ((24, 3, 31), (24, 3, 32), (30, 6, 31), (30, 7, 41), (20, 7, 42), (130, 3, 8))
+         for P, R in ((8, 5), (24, 3), (32, 4), (64, 3), (96, 6), (128, 2))] + [(700, 3, 128, 9, 9), (1000, 6, 64, 20, 30)]
+
+
+@pytest.mark.parametrize("cluster", [1, 2, 0])
+def test_batched_chain_forms_match_the_oracle(cluster):
+    """Every form of a batched chain (int8 rows in units of 1, 2 and 4 words, nibble and bit
+    words), resident and streamed, over two runs; cluster 0 is timed at create and then reused
+    from the cache, which has to bring its own groups to the device."""
+    probs = [_problem(*c, 100 + k) for k, c in enumerate(BATCH)]
+    for k, p in enumerate(probs):
+        p.n_sweeps, p.sweeps_per_swap = 4 + k % 3, 1 + k % 2
+    batches = [pt.Batch(probs, cluster_size=cluster)]
+    if cluster == 0:
+        assert batches[0].info().tuned_layouts >= 2
+        batches.append(pt.Batch(probs))
+        assert batches[1].info().tuned_layouts == 0
+    for b in batches:
+        orcs = [Oracle.from_problem(p, threads=THREADS) for p in probs]
+        for run in range(2):
+            b.run()
+            for k, (p, o) in enumerate(zip(probs, orcs)):
+                o.run(p.n_sweeps, p.sweeps_per_swap)
+                assert np.array_equal(b.read_state(k), o.read_state()), (BATCH[k], run)
+                og, oo = b.obs(k), o.obs()
+                for key in oo:
+                    assert np.array_equal(np.asarray(og[key]), np.asarray(oo[key])), (BATCH[k], run, key)
