@@ -165,27 +165,25 @@ struct ChainChange {
 template <typename Offsets, typename Unit>
 __device__ __forceinline__ void run_levels(const ChainSweep& c, const uint32_t* s_items, const int32_t* s_loff,
                                            int cols, Offsets offsets, Unit unit) {
-    int lg = 0;
-    while ((1 << lg) < cols) ++lg;
-    const int gmask = (1 << lg) - 1;
-    if ((c.gsize & gmask) == 0) {
+    if (c.gsize >= cols) {
         // this thread's column never changes: its row offsets are loop invariants
-        const int g = c.gtid & gmask, q_lane = c.gtid >> lg, q_step = c.gsize >> lg;
-        const UnitOffsets off = offsets((uint32_t)min(g, cols - 1));
+        const int q_step = c.gsize / cols, q_lane = c.gtid / cols, g = c.gtid - q_lane * cols;
+        const bool lane_ok = q_lane < q_step;
+        const UnitOffsets off = offsets((uint32_t)g);
         int base = s_loff[0];
         for (int lev = 0; lev < c.n_levels; ++lev) {
             const int end = s_loff[lev + 1];
-            if (g < cols)
+            if (lane_ok)
                 for (int q = base + q_lane; q < end; q += q_step) unit(s_items[q], (uint32_t)g, off);
             base = end;
             group_sync(c.bar, c.gsize);
         }
     } else {
         for (int lev = 0; lev < c.n_levels; ++lev) {
-            const int base = s_loff[lev], units = (s_loff[lev + 1] - base) << lg;
+            const int base = s_loff[lev], units = (s_loff[lev + 1] - base) * cols;
             for (int u = c.gtid; u < units; u += c.gsize) {
-                const int g = u & gmask;
-                if (g < cols) unit(s_items[base + (u >> lg)], (uint32_t)g, offsets((uint32_t)g));
+                const int q = u / cols, g = u - q * cols;
+                unit(s_items[base + q], (uint32_t)g, offsets((uint32_t)g));
             }
             group_sync(c.bar, c.gsize);
         }
@@ -853,10 +851,10 @@ static void choose_form(Prepared& pr, const std::vector<std::vector<int>>& adj, 
         if (P % (2 * copies)) continue;
         if (form >= kFormNibbles && pr.Lmax > kWordBitsLmax) continue;
         if (form > kFormBytes1 && form < kFormNibbles && IndexRule(pr.Lmax).wide) continue;
-        int cols = 1;
-        while (cols < P / (2 * copies)) cols <<= 1;
+        const int cols = P / (2 * copies), per = std::max(1, 32 / cols);
         // balanced levels fill whole rounds, but for the last of about every third level
-        const double rounds = std::max<double>(pr.n_levels, 2.0 * pr.N * cols / 32.0 + 0.35 * pr.n_levels);
+        const double rounds = std::max(1.0, cols / 32.0) *
+                              std::max<double>(pr.n_levels, 2.0 * pr.N / per + 0.35 * pr.n_levels);
         const size_t chain = (size_t)pr.N * form_row_bytes(form, P);
         const size_t fixed = (size_t)pr.N * (pr.dc == 4 ? 40 : 56) + 16384;
         const size_t fit = fixed < 230000 ? (230000 - fixed) / std::max<size_t>(chain, 16) : 0;
@@ -865,7 +863,7 @@ static void choose_form(Prepared& pr, const std::vector<std::vector<int>>& adj, 
         if (pr.form < 0 || cost < best) {
             best = cost;
             pr.form = form;
-            best_round = std::max(1, 32 / cols);
+            best_round = per;
         }
     }
     if (pr.form == kFormBytes1 && best_round == per_round) {
@@ -884,14 +882,13 @@ static void choose_form(Prepared& pr, const std::vector<std::vector<int>>& adj, 
 // off by at most 20 %, and names the faster of the two forms but for near ties.)
 static double sweep_cycles(const BatchInstance& I, int C) {
     const int instr = kFormInstr[I.dc == 4 ? 0 : 1][I.form];
-    int cols = 1;
-    while (cols < I.P / (2 * form_unit_copies(I.form))) cols <<= 1;
-    const double g = I.group_threads;
-    const double units = 2.0 * I.N / std::max(1, I.n_levels) * cols;
-    const double full = std::floor(units / g), rest = std::ceil((units - full * g) / 32.0);
+    const int cols = I.P / (2 * form_unit_copies(I.form)), g = I.group_threads;
+    const double items = 2.0 * I.N / std::max(1, I.n_levels);
+    const double per = g >= cols ? g / cols : (double)g / cols;  // items a round
+    const double full = std::floor(items / per), rest = std::ceil((items - full * per) * cols / 32.0);
     const int groups = std::min(C, I.n_groups);
     auto round = [&](double warps) { return instr * std::max(5.5, 1.65 * groups * warps / 4.0); };
-    const double level = full * round(g / 32.0) + (rest > 0.0 ? round(rest) : 0.0) + 150.0;
+    const double level = full * round(std::min(g / 32.0, std::ceil(per * cols / 32.0))) + (rest > 0.0 ? round(rest) : 0.0) + 150.0;
     return (I.n_levels * level + 4000.0) * std::max(1.0, (double)C / I.n_groups);
 }
 
@@ -1251,9 +1248,8 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
         auto work = [&](int first, int step) {
             char w[200];
             for (int k = first; k < count; k += step) {
-                int cols = 1;
-                while (cols < reqs[k].P / 8) cols <<= 1;
-                rcs[k] = prepare_request(reqs[k], pr[k], w, sizeof(w), reqs[k].P >= 8 ? std::max(1, 32 / cols) : 0);
+                rcs[k] = prepare_request(reqs[k], pr[k], w, sizeof(w),
+                                         reqs[k].P >= 8 ? std::max(1, 32 / (reqs[k].P / 8)) : 0);
                 if (rcs[k]) whys[k] = w;
             }
         };

@@ -680,6 +680,108 @@ __device__ __forceinline__ UnitOffsets row_offsets(uint32_t u, uint32_t half) {
     return o;
 }
 
+// Records: what an update reads of its site, one record for every update in schedule order, its
+// parity worked in. A descriptor takes the item first (another shared-memory latency) and about
+// eight instructions of parity arithmetic a unit, on a path whose every instruction costs a
+// level five to six cycles; a record takes twice the descriptors' memory and more.
+//   DC = 4:  C4, own words, opposite parity's, parity | off0..2, k0 | k1, k2, item, 0
+//   DC = 8:  C4, own words, opposite parity's, parity | J bytes (2), item, 0 | off0..3 | off4..6, 0
+template <int DC>
+struct UnitRecord {
+    static constexpr int kWords = DC == 4 ? 12 : 16;
+};
+__host__ __device__ inline int record_words(int dc) { return dc == 4 ? 12 : 16; }
+template <int DC>
+__device__ __forceinline__ void make_record(uint32_t* rec, const uint32_t* desc, uint32_t item, uint32_t half) {
+    const uint32_t par = item & 1u, shift = par * half;
+    const uint32_t row = DC == 4 ? desc[7] : desc[3];
+    rec[0] = desc[0];
+    rec[1] = row + shift;
+    rec[2] = row + half - shift;
+    rec[3] = par;
+    if constexpr (DC == 4) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            rec[4 + d] = desc[1 + d] + shift;
+            rec[7 + d] = desc[4 + d];
+        }
+        rec[10] = item;
+        rec[11] = 0u;
+    } else {
+        rec[4] = desc[1];
+        rec[5] = desc[2];
+        rec[6] = item;
+        rec[7] = 0u;
+#pragma unroll
+        for (int d = 0; d < 7; ++d) rec[8 + d] = desc[4 + d] + shift;
+        rec[15] = 0u;
+    }
+}
+// A record in registers: loaded a level ahead, it leaves the spins, the table and the flip
+// between two barriers.
+template <int DC>
+struct LoadedRecord {
+    SiteTerms<DC> s;  // (row: unused; offsets and own / opp carry the parity)
+    uint32_t own, opp, par, item;
+};
+template <int DC>
+__device__ __forceinline__ LoadedRecord<DC> load_record(const uint32_t* rec) {
+    LoadedRecord<DC> l;
+    const uint4 r0 = *reinterpret_cast<const uint4*>(rec), r1 = *reinterpret_cast<const uint4*>(rec + 4);
+    l.s.c4 = r0.x;
+    l.own = r0.y;
+    l.opp = r0.z;
+    l.par = r0.w;
+    if constexpr (DC == 4) {
+        const uint4 r2 = *reinterpret_cast<const uint4*>(rec + 8);
+        l.s.off[0] = r1.x;
+        l.s.off[1] = r1.y;
+        l.s.off[2] = r1.z;
+        l.s.k[0] = r1.w;
+        l.s.k[1] = r2.x;
+        l.s.k[2] = r2.y;
+        l.item = r2.z;
+    } else {
+        const uint4 r2 = *reinterpret_cast<const uint4*>(rec + 8), r3 = *reinterpret_cast<const uint4*>(rec + 12);
+        l.s.off[0] = r2.x;
+        l.s.off[1] = r2.y;
+        l.s.off[2] = r2.z;
+        l.s.off[3] = r2.w;
+        l.s.off[4] = r3.x;
+        l.s.off[5] = r3.y;
+        l.s.off[6] = r3.z;
+        l.s.k[0] = prmt(r1.x, 0u, 0x8880u);
+        l.s.k[1] = prmt(r1.x, 0u, 0x9991u);
+        l.s.k[2] = prmt(r1.x, 0u, 0xAAA2u);
+        l.s.k[3] = prmt(r1.x, 0u, 0xBBB3u);
+        l.s.k[4] = prmt(r1.y, 0u, 0x8880u);
+        l.s.k[5] = prmt(r1.y, 0u, 0x9991u);
+        l.s.k[6] = prmt(r1.y, 0u, 0xAAA2u);
+        l.item = r1.z;
+    }
+    return l;
+}
+// A unit of one word at column byte g4 = 4 g of its row half, edge copies at e0 (even) and e1 (odd)
+// of the opposite half.
+template <int DC, bool PRE, bool WIDE>
+__device__ __forceinline__ UnitEval<1> record_eval(int8_t* sp, const LoadedRecord<DC>& l, uint32_t g4, uint32_t e0,
+                                                   uint32_t e1, const uint4* rbq, uint32_t t, uint32_t slot,
+                                                   const UnitRule<WIDE>& rule, const PhiloxKey& key) {
+    UnitEval<1> e;
+    int8_t* spg = sp + g4;
+    e.own = spg + l.own;
+    uint32_t O[1], a[DC - 1];
+    load_words<1>(e.own, e.V);
+    load_words<1>(spg + l.opp, O);
+    const uint32_t edge = (uint8_t)sp[l.opp + e0 + l.par * (e1 - e0)];
+#pragma unroll
+    for (int d = 0; d < DC - 1; ++d) load_words<1>(spg + l.s.off[d], a + d);
+    unit_words<1, PRE>(e.u, l.item, rbq, t, slot, g4 >> 2, key);
+    trotter_differences<1, WIDE>(e.V, O, edge, l.par, e.D);
+    e.L[0] = site_index<DC>(l.s, a, e.V[0], rule.kM);
+    return e;
+}
+
 // ------------------------------------------------------------------------- any even P, any degree
 // The same unit (W = 1) for the shapes the classes above leave out: P not a multiple of 8, or
 // more than seven neighbours. Each parity's half of a row is padded to whole words (G words;
@@ -792,6 +894,30 @@ __device__ __forceinline__ CopyEval copy_eval(int8_t* sp, const uint32_t* desc, 
         const uint4 p1 = *reinterpret_cast<const uint4*>(t.rest + 2 * d - 4);
         f += (int)p0.y * sp[p0.x + own_off] + (int)p0.w * sp[p0.z + own_off];
         f += (int)p1.y * sp[p1.x + own_off] + (int)p1.w * sp[p1.z + own_off];
+    }
+    e.L = e.s * f;
+    e.m = e.s * nn;
+    e.u = word;
+    return e;
+}
+// The same from a record: the word-wise form's descriptor with the parity worked into every
+// offset (head: h, own row half, slots, opposite row half).
+__device__ __forceinline__ CopyEval copy_record_eval(int8_t* sp, const RowsTerms& t, uint32_t g, uint32_t e0,
+                                                     uint32_t e1, uint32_t word) {
+    CopyEval e;
+    int8_t* spg = sp + g;
+    e.own = spg + t.head.y;
+    e.s = *e.own;
+    const int nn = spg[t.head.w] + sp[t.head.w + (t.head.w < t.head.y ? e1 : e0)];
+    int f = (int)t.head.x;
+    f += (int)t.n0.y * spg[t.n0.x] + (int)t.n0.w * spg[t.n0.z];
+    f += (int)t.n1.y * spg[t.n1.x] + (int)t.n1.w * spg[t.n1.z];
+#pragma unroll 2
+    for (uint32_t d = 4; d < t.head.z; d += 4) {
+        const uint4 p0 = *reinterpret_cast<const uint4*>(t.rest + 2 * d - 8);
+        const uint4 p1 = *reinterpret_cast<const uint4*>(t.rest + 2 * d - 4);
+        f += (int)p0.y * spg[p0.x] + (int)p0.w * spg[p0.z];
+        f += (int)p1.y * spg[p1.x] + (int)p1.w * spg[p1.z];
     }
     e.L = e.s * f;
     e.m = e.s * nn;

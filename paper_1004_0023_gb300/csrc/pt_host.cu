@@ -653,14 +653,16 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     // time. 0 threads when a level is too large for that: beyond 384 copies a thread's second
     // round costs what the four-copy unit's longer instruction chain does.
     auto copy_threads = [&](int* producers) {
-        int ccols = 1;
-        while (ccols < P / 2) ccols <<= 1;
-        const long long copies = ((long long)items.size() * ccols + p.n_levels - 1) / p.n_levels;
-        if (P < 2 || p.slots == 0 || copies > 384 || ccols > 256) return 0;
-        const int unit = std::max(32, ccols);
-        const int consumers = std::max(64, (int)((copies + unit - 1) / unit) * unit);
+        const long long copies = ((long long)items.size() * (P / 2) + p.n_levels - 1) / p.n_levels;
+        if (P < 2 || p.slots == 0 || copies > 384 || P / 2 > 384) return 0;
+        const int consumers = std::max(64, (int)(std::max<long long>(copies, P / 2) + 31) / 32 * 32);
         *producers = std::min(128, std::max(32, (int)(copies / 3 + 31) / 32 * 32));
         return consumers + *producers <= 512 ? consumers + *producers : 0;
+    };
+    // records in shared memory where the rest leaves room, and every chain has an SM to itself
+    auto records_for = [&](int pth, int copy) {
+        return R <= n_sm && (copy || pth == kPathPacked || pth == kPathPackedInline || pth == kPathPeer ||
+                             pth == kPathCluster);
     };
     // a layout fits if it does with the threshold rows and / or the statistics moved out
     auto fits = [&](int pth) {
@@ -838,7 +840,11 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             cols = P / 16 + 1;
         } else {
             const int G = (path == kPathGeneric) ? ((P / 2) + 3) / 4 : (path == kPathBits && p.nibble ? P / 32 : P / 8);
-            while (cols < (c->plan.copy ? P / 2 : G)) cols <<= 1;
+            cols = c->plan.copy ? P / 2 : G;
+            if (path == kPathGeneric && !c->plan.rows && !c->plan.copy) {  // the byte-wise kernel pads to a power of two
+                cols = 1;
+                while (cols < G) cols <<= 1;
+            }
         }
         const int per_round = path == kPathClassical ? c->plan.threads / c->plan.chains_per_cta
                                                      : c->plan.n_consumer / cols;
@@ -851,6 +857,11 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             free_ctx(c);
             return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
                                c->plan.smem_bytes, max_smem);
+        }
+        if (records_for(path, c->plan.copy)) {
+            p.records = 1;
+            if (plan_smem() > (size_t)max_smem) p.records = 0;
+            c->plan.smem_bytes = plan_smem();
         }
     }
 
@@ -983,9 +994,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             free_ctx(c);
             return create_fail(PT_EINVAL, "kernel_path 7: the chains do not all fit the cluster's shared memory");
         }
-        int cols = 1;
-        while (cols < P / 8) cols <<= 1;
-        level_schedule(N, adj, items, level_off, std::max(1, pl.group_threads / cols), P / 4);
+        level_schedule(N, adj, items, level_off, std::max(1, pl.group_threads / (P / 8)), P / 4);
         cudaStream_t s = c->stream;
         if ((e = cudaMemcpyAsync(d_items, items.data(), items.size() * 4, cudaMemcpyHostToDevice, s)) !=
                 cudaSuccess ||
@@ -1081,6 +1090,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         auto make = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
                         std::vector<int32_t>& off_c) {
             pc = p;
+            pc.records = 0;
             if (cd.path == kPathClassical) {
                 pc.acc_in_smem = 1;
                 pc.tables_in_smem = 1;
@@ -1098,9 +1108,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             }
             if (cd.path == kPathPackedChains) {
                 if (!chains_plan(pc, packed_dc, cd.cluster, kGroupWidenDefault, pl, cd.group_threads)) return false;
-                int cols = 1;
-                while (cols < P / 8) cols <<= 1;
-                level_schedule(N, adj, it_c, off_c, std::max(1, pl.group_threads / cols), P / 4);
+                level_schedule(N, adj, it_c, off_c, std::max(1, pl.group_threads / (P / 8)), P / 4);
                 pc.n_levels = (int)off_c.size() - 1;
                 return true;
             }
@@ -1113,12 +1121,12 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                 pl.copy = 1;
                 pl.threads = cd.threads;
                 pl.n_consumer = cd.threads - cd.producers;
-                int cols = 1;
-                while (cols < P / 2) cols <<= 1;
-                level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / cols));
+                level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / (P / 2)));
                 pc.n_levels = (int)off_c.size() - 1;
                 if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.tables_in_smem = 0;
                 if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.acc_in_smem = 0;
+                pc.records = records_for(cd.path, 1);
+                if (pc.records && copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.records = 0;
                 pl.smem_bytes = copy_smem_bytes(pc, cl);
                 return pl.smem_bytes <= (size_t)max_smem;
             }
@@ -1132,14 +1140,15 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             pl.n_consumer = cd.threads - cd.producers;
             pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc, cpre);
             int cols = 1;
-            if (cd.path == kPathSplit || cd.path == kPathSplitInline) {
+            if (cd.path == kPathSplit || cd.path == kPathSplitInline)
                 cols = P / 16 + 1;
-            } else {
-                while (cols < P / 8) cols <<= 1;
-            }
+            else if (P >= 8)
+                cols = P / 8;
             level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / cols), row_words_for(cd.path));
             if (P == 1) drop_odd_updates(it_c, off_c);
             pc.n_levels = (int)off_c.size() - 1;
+            pc.records = records_for(cd.path, 0);
+            if (pc.records && sweep_smem_bytes(pc, cd.path, pl.dclass, cpre) > (size_t)max_smem) pc.records = 0;
             pl.smem_bytes = sweep_smem_bytes(pc, cd.path, pl.dclass, cpre);  // sized for this schedule
             return pl.smem_bytes <= (size_t)max_smem;
         };
@@ -1242,6 +1251,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                     c->cooperative = true;  // resident (checked above), cooperative launch available
                     p.acc_in_smem = pc.acc_in_smem;
                     p.tables_in_smem = pc.tables_in_smem;
+                    p.records = pc.records;
                     if (!cached) {
                         std::lock_guard<std::mutex> lock(g_plan_mutex);
                         const Cand& cb = cands[best];

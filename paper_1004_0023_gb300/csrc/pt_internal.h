@@ -92,6 +92,7 @@ struct DevProblem {
     int tables_in_smem;        // 1: every rung's threshold row resident in shared memory
     int slots;                 // path 1: neighbour slots of a site descriptor (a multiple of 4) when the
                                // word-wise kernel runs, 0: the byte-wise one
+    int records;               // 1: per-update records in schedule order in shared memory (see record_words)
     int nibble;                // path 4: 1 = the nibble form of the bit-packed chain
     int exact_swaps;           // test hook: 1 = always take the FP64 swap decision
     uint32_t key0, key1;

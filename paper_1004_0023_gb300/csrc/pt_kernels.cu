@@ -67,7 +67,7 @@ struct RowsLayout {
         const size_t N = p.N, G = ((size_t)p.P / 2 + 3) / 4;
         size_t o = 0;
         spins = o; o += up16(N * 8 * G);
-        desc = o;  o += N * rows_desc_words(p.slots) * 4;
+        desc = o;  o += (p.records ? 2 * N : N) * rows_desc_words(p.slots) * 4;
         items = o; o += up16(2 * N * 4);
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
         thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
@@ -97,7 +97,7 @@ struct FastLayout {
         size_t o = 0;
         spins = o; o += up16((size_t)N * row);
         lut = o;   o += bits && !p.nibble ? 2048 : 0;
-        desc = o;  o += (size_t)N * (dc == 4 ? 32 : 48);
+        desc = o;  o += p.records && !bits ? (size_t)2 * N * record_words(dc) * 4 : (size_t)N * (dc == 4 ? 32 : 48);
         items = o; o += up16((size_t)2 * N * 4);
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
         thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
@@ -132,6 +132,12 @@ size_t sweep_smem_bytes(const DevProblem& p, int path, int dclass, bool cluster_
 
 
 // ------------------------------------------------------------------------- end of a sweep
+// The other rung of `rung`'s pair in pass q, or -1.
+__device__ __forceinline__ int pair_rung(int rung, long long q, int R) {
+    const int other = (rung & 1) == (int)(q & 1) ? rung + 1 : rung - 1;
+    return other >= 0 && other < R ? other : -1;
+}
+
 // A chain's side of the swap pass that follows a sweep: rl is the lower rung of its pair,
 // partner the other rung; active = 0 when no pass follows or the chain has no partner.
 struct SwapSide {
@@ -150,7 +156,7 @@ __device__ SwapSide eos_publish(const DevProblem& p, int rung, long long& E, lon
     E += dE;
     M += dM;
     SwapSide w;
-    w.active = 0;
+    w.active = w.pass = 0;
     if (pass >= 0) {
         const int R = p.R;
         w.pass = pass;
@@ -204,50 +210,60 @@ __device__ __forceinline__ void eos_stats(const DevProblem& p, unsigned long lon
     }
 }
 
-// Thread 0 again: wait for the partner's mailbox (bounded by timeout_ns) and take the
-// decision both chains of the pair take. Returns the chain's rung for the next sweep; sets
-// *abort when the partner's mailbox never arrived within the time limit. count = false: the
+// Thread 0 again: wait for the partner's mailbox (bounded by timeout_ns) and take the decision
+// both chains of the pair take. Returns the chain's rung for the next sweep; sets *abort when
+// the partner's mailbox never arrived within the time limit. read(partner, wa, wb) loads the
+// partner's two tagged words. The pass's coefficients and random word do not depend on the
+// partner and are fetched before the wait, as is nothing but the loads and the comparison
+// after it; the clock is read only once the first polls have failed. count = false: the
 // pair's attempt and acceptance are counted by another CTA of the chain (split kernel).
-__device__ int eos_decide(const DevProblem& p, const SwapSide& w, int rung, long long E, long long M,
-                          long long timeout_ns, const PhiloxKey& key, int* abort, bool count = true) {
+template <typename Read>
+__device__ __forceinline__ int eos_decide_from(const DevProblem& p, const SwapSide& w, int rung, long long E,
+                                               long long M, long long timeout_ns, const PhiloxKey& key, int* abort,
+                                               bool count, Read read) {
     *abort = 0;
     if (!w.active) return rung;
-    const int R = p.R;
-    const Mailbox* mb = p.mbox + (size_t)w.pass * R;
-    long long pE, pM;
-    const unsigned long long start = globaltimer_ns();
-    // the first polls spin (the partner usually publishes within an L2 round trip); later
-    // ones back off with __nanosleep, doubling up to 256 ns, so that a CTA waiting on a slow
-    // partner leaves its issue slots and the L2 to the CTAs sharing its SM
+    const int R = p.R, rl = w.rl;
+    const bool lower = (rung == rl);
+    const double ca = p.coef[rl], cc = p.coef[(R - 1) + rl];
+    const uint32_t word = swap_word((uint32_t)w.q, (uint32_t)rl, key);
+    unsigned long long wa, wb, start = 0;
+    // the first polls spin (the partner usually publishes within a round trip); later ones back
+    // off with __nanosleep, doubling up to 256 ns, so that a CTA waiting on a slow partner
+    // leaves its issue slots and the L2 to the CTAs sharing its SM
     unsigned int nap = 0;
     for (int polls = 0;; ++polls) {
-        const unsigned long long wa = ld_relaxed_u64(&mb[w.partner].a);
-        const unsigned long long wb = ld_relaxed_u64(&mb[w.partner].b);
-        if ((wa & 0xFFFFFFull) == w.tag && (wb & 0xFFFFFFull) == w.tag) {
-            pE = (long long)wa >> 24;
-            pM = (long long)(int32_t)(uint32_t)(wb >> 32);
-            break;
-        }
-        if ((long long)(globaltimer_ns() - start) > timeout_ns) {
-            atomicCAS(p.status, 0, PT_ETIMEDOUT);
-            *abort = 1;
-            return rung;
-        }
+        read(w.partner, wa, wb);
+        if ((wa & 0xFFFFFFull) == w.tag && (wb & 0xFFFFFFull) == w.tag) break;
         if (polls >= 32) {
+            if (polls == 32) start = globaltimer_ns();
+            if ((long long)(globaltimer_ns() - start) > timeout_ns) {
+                atomicCAS(p.status, 0, PT_ETIMEDOUT);
+                *abort = 1;
+                return rung;
+            }
             nap = nap ? min(2u * nap, 256u) : 16u;
             __nanosleep(nap);
         }
     }
-    const int rl = w.rl;
-    const bool lower = (rung == rl);
-    const bool acc_swap = swap_accept_fast(lower ? E : pE, lower ? pE : E, lower ? M : pM, lower ? pM : M,
-                                           p.coef[rl], p.coef[(R - 1) + rl], (uint32_t)w.q, (uint32_t)rl, key,
-                                           p.exact_swaps != 0);
+    const long long pE = (long long)wa >> 24, pM = (long long)(int32_t)(uint32_t)(wb >> 32);
+    const bool acc_swap =
+        swap_accept_fast_by(lower ? E : pE, lower ? pE : E, lower ? M : pM, lower ? pM : M, ca, cc,
+                            [&] { return word; }, p.exact_swaps != 0);
     if (lower && count) {
         atomicAdd(p.swap_stats + 2 * rl, 1ull);
         if (acc_swap) atomicAdd(p.swap_stats + 2 * rl + 1, 1ull);
     }
     return acc_swap ? w.partner : rung;
+}
+__device__ __forceinline__ int eos_decide(const DevProblem& p, const SwapSide& w, int rung, long long E, long long M,
+                                          long long timeout_ns, const PhiloxKey& key, int* abort, bool count = true) {
+    const Mailbox* mb = p.mbox + (size_t)w.pass * p.R;
+    return eos_decide_from(p, w, rung, E, M, timeout_ns, key, abort, count,
+                           [&](int partner, unsigned long long& wa, unsigned long long& wb) {
+                               wa = ld_relaxed_u64(&mb[partner].a);
+                               wb = ld_relaxed_u64(&mb[partner].b);
+                           });
 }
 
 // Path 9 (one cluster holds every chain): the same decision with the partner's (E, M) read
@@ -256,43 +272,15 @@ __device__ int eos_decide(const DevProblem& p, const SwapSide& w, int rung, long
 // wait polls local shared memory. Four slots suffice: the chain that would overwrite the
 // slot a waiting chain reads (the holder of that rung three passes later) must first finish
 // the pass two later, in which it waits for the reader's own publication again.
-__device__ int eos_decide_cluster(const DevProblem& p, const unsigned long long* s_cmb, const SwapSide& w, int rung,
-                                  long long E, long long M, long long timeout_ns, const PhiloxKey& key, int* abort) {
-    *abort = 0;
-    if (!w.active) return rung;
-    const int R = p.R;
-    const unsigned long long* mb = s_cmb + ((size_t)(w.pass & (kClusterMailPasses - 1)) * R + w.partner) * 2;
-    long long pE, pM;
-    const unsigned long long start = globaltimer_ns();
-    unsigned int nap = 0;
-    for (int polls = 0;; ++polls) {
-        const unsigned long long wa = ld_cluster_local_u64(mb);
-        const unsigned long long wb = ld_cluster_local_u64(mb + 1);
-        if ((wa & 0xFFFFFFull) == w.tag && (wb & 0xFFFFFFull) == w.tag) {
-            pE = (long long)wa >> 24;
-            pM = (long long)(int32_t)(uint32_t)(wb >> 32);
-            break;
-        }
-        if ((long long)(globaltimer_ns() - start) > timeout_ns) {
-            atomicCAS(p.status, 0, PT_ETIMEDOUT);
-            *abort = 1;
-            return rung;
-        }
-        if (polls >= 32) {
-            nap = nap ? min(2u * nap, 256u) : 16u;
-            __nanosleep(nap);
-        }
-    }
-    const int rl = w.rl;
-    const bool lower = (rung == rl);
-    const bool acc_swap = swap_accept_fast(lower ? E : pE, lower ? pE : E, lower ? M : pM, lower ? pM : M,
-                                           p.coef[rl], p.coef[(R - 1) + rl], (uint32_t)w.q, (uint32_t)rl, key,
-                                           p.exact_swaps != 0);
-    if (lower) {
-        atomicAdd(p.swap_stats + 2 * rl, 1ull);
-        if (acc_swap) atomicAdd(p.swap_stats + 2 * rl + 1, 1ull);
-    }
-    return acc_swap ? w.partner : rung;
+__device__ __forceinline__ int eos_decide_cluster(const DevProblem& p, const unsigned long long* s_cmb,
+                                                  const SwapSide& w, int rung, long long E, long long M,
+                                                  long long timeout_ns, const PhiloxKey& key, int* abort) {
+    const unsigned long long* mb = s_cmb + (size_t)(w.pass & (kClusterMailPasses - 1)) * p.R * 2;
+    return eos_decide_from(p, w, rung, E, M, timeout_ns, key, abort, true,
+                           [&](int partner, unsigned long long& wa, unsigned long long& wb) {
+                               wa = ld_cluster_local_u64(mb + 2 * partner);
+                               wb = ld_cluster_local_u64(mb + 2 * partner + 1);
+                           });
 }
 
 // Both steps at once (the byte-wise kernel).
@@ -684,20 +672,23 @@ __global__ void __launch_bounds__(512, 1)
 // Random words of one sweep for the producer warps: word w of philox((t, i, slot,
 // p<<24 | g)) goes with copy 8g + p + 2w of site i (the same counter the update would use).
 __device__ __forceinline__ void produce_words(uint4* buf, uint32_t t, const uint32_t* s_items, int n_items, int G,
-                                              int lg, int gmask, int ptid, int np, uint32_t slot,
-                                              const PhiloxKey& key) {
+                                              int ptid, int np, uint32_t slot, const PhiloxKey& key) {
     if (ptid < 0 || np <= 0) return;  // producer threads only
-    const int total = n_items << lg;
-    for (int x = ptid; x < total; x += np) {
-        const int g = x & gmask;
-        if (g >= G) continue;
-        const int q = x >> lg;
+    auto make = [&](int q, int g) {
         const uint32_t it = s_items[q];
         // stored as min(u, 2^32 - 2): then u < thr alone is the acceptance rule, the
         // "accept always" entry 0xFFFFFFFF included
         const uint4 r = philox(make_uint4(t, it >> 1, slot, ((it & 1u) << 24) | (uint32_t)g), key);
         buf[q * G + g] = make_uint4(min(r.x, 0xFFFFFFFEu), min(r.y, 0xFFFFFFFEu), min(r.z, 0xFFFFFFFEu),
                                     min(r.w, 0xFFFFFFFEu));
+    };
+    if (np >= G) {  // a thread keeps one column
+        const int step = np / G, q0 = ptid / G, g = ptid - q0 * G;
+        if (q0 < step)
+            for (int q = q0; q < n_items; q += step) make(q, g);
+    } else {
+        for (int q = 0; q < n_items; ++q)
+            for (int g = ptid; g < G; g += np) make(q, g);
     }
 }
 
@@ -752,6 +743,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     const int G = NIB ? P >> 5 : ((P >> 1) + 3) >> 2;
     const uint32_t half = 4u * (uint32_t)G;
     const int desc_words = ROWS ? rows_desc_words(p.slots) : SiteDesc<ROWS ? 4 : DC>::DW;
+    const bool rec = !BITS && (COPY || !ROWS) && p.records;  // records in place of descriptors
 
     if constexpr (ROWS) {
         const int8_t* src = p.spins + (size_t)slot * p.slot_stride;
@@ -761,29 +753,32 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             const int par = c >= (int)half, h = c - par * (int)half;
             sp[x] = h < n_par ? src[(size_t)i * P + 2 * h + par] : (int8_t)1;
         }
-        // descriptors from the neighbour table: the sites with J = 0 are padding
+        // descriptors from the neighbour table (entries with J = 0 are padding), or (COPY) records:
+        // descriptors in schedule order with the parity worked in
         const uint32_t zero = (uint32_t)IndexRule(p.Lmax).zero();
-        for (int i = tid; i < N; i += nt) {
-            uint32_t* d = s_desc + (size_t)i * desc_words;
+        for (int x = tid; x < (rec ? 2 * N : N); x += nt) {
+            const uint32_t item = rec ? p.items[x] : 2u * (uint32_t)x;
+            const uint32_t i = item >> 1, shift = (item & 1u) * half, row = i * (uint32_t)RB;
+            uint32_t* d = s_desc + (size_t)x * desc_words;
             uint32_t sumJ = 0u, n = 0u;
             for (int k = 0; k < p.dmax; ++k) {
                 const uint32_t e = p.nbr[(size_t)i * p.dmax + k];
                 const uint32_t J = (uint32_t)(int)(int8_t)(e & 0xFFu);
                 if (J == 0u) continue;
-                d[4 + 2 * n] = (e >> 8) * (uint32_t)RB;
+                d[4 + 2 * n] = (e >> 8) * (uint32_t)RB + shift;
                 d[5 + 2 * n] = COPY ? J : J * (0u - kInv127);
                 sumJ += J;
                 ++n;
             }
             for (; n == 0u || (n & 3u); ++n) {  // at least the four slots every unit reads
-                d[4 + 2 * n] = (uint32_t)i * (uint32_t)RB;
+                d[4 + 2 * n] = row + shift;
                 d[5 + 2 * n] = 0u;
             }
             d[0] = COPY ? (uint32_t)(int)p.h[i]
                         : ((uint32_t)(int)p.h[i] + sumJ + zero + kInv127 * sumJ) * 0x01010101u;
-            d[1] = (uint32_t)i * (uint32_t)RB;
+            d[1] = row + shift;
             d[2] = n;
-            d[3] = 0u;
+            d[3] = row + half - shift;
         }
     } else if constexpr (NIB > 0) {
         load_bits<4>(reinterpret_cast<uint32_t*>(sp), p.spins + (size_t)slot * p.slot_stride, N, G, tid, nt);
@@ -813,9 +808,17 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     }
     {
         if constexpr (!ROWS) {
-            const int4* dsrc = reinterpret_cast<const int4*>(p.desc);
-            int4* ddst = reinterpret_cast<int4*>(s_desc);
-            for (int x = tid; x < N * desc_words / 4; x += nt) ddst[x] = dsrc[x];
+            if (rec) {
+                for (int x = tid; x < 2 * N; x += nt) {
+                    const uint32_t item = p.items[x];
+                    make_record<DC>(s_desc + (size_t)x * UnitRecord<DC>::kWords, p.desc + (item >> 1) * desc_words,
+                                    item, half);
+                }
+            } else {
+                const int4* dsrc = reinterpret_cast<const int4*>(p.desc);
+                int4* ddst = reinterpret_cast<int4*>(s_desc);
+                for (int x = tid; x < N * desc_words / 4; x += nt) ddst[x] = dsrc[x];
+            }
         }
         for (int x = tid; x < 2 * N; x += nt) s_items[x] = p.items[x];
         for (int x = tid; x <= p.n_levels; x += nt) s_loff[x] = p.level_off[x];
@@ -827,12 +830,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     long long E = p.E[slot], M = p.M[slot];  // meaningful in thread 0 only
 
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
-    int lgw = 0;
-    while ((1 << lgw) < G) ++lgw;
     const int cols = COPY ? P >> 1 : G;  // units of an item
-    int lg = 0;
-    while ((1 << lg) < cols) ++lg;
-    const int gmask = (1 << lg) - 1;
     const UnitRule<WIDE> rule(p.Lmax);
     // byte offset in shared memory at which the current rung's threshold row is looked up
     const int S = IndexRule(p.Lmax).S;
@@ -843,8 +841,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     const int n_items = 2 * N;
     const int lane = tid & 31;
     if (tid == 0) {
-        s_ctl[4] = -1;  // partner rung of the pending swap pass
-        s_ctl[5] = 0;   // a swap wait gave up
+        s_ctl[5] = 0;  // a swap wait gave up
         int* s_sum = reinterpret_cast<int*>(s_red);
         s_sum[0] = s_sum[1] = s_sum[2] = 0;  // the sweep's dE, dM and flips
     }
@@ -853,8 +850,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     __syncthreads();
     if (CSWAP) cluster_barrier();  // every CTA's mailboxes are clear before anyone publishes
     if (PRE && !PEER && !consumer)
-        produce_words(rbuf, (uint32_t)t0, s_items, n_items, G, lgw, (1 << lgw) - 1, tid - NC, nt - NC, (uint32_t)slot,
-                      key);
+        produce_words(rbuf, (uint32_t)t0, s_items, n_items, G, tid - NC, nt - NC, (uint32_t)slot, key);
     if (PEER) {
         // the peer CTA has written the first sweep's words (its arrival releases them); this
         // CTA's arrival orders nothing of its own, so it is relaxed
@@ -869,13 +865,22 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     // threshold row depends on the decision, and both candidate rows are in shared memory.
     // Up to two level-0 units per consumer thread are held in registers.
     // Warp 0 takes no level-0 unit, so that thread 0 can poll the partner's mailbox at once.
-    const int units0 = (s_loff[1] - s_loff[0]) << lg;
+    const int units0 = (s_loff[1] - s_loff[0]) * cols;
     const bool spec_ok = SPEC && !BITS && p.tables_in_smem && NC > 32 && units0 <= 2 * (NC - 32);
     bool spec_done = false;  // level 0 of sweep s was applied at the end of sweep s - 1
-    // units u = tid + k NC of a level have the same column g = u mod 2^lg when NC is a
-    // multiple of 2^lg: the thread then walks items q = base + (tid >> lg) + k (NC >> lg)
-    const bool g_fixed = (NC & gmask) == 0;
-    const int g_own = tid & gmask, q_lane = tid >> lg, q_step = NC >> lg;
+    int spec_q[2], spec_g[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int u = (tid - 32) + k * (NC - 32);
+        const bool ok = spec_ok && consumer && tid >= 32 && u < units0;
+        spec_q[k] = ok ? s_loff[0] + u / cols : -1;
+        spec_g[k] = ok ? u % cols : 0;
+    }
+    // With a thread for every column, a thread keeps its column g and walks the items q_lane,
+    // q_lane + q_step, ... of a level
+    const bool g_fixed = NC >= cols;
+    const int q_step = NC / cols, q_lane = tid / cols, g_own = tid - q_lane * cols;
+    const bool lane_ok = consumer && q_lane < q_step;
     FlipSums sums;
     sums.clear();
     BitSums nib_sums = {0, 0, 0};
@@ -892,12 +897,27 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         else
             return RowsColumn{row_offsets<1>((uint32_t)g, half), 0u, 0u};
     };
-    const Column col_own = column(min(g_own, cols - 1));  // this thread's fixed one
-    auto eval = [&](int q, int g, const Column& c, const uint4* rb, uint32_t t) -> Eval {
+    const Column col_own = column(g_own);  // this thread's fixed one
+    using Record = std::conditional_t<COPY, RowsTerms, LoadedRecord<ROWS ? 4 : DC>>;
+    auto load_rec = [&](int q) -> Record {
+        if constexpr (COPY)
+            return load_rows_site(s_desc + q * desc_words);
+        else
+            return load_record<ROWS ? 4 : DC>(s_desc + q * UnitRecord<ROWS ? 4 : DC>::kWords);
+    };
+    auto eval_rec = [&](const Record& r, int q, int g, const Column& c, const uint4* rb, uint32_t t) -> Eval {
+        if constexpr (COPY)
+            // word h % 4 of call h / 4: the words of an item's copies are consecutive
+            return copy_record_eval(sp, r, (uint32_t)g, c.edge[0] - half, c.edge[1],
+                                    reinterpret_cast<const uint32_t*>(rb + q * G)[g]);
+        else
+            return record_eval<ROWS ? 4 : DC, PRE, WIDE>(sp, r, 4u * (uint32_t)g, c.o.edge[0] - half, c.o.edge[1],
+                                                         rb + q * G + g, t, (uint32_t)slot, rule, key);
+    };
+    auto eval_desc = [&](int q, int g, const Column& c, const uint4* rb, uint32_t t) -> Eval {
         const uint32_t item = s_items[q];
         const uint32_t* desc = s_desc + (item >> 1) * (uint32_t)desc_words;
         if constexpr (COPY) {
-            // word h % 4 of call h / 4: the words of an item's copies are consecutive
             return copy_eval(sp, desc, item & 1u, c, reinterpret_cast<const uint32_t*>(rb + q * G)[g]);
         } else {
             UnitEval<1> e;
@@ -927,7 +947,8 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     SwapSide side;  // thread 0
     side.active = 0;
     const uint32_t qmod0 = (uint32_t)(q0 % kTagPeriod);
-    int since_pass = 0, next_pass = 0, sweep_flips = 0;  // thread 0
+    int since_pass = 0, next_pass = 0;
+    int sweep_flips = 0;  // thread 0
 
     for (int s = 0; s < n_sweeps; ++s) {
         const uint32_t t = (uint32_t)(t0 + s);
@@ -940,45 +961,75 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             if constexpr (NIB > 0) {
                 const IndexRule index(p.Lmax);
                 nib_sums.clear();
+                auto unit = [&](int q, uint32_t g, const UnitOffsets& off) {
+                    bits_unit<DC, NIB, 4>(sp, s_desc, s_items[q], off, g, t, (uint32_t)slot, key, smem,
+                                          (uint32_t)index.S, (uint32_t)(2 * p.Lmax - 255) * kInv255, thr_c, nib_sums);
+                };
+                const UnitOffsets off = word_offsets((uint32_t)g_own, (uint32_t)G);
                 for (int lev = 0; lev < p.n_levels; ++lev) {
-                    const int base = s_loff[lev];
-                    const int units = (s_loff[lev + 1] - base) << lg;
-                    for (int u = tid; u < units; u += NC) {
-                        const int g = u & gmask;
-                        if (g >= cols) continue;
-                        bits_unit<DC, NIB, 4>(sp, s_desc, s_items[base + (u >> lg)],
-                                              word_offsets((uint32_t)g, (uint32_t)G), (uint32_t)g, t, (uint32_t)slot,
-                                              key, smem, (uint32_t)index.S, (uint32_t)(2 * p.Lmax - 255) * kInv255,
-                                              thr_c, nib_sums);
+                    const int base = s_loff[lev], end = s_loff[lev + 1];
+                    if (g_fixed) {
+                        if (lane_ok)
+                            for (int q = base + q_lane; q < end; q += q_step) unit(q, (uint32_t)g_own, off);
+                    } else {
+                        for (int u = tid; u < (end - base) * cols; u += NC) {
+                            const int q = u / cols;
+                            unit(base + q, (uint32_t)(u - q * cols), word_offsets((uint32_t)(u - q * cols), (uint32_t)G));
+                        }
                     }
                     __syncthreads();
                 }
             } else {
-                for (int lev = spec_done ? 1 : 0; lev < p.n_levels; ++lev) {
-                    const int base = s_loff[lev];
-                    auto unit = [&](int q, int g, const Column& c) {
-                        if constexpr (BITS) {
-                            packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot, key,
-                                                       smem, rule, thr_c, sums);
-                        } else {
-                            const Eval e = eval(q, g, c, rb, t);
-                            commit(e, flips(e, c, thr_c));
+                const int lev0 = spec_done ? 1 : 0;
+                if (rec && g_fixed) {
+                    // this thread's column never changes: its row offsets are loop invariants. Each
+                    // level's first record is loaded before the barrier that ends the level before.
+                    int end = s_loff[min(lev0 + 1, p.n_levels)], q = s_loff[lev0] + q_lane;
+                    bool have = lane_ok && q < end;
+                    Record r = {};
+                    if (have) r = load_rec(q);
+                    for (int lev = lev0; lev < p.n_levels; ++lev) {
+                        const int end2 = s_loff[min(lev + 2, p.n_levels)];
+                        if (have) {
+                            Eval e = eval_rec(r, q, g_own, col_own, rb, t);
+                            commit(e, flips(e, col_own, thr_c));
+                            for (q += q_step; q < end; q += q_step) {
+                                e = eval_rec(load_rec(q), q, g_own, col_own, rb, t);
+                                commit(e, flips(e, col_own, thr_c));
+                            }
                         }
-                    };
-                    if (g_fixed) {
-                        // this thread's column never changes: its row offsets are loop invariants
-                        if (g_own < cols) {
-                            const int end = s_loff[lev + 1];
-                            for (int q = base + q_lane; q < end; q += q_step) unit(q, g_own, col_own);
-                        }
-                    } else {
-                        const int units = (s_loff[lev + 1] - base) << lg;
-                        for (int u = tid; u < units; u += NC) {
-                            const int g = u & gmask;
-                            if (g < cols) unit(base + (u >> lg), g, column(g));
-                        }
+                        q = end + q_lane;
+                        end = end2;
+                        have = lane_ok && q < end;
+                        if (have) r = load_rec(q);
+                        if (PRE) named_barrier(1, NC); else __syncthreads();
                     }
-                    if (PRE) named_barrier(1, NC); else __syncthreads();
+                } else {
+                    for (int lev = lev0; lev < p.n_levels; ++lev) {
+                        const int base = s_loff[lev];
+                        auto unit = [&](int q, int g, const Column& c) {
+                            if constexpr (BITS) {
+                                packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot,
+                                                           key, smem, rule, thr_c, sums);
+                            } else {
+                                const Eval e = rec ? eval_rec(load_rec(q), q, g, c, rb, t) : eval_desc(q, g, c, rb, t);
+                                commit(e, flips(e, c, thr_c));
+                            }
+                        };
+                        if (g_fixed) {
+                            if (lane_ok) {
+                                const int end = s_loff[lev + 1];
+                                for (int q = base + q_lane; q < end; q += q_step) unit(q, g_own, col_own);
+                            }
+                        } else {
+                            const int units = (s_loff[lev + 1] - base) * cols;
+                            for (int u = tid; u < units; u += NC) {
+                                const int q = u / cols, g = u - q * cols;
+                                unit(base + q, g, column(g));
+                            }
+                        }
+                        if (PRE) named_barrier(1, NC); else __syncthreads();
+                    }
                 }
             }
             // a chain's per-sweep changes fit in 32 bits: each warp adds its sums to three
@@ -1003,51 +1054,52 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                 atomicAdd(s_sum + 1, dM);
                 atomicAdd(s_sum + 2, dF);
             }
-            if (PRE) named_barrier(1, NC); else __syncthreads();
-            if (tid == 0) {
-                const int sE = s_sum[0], sM = s_sum[1];
-                sweep_flips = s_sum[2];
-                s_sum[0] = s_sum[1] = s_sum[2] = 0;
-                // a swap pass follows every sweeps_per_swap-th sweep (counted, not divided)
-                int pass = -1;
-                if (sweeps_per_swap > 0 && ++since_pass == sweeps_per_swap) {
-                    since_pass = 0;
-                    pass = next_pass++;
-                }
-                side = eos_publish(p, rung, E, M, sE, sM, pass, q0, qmod0, !CSWAP);
-                s_ctl[4] = side.active ? side.partner : -1;
-                if (CSWAP && side.active && rung != p.withhold_rung) {
-                    // the publication, into every CTA of the cluster (thread 0 alone: having
-                    // warp 0's lanes share the stores would make them wait for this thread,
-                    // which measured slower)
-                    const int idx = ((side.pass & (kClusterMailPasses - 1)) * p.R + rung) * 2;
-                    const unsigned long long wa = ((unsigned long long)E << 24) | side.tag;
-                    const unsigned long long wb = ((unsigned long long)(uint32_t)(int32_t)M << 32) | side.tag;
-                    for (int r = 0; r < p.R; ++r) st_cluster_u64x2(s_cmb + idx, (unsigned)r, wa, wb);
-                }
-            }
         } else if (PRE && !consumer && s + 1 < n_sweeps) {
             // producer warps only: a consumer whose swap wait gave up skips to the barrier below
-            produce_words(rbuf + (size_t)((s + 1) & 1) * n_items * G, t + 1u, s_items, n_items, G, lgw,
-                          (1 << lgw) - 1, tid - NC, nt - NC, (uint32_t)slot, key);
+            produce_words(rbuf + (size_t)((s + 1) & 1) * n_items * G, t + 1u, s_items, n_items, G, tid - NC, nt - NC,
+                          (uint32_t)slot, key);
         }
-        // the next sweep's random words are complete and every consumer has finished sweep s;
-        // a wait that gave up in the previous sweep ends the launch here, for every thread
+        // a swap pass follows every sweeps_per_swap-th sweep (counted, not divided)
+        int pass = -1;
+        if (sweeps_per_swap > 0 && ++since_pass == sweeps_per_swap) {
+            since_pass = 0;
+            pass = next_pass++;
+        }
+        // the sweep's sums and the next sweep's random words are complete, and every consumer has
+        // finished sweep s; a wait that gave up in the previous sweep ends the launch here, for
+        // every thread
         if constexpr (PEER) {
-            // the peer CTA learns at the same barrier that this CTA leaves, and leaves too.
-            // Otherwise the arrival is relaxed: a release would first wait for this sweep's
-            // mailbox store to reach L2, on the way to the swap decision. The words this CTA
-            // read are in registers by now, so the peer may overwrite their buffer.
+            // The peer CTA learns at the cluster barrier that this CTA leaves, and leaves too.
+            // Otherwise the arrival is relaxed: a release would first wait for earlier global
+            // stores to reach L2, on the way to the swap decision. The words this CTA read are in
+            // registers by now, so the peer may overwrite their buffer.
+            named_barrier(1, NC);
             if (s_ctl[5]) {
                 if (tid == 0) cg::this_cluster().map_shared_rank(s_ctl, 1)[6] = 1;
                 cluster_arrive_release();
             } else {
                 cluster_arrive_relaxed();
             }
-            cluster_wait_acquire();
         } else {
             __syncthreads();
         }
+        if (tid == 0 && !s_ctl[5]) {
+            int* s_sum = reinterpret_cast<int*>(s_red);
+            const int sE = s_sum[0], sM = s_sum[1];
+            sweep_flips = s_sum[2];
+            s_sum[0] = s_sum[1] = s_sum[2] = 0;
+            side = eos_publish(p, rung, E, M, sE, sM, pass, q0, qmod0, !CSWAP);
+            if (CSWAP && side.active && rung != p.withhold_rung) {
+                // the publication, into every CTA of the cluster (thread 0 alone: having
+                // warp 0's lanes share the stores would make them wait for this thread,
+                // which measured slower)
+                const int idx = ((side.pass & (kClusterMailPasses - 1)) * p.R + rung) * 2;
+                const unsigned long long wa = ((unsigned long long)E << 24) | side.tag;
+                const unsigned long long wb = ((unsigned long long)(uint32_t)(int32_t)M << 32) | side.tag;
+                for (int r = 0; r < p.R; ++r) st_cluster_u64x2(s_cmb + idx, (unsigned)r, wa, wb);
+            }
+        }
+        if constexpr (PEER) cluster_wait_acquire();
         if (s_ctl[5]) {  // status holds PT_ETIMEDOUT
             if (CSWAP) break;  // to the cluster barrier that every CTA passes before leaving
             return;
@@ -1056,7 +1108,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
 
         // level 0 of sweep s + 1 under both candidate rungs
         const bool spec = spec_ok && s + 1 < n_sweeps;
-        const int prung = s_ctl[4];
+        const int prung = pass >= 0 ? pair_rung(rung, q0 + pass, p.R) : -1;
         Eval ev[2];
         uint32_t Fa[2] = {0u, 0u}, Fb[2] = {0u, 0u};
         bool valid[2] = {false, false};
@@ -1065,13 +1117,11 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             const uint32_t thr_b = prung >= 0 ? thr0 + thr_step * (uint32_t)prung : thr_c;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                const int u = (tid - 32) + k * (NC - 32);
-                const int g = u & gmask;
-                valid[k] = tid >= 32 && u < units0 && g < cols;
+                valid[k] = spec_q[k] >= 0;
                 if (valid[k]) {
-                    const int q = s_loff[0] + (u >> lg);
+                    const int q = spec_q[k], g = spec_g[k];
                     const Column c = column(g);
-                    ev[k] = eval(q, g, c, rb1, t + 1u);
+                    ev[k] = rec ? eval_rec(load_rec(q), q, g, c, rb1, t + 1u) : eval_desc(q, g, c, rb1, t + 1u);
                     Fa[k] = flips(ev[k], c, thr_c);
                     Fb[k] = prung >= 0 ? flips(ev[k], c, thr_b) : Fa[k];
                 }
@@ -1086,14 +1136,17 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                                        : eos_decide(p, side, rung, E, M, timeout_ns, key, &abort_flag);
             if (abort_flag) s_ctl[5] = 1;  // a partner never arrived
         }
-        if (PRE) named_barrier(1, NC); else __syncthreads();
-        if (s_ctl[5]) continue;  // skip to the next barrier with the producers, then leave
-        const int nr = s_ctl[2 * (s & 1)];
-        const bool moved = nr != rung;
-        if (moved) {
-            rung = nr;
-            if (!p.tables_in_smem) load_thr_columns(p, s_thr, rung, tid, NC);
-            thr_c = thr0 + thr_step * (uint32_t)rung;
+        bool moved = false;
+        if (prung >= 0) {  // nobody waits for a decision that is not to be taken
+            if (PRE) named_barrier(1, NC); else __syncthreads();
+            if (s_ctl[5]) continue;  // skip to the next barrier with the producers, then leave
+            const int nr = s_ctl[2 * (s & 1)];
+            moved = nr != rung;
+            if (moved) {
+                rung = nr;
+                if (!p.tables_in_smem) load_thr_columns(p, s_thr, rung, tid, NC);
+                thr_c = thr0 + thr_step * (uint32_t)rung;
+            }
         }
         spec_done = spec;
         if (spec) {
@@ -1158,19 +1211,16 @@ __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n
     int* s_ctl = reinterpret_cast<int*>(smem + L.ctl);
     uint4* peer_rbuf = cluster.map_shared_rank(reinterpret_cast<uint4*>(smem + L.rbuf), 0);
     const int n_items = 2 * p.N, G = p.P >> 3;
-    int lg = 0;
-    while ((1 << lg) < G) ++lg;
-    const int gmask = (1 << lg) - 1;
     for (int x = tid; x < n_items; x += nt) s_items[x] = p.items[x];
     if (tid == 0) s_ctl[6] = 0;
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
     __syncthreads();
-    produce_words(peer_rbuf, (uint32_t)t0, s_items, n_items, G, lg, gmask, tid, nt, (uint32_t)slot, key);
+    produce_words(peer_rbuf, (uint32_t)t0, s_items, n_items, G, tid, nt, (uint32_t)slot, key);
     cluster_barrier();  // release: the words are visible to rank 0 after its wait
     for (int s = 0; s < n_sweeps; ++s) {
         if (s + 1 < n_sweeps)
             produce_words(peer_rbuf + (size_t)((s + 1) & 1) * n_items * G, (uint32_t)(t0 + s + 1), s_items, n_items, G,
-                          lg, gmask, tid, nt, (uint32_t)slot, key);
+                          tid, nt, (uint32_t)slot, key);
         cluster_barrier();
         if (s_ctl[6]) return;  // rank 0's swap wait gave up; it leaves after this barrier too
     }
