@@ -210,8 +210,8 @@ __device__ __forceinline__ void eos_stats(const DevProblem& p, unsigned long lon
     }
 }
 
-// Thread 0 again: wait for the partner's mailbox (bounded by timeout_ns) and take the decision
-// both chains of the pair take. Returns the chain's rung for the next sweep; sets *abort when
+// One thread, or a warp whose lanes all follow E and M (count in one of them): wait for the
+// partner's mailbox (bounded by timeout_ns) and take the decision both chains of the pair take. Returns the chain's rung for the next sweep; sets *abort when
 // the partner's mailbox never arrived within the time limit. read(partner, wa, wb) loads the
 // partner's two tagged words. The pass's coefficients and random word do not depend on the
 // partner and are fetched before the wait, as is nothing but the loads and the comparison
@@ -274,9 +274,10 @@ __device__ __forceinline__ int eos_decide(const DevProblem& p, const SwapSide& w
 // the pass two later, in which it waits for the reader's own publication again.
 __device__ __forceinline__ int eos_decide_cluster(const DevProblem& p, const unsigned long long* s_cmb,
                                                   const SwapSide& w, int rung, long long E, long long M,
-                                                  long long timeout_ns, const PhiloxKey& key, int* abort) {
+                                                  long long timeout_ns, const PhiloxKey& key, int* abort,
+                                                  bool count = true) {
     const unsigned long long* mb = s_cmb + (size_t)(w.pass & (kClusterMailPasses - 1)) * p.R * 2;
-    return eos_decide_from(p, w, rung, E, M, timeout_ns, key, abort, true,
+    return eos_decide_from(p, w, rung, E, M, timeout_ns, key, abort, count,
                            [&](int partner, unsigned long long& wa, unsigned long long& wb) {
                                wa = ld_cluster_local_u64(mb + 2 * partner);
                                wb = ld_cluster_local_u64(mb + 2 * partner + 1);
@@ -944,11 +945,12 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         else
             unit_commit<1>(e, &F, sums);
     };
-    SwapSide side;  // thread 0
+    const bool ender = CSWAP ? tid < 32 : tid == 0;  // follows E and M and ends the sweeps
+    SwapSide side;  // ender
     side.active = 0;
     const uint32_t qmod0 = (uint32_t)(q0 % kTagPeriod);
     int since_pass = 0, next_pass = 0;
-    int sweep_flips = 0;  // thread 0
+    int sweep_flips = 0;  // ender
 
     for (int s = 0; s < n_sweeps; ++s) {
         const uint32_t t = (uint32_t)(t0 + s);
@@ -1083,20 +1085,22 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         } else {
             __syncthreads();
         }
-        if (tid == 0 && !s_ctl[5]) {
+        // Thread 0 ends the sweep. On path 9 all of warp 0 does, every lane with the same E and M, so
+        // that lane r writes the publication into CTA r (one store instruction; thread 0 alone took
+        // 17 cycles a copy: 2.42 -> 2.32 us per sweep on N=16, P=32, R=16; through global mailboxes
+        // a warp's polls measured 0.1 us slower than one thread's).
+        if (ender && !s_ctl[5]) {
             int* s_sum = reinterpret_cast<int*>(s_red);
             const int sE = s_sum[0], sM = s_sum[1];
             sweep_flips = s_sum[2];
-            s_sum[0] = s_sum[1] = s_sum[2] = 0;
-            side = eos_publish(p, rung, E, M, sE, sM, pass, q0, qmod0, !CSWAP);
-            if (CSWAP && side.active && rung != p.withhold_rung) {
-                // the publication, into every CTA of the cluster (thread 0 alone: having
-                // warp 0's lanes share the stores would make them wait for this thread,
-                // which measured slower)
+            if (CSWAP) __syncwarp();
+            if (lane == 0) s_sum[0] = s_sum[1] = s_sum[2] = 0;
+            side = eos_publish(p, rung, E, M, sE, sM, pass, q0, qmod0, !CSWAP && lane == 0);
+            if (CSWAP && side.active && rung != p.withhold_rung && lane < p.R) {
                 const int idx = ((side.pass & (kClusterMailPasses - 1)) * p.R + rung) * 2;
                 const unsigned long long wa = ((unsigned long long)E << 24) | side.tag;
                 const unsigned long long wb = ((unsigned long long)(uint32_t)(int32_t)M << 32) | side.tag;
-                for (int r = 0; r < p.R; ++r) st_cluster_u64x2(s_cmb + idx, (unsigned)r, wa, wb);
+                st_cluster_u64x2(s_cmb + idx, (unsigned)lane, wa, wb);
             }
         }
         if constexpr (PEER) cluster_wait_acquire();
@@ -1127,14 +1131,21 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                 }
             }
         }
-        if (tid == 0) {
+        if (ender) {
             // the statistics of sweep s (rung unchanged until the decision below), while
             // the partner's mailbox may still be on its way
-            eos_stats(p, p.acc_in_smem ? s_acc : p.acc, rung, E, M, sweep_flips);
-            int abort_flag = 0;
-            s_ctl[2 * (s & 1)] = CSWAP ? eos_decide_cluster(p, s_cmb, side, rung, E, M, timeout_ns, key, &abort_flag)
-                                       : eos_decide(p, side, rung, E, M, timeout_ns, key, &abort_flag);
-            if (abort_flag) s_ctl[5] = 1;  // a partner never arrived
+            if (lane == 0) eos_stats(p, p.acc_in_smem ? s_acc : p.acc, rung, E, M, sweep_flips);
+            if (prung >= 0) {
+                int abort_flag = 0;
+                const int next =
+                    CSWAP ? eos_decide_cluster(p, s_cmb, side, rung, E, M, timeout_ns, key, &abort_flag, lane == 0)
+                          : eos_decide(p, side, rung, E, M, timeout_ns, key, &abort_flag, lane == 0);
+                if (CSWAP) __syncwarp();
+                if (lane == 0) {
+                    s_ctl[2 * (s & 1)] = next;
+                    if (abort_flag) s_ctl[5] = 1;  // a partner never arrived
+                }
+            }
         }
         bool moved = false;
         if (prung >= 0) {  // nobody waits for a decision that is not to be taken
