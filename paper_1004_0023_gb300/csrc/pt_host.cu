@@ -699,24 +699,30 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         }
         return resident >= R;
     };
-    // path 8 when the produced-words layout fits and all R two-CTA clusters can be resident
-    auto peer_fits = [&](int th) {
-        if (!fits(kPathPacked) || th < 64) return false;
-        DevProblem q = p;
-        if (sweep_smem_bytes(q, kPathPeer, packed_dc) > (size_t)max_smem) q.tables_in_smem = 0;
-        if (sweep_smem_bytes(q, kPathPeer, packed_dc) > (size_t)max_smem) q.acc_in_smem = 0;
-        LaunchPlan probe;
-        probe.path = kPathPeer;
-        probe.dclass = packed_dc;
-        probe.threads = th;
-        probe.n_consumer = th;
-        probe.smem_bytes = sweep_smem_bytes(q, kPathPeer, packed_dc);
-        long long resident = 0;
-        if (prepare_sweep_kernel(probe) != cudaSuccess || sweep_resident_chains(q, probe, &resident) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return false;
+    // path 8's pieces of a sweep: levels in turn while their updates number at most `cap`
+    auto cut_sweep = [&](DevProblem& q, const std::vector<int32_t>& off, int pieces) {
+        const int n_lev = (int)off.size() - 1;
+        q.n_chunks = 0;
+        q.chunk_items = 0;
+        if (pieces <= 1) return true;
+        int cap = (off[n_lev] + pieces - 1) / pieces;
+        for (;; cap += std::max(1, cap / 32)) {  // the first capacity that needs no more than `pieces`
+            int n = 0, most = 0;
+            for (int l = 0; l < n_lev; ++n) {
+                int m = l + 1;
+                while (m < n_lev && off[m + 1] - off[l] <= cap) ++m;
+                if (n < kMaxChunks) q.chunk_level[n] = (int16_t)l;
+                most = std::max(most, off[m] - off[l]);
+                l = m;
+            }
+            if (n <= pieces) {
+                q.n_chunks = n;
+                q.chunk_items = most;
+                q.chunk_level[n] = (int16_t)n_lev;
+                return n_lev < 32768;
+            }
+            if (cap >= off[n_lev]) return false;
         }
-        return resident >= R;
     };
     if (path == 0) {
         path = kPathGeneric;
@@ -1062,8 +1068,9 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                     if (th >= P / 16 + 1) cands.push_back({kPathSplitInline, th, 0});
             if (fits(kPathPackedInline))
                 for (int th : {256, 384, 512}) cands.push_back({kPathPackedInline, th, 0});
-            for (int th : {384, 512})
-                if (peer_fits(th)) cands.push_back({kPathPeer, th, 0});
+            // path 8, its random words in pieces of a sweep where whole sweeps do not fit (make)
+            if (2 * R <= n_sm)
+                for (int th : {384, 512}) cands.push_back({kPathPeer, th, 0});
             // every chain's CTA in one cluster, swap mailboxes in shared memory (R <= 16), with
             // the random words inline or from producer warps
             if (R <= 16)
@@ -1090,7 +1097,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         auto make = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
                         std::vector<int32_t>& off_c) {
             pc = p;
-            pc.records = 0;
+            pc.records = pc.n_chunks = 0;
             if (cd.path == kPathClassical) {
                 pc.acc_in_smem = 1;
                 pc.tables_in_smem = 1;
@@ -1147,6 +1154,23 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / cols), row_words_for(cd.path));
             if (P == 1) drop_odd_updates(it_c, off_c);
             pc.n_levels = (int)off_c.size() - 1;
+            if (cd.path == kPathPeer) {
+                // The fewest pieces of a sweep (cut_sweep) with which the layout fits, with records in
+                // at most four, else without: N=512, P=64, R=64 runs 6.47 us per sweep with swaps in
+                // pieces; path 6, the fastest otherwise, 7.70. From P = 128 the split kernels
+                // (paths 5 and 6) hold such chains in two CTAs, and are what is timed.
+                pl.dclass = packed_dc;
+                for (pc.records = records_for(cd.path, 0); pc.records >= 0; --pc.records)
+                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : pc.records ? 4 : kMaxChunks); ++pieces) {
+                        pc.tables_in_smem = (size_t)R * p.nL3 * 4 <= 49152 ? 1 : 0;
+                        pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
+                        if (!cut_sweep(pc, off_c, pieces)) continue;
+                        pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc);
+                        pl.pieces = pc.n_chunks;
+                        if (pl.smem_bytes <= (size_t)max_smem) return true;
+                    }
+                return false;
+            }
             pc.records = records_for(cd.path, 0);
             if (pc.records && sweep_smem_bytes(pc, cd.path, pl.dclass, cpre) > (size_t)max_smem) pc.records = 0;
             pl.smem_bytes = sweep_smem_bytes(pc, cd.path, pl.dclass, cpre);  // sized for this schedule
@@ -1252,6 +1276,9 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                     p.acc_in_smem = pc.acc_in_smem;
                     p.tables_in_smem = pc.tables_in_smem;
                     p.records = pc.records;
+                    p.n_chunks = pc.n_chunks;
+                    p.chunk_items = pc.chunk_items;
+                    memcpy(p.chunk_level, pc.chunk_level, sizeof(p.chunk_level));
                     if (!cached) {
                         std::lock_guard<std::mutex> lock(g_plan_mutex);
                         const Cand& cb = cands[best];

@@ -27,6 +27,7 @@ struct alignas(16) Mailbox {
     unsigned long long b;
 };
 constexpr long long kTagPeriod = 16777215ll;
+constexpr int kMaxChunks = 8;          // path 8: pieces of a sweep whose random words are made at a time
 constexpr int kClusterMailPasses = 4;  // path 9: swap passes whose mailboxes each CTA holds at once
 
 // Multiplicative inverses modulo 2^32 (Newton's iteration doubles the correct low bits).
@@ -92,6 +93,10 @@ struct DevProblem {
     int tables_in_smem;        // 1: every rung's threshold row resident in shared memory
     int slots;                 // path 1: neighbour slots of a site descriptor (a multiple of 4) when the
                                // word-wise kernel runs, 0: the byte-wise one
+    // Path 8: a sweep's random words come in n_chunks pieces, the words of levels chunk_level[c] to
+    // chunk_level[c + 1] - 1 (at most chunk_items updates); n_chunks <= 1: the whole sweep at once.
+    int n_chunks, chunk_items;
+    int16_t chunk_level[kMaxChunks + 1];
     int records;               // 1: per-update records in schedule order in shared memory (see record_words)
     int nibble;                // path 4: 1 = the nibble form of the bit-packed chain
     int exact_swaps;           // test hook: 1 = always take the FP64 swap decision
@@ -128,6 +133,7 @@ struct LaunchPlan {
     int thr_resident = 0;   // path 7: every rung's threshold row in shared memory
     int form = 0, form_t = 0;  // path 7: kForm* of a chain
     int n_groups = 0;       // path 7: chain groups of a CTA
+    int pieces = 0;         // path 8: > 1 where the random words come in pieces of a sweep
     int copy = 0;           // paths 1, 3 and 9: one copy a thread (sweep_copy_kernel)
     int nibble = 0;         // path 4: neighbour slots of the nibble form, 0 = one bit a copy
     int rows = 0;           // path 1: the word-wise kernel (DevProblem::slots > 0)

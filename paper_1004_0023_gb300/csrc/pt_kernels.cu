@@ -106,7 +106,7 @@ struct FastLayout {
         ctl = o;   o += 32;
         cmb = o;   o += cswap ? (size_t)kClusterMailPasses * p.R * 16 : 0;
         rbuf = o;
-        if (pre) o += (size_t)2 * (2 * N) * (P / 8) * 16;
+        if (pre) o += (size_t)2 * (p.n_chunks > 1 ? p.chunk_items : 2 * N) * (P / 8) * 16;
         total = o;
     }
 };
@@ -706,9 +706,10 @@ __device__ __forceinline__ void produce_words(uint4* buf, uint32_t t, const uint
 // cluster barrier only after the mailboxes are cleared and before they leave.
 // DC = 0: path 1's word-wise kernel (RowsLayout, rows_unit_eval) on the same loop.
 // COPY (with DC = 0 and PRE): one copy a thread.
+// PIECES (with PEER): a sweep's random words come in p.n_chunks pieces (pt_internal.h).
 // NIB > 0: the nibble form of the bit-packed chain with NIB neighbour slots in use.
 template <int DC, bool PRE, bool WIDE, bool BITS = false, bool SPEC = true, bool PEER = false, bool CSWAP = false,
-          int NIB = 0, bool COPY = false>
+          int NIB = 0, bool COPY = false, bool PIECES = false>
 __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot, long long t0, long long q0,
                                                   int n_sweeps, int sweeps_per_swap, long long timeout_ns,
                                                   int n_consumer, unsigned char* smem) {
@@ -882,6 +883,9 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     const bool g_fixed = NC >= cols;
     const int q_step = NC / cols, q_lane = tid / cols, g_own = tid - q_lane * cols;
     const bool lane_ok = consumer && q_lane < q_step;
+    // words of one of the two buffers; PIECES: pieces used so far
+    const size_t buf_words = (size_t)(PIECES ? p.chunk_items : n_items) * G;
+    int chunk = 0;
     FlipSums sums;
     sums.clear();
     BitSums nib_sums = {0, 0, 0};
@@ -955,7 +959,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     for (int s = 0; s < n_sweeps; ++s) {
         const uint32_t t = (uint32_t)(t0 + s);
         if (consumer && !s_ctl[5]) {
-            const uint4* rb = rbuf + (size_t)(s & 1) * n_items * G;
+            const uint4* rb = rbuf + (size_t)((PIECES ? chunk : s) & 1) * buf_words;
             if (!spec_done) {
                 sums.clear();
                 copy_sums = CopySums{0, 0, 0};
@@ -982,55 +986,64 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                     __syncthreads();
                 }
             } else {
-                const int lev0 = spec_done ? 1 : 0;
-                if (rec && g_fixed) {
-                    // this thread's column never changes: its row offsets are loop invariants. Each
-                    // level's first record is loaded before the barrier that ends the level before.
-                    int end = s_loff[min(lev0 + 1, p.n_levels)], q = s_loff[lev0] + q_lane;
-                    bool have = lane_ok && q < end;
-                    Record r = {};
-                    if (have) r = load_rec(q);
-                    for (int lev = lev0; lev < p.n_levels; ++lev) {
-                        const int end2 = s_loff[min(lev + 2, p.n_levels)];
-                        if (have) {
-                            Eval e = eval_rec(r, q, g_own, col_own, rb, t);
-                            commit(e, flips(e, col_own, thr_c));
-                            for (q += q_step; q < end; q += q_step) {
-                                e = eval_rec(load_rec(q), q, g_own, col_own, rb, t);
-                                commit(e, flips(e, col_own, thr_c));
-                            }
-                        }
-                        q = end + q_lane;
-                        end = end2;
-                        have = lane_ok && q < end;
-                        if (have) r = load_rec(q);
-                        if (PRE) named_barrier(1, NC); else __syncthreads();
+                for (int piece = 0; piece < (PIECES ? p.n_chunks : 1); ++piece) {
+                    if (PIECES && piece > 0) {  // the next piece's words; this one's are no longer needed
+                        cluster_arrive_relaxed();
+                        cluster_wait_acquire();
+                        ++chunk;
+                        rb = rbuf + (size_t)(chunk & 1) * buf_words - (size_t)s_loff[p.chunk_level[piece]] * G;
                     }
-                } else {
-                    for (int lev = lev0; lev < p.n_levels; ++lev) {
-                        const int base = s_loff[lev];
-                        auto unit = [&](int q, int g, const Column& c) {
-                            if constexpr (BITS) {
-                                packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot,
-                                                           key, smem, rule, thr_c, sums);
-                            } else {
-                                const Eval e = rec ? eval_rec(load_rec(q), q, g, c, rb, t) : eval_desc(q, g, c, rb, t);
-                                commit(e, flips(e, c, thr_c));
+                    const int lev0 = piece > 0 ? p.chunk_level[piece] : spec_done ? 1 : 0;
+                    const int lev_end = PIECES ? p.chunk_level[piece + 1] : p.n_levels;
+                    if (rec && g_fixed) {
+                        // this thread's column never changes: its row offsets are loop invariants. Each
+                        // level's first record is loaded before the barrier that ends the level before.
+                        int end = s_loff[min(lev0 + 1, lev_end)], q = s_loff[lev0] + q_lane;
+                        bool have = lane_ok && q < end;
+                        Record r = {};
+                        if (have) r = load_rec(q);
+                        for (int lev = lev0; lev < lev_end; ++lev) {
+                            const int end2 = s_loff[min(lev + 2, lev_end)];
+                            if (have) {
+                                Eval e = eval_rec(r, q, g_own, col_own, rb, t);
+                                commit(e, flips(e, col_own, thr_c));
+                                for (q += q_step; q < end; q += q_step) {
+                                    e = eval_rec(load_rec(q), q, g_own, col_own, rb, t);
+                                    commit(e, flips(e, col_own, thr_c));
+                                }
                             }
-                        };
-                        if (g_fixed) {
-                            if (lane_ok) {
-                                const int end = s_loff[lev + 1];
-                                for (int q = base + q_lane; q < end; q += q_step) unit(q, g_own, col_own);
-                            }
-                        } else {
-                            const int units = (s_loff[lev + 1] - base) * cols;
-                            for (int u = tid; u < units; u += NC) {
-                                const int q = u / cols, g = u - q * cols;
-                                unit(base + q, g, column(g));
-                            }
+                            q = end + q_lane;
+                            end = end2;
+                            have = lane_ok && q < end;
+                            if (have) r = load_rec(q);
+                            if (PRE) named_barrier(1, NC); else __syncthreads();
                         }
-                        if (PRE) named_barrier(1, NC); else __syncthreads();
+                    } else {
+                        for (int lev = lev0; lev < lev_end; ++lev) {
+                            const int base = s_loff[lev];
+                            auto unit = [&](int q, int g, const Column& c) {
+                                if constexpr (BITS) {
+                                    packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot,
+                                                               key, smem, rule, thr_c, sums);
+                                } else {
+                                    const Eval e = rec ? eval_rec(load_rec(q), q, g, c, rb, t) : eval_desc(q, g, c, rb, t);
+                                    commit(e, flips(e, c, thr_c));
+                                }
+                            };
+                            if (g_fixed) {
+                                if (lane_ok) {
+                                    const int end = s_loff[lev + 1];
+                                    for (int q = base + q_lane; q < end; q += q_step) unit(q, g_own, col_own);
+                                }
+                            } else {
+                                const int units = (s_loff[lev + 1] - base) * cols;
+                                for (int u = tid; u < units; u += NC) {
+                                    const int q = u / cols, g = u - q * cols;
+                                    unit(base + q, g, column(g));
+                                }
+                            }
+                            if (PRE) named_barrier(1, NC); else __syncthreads();
+                        }
                     }
                 }
             }
@@ -1061,6 +1074,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             produce_words(rbuf + (size_t)((s + 1) & 1) * n_items * G, t + 1u, s_items, n_items, G, tid - NC, nt - NC,
                           (uint32_t)slot, key);
         }
+        ++chunk;
         // a swap pass follows every sweeps_per_swap-th sweep (counted, not divided)
         int pass = -1;
         if (sweeps_per_swap > 0 && ++since_pass == sweeps_per_swap) {
@@ -1117,7 +1131,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         uint32_t Fa[2] = {0u, 0u}, Fb[2] = {0u, 0u};
         bool valid[2] = {false, false};
         if (spec) {
-            const uint4* rb1 = rbuf + (size_t)((s + 1) & 1) * n_items * G;
+            const uint4* rb1 = rbuf + (size_t)((PIECES ? chunk : s + 1) & 1) * buf_words;
             const uint32_t thr_b = prung >= 0 ? thr0 + thr_step * (uint32_t)prung : thr_c;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -1209,11 +1223,12 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
 }
 
 // Path 8, rank 1 of each cluster: the random words of every sweep of chain `slot`, written
-// one sweep ahead into rank 0's double buffer through distributed shared memory (the words
+// one sweep (or piece of a sweep, where two whole sweeps' words do not fit: DevProblem::n_chunks)
+// ahead into rank 0's double buffer through distributed shared memory (the words
 // are a function of the chain, the sweep and the update, never of the rung, so they need no
 // swap decision). It passes the same cluster barriers as rank 0 (one before the first sweep,
 // one per sweep) and leaves after the one at which rank 0 reports that it leaves.
-template <int DC>
+template <int DC, bool PIECES>
 __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n_sweeps, unsigned char* smem) {
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -1222,25 +1237,38 @@ __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n
     int* s_ctl = reinterpret_cast<int*>(smem + L.ctl);
     uint4* peer_rbuf = cluster.map_shared_rank(reinterpret_cast<uint4*>(smem + L.rbuf), 0);
     const int n_items = 2 * p.N, G = p.P >> 3;
+    int32_t* s_loff = reinterpret_cast<int32_t*>(smem + L.loff);
     for (int x = tid; x < n_items; x += nt) s_items[x] = p.items[x];
+    for (int x = tid; x <= p.n_levels; x += nt) s_loff[x] = p.level_off[x];
     if (tid == 0) s_ctl[6] = 0;
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
     __syncthreads();
-    produce_words(peer_rbuf, (uint32_t)t0, s_items, n_items, G, tid, nt, (uint32_t)slot, key);
+    const int pieces = PIECES ? p.n_chunks : 1;
+    const size_t buf_words = (size_t)(PIECES ? p.chunk_items : n_items) * G;
+    // piece k of the launch (piece k % pieces of sweep t0 + k / pieces), into buffer k & 1
+    auto produce = [&](int sweep, int piece, int buffer) {
+        const int first = PIECES ? s_loff[p.chunk_level[piece]] : 0;
+        const int end = PIECES ? s_loff[p.chunk_level[piece + 1]] : n_items;
+        produce_words(peer_rbuf + (size_t)buffer * buf_words, (uint32_t)(t0 + sweep), s_items + first, end - first, G,
+                      tid, nt, (uint32_t)slot, key);
+    };
+    produce(0, 0, 0);
     cluster_barrier();  // release: the words are visible to rank 0 after its wait
-    for (int s = 0; s < n_sweeps; ++s) {
-        if (s + 1 < n_sweeps)
-            produce_words(peer_rbuf + (size_t)((s + 1) & 1) * n_items * G, (uint32_t)(t0 + s + 1), s_items, n_items, G,
-                          tid, nt, (uint32_t)slot, key);
-        cluster_barrier();
-        if (s_ctl[6]) return;  // rank 0's swap wait gave up; it leaves after this barrier too
-    }
+    int buffer = 0;
+    for (int s = 0; s < n_sweeps; ++s)
+        for (int piece = 0; piece < pieces; ++piece) {
+            buffer ^= 1;
+            const bool wrap = piece + 1 == pieces;
+            if (!wrap || s + 1 < n_sweeps) produce(wrap ? s + 1 : s, wrap ? 0 : piece + 1, buffer);
+            cluster_barrier();
+            if (s_ctl[6]) return;  // rank 0's swap wait gave up; it leaves after this barrier too
+        }
 }
 
 // Path 8: R clusters of two CTAs; rank 0 sweeps chain (cluster index) with every thread,
 // rank 1 produces its random words. The cluster shape is compiled in, and checked on entry
 // (both CTAs return before any barrier or remote access if it is not 2).
-template <int DC>
+template <int DC, bool PIECES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     sweep_peer_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                       long long timeout_ns, int n_consumer) {
@@ -1253,13 +1281,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     const int slot = (int)(blockIdx.x >> 1);
     if (cluster.block_rank() == 0) {
         if (IndexRule(p.Lmax).wide)
-            sweep_packed_body<DC, true, true, false, true, true>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
+            sweep_packed_body<DC, true, true, false, true, true, false, 0, false, PIECES>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
                                                                  timeout_ns, blockDim.x, smem);
         else
-            sweep_packed_body<DC, true, false, false, true, true>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
+            sweep_packed_body<DC, true, false, false, true, true, false, 0, false, PIECES>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
                                                                   timeout_ns, blockDim.x, smem);
     } else
-        peer_producer<DC>(p, slot, t0, n_sweeps, smem);
+        peer_producer<DC, PIECES>(p, slot, t0, n_sweeps, smem);
 }
 
 template <int DC, bool PRE, int MAXT, bool BITS = false>
@@ -1871,8 +1899,11 @@ static const void* sweep_fn(const LaunchPlan& plan) {
             default: return (const void*)sweep_kernel<32>;
         }
     }
-    if (plan.path == kPathPeer)
-        return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4> : (const void*)sweep_peer_kernel<8>;
+    if (plan.path == kPathPeer) {
+        if (plan.pieces > 1)
+            return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, true> : (const void*)sweep_peer_kernel<8, true>;
+        return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, false> : (const void*)sweep_peer_kernel<8, false>;
+    }
     if (plan.path == kPathCluster) {
         const bool pre = plan.n_consumer < plan.threads;
         if (plan.dclass == 4)

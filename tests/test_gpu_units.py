@@ -113,3 +113,23 @@ def test_batched_chain_forms_match_the_oracle(cluster):
                 og, oo = b.obs(k), o.obs()
                 for key in oo:
                     assert np.array_equal(np.asarray(og[key]), np.asarray(oo[key])), (BATCH[k], run, key)
+
+
+@pytest.mark.parametrize("n,degree,P,R,lmax,pieces", [
+    (512, 3, 64, 6, 13, True), (512, 1, 64, 4, 5, False), (500, 7, 64, 5, 41, False), (512, 7, 64, 4, 42, False),
+    (420, 3, 72, 5, 31, False), (300, 5, 120, 3, 60, False),
+])
+def test_chains_whose_random_words_do_not_fit_whole_match_the_oracle(n, degree, P, R, lmax, pieces):
+    """Automatic plans of chains too large for two sweeps of produced words: path 8 makes them in
+    pieces of a sweep. `pieces`: it is the fastest there by a quarter, so it has to be the plan."""
+    prob = _problem(n, degree, P, R, lmax, n + P)
+    g, o = pt.PT.from_problem(prob), Oracle.from_problem(prob, threads=THREADS)
+    assert g.info.kernel_path == 8 or not pieces
+    for sweeps, sps in ((1, 1), (2, 1), (7, 0), (12, 3)):
+        g.run(sweeps, sps)
+        o.run(sweeps, sps)
+        assert np.array_equal(g.read_state(), o.read_state())
+    og, oo = g.obs(), o.obs()
+    for k in oo:
+        assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
+    g.close()
