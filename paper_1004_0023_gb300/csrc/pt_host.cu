@@ -1314,6 +1314,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         TUNE_CUDA(cudaStreamSynchronize(s));
 #undef TUNE_CUDA
     }
+    c->plan.overlap = 1;  // its tables, schedule and descriptors are final
     *out = c;
     return PT_OK;
 }
@@ -1396,7 +1397,7 @@ extern "C" int pt_swap(pt_ctx* c) {
     int g = guard(c);
     if (g) return g;
     if (c->q + 1 > 0xFFFFFFFFll) return ctx_fail(c, PT_EOVERFLOW, "swap pass counter exhausted");
-    CUDA_OR_FAIL(c, launch_swap(c->dp, c->q, c->stream));
+    CUDA_OR_FAIL(c, launch_swap(c->dp, c->q, c->stream, c->plan.overlap));
     c->launches += 1;
     c->q += 1;
     return PT_OK;
@@ -1425,7 +1426,7 @@ extern "C" int pt_run(pt_ctx* c, int64_t n_sweeps, int32_t sps) {
     for (long long s = 0; s + sps <= n_sweeps; s += sps) {
         int rc = enqueue_sweeps(c, sps, 0);
         if (rc) return rc;
-        CUDA_OR_FAIL(c, launch_swap(c->dp, c->q, c->stream));
+        CUDA_OR_FAIL(c, launch_swap(c->dp, c->q, c->stream, c->plan.overlap));
         c->launches += 1;
         c->q += 1;
     }

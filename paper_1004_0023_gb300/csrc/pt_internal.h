@@ -133,6 +133,8 @@ struct LaunchPlan {
     int thr_resident = 0;   // path 7: every rung's threshold row in shared memory
     int form = 0, form_t = 0;  // path 7: kForm* of a chain
     int n_groups = 0;       // path 7: chain groups of a CTA
+    // a context's own launches: set-up overlaps the kernel before (wait_for_earlier_kernels)
+    int overlap = 0;
     int pieces = 0;         // path 8: > 1 where the random words come in pieces of a sweep
     int copy = 0;           // paths 1, 3 and 9: one copy a thread (sweep_copy_kernel)
     int nibble = 0;         // path 4: neighbour slots of the nibble form, 0 = one bit a copy
@@ -211,7 +213,7 @@ cudaError_t launch_energy(const DevProblem& p, cudaStream_t s);
 cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long t0,
                           long long q0, int n_sweeps, int sweeps_per_swap, long long timeout_ns,
                           bool cooperative, cudaStream_t s);
-cudaError_t launch_swap(const DevProblem& p, long long q, cudaStream_t s);
+cudaError_t launch_swap(const DevProblem& p, long long q, cudaStream_t s, bool overlap = false);
 cudaError_t launch_gather_state(const DevProblem& p, int8_t* out, cudaStream_t s);
 cudaError_t launch_scatter_state(const DevProblem& p, const int8_t* in, cudaStream_t s);
 cudaError_t sweep_kernel_occupancy(const DevProblem& p, const LaunchPlan& plan, int* blocks_per_sm);

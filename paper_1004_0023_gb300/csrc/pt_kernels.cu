@@ -294,6 +294,14 @@ __device__ int end_of_sweep(const DevProblem& p, unsigned long long* acc, int ru
     return eos_decide(p, w, rung, E, M, timeout_ns, key, abort);
 }
 
+// Programmatic dependent launch (LaunchPlan::overlap). A kernel first does what no earlier kernel
+// of the context writes (tables, schedule, records, random words); after wait_for_earlier_kernels
+// everything before it in the stream is complete and visible. allow_next_kernel lets the next
+// one's blocks start as soon as all of this kernel's have got there. Both do nothing in a launch
+// without the attribute.
+__device__ __forceinline__ void wait_for_earlier_kernels() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Shared-memory threshold rows: every rung's row when they fit, else the current one. The
 // byte-wise kernels keep the public layout ...
 __device__ __forceinline__ void load_thr(const DevProblem& p, uint32_t* s_thr, int rung, int tid, int nt) {
@@ -747,14 +755,9 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     const int desc_words = ROWS ? rows_desc_words(p.slots) : SiteDesc<ROWS ? 4 : DC>::DW;
     const bool rec = !BITS && (COPY || !ROWS) && p.records;  // records in place of descriptors
 
+    // what no earlier kernel writes
     if constexpr (ROWS) {
-        const int8_t* src = p.spins + (size_t)slot * p.slot_stride;
-        const int RB = 2 * (int)half, n_par = P >> 1;
-        for (int x = tid; x < N * RB; x += nt) {
-            const int i = x / RB, c = x - i * RB;
-            const int par = c >= (int)half, h = c - par * (int)half;
-            sp[x] = h < n_par ? src[(size_t)i * P + 2 * h + par] : (int8_t)1;
-        }
+        const int RB = 2 * (int)half;
         // descriptors from the neighbour table (entries with J = 0 are padding), or (COPY) records:
         // descriptors in schedule order with the parity worked in
         const uint32_t zero = (uint32_t)IndexRule(p.Lmax).zero();
@@ -782,21 +785,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             d[2] = n;
             d[3] = row + half - shift;
         }
-    } else if constexpr (NIB > 0) {
-        load_bits<4>(reinterpret_cast<uint32_t*>(sp), p.spins + (size_t)slot * p.slot_stride, N, G, tid, nt);
-    } else if constexpr (BITS) {
-        // int8 chain in global memory -> one bit per copy in shared memory
-        const uint2* src = reinterpret_cast<const uint2*>(p.spins + (size_t)slot * p.slot_stride);
-        for (int x = tid; x < N * (P / 8); x += nt) {
-            const uint2 v = src[x];
-            uint32_t b = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                b |= ((v.x >> (8 * k + 7)) & 1u) << k;
-                b |= ((v.y >> (8 * k + 7)) & 1u) << (k + 4);
-            }
-            bp[x] = (uint8_t)b;
-        }
+    } else if constexpr (BITS && NIB == 0) {
         for (int x = tid; x < 512; x += nt) {
             const uint32_t par = (uint32_t)x >> 8, byte = (uint32_t)x & 0xFFu;
             uint32_t v = 0;
@@ -804,9 +793,6 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
             for (int w = 0; w < 4; ++w) v |= (((byte >> (par + 2 * w)) & 1u) ? 0xFFu : 0x01u) << (8 * w);
             s_lut[x] = v;
         }
-    } else {
-        // interleaved int8 chain in global memory -> parity-split rows in shared memory
-        load_split(sp, p.spins + (size_t)slot * p.slot_stride, N, P, P >> 3, chunk_ginv(P >> 3), tid, nt);
     }
     {
         if constexpr (!ROWS) {
@@ -825,11 +811,59 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         for (int x = tid; x < 2 * N; x += nt) s_items[x] = p.items[x];
         for (int x = tid; x <= p.n_levels; x += nt) s_loff[x] = p.level_off[x];
     }
-    int rung = p.rung_of_slot[slot];
-    load_thr_columns(p, s_thr, rung, tid, nt);
+    if (p.tables_in_smem) load_thr_columns(p, s_thr, 0, tid, nt);
     if (p.acc_in_smem)
         for (int x = tid; x < p.R * kAccCount; x += nt) s_acc[x] = 0ull;
-    long long E = p.E[slot], M = p.M[slot];  // meaningful in thread 0 only
+    if (tid == 0) {
+        s_ctl[5] = 0;  // a swap wait gave up
+        int* s_sum = reinterpret_cast<int*>(s_red);
+        s_sum[0] = s_sum[1] = s_sum[2] = 0;  // the sweep's dE, dM and flips
+    }
+    if (CSWAP)
+        for (int x = tid; x < kClusterMailPasses * p.R * 2; x += nt) s_cmb[x] = 0ull;
+    const int n_items = 2 * N;
+    if (PRE && !PEER) {
+        __syncthreads();
+        if (!consumer)
+            produce_words(rbuf, (uint32_t)t0, s_items, n_items, G, tid - NC, nt - NC, (uint32_t)slot,
+                          philox_schedule(p.key0, p.key1));
+    }
+    wait_for_earlier_kernels();
+    allow_next_kernel();
+
+    // the chain, its energies and its rung
+    if constexpr (ROWS) {
+        const int8_t* src = p.spins + (size_t)slot * p.slot_stride;
+        const int RB = 2 * (int)half, n_par = P >> 1;
+        for (int x = tid; x < N * RB; x += nt) {
+            const int i = x / RB, c = x - i * RB;
+            const int par = c >= (int)half, h = c - par * (int)half;
+            sp[x] = h < n_par ? src[(size_t)i * P + 2 * h + par] : (int8_t)1;
+        }
+    } else if constexpr (NIB > 0) {
+        load_bits<4>(reinterpret_cast<uint32_t*>(sp), p.spins + (size_t)slot * p.slot_stride, N, G, tid, nt);
+    } else if constexpr (BITS) {
+        // int8 chain in global memory -> one bit per copy in shared memory
+        const uint2* src = reinterpret_cast<const uint2*>(p.spins + (size_t)slot * p.slot_stride);
+        for (int x = tid; x < N * (P / 8); x += nt) {
+            const uint2 v = src[x];
+            uint32_t b = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                b |= ((v.x >> (8 * k + 7)) & 1u) << k;
+                b |= ((v.y >> (8 * k + 7)) & 1u) << (k + 4);
+            }
+            bp[x] = (uint8_t)b;
+        }
+    } else {
+        // interleaved int8 chain in global memory -> parity-split rows in shared memory
+        load_split(sp, p.spins + (size_t)slot * p.slot_stride, N, P, P >> 3, chunk_ginv(P >> 3), tid, nt);
+    }
+    int rung = p.rung_of_slot[slot];
+    if (!p.tables_in_smem) load_thr_columns(p, s_thr, rung, tid, nt);
+    long long E = p.E[slot], M = p.M[slot];  // meaningful in the threads that end the sweeps
+    __syncthreads();
+    if (CSWAP) cluster_barrier();  // every CTA's mailboxes are clear before anyone publishes
 
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
     const int cols = COPY ? P >> 1 : G;  // units of an item
@@ -840,26 +874,12 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
         COPY ? (uint32_t)L.thr + 4u * (uint32_t)(p.Lmax + S) : thr_base<WIDE>((uint32_t)L.thr, p.Lmax);
     const uint32_t thr_step = p.tables_in_smem ? 12u * (uint32_t)S : 0u;
     uint32_t thr_c = thr0 + thr_step * (uint32_t)rung;
-    const int n_items = 2 * N;
     const int lane = tid & 31;
-    if (tid == 0) {
-        s_ctl[5] = 0;  // a swap wait gave up
-        int* s_sum = reinterpret_cast<int*>(s_red);
-        s_sum[0] = s_sum[1] = s_sum[2] = 0;  // the sweep's dE, dM and flips
-    }
-    if (CSWAP)
-        for (int x = tid; x < kClusterMailPasses * p.R * 2; x += nt) s_cmb[x] = 0ull;
-    __syncthreads();
-    if (CSWAP) cluster_barrier();  // every CTA's mailboxes are clear before anyone publishes
-    if (PRE && !PEER && !consumer)
-        produce_words(rbuf, (uint32_t)t0, s_items, n_items, G, tid - NC, nt - NC, (uint32_t)slot, key);
     if (PEER) {
         // the peer CTA has written the first sweep's words (its arrival releases them); this
         // CTA's arrival orders nothing of its own, so it is relaxed
         cluster_arrive_relaxed();
         cluster_wait_acquire();
-    } else if (PRE) {
-        __syncthreads();
     }
 
     // Level 0 of the next sweep can be evaluated while the swap decision is still pending:
@@ -1253,6 +1273,8 @@ __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n
                       tid, nt, (uint32_t)slot, key);
     };
     produce(0, 0, 0);
+    wait_for_earlier_kernels();  // no CTA may end before the kernels before this one
+    allow_next_kernel();
     cluster_barrier();  // release: the words are visible to rank 0 after its wait
     int buffer = 0;
     for (int s = 0; s < n_sweeps; ++s)
@@ -1842,10 +1864,23 @@ __global__ void energy_kernel(DevProblem p) {
 // One swap pass q with chains in place (state already in global memory).
 __global__ void swap_kernel(DevProblem p, long long q) {
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
-    for (int rl = (int)(q & 1) + 2 * (int)threadIdx.x; rl + 1 < p.R; rl += 2 * (int)blockDim.x) {
+    allow_next_kernel();  // the next sweeps' set-up waits for this kernel all the same
+    // the first pair's coefficients and random word depend on no earlier kernel either
+    const int rl0 = (int)(q & 1) + 2 * (int)threadIdx.x;
+    double ca = 0.0, cc = 0.0;
+    uint32_t word = 0u;
+    auto pair_inputs = [&](int rl) {
+        ca = p.coef[rl];
+        cc = p.coef[(p.R - 1) + rl];
+        word = swap_word((uint32_t)q, (uint32_t)rl, key);
+    };
+    if (rl0 + 1 < p.R) pair_inputs(rl0);
+    wait_for_earlier_kernels();
+    for (int rl = rl0; rl + 1 < p.R; rl += 2 * (int)blockDim.x) {
+        if (rl != rl0) pair_inputs(rl);
         const int X = p.slot_of_rung[rl], Y = p.slot_of_rung[rl + 1];
-        const bool acc = swap_accept_fast(p.E[X], p.E[Y], p.M[X], p.M[Y], p.coef[rl], p.coef[(p.R - 1) + rl],
-                                          (uint32_t)q, (uint32_t)rl, key, p.exact_swaps != 0);
+        const bool acc = swap_accept_fast_by(p.E[X], p.E[Y], p.M[X], p.M[Y], ca, cc, [&] { return word; },
+                                             p.exact_swaps != 0);
         p.swap_stats[2 * rl] += 1ull;
         if (acc) {
             p.swap_stats[2 * rl + 1] += 1ull;
@@ -2019,6 +2054,19 @@ cudaError_t sweep_resident_chains(const DevProblem& p, const LaunchPlan& plan, l
     return e;
 }
 
+// The launch attribute of LaunchPlan::overlap: 1 where it was appended (not under capture, where
+// the graph would get edges of a kind its user may not expect).
+static unsigned overlap_attr(bool overlap, cudaStream_t s, cudaLaunchAttribute* attr) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!overlap || cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        if (overlap) (void)cudaGetLastError();
+        return 0;
+    }
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
+    return 1;
+}
+
 cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long t0, long long q0,
                           int n_sweeps, int sweeps_per_swap, long long timeout_ns, bool cooperative,
                           cudaStream_t s) {
@@ -2029,8 +2077,9 @@ cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long
     const void* fn = sweep_fn(plan);
     if (plan.path == kPathCluster || plan.path == kPathClassical) {
         // one cluster holds every chain, so the swap passes never need a cooperative launch
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = cluster_config(p, plan, s, attr);
+        cfg.numAttrs += overlap_attr(plan.overlap && plan.path == kPathCluster, s, attr + cfg.numAttrs);
         const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
         if (e != cudaSuccess) (void)cudaGetLastError();
         return e;
@@ -2038,13 +2087,25 @@ cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long
     if (plan.path == kPathSplit || plan.path == kPathSplitInline || plan.path == kPathPeer) {
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = split_config(p, plan, cooperative, s, attr);
+        if (!cooperative) cfg.numAttrs += overlap_attr(plan.overlap && plan.path == kPathPeer, s, attr);
         const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
         if (e != cudaSuccess) (void)cudaGetLastError();  // a rejected launch leaves no error for the next one
         return e;
     }
     if (cooperative)
         return cudaLaunchCooperativeKernel(fn, dim3(p.R), dim3(plan.threads), args, plan.smem_bytes, s);
-    return cudaLaunchKernel(fn, dim3(p.R), dim3(plan.threads), args, plan.smem_bytes, s);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.R);
+    cfg.blockDim = dim3(plan.threads);
+    cfg.dynamicSmemBytes = plan.smem_bytes;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    // (the byte-wise kernel has no wait of its own)
+    cfg.numAttrs = overlap_attr(plan.overlap && (plan.path != kPathGeneric || plan.rows || plan.copy), s, attr);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_init(const DevProblem& p, cudaStream_t s) {
@@ -2057,9 +2118,17 @@ cudaError_t launch_energy(const DevProblem& p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_swap(const DevProblem& p, long long q, cudaStream_t s) {
-    swap_kernel<<<1, 256, 0, s>>>(p, q);
-    return cudaGetLastError();
+cudaError_t launch_swap(const DevProblem& p, long long q, cudaStream_t s, bool overlap) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap_attr(overlap, s, attr);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, swap_kernel, p, q);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_gather_state(const DevProblem& p, int8_t* out, cudaStream_t s) {

@@ -133,3 +133,33 @@ def test_chains_whose_random_words_do_not_fit_whole_match_the_oracle(n, degree, 
     for k in oo:
         assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
     g.close()
+
+
+@pytest.mark.parametrize("kw", [dict(), *[dict(kernel_path=k) for k in (1, 2, 3, 4, 5, 8, 9)],
+                                dict(kernel_path=9, threads_per_block=96, producer_threads=32)])
+def test_back_to_back_launches_match_the_oracle(kw):
+    """Sweep, swap and run launches of two contexts enqueued in turn without a wait between them:
+    a launch's set-up may overlap the one before, its sweeps may not."""
+    probs = [_problem(16, 3, 32, 6, 9, 7), _problem(40, 5, 48, 9, 30, 8)]
+    gs = [pt.PT.from_problem(p, **kw) for p in probs]
+    os_ = [Oracle.from_problem(p, threads=THREADS) for p in probs]
+    x = [np.where(np.random.default_rng(k).random(o.read_state().shape) < 0.5, 1, -1).astype(np.int8)
+         for k, o in enumerate(os_)]
+    for round_ in range(3):
+        for step in range(12):
+            for c in gs + os_:
+                c.sweep(1 + step % 3)
+                c.swap()
+                if step % 4 == 3:
+                    c.run(4, 2)
+        for g, o in zip(gs, os_):
+            assert np.array_equal(g.read_state(), o.read_state()), round_
+        if round_ == 0:
+            for k in range(2):
+                gs[k].write_state(x[k])
+                os_[k].write_state(x[k])
+    for g, o in zip(gs, os_):
+        og, oo = g.obs(), o.obs()
+        for k in oo:
+            assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
+        g.close()
