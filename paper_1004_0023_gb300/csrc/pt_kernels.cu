@@ -342,6 +342,8 @@ __global__ void __launch_bounds__(512, 1)
 sweep_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
              long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
+    wait_for_earlier_kernels();
+    allow_next_kernel();
     const int N = p.N, P = p.P;
     const int tid = threadIdx.x, nt = blockDim.x;
     const int slot = blockIdx.x;
@@ -521,6 +523,8 @@ __global__ void __launch_bounds__(512, 1)
     sweep_classical_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                            long long timeout_ns, int C) {
     extern __shared__ __align__(16) unsigned char smem[];
+    wait_for_earlier_kernels();
+    allow_next_kernel();
     cg::cluster_group cluster = cg::this_cluster();
     const int K = (p.R + C - 1) / C;
     if (cluster.num_blocks() != (unsigned)K || gridDim.x != (unsigned)K || p.P != 1 || C < 1 || (C & (C - 1)) ||
@@ -1784,6 +1788,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                        long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
+    wait_for_earlier_kernels();
+    allow_next_kernel();
     cg::cluster_group cluster = cg::this_cluster();
     // the cluster shape is compiled in; should a launch ever run without it, no CTA touches
     // a peer's shared memory or waits at a cluster barrier
@@ -2079,7 +2085,7 @@ cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long
         // one cluster holds every chain, so the swap passes never need a cooperative launch
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = cluster_config(p, plan, s, attr);
-        cfg.numAttrs += overlap_attr(plan.overlap && plan.path == kPathCluster, s, attr + cfg.numAttrs);
+        cfg.numAttrs += overlap_attr(plan.overlap, s, attr + cfg.numAttrs);
         const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
         if (e != cudaSuccess) (void)cudaGetLastError();
         return e;
@@ -2087,7 +2093,7 @@ cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long
     if (plan.path == kPathSplit || plan.path == kPathSplitInline || plan.path == kPathPeer) {
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = split_config(p, plan, cooperative, s, attr);
-        if (!cooperative) cfg.numAttrs += overlap_attr(plan.overlap && plan.path == kPathPeer, s, attr);
+        if (!cooperative) cfg.numAttrs += overlap_attr(plan.overlap, s, attr);
         const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
         if (e != cudaSuccess) (void)cudaGetLastError();  // a rejected launch leaves no error for the next one
         return e;
@@ -2101,8 +2107,7 @@ cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long
     cfg.dynamicSmemBytes = plan.smem_bytes;
     cfg.stream = s;
     cfg.attrs = attr;
-    // (the byte-wise kernel has no wait of its own)
-    cfg.numAttrs = overlap_attr(plan.overlap && (plan.path != kPathGeneric || plan.rows || plan.copy), s, attr);
+    cfg.numAttrs = overlap_attr(plan.overlap, s, attr);
     const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
     if (e != cudaSuccess) (void)cudaGetLastError();
     return e;

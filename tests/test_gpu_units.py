@@ -136,11 +136,17 @@ def test_chains_whose_random_words_do_not_fit_whole_match_the_oracle(n, degree, 
 
 
 @pytest.mark.parametrize("kw", [dict(), *[dict(kernel_path=k) for k in (1, 2, 3, 4, 5, 8, 9)],
-                                dict(kernel_path=9, threads_per_block=96, producer_threads=32)])
+                                dict(kernel_path=9, threads_per_block=96, producer_threads=32),
+                                dict(P=1, kernel_path=1), dict(P=1, kernel_path=10)])
 def test_back_to_back_launches_match_the_oracle(kw):
     """Sweep, swap and run launches of two contexts enqueued in turn without a wait between them:
     a launch's set-up may overlap the one before, its sweeps may not."""
-    probs = [_problem(16, 3, 32, 6, 9, 7), _problem(40, 5, 48, 9, 30, 8)]
+    kw = dict(kw)
+    P = kw.pop("P", 0)
+    probs = [_problem(16, 3, P or 32, 6, 9, 7), _problem(40, 5, P or 48, 9, 30, 8)]
+    if P == 1:  # classical chains have no transverse field
+        for p in probs:
+            p.gamma = np.zeros_like(p.gamma)
     gs = [pt.PT.from_problem(p, **kw) for p in probs]
     os_ = [Oracle.from_problem(p, threads=THREADS) for p in probs]
     x = [np.where(np.random.default_rng(k).random(o.read_state().shape) < 0.5, 1, -1).astype(np.int8)
