@@ -892,6 +892,10 @@ static double sweep_cycles(const BatchInstance& I, int C) {
     return (I.n_levels * level + 4000.0) * std::max(1.0, (double)C / I.n_groups);
 }
 
+double ptq::request_cycles(const BatchInstance& I, int cluster) {
+    return (double)I.n_sweeps * sweep_cycles(I, (I.R + cluster - 1) / cluster);
+}
+
 int ptq::prepare_request(const pt_request& r, Prepared& pr, char* why, size_t why_len, int per_round) {
     const pt_instance* inst = &r.inst;
     const int N = inst->n, nE = inst->n_edges, P = r.P, R = r.R;

@@ -159,7 +159,10 @@ void ptq::level_schedule(int N, const std::vector<std::vector<int>>& adj, std::v
             b1[i] = b;
             b0[i] = std::min(a, b - 1);
         }
-        auto latest = [&](int x) { return (x & 1) ? b1[x >> 1] : b0[x >> 1]; };
+        // an item by urgency: its latest level above its number. `ready` stays in this order: what
+        // a level releases is sorted and merged in (sorting all that is ready for every level took
+        // most of a request's preparation).
+        auto urgency = [&](int x) { return (uint64_t)((x & 1) ? b1[x >> 1] : b0[x >> 1]) << 32 | (uint32_t)x; };
         std::vector<int> waiting(2 * (size_t)N, 0), level(2 * (size_t)N, -1);
         for (int i = 0; i < N; ++i) {
             for (int j : adj[i])
@@ -169,34 +172,33 @@ void ptq::level_schedule(int N, const std::vector<std::vector<int>>& adj, std::v
                 }
             waiting[2 * i + 1]++;
         }
-        std::vector<int> ready, next;
+        std::vector<uint64_t> ready, next, merged;
         for (int x = 0; x < 2 * N; ++x)
-            if (waiting[x] == 0) ready.push_back(x);
+            if (waiting[x] == 0) ready.push_back(urgency(x));
+        std::sort(ready.begin(), ready.end());
         int left = 2 * N;
         for (int l = 0; l < nlev; ++l) {
-            std::sort(ready.begin(), ready.end(), [&](int x, int y) {
-                const int bx = latest(x), by = latest(y);
-                return bx != by ? bx < by : x < y;
-            });
             int must = 0;
-            while (must < (int)ready.size() && latest(ready[must]) == l) ++must;
+            while (must < (int)ready.size() && (int)(ready[must] >> 32) == l) ++must;
             const int even_share = (left + (nlev - l) - 1) / (nlev - l);
             const int cap = std::max(must, (even_share + per_round - 1) / per_round * per_round);
             const int take = std::min(cap, (int)ready.size());
             next.clear();
             for (int k = 0; k < take; ++k) {
-                const int x = ready[k], i = x >> 1;
+                const int x = (int)(uint32_t)ready[k], i = x >> 1;
                 level[x] = l;
                 auto release = [&](int y) {
-                    if (--waiting[y] == 0) next.push_back(y);
+                    if (--waiting[y] == 0) next.push_back(urgency(y));
                 };
                 for (int j : adj[i])
                     if (j > i) release(2 * j + (x & 1));
                 if (!(x & 1)) release(x + 1);
             }
             left -= take;
-            ready.erase(ready.begin(), ready.begin() + take);
-            ready.insert(ready.end(), next.begin(), next.end());
+            std::sort(next.begin(), next.end());
+            merged.resize(ready.size() - take + next.size());
+            std::merge(ready.begin() + take, ready.end(), next.begin(), next.end(), merged.begin());
+            ready.swap(merged);
         }
         // keep the as-early-as-possible levels where the fill takes more rounds than they do
         // (it can, by one, on long chains with small rounds)
@@ -239,25 +241,20 @@ void ptq::level_schedule(int N, const std::vector<std::vector<int>>& adj, std::v
         // robin over those start banks puts items with different starts side by side, so a
         // warp's loads of its items' own words (and, for rows of 32 words, of every
         // neighbour word) fall in different banks.
-        std::vector<uint32_t> lev_items;
-        std::vector<std::vector<uint32_t>> by_bank(32);
+        std::vector<uint64_t> dealt;  // (round, bank, item), to be sorted
         for (int l = 0; l < nlev; ++l) {
-            for (auto& b : by_bank) b.clear();
+            uint32_t rounds[32] = {};
+            dealt.clear();
+            bool sorted = true;
             for (int x = level_off[l]; x < level_off[l + 1]; ++x) {
                 const uint32_t it = items[x], i = it >> 1, par = it & 1u;
-                by_bank[(i * (uint32_t)row_words + par * (uint32_t)(row_words / 2)) & 31u].push_back(it);
+                const uint32_t bank = (i * (uint32_t)row_words + par * (uint32_t)(row_words / 2)) & 31u;
+                dealt.push_back((uint64_t)(rounds[bank]++ * 32u + bank) << 32 | it);
+                sorted = sorted && (dealt.size() < 2 || dealt[dealt.size() - 2] < dealt.back());
             }
-            lev_items.clear();
-            for (size_t k = 0;; ++k) {
-                bool any = false;
-                for (auto& b : by_bank)
-                    if (k < b.size()) {
-                        lev_items.push_back(b[k]);
-                        any = true;
-                    }
-                if (!any) break;
-            }
-            std::copy(lev_items.begin(), lev_items.end(), items.begin() + level_off[l]);
+            if (sorted) continue;
+            std::sort(dealt.begin(), dealt.end());
+            for (size_t k = 0; k < dealt.size(); ++k) items[level_off[l] + k] = (uint32_t)dealt[k];
         }
     }
 }

@@ -263,6 +263,9 @@ void fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base, con
 // Group width of a fixed layout: narrowest that fits (one warp per chain where possible),
 // which the autotuner picks on the batched size mix.
 constexpr int kGroupWidenDefault = -4;
+// Cycles the n_sweeps of a request take on one cluster, by the model choose_groups compares forms
+// with (the layout choose_groups picked for that cluster).
+double request_cycles(const BatchInstance& I, int cluster);
 void choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen = kGroupWidenDefault);
 
 // Batched launchers (pt_batch.cu).

@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <atomic>
 #include <deque>
+#include <functional>
 #include <map>
 #include <vector>
 
@@ -582,22 +583,53 @@ static int launch_group(pt_server* s, const std::vector<ServeReq*>& g) {
     // gets a cluster of its own at once (2 when even that is too many). A member runs on one
     // cluster, so a short backlog gets wide clusters (each request's chains over more SMs,
     // lower latency) and a long one narrow clusters (the most requests at once: on this GPU
-    // clusters of 2 also sweep the most attempts per second). 16 is not used: fewer of them
-    // fit the GPU's SMs, and they lost to 8 on latency as well in measured replays.
+    // clusters of 2 also sweep the most attempts per second). Wider clusters than that, up to
+    // 16, where the members taken longest first onto as many of them as fit end a seventh
+    // sooner by the model of a sweep: a backlog of unequal requests waits for its largest, and
+    // the SMs beyond one cluster each stay idle (12 requests of N = 128 to 444, P = 32 to 128,
+    // R = 8 to 31, 600 sweeps: 22.0 ms on 12 clusters of 8, 13.0 ms on 7 of 16; a margin below
+    // the model's error would move equal requests, which lose when some wait for a cluster).
     int K = s->cluster, ncl = s->n_clusters;
     if (s->adaptive_cluster) {
+        // the members' modelled cycles on clusters of 2^l CTAs; false: one does not fit
+        // (narrower clusters hold more chains per CTA but never need more room than streaming
+        // one chain per group)
+        std::vector<double> t;
+        auto cycles = [&](int l) {
+            bool ok = true;
+            t.resize(n);
+            for (int k = 0; k < n && ok; ++k) {
+                BatchInstance I = g[k]->inst;
+                I.n_sweeps = (int)g[k]->remaining;
+                choose_groups(I, 1 << l, s->threads, s->smem_cap);
+                ok = batch_smem_bytes(I, 1 << l, s->threads) <= s->smem_cap;
+                t[k] = request_cycles(I, 1 << l);
+            }
+            return ok;
+        };
+        // when the last member ends, longest first, on the clusters the other launches leave
+        auto makespan = [&](int l) {
+            std::sort(t.begin(), t.end(), std::greater<double>());
+            const int room = (int)(s->ncl_by_log2[l] * std::max<long long>(0, s->n_sm - s->inflight_sms) / s->n_sm);
+            std::vector<double> end(std::max(1, std::min(room, n)), 0.0);
+            for (double x : t) *std::min_element(end.begin(), end.end()) += x;
+            return *std::max_element(end.begin(), end.end());
+        };
         int l = 3;
         while (l > 1 && s->ncl_by_log2[l] < n) --l;
-        // every member must fit a CTA of that cluster size (narrower clusters hold more chains
-        // per CTA but never need more room than streaming one chain per group)
-        for (; l > 1; --l) {
-            bool ok = true;
-            for (ServeReq* q : g) {
-                BatchInstance I = q->inst;
-                choose_groups(I, 1 << l, s->threads, s->smem_cap);
-                if (batch_smem_bytes(I, 1 << l, s->threads) > s->smem_cap) ok = false;
-            }
-            if (ok) break;
+        bool fits = false;
+        for (; l > 1; --l)
+            if ((fits = cycles(l))) break;
+        if (fits && s->ncl_by_log2[l] > 0) {
+            double best = makespan(l);
+            for (int w = l + 1; w <= 4; ++w)
+                if (s->ncl_by_log2[w] > 0 && cycles(w)) {
+                    const double m = makespan(w);
+                    if (m < best * 6.0 / 7.0) {
+                        best = m;
+                        l = w;
+                    }
+                }
         }
         K = 1 << l;
         ncl = s->ncl_by_log2[l] > 0 ? s->ncl_by_log2[l] : s->n_clusters;

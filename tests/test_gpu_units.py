@@ -169,3 +169,25 @@ def test_back_to_back_launches_match_the_oracle(kw):
         for k in oo:
             assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
         g.close()
+
+
+def test_an_unequal_backlog_on_wide_clusters_matches_the_oracle():
+    """Nine requests admitted together, the longest by far the largest: clusters wider than one for
+    each member, which the shorter ones take in turn."""
+    probs = [_problem(120, 7, 64, 32, 30, 3)] + [_problem(12 + k, 3, 16 + 8 * (k % 3), 4 + k, 9, k) for k in range(8)]
+    for k, p in enumerate(probs):
+        p.n_sweeps, p.sweeps_per_swap = 30 if k == 0 else 12, 1 + k % 3
+    srv = pt.Server(arena_bytes=1 << 28)
+    ids = [srv.submit(p) for p in probs]
+    done = set()
+    while len(done) < len(ids):
+        done |= set(srv.step())
+    for rid, p in zip(ids, probs):
+        state, obs = srv.result(rid)
+        o = Oracle.from_problem(p, threads=THREADS)
+        o.run(p.n_sweeps, p.sweeps_per_swap)
+        assert np.array_equal(state, o.read_state())
+        want = o.obs()
+        for k in want:
+            assert np.array_equal(np.asarray(obs[k]), np.asarray(want[k])), k
+    srv.close()
