@@ -1156,16 +1156,28 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                 // at most four, else without: N=512, P=64, R=64 runs 6.47 us per sweep with swaps in
                 // pieces; path 6, the fastest otherwise, 7.70. From P = 128 the split kernels
                 // (paths 5 and 6) hold such chains in two CTAs, and are what is timed.
+                // Threshold tables of 48 to 96 KB too stay in shared memory if two pieces make the
+                // room: the next sweep's level 0 is then evaluated while the partner's mailbox is
+                // awaited (N=300, P=40, R=48, Lmax=58: 7.31 -> 6.89 us per sweep with a swap each,
+                // 6.23 -> 6.14 without; calls of five sweeps, which load the tables each time, are
+                // no slower).
                 pl.dclass = packed_dc;
-                for (pc.records = records_for(cd.path, 0); pc.records >= 0; --pc.records)
-                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : pc.records ? 4 : kMaxChunks); ++pieces) {
-                        pc.tables_in_smem = (size_t)R * p.nL3 * 4 <= 49152 ? 1 : 0;
-                        pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
-                        if (!cut_sweep(pc, off_c, pieces)) continue;
-                        pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc);
-                        pl.pieces = pc.n_chunks;
-                        if (pl.smem_bytes <= (size_t)max_smem) return true;
-                    }
+                const size_t table_bytes = (size_t)R * p.nL3 * 4;
+                auto fits_in = [&](int pieces, size_t max_tables) {
+                    pc.tables_in_smem = table_bytes <= max_tables ? 1 : 0;
+                    pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
+                    if (!cut_sweep(pc, off_c, pieces)) return false;
+                    pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc);
+                    pl.pieces = pc.n_chunks;
+                    return pl.smem_bytes <= (size_t)max_smem;
+                };
+                pc.records = records_for(cd.path, 0);
+                if (table_bytes > 49152 && table_bytes <= 98304)
+                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : 2); ++pieces)
+                        if (fits_in(pieces, 98304)) return true;
+                for (; pc.records >= 0; --pc.records)
+                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : pc.records ? 4 : kMaxChunks); ++pieces)
+                        if (fits_in(pieces, 49152)) return true;
                 return false;
             }
             pc.records = records_for(cd.path, 0);
