@@ -75,10 +75,14 @@ typedef struct {
     int32_t test_withhold_rung; /* test hook, 0 = off: if r+1, the chain on rung r never
                                    publishes its swap mailbox, so its partner's wait runs out
                                    and the call fails with PT_ETIMEDOUT (no fault, no hang) */
-    int32_t kernel_path;        /* 0 = auto, 1 = byte-wise, 2 = packed with inline random
+    int32_t kernel_path;        /* 0 = auto, 1 = any shape (words of
+                                   four copies, or one copy a thread on small levels, with
+                                   inline or produced random words; byte-wise for P = 1 and
+                                   where the words' layout does not fit), 2 = packed with inline random
                                    words, 3 = packed with random words produced one sweep
-                                   ahead by dedicated warps, 4 = packed with one bit per
-                                   copy in shared memory (paths 2-6 need P % 8 == 0 and
+                                   ahead by dedicated warps, 4 = packed with four bits
+                                   (P % 32 == 0, Lmax <= 31, if it fits) or one bit per copy
+                                   in shared memory (paths 2-6 need P % 8 == 0 and
                                    degree <= 7), 5 = path 3 with each chain split over a
                                    cluster of two CTAs, one half of the Trotter copies each
                                    (needs P % 16 == 0 and all R chains resident at once;
@@ -93,8 +97,9 @@ typedef struct {
                                    mailboxes between SMs), 8 = path 3 with every thread
                                    sweeping and the random words made by a second CTA of a
                                    two-CTA cluster per chain, written into the first one's
-                                   shared memory one sweep ahead (needs all R clusters
-                                   resident at once; for ladders that leave SMs idle),
+                                   shared memory one sweep ahead (the automatic plan also in
+                                   pieces of a sweep where two whole sweeps' words do not fit;
+                                   needs all R clusters resident at once; for ladders that leave SMs idle),
                                    9 = path 2 (or path 3 with producer_threads > 0) with the
                                    CTAs of all R chains in one thread-block cluster and the
                                    swap mailboxes in every CTA's shared memory, so that a
@@ -167,7 +172,7 @@ typedef struct {
  *   P           Trotter copies, even, 2 <= P <= 4096; or P = 1 with gamma = 0 on every rung:
  *               classical parallel tempering over the temperatures (one copy per chain,
  *               no Trotter coupling: K = 0, m = 0, M = N). Classical chains run on the
- *               byte-wise kernel; batched launches and the server need P % 8 == 0.
+ *               byte-wise kernel (path 1) or packed several to a CTA (path 10); batched launches and the server need P % 8 == 0.
  *   ladder, R   R >= 1 rungs (copied), 1 <= R <= 65535.
  *   flip_thr    NULL to build the Metropolis table in FP64 on the host, or R*(2*Lmax+1)*3
  *               uint32 thresholds [r][L+Lmax][m/2+1] (accept iff thr == 0xFFFFFFFF or
@@ -331,7 +336,9 @@ typedef struct {
     int32_t cluster_size;   /* CTAs per cluster of batched launches (1..16), or 0: 2 in
                                stepped mode; a backlog launch in streamed mode takes the
                                largest of 8, 4 and 2 at which every request of the backlog
-                               gets a cluster of its own at once (else 2) */
+                               gets a cluster of its own at once (else 2), or
+                               wider ones, up to 16, where the requests taken
+                               longest first on those that fit end clearly sooner */
     int32_t reserved[3];    /* reserved[1] = 1: stepped mode (a quantum of sweeps per launch);
                                reserved[0] = 1: stepped mode with chains packed on clusters only */
 } pt_server_options;

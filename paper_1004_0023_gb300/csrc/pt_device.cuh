@@ -21,13 +21,6 @@ struct PhiloxKey {
     __device__ __forceinline__ uint32_t b(int r) const { return k1[r]; }
 };
 
-// The same round keys read from shared memory, for kernels that cannot spare 20 registers
-// per thread for them: rounds 2j and 2j+1 in one 16-byte word k[j] = (k0, k1, k0', k1'), so a
-// pair of rounds costs one shared load.
-struct PhiloxKeyShared {
-    const uint4* k;
-};
-
 __device__ __forceinline__ PhiloxKey philox_schedule(uint32_t key0, uint32_t key1) {
     PhiloxKey k;
 #pragma unroll
@@ -50,15 +43,6 @@ __device__ __forceinline__ uint4 philox(uint4 c, const PhiloxKey& k) {
     return c;
 }
 
-__device__ __forceinline__ uint4 philox(uint4 c, const PhiloxKeyShared& k) {
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        const uint4 kk = k.k[j];
-        c = philox_round(c, kk.x, kk.y);
-        c = philox_round(c, kk.z, kk.w);
-    }
-    return c;
-}
 
 // ------------------------------------------------------------------------- det_exp
 // exp(x) for x in (-23, 0] from IEEE round-to-nearest basic operations only (Cody & Waite
@@ -138,12 +122,6 @@ __device__ __forceinline__ bool swap_accept_fast_by(long long EX, long long EY, 
 
 // The two rules with the word drawn from (q, rl) under `key` when needed.
 template <typename Key = PhiloxKey>
-__device__ __forceinline__ bool swap_accept(long long EX, long long EY, long long MX, long long MY,
-                                            double a, double c, uint32_t q, uint32_t rl,
-                                            const Key& key) {
-    return swap_accept_by(EX, EY, MX, MY, a, c, [&] { return swap_word(q, rl, key); });
-}
-template <typename Key = PhiloxKey>
 __device__ __forceinline__ bool swap_accept_fast(long long EX, long long EY, long long MX, long long MY,
                                                  double a, double c, uint32_t q, uint32_t rl,
                                                  const Key& key, bool exact_only) {
@@ -156,16 +134,6 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ long long ld_relaxed_s64(const long long* p) {
-    long long v;
-    asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -173,12 +141,6 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 }
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_relaxed_s64(long long* p, long long v) {
-    asm volatile("st.relaxed.gpu.global.s64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Tag of pass q0 + pass, from qmod0 = q0 mod kTagPeriod (taken once per launch): a 32-bit

@@ -103,9 +103,9 @@ struct DevProblem {
     uint32_t key0, key1;
 };
 
-// Sweep kernel variants: byte-wise (any shape), packed with Philox inline, packed with the
-// random words produced one sweep ahead by dedicated warps, bit-packed, and the produced-words
-// kernel with each chain split over a cluster of two CTAs.
+// Sweep kernel variants: any shape (word-wise, one copy a thread, or byte-wise), packed with Philox
+// inline, packed with the random words produced one sweep ahead by dedicated warps, bit-packed, and
+// the produced-words kernel with each chain split over a cluster of two CTAs.
 // Path 7 runs the batched kernel on the one problem: all chains packed on the CTAs of one
 // cluster (thread groups per chain), resident in shared memory, swaps in shared memory.
 enum {

@@ -335,8 +335,9 @@ __device__ __forceinline__ void flush_acc(const DevProblem& p, const unsigned lo
 }
 
 // ------------------------------------------------------------------------- generic sweep
-// One CTA per chain (slot); byte-wise spins, Philox inline in each 4-copy unit. Used when
-// P is not a multiple of 8 or a site has more than 7 neighbours.
+// One CTA per chain (slot); byte-wise spins, Philox inline in each 4-copy unit. Used for P = 1
+// and where the word-wise kernel's layout does not fit; other shapes
+// that the packed kernels refuse run word-wise (sweep_rows_kernel, sweep_copy_kernel).
 template <int DCLASS>
 __global__ void __launch_bounds__(512, 1)
 sweep_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,

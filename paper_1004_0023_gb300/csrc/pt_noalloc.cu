@@ -1,5 +1,5 @@
-// pt_noalloc.cu -- pt_run_noalloc: the byte-wise sweep kernel with in-launch swaps, run on
-// device buffers the caller owns, with no allocation of any kind.
+// pt_noalloc.cu -- pt_run_noalloc: path 1's sweep kernel (word-wise, byte-wise where its layout
+// does not fit) with in-launch swaps, run on device buffers the caller owns, with no allocation of any kind.
 //
 // Who needs this: callers that cannot allocate device memory, neither themselves nor
 // through this library. Latency-critical loops must not enter the allocator (cudaMalloc
