@@ -431,15 +431,18 @@ static int upload_request(pt_server* s, ServeReq* q, cudaStream_t st) {
     memcpy(&host[pr.off_tloff], pr.tlevel_off.data(), pr.tlevel_off.size() * 4);
     memcpy(&host[pr.off_thr], pr.thr.data(), pr.thr.size() * 4);
     memcpy(&host[pr.off_coef], pr.coef.data(), pr.coef.size() * 8);
-    std::vector<int2> map(pr.R);
-    for (int rho = 0; rho < pr.R; ++rho) map[rho] = make_int2(0, rho);
+    // the record and the map behind it in one copy
+    std::vector<unsigned char> tail(pr.off_map - pr.off_inst + (size_t)pr.R * sizeof(int2), 0);
+    memcpy(&tail[0], &q->inst, sizeof(BatchInstance));
+    for (int rho = 0; rho < pr.R; ++rho) {
+        const int2 m = make_int2(0, rho);
+        memcpy(&tail[pr.off_map - pr.off_inst + (size_t)rho * sizeof(int2)], &m, sizeof(m));
+    }
     cudaError_t e;
     if ((e = cudaMemcpyAsync(base, host.data(), host.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaMemsetAsync(base + pr.off_spins, 0, q->block_bytes - pr.off_spins, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(base + pr.off_inst, &q->inst, sizeof(BatchInstance), cudaMemcpyHostToDevice, st)) !=
+        (e = cudaMemcpyAsync(base + pr.off_inst, tail.data(), tail.size(), cudaMemcpyHostToDevice, st)) !=
             cudaSuccess ||
-        (e = cudaMemcpyAsync(base + pr.off_map, map.data(), map.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                             st)) != cudaSuccess ||
         (e = launch_batch_init((const BatchInstance*)(base + pr.off_inst), (const int2*)(base + pr.off_map), pr.R,
                                st)) != cudaSuccess)
         return sfail(s, PT_ECUDA, "streamed admission: %s", cudaGetErrorString(e));
