@@ -31,6 +31,7 @@
 #include <deque>
 #include <functional>
 #include <map>
+#include <memory>
 #include <vector>
 
 #include "pt.h"
@@ -1000,31 +1001,28 @@ extern "C" int pt_server_read_result(pt_server* s, int64_t id, int8_t* state, si
     if (q->state != 2) return sfail(s, PT_EBUSY, "request %lld has not finished", (long long)id);
     const BatchInstance& I = q->inst;
     const int R = I.R;
-    std::vector<int32_t> slot_of(R);
-    std::vector<long long> E(R), M(R);
-    std::vector<unsigned long long> acc((size_t)R * kAccCount), sw(2 * (size_t)R);
-    std::vector<int8_t> spins;
+    const size_t chain = (size_t)I.N * I.P;
+    if (state && bytes < (size_t)R * chain) return sfail(s, PT_EINVAL, "state buffer needs %zu bytes", (size_t)R * chain);
+    // The chains and everything behind them up to the swap counts lie in one piece of the request's
+    // block (request_block_layout): one copy (six took about 8 us each).
+    const unsigned char* first = state ? (const unsigned char*)I.spins : (const unsigned char*)I.E;
+    const size_t span = (size_t)((const unsigned char*)(I.swap_stats + 2 * (size_t)R) - first);
+    std::unique_ptr<unsigned char[]> host(new unsigned char[span]);
     cudaError_t e;
     cudaStream_t st = s->stream;
-    if ((e = cudaMemcpyAsync(slot_of.data(), I.slot_of_rung, R * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(E.data(), I.E, R * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(M.data(), I.M, R * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(acc.data(), I.acc, acc.size() * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(sw.data(), I.swap_stats, sw.size() * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(host.get(), first, span, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return sfail(s, PT_ECUDA, "%s", cudaGetErrorString(e));
-    if (state) {
-        const size_t need = (size_t)R * I.N * I.P;
-        if (bytes < need) return sfail(s, PT_EINVAL, "state buffer needs %zu bytes", need);
-        spins.resize((size_t)R * I.slot_stride);
-        if ((e = cudaMemcpyAsync(spins.data(), I.spins, spins.size(), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-            return sfail(s, PT_ECUDA, "%s", cudaGetErrorString(e));
-    }
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return sfail(s, PT_ECUDA, "%s", cudaGetErrorString(e));
-    if (state) {
-        // replica order on the device, rung order across the boundary
-        const size_t chain = (size_t)I.N * I.P;
-        for (int r = 0; r < R; ++r) memcpy(state + (size_t)r * chain, &spins[(size_t)slot_of[r] * I.slot_stride], chain);
-    }
+    // (blocks and their parts start on 256-byte boundaries, so every part is aligned in `host` too)
+    auto part = [&](const void* device) { return host.get() + ((const unsigned char*)device - first); };
+    const int32_t* slot_of = (const int32_t*)part(I.slot_of_rung);
+    const long long *E = (const long long*)part(I.E), *M = (const long long*)part(I.M);
+    const unsigned long long *acc = (const unsigned long long*)part(I.acc),
+                             *sw = (const unsigned long long*)part(I.swap_stats);
+    // replica order on the device, rung order across the boundary
+    if (state)
+        for (int r = 0; r < R; ++r)
+            memcpy(state + (size_t)r * chain, part(I.spins) + (size_t)slot_of[r] * I.slot_stride, chain);
     if (o) {
         o->t = I.t0;
         o->q = I.q0;
