@@ -52,7 +52,7 @@ struct BatchLayout {
         C = (I.R + K - 1) / K;
         ngroups = I.n_groups;
         chain_stride = (int)up16((size_t)I.N * form_row_bytes(I.form, I.P));
-        nbufs = I.resident ? C : ngroups;
+        nbufs = CtaShare::buffers(I, K);
         thr_words = (int)(up16((size_t)IndexRule(I.Lmax).row_words() * 4) / 4);
         size_t o = 0;
         sdesc = o;  o += (size_t)I.N * DW * 4;
@@ -282,9 +282,10 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
     unsigned long long* mail =
         I.mail_smem ? reinterpret_cast<unsigned long long*>(smem + L.mail) : reinterpret_cast<unsigned long long*>(I.mail);
 
-    const int N = I.N, P = I.P, R = I.R, C = L.C;
-    const int c_begin = rank * C;
-    const int c_count = max(0, min(C, R - c_begin));
+    const int N = I.N, P = I.P, R = I.R;
+    const CtaShare share(I, rank, K);
+    const int c_begin = share.begin, c_count = share.count;
+    const bool in_place = share.in_place;
     const IndexRule index(I.Lmax);
     const int gsize = I.group_threads, ngroups = L.ngroups;
     const int grp = tid / gsize, gtid = tid - grp * gsize;
@@ -314,7 +315,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                 for (int c = 0; c < 3; ++c) s_thr[(size_t)r * L.thr_words + c * index.S + l] = I.thr[3 * x + c];
             }
         }
-        if (I.resident)
+        if (in_place)
             for (int lc = 0; lc < c_count; ++lc)
                 load_chain(I, reinterpret_cast<int8_t*>(s_chains + (size_t)lc * L.chain_stride),
                            I.spins + (size_t)(c_begin + lc) * I.slot_stride, tid, nt);
@@ -330,7 +331,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
     const int lane = tid & 31, gwarp = gtid >> 5;
     const bool one_warp = gsize == 32, lead = gwarp == 0;
     const int sps = I.sweeps_per_swap;
-    const bool keep = c_count <= ngroups;  // each group keeps one chain
+    const bool keep = share.keep;
     const uint32_t qmod0 = (uint32_t)(I.q0 % kTagPeriod);
     uint32_t phase = grp < 16 ? sh.phase[grp] : 0u;
     bool stored = false;  // lead: a bulk store of chain `stored_lc` is in flight
@@ -432,15 +433,15 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
         // ---- the chain, and its rung's thresholds
         const int rho = c_begin + lc;
         int8_t* g_chain = I.spins + (size_t)rho * I.slot_stride;
-        int8_t* buf = reinterpret_cast<int8_t*>(s_chains + (size_t)(I.resident ? lc : grp) * L.chain_stride);
-        const bool bulk_in = !I.resident && s > 0;
+        int8_t* buf = reinterpret_cast<int8_t*>(s_chains + (size_t)(in_place ? lc : grp) * L.chain_stride);
+        const bool bulk_in = !in_place && s > 0;
         if (bulk_in) {
                 // the chain in its shared-memory form, as an earlier sweep's bulk store left it
             if (lead && lane == 0) {
                 fence_async();
                 bulk_load(buf, g_chain, (uint32_t)L.chain_stride, &sh.mbar[grp]);
             }
-        } else if (!I.resident) {
+        } else if (!in_place) {
             load_chain(I, buf, g_chain, gtid, gsize);
         }
         const uint32_t thr_c = (uint32_t)L.thr + 4u * (uint32_t)L.thr_words * (uint32_t)(I.thr_resident ? rung : grp);
@@ -464,7 +465,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
 
         // ---- sweep s
         const ChainSweep job = {(uint32_t)L.sdesc, (uint32_t)L.items, (uint32_t)L.loff, thr_c,
-                                (uint32_t)(L.chains + (size_t)(I.resident ? lc : grp) * L.chain_stride),
+                                (uint32_t)(L.chains + (size_t)(in_place ? lc : grp) * L.chain_stride),
                                 I.key0, I.key1, (uint32_t)(I.t0 + s), (uint32_t)rho, I.n_levels, I.Lmax, P, gsize,
                                 gtid, bar};
         const ChainChange ch =
@@ -473,7 +474,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
         // ---- the chain back (a bulk store takes it in its shared-memory form; the last sweep's
         // is converted again), and the sweep's statistics and publication
         const bool last = s + 1 == I.n_sweeps;
-        if (!I.resident) {
+        if (!in_place) {
             if (!last) {
                 fence_async();  // this thread's flips, for the copy the lead starts
             } else {
@@ -494,7 +495,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
             __syncwarp();
         }
         if (lead) {
-            if (!I.resident && !last) {
+            if (!in_place && !last) {
                 if (lane == 0) bulk_store(g_chain, buf, (uint32_t)L.chain_stride);
                 stored = true;
                 stored_lc = lc;
@@ -542,7 +543,6 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
             }
         }
     }
-    if (lead && stored && lane == 0) bulk_stores_done();  // only after a wait that gave up
     __syncthreads();
     if (gtid == 0 && grp < ngroups && grp < 16) sh.phase[grp] = phase;
 
@@ -553,7 +553,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
         I.rung_of_slot[c_begin + x] = s_rung[x];
         I.slot_of_rung[s_rung[x]] = c_begin + x;
     }
-    if (I.resident)
+    if (in_place)
         for (int lc = 0; lc < c_count; ++lc)
             store_chain(I, I.spins + (size_t)(c_begin + lc) * I.slot_stride,
                         reinterpret_cast<const int8_t*>(s_chains + (size_t)lc * L.chain_stride), tid, nt);

@@ -194,6 +194,29 @@ struct BatchInstance {
     int n_sweeps, sweeps_per_swap;
 };
 
+// CTA `rank` of a cluster of K: its chains of the problem, and where they are during a run.
+struct CtaShare {
+    int begin, count;
+    bool keep;      // no more chains than groups: each group keeps one
+    bool in_place;  // chain lc stays in buffer lc; else chains are streamed, a buffer a group
+    __host__ __device__ CtaShare(const BatchInstance& I, int rank, int K) {
+        const int C = (I.R + K - 1) / K;
+        begin = rank * C;
+        count = I.R - begin < C ? I.R - begin : C;
+        if (count < 0) count = 0;
+        keep = count <= I.n_groups;
+        // The last CTA of a streamed problem has fewer chains than the others, and may keep them: a
+        // kept chain has its group's buffer to itself, so it stays there. (Streaming it would need a
+        // wait between the store after one sweep and the load before the next: bulk copies have no
+        // order among themselves.)
+        in_place = I.resident != 0 || keep;
+    }
+    // chain buffers of every CTA of the cluster
+    __host__ __device__ static int buffers(const BatchInstance& I, int K) {
+        return I.resident ? (I.R + K - 1) / K : I.n_groups;
+    }
+};
+
 struct BatchParams {
     BatchInstance* inst;        // [count]; t0 / q0 of a finished problem advance in place
     const int32_t* order;       // [count] request indices, most work first
