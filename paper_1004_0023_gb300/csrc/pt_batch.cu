@@ -73,9 +73,9 @@ struct BatchLayout {
 
 // Shared memory of the persistent kernel that outlives a problem.
 struct BatchShared {
+    unsigned long long next;      // next task of this CTA
     unsigned long long mbar[16];  // per group: arrival of a streamed chain
     uint32_t phase[16];           // its parity of the next arrival
-    int next;                     // next task of this CTA
     int abort;                    // a wait gave up
     int job;
 };
@@ -319,7 +319,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
             for (int lc = 0; lc < c_count; ++lc)
                 load_chain(I, reinterpret_cast<int8_t*>(s_chains + (size_t)lc * L.chain_stride),
                            I.spins + (size_t)(c_begin + lc) * I.slot_stride, tid, nt);
-        if (tid == 0) sh.next = 0;
+        if (tid == 0) sh.next = 0ull;
     }
     __syncthreads();
     if (K > 1) cluster_barrier();  // every mailbox is clear before anyone publishes
@@ -337,6 +337,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
     bool stored = false;  // lead: a bulk store of chain `stored_lc` is in flight
     int stored_lc = 0, stored_seq = 0;
     int kept_s = 0;
+    TaskCursor at;
 
     for (;;) {
         // ---- the next task, its chain's last sweep and that sweep's swap decision
@@ -357,11 +358,11 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                     }
                     stored = false;
                 }
-                int task = 0;
-                if (lane == 0) task = atomicAdd(&sh.next, 1);
-                task = __shfl_sync(0xFFFFFFFFu, task, 0);
-                s = task / c_count;
-                lc = task - s * c_count;
+                unsigned long long task = 0;
+                if (lane == 0) task = atomicAdd(&sh.next, 1ull);
+                at.move_to(__shfl_sync(0xFFFFFFFFu, task, 0), c_count);
+                s = at.s;
+                lc = at.lc;
                 stop = s > I.n_sweeps;
                 if (!stop && s > 0) {
                     volatile int* seq = s_seq + lc;

@@ -217,6 +217,27 @@ struct CtaShare {
     }
 };
 
+// A group's place in its CTA's sequence of tasks: task number s * count + lc is sweep s of chain
+// lc. The number needs 64 bits (2^30 sweeps of 1024 chains), but a group's next task is close to
+// its last one, so a 32-bit division of the step finds it.
+struct TaskCursor {
+    unsigned long long task = 0;
+    int s = 0, lc = 0;
+    __host__ __device__ void move_to(unsigned long long next, int count) {
+        const unsigned long long step = next - task;
+        task = next;
+        if (step < 0x40000000ull) {
+            const unsigned x = (unsigned)lc + (unsigned)step;
+            const unsigned sweeps = x / (unsigned)count;
+            s += (int)sweeps;
+            lc = (int)(x - sweeps * (unsigned)count);
+        } else {
+            s = (int)(next / (unsigned)count);
+            lc = (int)(next - (unsigned long long)s * (unsigned)count);
+        }
+    }
+};
+
 struct BatchParams {
     BatchInstance* inst;        // [count]; t0 / q0 of a finished problem advance in place
     const int32_t* order;       // [count] request indices, most work first

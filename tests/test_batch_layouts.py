@@ -1,5 +1,5 @@
-"""Batched layouts with streamed chains: which CTAs stream and which keep their chains (host
-code, on the CPU), and the bits of the requests that have both (GPU)."""
+"""Batched layouts with streamed chains: which CTAs stream and which keep their chains, and the
+sequence of their tasks (host code, on the CPU), and the bits of the requests that have both (GPU)."""
 import os
 import subprocess
 
@@ -22,8 +22,22 @@ STREAMED = [(294, 6, 128, 45, 20, 1), (900, 7, 40, 35, 60, 2)]
 
 
 @pytest.fixture(scope="module")
-def layouts(libpt, tmp_path_factory):
-    exe = compile_host("batch_layouts", tmp_path_factory.mktemp("native"))
+def native(libpt, tmp_path_factory):
+    """native(name): the host program tests/native/<name>.cu, compiled once."""
+    out_dir = tmp_path_factory.mktemp("native")
+    built = {}
+
+    def program(name):
+        if name not in built:
+            built[name] = compile_host(name, out_dir)
+        return built[name]
+
+    return program
+
+
+@pytest.fixture(scope="module")
+def layouts(native):
+    exe = native("batch_layouts")
 
     def run(problems):
         text = []
@@ -72,6 +86,18 @@ def test_a_cta_that_keeps_its_chains_does_not_stream_them(layouts):
         assert lay["bytes"] > 0 and not lay["resident"], c
         kept = [x["in_place"] for x in lay["ctas"] if x["count"]]
         assert any(kept) == (c in MIXED) and not all(kept), c
+
+
+@pytest.mark.parametrize("chains,first", [
+    (1024, 0), (1024, 2 ** 21 - 3), (1024, 2 ** 22 - 3), (1024, 2 ** 30 - 40), (32, 2 ** 26 - 40), (32, 2 ** 30 - 40),
+    (17, 2 ** 31 // 17 - 5), (1, 2 ** 30 - 40),
+])
+def test_tasks_of_the_longest_runs_stay_in_range(native, chains, first):
+    """2^30 sweeps of 1024 chains: the task number passes 2^31, 2^32 and ends at 2^40."""
+    r = subprocess.run([native("batch_tasks"), str(chains), str(2 ** 30), str(first), "60000"], capture_output=True,
+                       text=True)
+    assert r.returncode == 0, r.stdout
+    assert int(r.stdout) == min(60000, (2 ** 30 + 1 - first) * chains)
 
 
 @pytest.mark.gpu
