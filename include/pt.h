@@ -69,12 +69,13 @@ typedef struct {
 /* Optional settings (zero-initialised = defaults). */
 typedef struct {
     int32_t threads_per_block;  /* 0 = choose automatically; else a multiple of 32 <= 1024 */
-    int32_t wait_timeout_ms;    /* limit of every device-side wait; 0 = 5000 ms */
+    int32_t wait_timeout_ms;    /* limit of every device-side wait, of batched launches too; 0 = 5000 ms */
     int32_t swap_mode;          /* 0 = auto, 1 = swaps inside one cooperative launch,
                                    2 = one launch per sweep interval + a swap launch */
     int32_t test_withhold_rung; /* test hook, 0 = off: if r+1, the chain on rung r never
                                    publishes its swap mailbox, so its partner's wait runs out
-                                   and the call fails with PT_ETIMEDOUT (no fault, no hang) */
+                                   and the call fails with PT_ETIMEDOUT (no fault, no hang);
+                                   batched launches: in every request */
     int32_t kernel_path;        /* 0 = auto, 1 = any shape (words of
                                    four copies, or one copy a thread on small levels, with
                                    inline or produced random words; byte-wise for P = 1 and

@@ -40,9 +40,6 @@ namespace cg = cooperative_groups;
 
 namespace ptq {
 
-// Swap mailboxes of a problem: kClusterMailPasses passes of R entries.
-constexpr long long kBatchWaitNs = 20000000000ll;  // limit of every wait inside the kernel
-
 // Shared memory of one CTA while it owns problem I.
 struct BatchLayout {
     size_t sdesc, items, loff, rung, seq, E, M, mail, thr, red, ctl, chains, total;
@@ -125,10 +122,16 @@ __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t 
 __device__ __forceinline__ void bulk_stores_done() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
-// Polls ready() until it holds, with a time limit (then status and sh.abort say so) and back-off;
+// The time limit of every wait inside the kernel, and the word that says PT_ETIMEDOUT when one ran out.
+struct WaitLimit {
+    long long ns;
+    int* status;
+};
+
+// Polls ready() until it holds, with a time limit (then the status and sh.abort say so) and back-off;
 // false when some wait of this CTA gave up. The whole warp, converged.
 template <typename Ready>
-__device__ __forceinline__ bool wait_for(BatchShared& sh, int* status, Ready ready) {
+__device__ __forceinline__ bool wait_for(BatchShared& sh, const WaitLimit& limit, Ready ready) {
     const unsigned long long start = globaltimer_ns();
     unsigned int nap = 0;
     for (int polls = 0;; ++polls) {
@@ -137,9 +140,9 @@ __device__ __forceinline__ bool wait_for(BatchShared& sh, int* status, Ready rea
             nap = nap ? min(2u * nap, 256u) : 16u;
             __nanosleep(nap);
             if (*(volatile int*)&sh.abort) return false;
-            if ((long long)(globaltimer_ns() - start) > kBatchWaitNs) {
+            if ((long long)(globaltimer_ns() - start) > limit.ns) {
                 if ((threadIdx.x & 31) == 0) {
-                    if (status) atomicCAS(status, 0, PT_ETIMEDOUT);
+                    atomicCAS(limit.status, 0, PT_ETIMEDOUT);
                     *(volatile int*)&sh.abort = 1;
                 }
                 return false;
@@ -266,7 +269,7 @@ __device__ void store_chain(const BatchInstance& I, int8_t* dst, const int8_t* b
 }
 
 __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchShared& sh, cg::cluster_group& cluster,
-                            int rank, int K, int* status) {
+                            int rank, int K, const WaitLimit& limit) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const BatchLayout L(I, K, nt);
     uint32_t* s_sdesc = reinterpret_cast<uint32_t*>(smem + L.sdesc);
@@ -366,7 +369,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                 stop = s > I.n_sweeps;
                 if (!stop && s > 0) {
                     volatile int* seq = s_seq + lc;
-                    stop = !wait_for(sh, status, [&] { return *seq >= s; });
+                    stop = !wait_for(sh, limit, [&] { return *seq >= s; });
                     __threadfence_block();
                 }
             }
@@ -384,7 +387,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                         const unsigned long long* mb =
                             mail + ((size_t)(pass & (kClusterMailPasses - 1)) * R + partner) * 2;
                         unsigned long long wa = 0, wb = 0;
-                        stop = !wait_for(sh, status, [&] {
+                        stop = !wait_for(sh, limit, [&] {
                             if (I.mail_smem) {
                                 wa = ld_cluster_local_u64(mb);
                                 wb = ld_cluster_local_u64(mb + 1);
@@ -454,8 +457,8 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
             // (the copy completes by itself; the limit only bounds the wait)
             const unsigned long long start = globaltimer_ns();
             while (!mbar_try_wait(&sh.mbar[grp], phase)) {
-                if ((long long)(globaltimer_ns() - start) > kBatchWaitNs) {
-                    if (status) atomicCAS(status, 0, PT_ETIMEDOUT);
+                if ((long long)(globaltimer_ns() - start) > limit.ns) {
+                    atomicCAS(limit.status, 0, PT_ETIMEDOUT);
                     *(volatile int*)&sh.abort = 1;
                     break;
                 }
@@ -516,7 +519,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                 s_E[lc] = E;
                 s_M[lc] = M;
             }
-            if (sps > 0 && (s + 1) % sps == 0) {
+            if (sps > 0 && (s + 1) % sps == 0 && rung + 1 != I.withhold) {
                 const int pass = (s + 1) / sps - 1;
                 const unsigned long long tag = mbox_tag(qmod0, pass);
                 const unsigned long long wa = ((unsigned long long)E << 24) | tag;
@@ -575,9 +578,10 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int K = (int)cluster.num_blocks();
+    const WaitLimit limit = {bp.timeout_ns, bp.status};
     if (bp.single) {
         // one problem on this one cluster; the host keeps its counters
-        run_problem(bp.one, smem, sh, cluster, rank, K, bp.status);
+        run_problem(bp.one, smem, sh, cluster, rank, K, limit);
         if (K > 1) cluster.sync();  // peers are done reading this CTA's published (E, M)
         return;
     }
@@ -588,7 +592,7 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
         cluster.sync();  // every CTA has read the job before rank 0 may reuse or release sh.job
         if (job >= bp.count) break;
         const BatchInstance I = bp.inst[bp.order[job]];
-        run_problem(I, smem, sh, cluster, rank, K, bp.status);
+        run_problem(I, smem, sh, cluster, rank, K, limit);
         cluster.sync();  // peers are done reading this CTA's published (E, M)
         if (rank == 0 && threadIdx.x == 0) {
             // a finished problem's counters advance on the device, so the same launch can be
@@ -725,13 +729,14 @@ size_t batch_smem_cap() {
 }
 
 cudaError_t launch_batch_single(const BatchInstance& I, int cluster, int threads, size_t smem, int* status,
-                                cudaStream_t s) {
+                                long long timeout_ns, cudaStream_t s) {
     BatchParams bp;
     bp.inst = nullptr;
     bp.order = nullptr;
     bp.count = 1;
     bp.next_job = nullptr;
     bp.status = status;
+    bp.timeout_ns = timeout_ns;
     bp.single = 1;
     bp.one = I;
     return launch_batch(bp, cluster, 1, threads, smem, s);
@@ -759,6 +764,7 @@ struct pt_batch {
     int32_t* d_order;
     int* d_counter;
     int* d_status;
+    long long timeout_ns;
     int8_t* d_staging;
     std::vector<BatchInstance> h_inst;
     std::vector<long long> sweep_limit;
@@ -1167,6 +1173,7 @@ static cudaError_t enqueue_run(pt_batch* b) {
     bp.count = b->count;
     bp.next_job = b->d_counter;
     bp.status = b->d_status;
+    bp.timeout_ns = b->timeout_ns;
     return launch_batch(bp, b->cluster, b->n_clusters, b->threads, b->smem, b->stream);
 }
 
@@ -1176,9 +1183,11 @@ static cudaError_t enqueue_run(pt_batch* b) {
 // the choice cannot change any result; the state is reset afterwards.
 static int autotune(pt_batch* b) {
     static const int kClusters[] = {1, 2, 4, 8};
-    std::vector<int> full(b->count);
+    std::vector<int> full(b->count), withhold(b->count);
     for (int k = 0; k < b->count; ++k) {
         full[k] = b->h_inst[k].n_sweeps;
+        withhold[k] = b->h_inst[k].withhold;
+        b->h_inst[k].withhold = 0;
         b->h_inst[k].n_sweeps = std::min(full[k], std::max(2, full[k] / 100));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1224,7 +1233,10 @@ static int autotune(pt_batch* b) {
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    for (int k = 0; k < b->count; ++k) b->h_inst[k].n_sweeps = full[k];
+    for (int k = 0; k < b->count; ++k) {
+        b->h_inst[k].n_sweeps = full[k];
+        b->h_inst[k].withhold = withhold[k];
+    }
     if (e != cudaSuccess) return bfail(b, PT_ECUDA, "autotuner: %s", cudaGetErrorString(e));
     int st = 0;
     if ((e = cudaMemcpy(&st, b->d_status, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess || st)
@@ -1287,6 +1299,7 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
     b->h_obs_bytes = 0;
     b->tuned = 0;
     b->widen = 0;
+    b->timeout_ns = (opt && opt->wait_timeout_ms > 0 ? opt->wait_timeout_ms : 5000) * 1000000ll;
     b->err = 0;
     b->msg[0] = 0;
     if (!b->stream) {
@@ -1345,6 +1358,7 @@ extern "C" int pt_batch_create(const pt_request* reqs, int32_t count, const pt_o
         I.n_levels = p.n_levels;
         I.dc = p.dc;
         I.form = I.form_t = p.form;
+        I.withhold = opt && opt->test_withhold_rung > 0 ? opt->test_withhold_rung : 0;
         I.slot_stride = p.slot_stride;
         I.key0 = (uint32_t)(reqs[k].seed & 0xFFFFFFFFu);
         I.key1 = (uint32_t)(reqs[k].seed >> 32);

@@ -399,7 +399,7 @@ static cudaError_t launch_plan_sweeps(const DevProblem& p, const LaunchPlan& pla
                                       int sps, long long timeout_ns, bool cooperative, cudaStream_t s) {
     if (plan.path == kPathPackedChains)
         return launch_batch_single(chains_instance(p, plan, t0, q0, n, sps), plan.cluster, plan.threads,
-                                   plan.smem_bytes, p.status, s);
+                                   plan.smem_bytes, p.status, timeout_ns, s);
     return launch_sweeps(p, plan, t0, q0, n, sps, timeout_ns, cooperative, s);
 }
 
@@ -1357,7 +1357,8 @@ static int enqueue_sweeps(pt_ctx* c, long long n, int sps) {
             long long chunk = n - done;
             chunk = std::min<long long>(chunk, sps > 0 ? ((1ll << 30) / sps) * sps : (1ll << 30));
             CUDA_OR_FAIL(c, launch_batch_single(chains_instance(c->dp, c->plan, c->t, c->q, (int)chunk, sps),
-                                                c->plan.cluster, c->plan.threads, c->plan.smem_bytes, c->dp.status, c->stream));
+                                                c->plan.cluster, c->plan.threads, c->plan.smem_bytes, c->dp.status,
+                                                c->timeout_ns, c->stream));
             c->launches += 1;
             c->t += chunk;
             if (sps > 0) c->q += chunk / sps;

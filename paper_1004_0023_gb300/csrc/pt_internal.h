@@ -189,6 +189,7 @@ struct BatchInstance {
     int form;                  // kForm*: how a chain lies in shared memory (form_t, or kFormBytes1)
     int form_t;                // the form with the least instructions for the chain on one-warp groups
     int n_groups;              // groups of group_threads threads at work in a CTA
+    int withhold;              // test hook: 1 + the rung whose chain never publishes (0 = off)
     uint32_t key0, key1;
     long long t0, q0;          // counters before this run
     int n_sweeps, sweeps_per_swap;
@@ -244,6 +245,7 @@ struct BatchParams {
     int count;
     int* next_job;              // work counter, zero at launch
     int* status;
+    long long timeout_ns = 5000000000ll;  // limit of every wait inside the launch
     int* done = nullptr;        // [count] or null: done[k] = done_token once problem k is written back
     int done_token = 1;         // nonzero, different per launch, so stale flags never match
     int single = 0;             // 1: one cluster runs `one` (passed by value) once; inst, order,
@@ -320,7 +322,7 @@ cudaError_t batch_max_clusters(int cluster, int threads, size_t smem, int* n_clu
 cudaError_t launch_batch_init(const BatchInstance* inst, const int2* map, int n_chains, cudaStream_t s);
 // One problem on one cluster of `cluster` CTAs (path 7); I carries t0, q0, n_sweeps, sweeps_per_swap.
 cudaError_t launch_batch_single(const BatchInstance& I, int cluster, int threads, size_t smem, int* status,
-                                cudaStream_t s);
+                                long long timeout_ns, cudaStream_t s);
 // The largest shared-memory need of the batched kernel: the device's opt-in maximum less
 // the kernel's static shared memory.
 size_t batch_smem_cap();

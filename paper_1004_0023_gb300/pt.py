@@ -339,7 +339,7 @@ def _read_obs(R, call, check):
 class Batch:
     """Many independent problems in one persistent launch (include/pt.h, pt_batch_*)."""
 
-    def __init__(self, problems, cluster_size=0, stream=None):
+    def __init__(self, problems, cluster_size=0, stream=None, wait_timeout_ms=0, test_withhold_rung=-1):
         self.lib = load()
         self.problems = list(problems)
         keep = []
@@ -352,6 +352,8 @@ class Batch:
                                  int(prob.seed) & 0xFFFFFFFFFFFFFFFF, int(prob.n_sweeps), int(prob.sweeps_per_swap))
         opt = pt_options()
         opt.cluster_size = int(cluster_size)
+        opt.wait_timeout_ms = int(wait_timeout_ms)
+        opt.test_withhold_rung = int(test_withhold_rung) + 1
         h = _vp()
         rc = self.lib.pt_batch_create(reqs, len(self.problems), ctypes.byref(opt),
                                       None if stream is None else _vp(int(stream)), ctypes.byref(h))

@@ -2,6 +2,7 @@
 sequence of their tasks (host code, on the CPU), and the bits of the requests that have both (GPU)."""
 import os
 import subprocess
+import time
 
 import numpy as np
 import pytest
@@ -114,3 +115,28 @@ def test_streamed_and_kept_chains_of_one_request_match_the_oracle(libpt, case):
         og, oo = b.obs(0), o.obs()
         for key in oo:
             assert np.array_equal(np.asarray(og[key]), np.asarray(oo[key])), (run, key)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", [(16, 3, 32, 6, 9, 1), (24, 3, 32, 40, 9, 2), (24, 3, 32, 5, 9, 4), MIXED[0], MIXED[1],
+                                  STREAMED[1]])
+def test_batched_waits_end_at_the_given_limit(libpt, case):
+    """The chain on rung 2 never publishes: its partner's wait ends after wait_timeout_ms and the
+    call returns PT_ETIMEDOUT, with chains kept, taken as tasks and streamed; a new batch then runs."""
+    prob = _problem(*case[:5], 60 + case[0])
+    prob.n_sweeps, prob.sweeps_per_swap = 8, 1
+    b = pt.Batch([prob, prob], cluster_size=case[5], wait_timeout_ms=150, test_withhold_rung=2)
+    start = time.monotonic()
+    b.run()
+    with pytest.raises(pt.PTError) as e:
+        b.sync()
+    assert e.value.code == pt.PT_ETIMEDOUT
+    assert time.monotonic() - start < 4.0
+    with pytest.raises(pt.PTError):  # sticky
+        b.run()
+    b.close()
+    b = pt.Batch([prob], cluster_size=case[5])
+    b.run()
+    o = Oracle.from_problem(prob, threads=THREADS)
+    o.run(prob.n_sweeps, prob.sweeps_per_swap)
+    assert np.array_equal(b.read_state(0), o.read_state())
