@@ -796,7 +796,7 @@ static std::map<std::vector<long long>, BatchLayoutChoice> g_layout_cache;
 
 static std::vector<long long> batch_shape_key(const std::vector<BatchInstance>& insts, int threads) {
     std::vector<long long> key;
-    key.reserve(insts.size() * 7 + 1);
+    key.reserve(insts.size() * 9 + 1);
     key.push_back(threads);
     for (const BatchInstance& I : insts) {
         key.push_back(I.N);
@@ -804,6 +804,8 @@ static std::vector<long long> batch_shape_key(const std::vector<BatchInstance>& 
         key.push_back(I.R);
         key.push_back(I.dc);
         key.push_back(I.n_levels);
+        key.push_back(I.form_t);  // the forms a chain can take: Lmax decides
+        key.push_back(IndexRule(I.Lmax).wide ? 1 : 0);
         key.push_back(I.n_sweeps);
         key.push_back(I.sweeps_per_swap);
     }

@@ -46,11 +46,14 @@ struct pt_ctx {
     int tuned_plans;             // candidate plans timed at create
 };
 
-// Plans chosen by the create-time autotuner, per problem shape, for the process.
+// Plans chosen by the create-time autotuner, per problem shape, for the process. Lmax and the
+// largest degree count by what they decide: the index form, where the threshold rows of a ladder
+// can be (48 KB and 96 KB, see the candidates' plans) and the slots of the any-shape descriptors.
 struct PlanKey {
-    int N, P, R, dc, n_levels, n_edges;
+    int N, P, R, dc, n_levels, n_edges, slots, wide, tables;
     bool operator<(const PlanKey& o) const {
-        return std::tie(N, P, R, dc, n_levels, n_edges) < std::tie(o.N, o.P, o.R, o.dc, o.n_levels, o.n_edges);
+        return std::tie(N, P, R, dc, n_levels, n_edges, slots, wide, tables) <
+               std::tie(o.N, o.P, o.R, o.dc, o.n_levels, o.n_edges, o.slots, o.wide, o.tables);
     }
 };
 struct PlanChoice {
@@ -1030,7 +1033,113 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             int cluster = 1, group_threads = 0;  // path 7; path 10: CTAs and chains per CTA
             int copy = 0;
         };
-        const PlanKey key{N, P, R, packed_dc, p.n_levels, nE};
+        const size_t table_bytes = (size_t)R * p.nL3 * 4;
+        const PlanKey key{N, P, R, packed_dc, p.n_levels, nE, p.slots, IndexRule(Lmax).wide ? 1 : 0,
+                          table_bytes <= 49152 ? 0 : (table_bytes <= 98304 ? 1 : 2)};
+        // a candidate's plan, shared-memory flags and level schedule
+        auto make = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
+                        std::vector<int32_t>& off_c) {
+            pc = p;
+            pc.records = pc.n_chunks = 0;
+            if (cd.path == kPathClassical) {
+                pc.acc_in_smem = 1;
+                pc.tables_in_smem = 1;
+                pl.path = kPathClassical;
+                pl.dclass = dclass;
+                pl.threads = cd.threads;
+                pl.n_consumer = cd.threads;
+                pl.chains_per_cta = cd.group_threads;
+                pl.cluster = cd.cluster;
+                level_schedule(N, adj, it_c, off_c, std::max(1, cd.threads / cd.group_threads));
+                drop_odd_updates(it_c, off_c);
+                pc.n_levels = (int)off_c.size() - 1;
+                pl.smem_bytes = classical_smem_bytes(pc, cd.group_threads);  // sized for this schedule
+                return pl.smem_bytes <= (size_t)max_smem;
+            }
+            if (cd.path == kPathPackedChains) {
+                if (!chains_plan(pc, packed_dc, cd.cluster, kGroupWidenDefault, pl, cd.group_threads)) return false;
+                level_schedule(N, adj, it_c, off_c, std::max(1, pl.group_threads / (P / 8)), P / 4);
+                pc.n_levels = (int)off_c.size() - 1;
+                return true;
+            }
+            pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
+            pc.tables_in_smem = (size_t)R * p.nL3 * 4 <= 49152 ? 1 : 0;
+            if (cd.copy) {
+                if (p.slots == 0) return false;
+                const bool cl = cd.path == kPathCluster;
+                pl.path = cd.path;
+                pl.dclass = packed_dc;
+                pl.copy = 1;
+                pl.threads = cd.threads;
+                pl.n_consumer = cd.threads - cd.producers;
+                level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / (P / 2)));
+                pc.n_levels = (int)off_c.size() - 1;
+                if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.tables_in_smem = 0;
+                if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.acc_in_smem = 0;
+                pc.records = records_for(cd.path, 1);
+                if (pc.records && copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.records = 0;
+                pl.smem_bytes = copy_smem_bytes(pc, cl);
+                return pl.smem_bytes <= (size_t)max_smem;
+            }
+            const bool cpre = cd.path == kPathCluster && cd.producers > 0;
+            if (pc.tables_in_smem && sweep_smem_bytes(pc, cd.path, packed_dc, cpre) > (size_t)max_smem)
+                pc.tables_in_smem = 0;
+            if (pc.acc_in_smem && sweep_smem_bytes(pc, cd.path, packed_dc, cpre) > (size_t)max_smem) pc.acc_in_smem = 0;
+            pl.path = cd.path;
+            pl.dclass = cd.path == kPathGeneric ? dclass : packed_dc;
+            pl.threads = cd.threads;
+            pl.n_consumer = cd.threads - cd.producers;
+            pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc, cpre);
+            int cols = 1;
+            if (cd.path == kPathSplit || cd.path == kPathSplitInline)
+                cols = P / 16 + 1;
+            else if (P >= 8)
+                cols = P / 8;
+            level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / cols), row_words_for(cd.path));
+            if (P == 1) drop_odd_updates(it_c, off_c);
+            pc.n_levels = (int)off_c.size() - 1;
+            if (cd.path == kPathPeer) {
+                // The fewest pieces of a sweep (cut_sweep) with which the layout fits, with records in
+                // at most four, else without: N=512, P=64, R=64 runs 6.47 us per sweep with swaps in
+                // pieces; path 6, the fastest otherwise, 7.70. From P = 128 the split kernels
+                // (paths 5 and 6) hold such chains in two CTAs, and are what is timed.
+                // Threshold tables of 48 to 96 KB too stay in shared memory if two pieces make the
+                // room: the next sweep's level 0 is then evaluated while the partner's mailbox is
+                // awaited (N=300, P=40, R=48, Lmax=58: 7.31 -> 6.89 us per sweep with a swap each,
+                // 6.23 -> 6.14 without; calls of five sweeps, which load the tables each time, are
+                // no slower).
+                pl.dclass = packed_dc;
+                auto fits_in = [&](int pieces, size_t max_tables) {
+                    pc.tables_in_smem = table_bytes <= max_tables ? 1 : 0;
+                    pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
+                    if (!cut_sweep(pc, off_c, pieces)) return false;
+                    pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc);
+                    pl.pieces = pc.n_chunks;
+                    return pl.smem_bytes <= (size_t)max_smem;
+                };
+                pc.records = records_for(cd.path, 0);
+                if (table_bytes > 49152 && table_bytes <= 98304)
+                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : 2); ++pieces)
+                        if (fits_in(pieces, 98304)) return true;
+                for (; pc.records >= 0; --pc.records)
+                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : pc.records ? 4 : kMaxChunks); ++pieces)
+                        if (fits_in(pieces, 49152)) return true;
+                return false;
+            }
+            pc.records = records_for(cd.path, 0);
+            if (pc.records && sweep_smem_bytes(pc, cd.path, pl.dclass, cpre) > (size_t)max_smem) pc.records = 0;
+            pl.smem_bytes = sweep_smem_bytes(pc, cd.path, pl.dclass, cpre);  // sized for this schedule
+            return pl.smem_bytes <= (size_t)max_smem;
+        };
+        // every chain of a made plan resident at once
+        auto runs_here = [&](const LaunchPlan& pl, const DevProblem& pc) {
+            if (pl.path == kPathPackedChains) return true;  // checked by chains_plan
+            long long res = 0;
+            const bool ok = prepare_sweep_kernel(pl) == cudaSuccess &&
+                            sweep_resident_chains(pc, pl, &res) == cudaSuccess && res >= R;
+            if (!ok) (void)cudaGetLastError();
+            return ok;
+        };
         std::vector<Cand> cands;
         {
             std::lock_guard<std::mutex> lock(g_plan_mutex);
@@ -1038,6 +1147,14 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             if (it != g_plan_cache.end())
                 cands.push_back({it->second.path, it->second.threads, it->second.producers, it->second.cluster,
                                  it->second.group_threads, it->second.copy});
+        }
+        if (!cands.empty()) {
+            // a choice that this problem's plan cannot follow does not count: its candidates are timed
+            LaunchPlan pl;
+            DevProblem pc;
+            std::vector<uint32_t> it_c;
+            std::vector<int32_t> off_c;
+            if (!make(cands[0], pl, pc, it_c, off_c) || !runs_here(pl, pc)) cands.clear();
         }
         const bool cached = !cands.empty();
         if (!cached && P == 1) {
@@ -1090,101 +1207,6 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                     if (!dup) cands.push_back({kPathPackedChains, 512, 0, K, pl.group_threads});
                 }
         }
-        // a candidate's plan, shared-memory flags and level schedule
-        auto make = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
-                        std::vector<int32_t>& off_c) {
-            pc = p;
-            pc.records = pc.n_chunks = 0;
-            if (cd.path == kPathClassical) {
-                pc.acc_in_smem = 1;
-                pc.tables_in_smem = 1;
-                pl.path = kPathClassical;
-                pl.dclass = dclass;
-                pl.threads = cd.threads;
-                pl.n_consumer = cd.threads;
-                pl.chains_per_cta = cd.group_threads;
-                pl.cluster = cd.cluster;
-                level_schedule(N, adj, it_c, off_c, std::max(1, cd.threads / cd.group_threads));
-                drop_odd_updates(it_c, off_c);
-                pc.n_levels = (int)off_c.size() - 1;
-                pl.smem_bytes = classical_smem_bytes(pc, cd.group_threads);  // sized for this schedule
-                return pl.smem_bytes <= (size_t)max_smem;
-            }
-            if (cd.path == kPathPackedChains) {
-                if (!chains_plan(pc, packed_dc, cd.cluster, kGroupWidenDefault, pl, cd.group_threads)) return false;
-                level_schedule(N, adj, it_c, off_c, std::max(1, pl.group_threads / (P / 8)), P / 4);
-                pc.n_levels = (int)off_c.size() - 1;
-                return true;
-            }
-            pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
-            pc.tables_in_smem = (size_t)R * p.nL3 * 4 <= 49152 ? 1 : 0;
-            if (cd.copy) {
-                const bool cl = cd.path == kPathCluster;
-                pl.path = cd.path;
-                pl.dclass = packed_dc;
-                pl.copy = 1;
-                pl.threads = cd.threads;
-                pl.n_consumer = cd.threads - cd.producers;
-                level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / (P / 2)));
-                pc.n_levels = (int)off_c.size() - 1;
-                if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.tables_in_smem = 0;
-                if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.acc_in_smem = 0;
-                pc.records = records_for(cd.path, 1);
-                if (pc.records && copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.records = 0;
-                pl.smem_bytes = copy_smem_bytes(pc, cl);
-                return pl.smem_bytes <= (size_t)max_smem;
-            }
-            const bool cpre = cd.path == kPathCluster && cd.producers > 0;
-            if (pc.tables_in_smem && sweep_smem_bytes(pc, cd.path, packed_dc, cpre) > (size_t)max_smem)
-                pc.tables_in_smem = 0;
-            if (pc.acc_in_smem && sweep_smem_bytes(pc, cd.path, packed_dc, cpre) > (size_t)max_smem) pc.acc_in_smem = 0;
-            pl.path = cd.path;
-            pl.dclass = cd.path == kPathGeneric ? dclass : packed_dc;
-            pl.threads = cd.threads;
-            pl.n_consumer = cd.threads - cd.producers;
-            pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc, cpre);
-            int cols = 1;
-            if (cd.path == kPathSplit || cd.path == kPathSplitInline)
-                cols = P / 16 + 1;
-            else if (P >= 8)
-                cols = P / 8;
-            level_schedule(N, adj, it_c, off_c, std::max(1, pl.n_consumer / cols), row_words_for(cd.path));
-            if (P == 1) drop_odd_updates(it_c, off_c);
-            pc.n_levels = (int)off_c.size() - 1;
-            if (cd.path == kPathPeer) {
-                // The fewest pieces of a sweep (cut_sweep) with which the layout fits, with records in
-                // at most four, else without: N=512, P=64, R=64 runs 6.47 us per sweep with swaps in
-                // pieces; path 6, the fastest otherwise, 7.70. From P = 128 the split kernels
-                // (paths 5 and 6) hold such chains in two CTAs, and are what is timed.
-                // Threshold tables of 48 to 96 KB too stay in shared memory if two pieces make the
-                // room: the next sweep's level 0 is then evaluated while the partner's mailbox is
-                // awaited (N=300, P=40, R=48, Lmax=58: 7.31 -> 6.89 us per sweep with a swap each,
-                // 6.23 -> 6.14 without; calls of five sweeps, which load the tables each time, are
-                // no slower).
-                pl.dclass = packed_dc;
-                const size_t table_bytes = (size_t)R * p.nL3 * 4;
-                auto fits_in = [&](int pieces, size_t max_tables) {
-                    pc.tables_in_smem = table_bytes <= max_tables ? 1 : 0;
-                    pc.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
-                    if (!cut_sweep(pc, off_c, pieces)) return false;
-                    pl.smem_bytes = sweep_smem_bytes(pc, cd.path, packed_dc);
-                    pl.pieces = pc.n_chunks;
-                    return pl.smem_bytes <= (size_t)max_smem;
-                };
-                pc.records = records_for(cd.path, 0);
-                if (table_bytes > 49152 && table_bytes <= 98304)
-                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : 2); ++pieces)
-                        if (fits_in(pieces, 98304)) return true;
-                for (; pc.records >= 0; --pc.records)
-                    for (int pieces = 1; pieces <= (P >= 128 ? 1 : pc.records ? 4 : kMaxChunks); ++pieces)
-                        if (fits_in(pieces, 49152)) return true;
-                return false;
-            }
-            pc.records = records_for(cd.path, 0);
-            if (pc.records && sweep_smem_bytes(pc, cd.path, pl.dclass, cpre) > (size_t)max_smem) pc.records = 0;
-            pl.smem_bytes = sweep_smem_bytes(pc, cd.path, pl.dclass, cpre);  // sized for this schedule
-            return pl.smem_bytes <= (size_t)max_smem;
-        };
         cudaStream_t s = c->stream;
         int best = -1, timed_plans = 0;
         if (cands.size() == 1) {
@@ -1209,14 +1231,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                 DevProblem pc;
                 std::vector<uint32_t> it_c;
                 std::vector<int32_t> off_c;
-                if (!make(cands[k], pl, pc, it_c, off_c)) continue;
-                long long res = 0;
-                if (pl.path != kPathPackedChains &&
-                    (prepare_sweep_kernel(pl) != cudaSuccess || sweep_resident_chains(pc, pl, &res) != cudaSuccess ||
-                     res < R)) {
-                    (void)cudaGetLastError();
-                    continue;
-                }
+                if (!make(cands[k], pl, pc, it_c, off_c) || !runs_here(pl, pc)) continue;
                 cudaError_t e1 = cudaMemcpyAsync(d_items, it_c.data(), it_c.size() * 4, cudaMemcpyHostToDevice, s);
                 if (e1 == cudaSuccess)
                     e1 = cudaMemcpyAsync(d_loff, off_c.data(), off_c.size() * 4, cudaMemcpyHostToDevice, s);
@@ -1272,10 +1287,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             std::vector<uint32_t> it_b;
             std::vector<int32_t> off_b;
             if (make(cands[best], pl, pc, it_b, off_b)) {
-                long long res = 0;
-                if (pl.path == kPathPackedChains ||
-                    (prepare_sweep_kernel(pl) == cudaSuccess && sweep_resident_chains(pc, pl, &res) == cudaSuccess &&
-                     res >= R)) {
+                if (runs_here(pl, pc)) {
                     // the plan with the schedule its shared memory was sized for
                     items.swap(it_b);
                     level_off.swap(off_b);

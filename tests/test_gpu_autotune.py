@@ -68,3 +68,43 @@ def test_autotuned_short_ladder_may_take_the_one_cluster_plan():
     g.run(200, 1)
     o.run(200, 1)
     _same(g, o)
+
+
+def _coupled(n, degree, P, R, j, h, seed):
+    """Regular couplings of one size, so that Lmax = degree * j + h at every site."""
+    ei, ej = instances.random_regular_graph(n, degree, np.random.default_rng(seed))
+    rng = np.random.default_rng(seed + 1)
+    J = j * rng.choice([-1, 1], ei.size)
+    T = np.full(R, 0.05 * j)
+    return instances.Problem(n, ei, ej, J.astype(np.int32), (h * rng.choice([-1, 1], n)).astype(np.int32), P, T,
+                             instances.gamma_ladder("geometric", 0.05 * j, 4.0 * j, R), 1, 20, 1, "")
+
+
+@pytest.mark.parametrize("n,order", [(54, (2, 20)), (58, (20, 2))])
+def test_problems_that_differ_in_lmax_alone_are_tuned_apart(n, order):
+    """Lmax 7 and 61 on one graph: the index form differs, so neither takes the other's plan; each
+    takes its own again."""
+    for j in order:
+        prob = _coupled(n, 3, 48, 9, j, 1, 77)
+        g = pt.PT.from_problem(prob)
+        assert g.info.lmax == 3 * j + 1 and g.info.tuned_plans >= 2
+        again = pt.PT.from_problem(_coupled(n, 3, 48, 9, j, 1, 77))
+        assert again.info.tuned_plans == 0 and again.info.kernel_path == g.info.kernel_path
+        o = Oracle.from_problem(prob, threads=THREADS)
+        g.run(40, 1)
+        o.run(40, 1)
+        _same(g, o)
+
+
+@pytest.mark.parametrize("n,order", [(84, (2, 20)), (88, (20, 2))])
+def test_batches_that_differ_in_lmax_alone_are_tuned_apart(n, order):
+    for j in order:
+        probs = [_coupled(n, 3, 64, 9, j, 1, 78), _coupled(n + 2, 3, 64, 9, j, 1, 79)]
+        b = pt.Batch(probs)
+        assert b.info().tuned_layouts >= 1
+        assert pt.Batch(probs).info().tuned_layouts == 0
+        b.run()
+        for k, p in enumerate(probs):
+            o = Oracle.from_problem(p, threads=THREADS)
+            o.run(p.n_sweeps, p.sweeps_per_swap)
+            assert np.array_equal(b.read_state(k), o.read_state()), (j, k)
