@@ -881,8 +881,10 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     uint32_t thr_c = thr0 + thr_step * (uint32_t)rung;
     const int lane = tid & 31;
     if (PEER) {
-        // the peer CTA has written the first sweep's words (its arrival releases them); this
-        // CTA's arrival orders nothing of its own, so it is relaxed
+        // the barrier entered at the start of the kernel, then: the peer CTA has written the first
+        // sweep's words (its arrival releases them); this CTA's arrival orders nothing of its own,
+        // so it is relaxed
+        cluster_wait_acquire();
         cluster_arrive_relaxed();
         cluster_wait_acquire();
     }
@@ -1251,8 +1253,9 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
 // one sweep (or piece of a sweep, where two whole sweeps' words do not fit: DevProblem::n_chunks)
 // ahead into rank 0's double buffer through distributed shared memory (the words
 // are a function of the chain, the sweep and the update, never of the rung, so they need no
-// swap decision). It passes the same cluster barriers as rank 0 (one before the first sweep,
-// one per sweep) and leaves after the one at which rank 0 reports that it leaves.
+// swap decision). It passes the same cluster barriers as rank 0 (one entered at the start of the
+// kernel, which shows that both CTAs run, one before the first sweep, one per sweep or piece) and
+// leaves after the one at which rank 0 reports that it leaves.
 template <int DC, bool PIECES>
 __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n_sweeps, unsigned char* smem) {
     cg::cluster_group cluster = cg::this_cluster();
@@ -1268,6 +1271,7 @@ __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n
     if (tid == 0) s_ctl[6] = 0;
     const PhiloxKey key = philox_schedule(p.key0, p.key1);
     __syncthreads();
+    cluster_wait_acquire();  // rank 0 has started: its shared memory may be written
     const int pieces = PIECES ? p.n_chunks : 1;
     const size_t buf_words = (size_t)(PIECES ? p.chunk_items : n_items) * G;
     // piece k of the launch (piece k % pieces of sweep t0 + k / pieces), into buffer k & 1
@@ -1306,6 +1310,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
         return;
     }
     const int slot = (int)(blockIdx.x >> 1);
+    // no CTA touches the other's shared memory before its wait on this barrier shows that the other
+    // has started; arriving first and waiting only then leaves the set-up in between
+    cluster_arrive_relaxed();
     if (cluster.block_rank() == 0) {
         if (IndexRule(p.Lmax).wide)
             sweep_packed_body<DC, true, true, false, true, true, false, 0, false, PIECES>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
