@@ -131,7 +131,10 @@ typedef struct {
                                    on it. 1: off. */
     int32_t group_threads;      /* kernel_path 7: threads sweeping one chain (32, 64, ..., 512),
                                    0 = the narrowest that keeps every chain resident */
-    int32_t reserved[2];
+    int32_t test_pieces;        /* test hook, kernel_path 8 only: 2..8 = its random words made in at
+                                   most so many pieces of a sweep, as the automatic plan does where
+                                   whole sweeps' words do not fit (results are identical) */
+    int32_t reserved;
 } pt_options;
 
 /* Statistics (Fig. 4 "gather statistics"; Sec. 5 accumulates in high precision).
@@ -164,7 +167,8 @@ typedef struct {
     int64_t kernel_launches;   /* kernels this context has launched so far */
     int64_t h2d_bytes;         /* bytes copied host -> device so far */
     int32_t tuned_plans;       /* candidate plans timed by pt_create (0: none, or cached) */
-    int32_t reserved;
+    int32_t pieces;            /* path 8: pieces of a sweep its random words are made in (1 = whole
+                                  sweeps); 0 on other paths */
 } pt_info;
 
 /* Create a PT-QMC problem on the current CUDA device (Sec. 2: chains and temperatures

@@ -748,6 +748,9 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                    sweep_smem_bytes(q, kPathBits, packed_dc) <= (size_t)max_smem;
         c->plan.nibble = !p.nibble ? 0 : (packed_dc == 4 ? 3 : (dmax <= 6 ? 6 : 7));
     }
+    // test hook: path 8's words in pieces of a sweep (the levels are balanced again below)
+    const int cut = path == kPathPeer && opt ? std::max(0, std::min(opt->test_pieces, kMaxChunks)) : 0;
+    if (cut > 1 && !cut_sweep(p, level_off, cut)) p.n_chunks = 0;
     c->plan.path = path;
     c->plan.rows = path == kPathGeneric && p.slots > 0;
     c->plan.dclass = (path == kPathGeneric || path == kPathClassical) ? dclass : packed_dc;
@@ -857,6 +860,8 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         level_schedule(N, adj, items, level_off, std::max(1, per_round), row_words_for(path));
         if (P == 1) drop_odd_updates(items, level_off);
         p.n_levels = (int)level_off.size() - 1;
+        if (cut > 1 && !cut_sweep(p, level_off, cut)) p.n_chunks = 0;
+        c->plan.pieces = p.n_chunks;
         // the level offsets live in shared memory: size it for this schedule's level count
         c->plan.smem_bytes = plan_smem();
         if ((long long)c->plan.smem_bytes > (long long)max_smem) {
@@ -1608,7 +1613,7 @@ extern "C" int pt_get_info(const pt_ctx* c, pt_info* o) {
     o->kernel_launches = c->launches;
     o->h2d_bytes = c->h2d_bytes;
     o->tuned_plans = c->tuned_plans;
-    o->reserved = 0;
+    o->pieces = c->plan.path == kPathPeer ? std::max(1, c->plan.pieces) : 0;
     return PT_OK;
 }
 

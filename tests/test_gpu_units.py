@@ -191,3 +191,45 @@ def test_an_unequal_backlog_on_wide_clusters_matches_the_oracle():
         for k in want:
             assert np.array_equal(np.asarray(obs[k]), np.asarray(want[k])), k
     srv.close()
+
+
+# both neighbour classes, narrow and wide index, copies that don't fill 16; the last four with
+# records that don't fit beside the words (two pieces) and with whole sweeps' words that don't
+PIECES = [(60, 3, 64, 6, 13), (60, 7, 64, 5, 41), (60, 7, 64, 4, 42), (60, 3, 40, 4, 127)]
+PIECES = [(*c, k) for c in PIECES for k in (2, 3, 5, 8)] + [
+    (500, 7, 64, 4, 41, 2), (500, 7, 64, 4, 60, 2), (512, 3, 64, 5, 13, 4), (512, 3, 64, 5, 42, 8)]
+
+
+@pytest.mark.parametrize("case", PIECES)
+def test_random_words_in_pieces_match_the_oracle(case):
+    """Path 8 with its words in a given number of pieces, whatever plan would be the fastest."""
+    prob = _problem(*case[:5], 300 + case[5])
+    g, o = pt.PT.from_problem(prob, kernel_path=8, test_pieces=case[5]), Oracle.from_problem(prob, threads=THREADS)
+    assert g.info.kernel_path == 8 and 2 <= g.info.pieces <= case[5]
+    for sweeps, sps in ((1, 1), (2, 1), (7, 0), (12, 3), (1, 0)):
+        g.run(sweeps, sps)
+        o.run(sweeps, sps)
+        assert np.array_equal(g.read_state(), o.read_state()), (sweeps, sps)
+    og, oo = g.obs(), o.obs()
+    for k in oo:
+        assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
+    g.close()
+
+
+@pytest.mark.parametrize("pieces", [2, 3, 8])
+def test_partner_that_never_publishes_times_out_with_words_in_pieces(pieces):
+    """The sweeping CTA gives up with sweeps left and skips to the sweep's last barrier; the word CTA
+    meets it at its next piece's, learns of it there and leaves with it."""
+    prob = _problem(60, 3, 64, 6, 13, 9)
+    g = pt.PT.from_problem(prob, kernel_path=8, test_pieces=pieces, wait_timeout_ms=200, test_withhold_rung=3,
+                           swap_mode=1)
+    assert g.info.pieces >= 2
+    g.run(4, 1)
+    with pytest.raises(pt.PTError) as e:
+        g.sync()
+    assert e.value.code == pt.PT_ETIMEDOUT
+    g.close()
+    h, o = pt.PT.from_problem(prob), Oracle.from_problem(prob, threads=THREADS)
+    h.run(20, 1)
+    o.run(20, 1)
+    assert np.array_equal(h.read_state(), o.read_state())
