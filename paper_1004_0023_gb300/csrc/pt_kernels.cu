@@ -72,7 +72,7 @@ struct RowsLayout {
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
         thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
         acc = o;   o += acc_bytes(p);
-        red = o;   o += 32 * 3 * 8;
+        red = o;   o += 16;  // the sweep's three sums
         ctl = o;   o += 32;
         cmb = o;   o += cswap ? (size_t)kClusterMailPasses * p.R * 16 : 0;
         rbuf = o;  o += pre ? 2 * (2 * N) * G * 16 : 0;
@@ -102,7 +102,7 @@ struct FastLayout {
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
         thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
         acc = o;   o += acc_bytes(p);
-        red = o;   o += 32 * 3 * 8;
+        red = o;   o += 16;  // the sweep's three sums
         ctl = o;   o += 32;
         cmb = o;   o += cswap ? (size_t)kClusterMailPasses * p.R * 16 : 0;
         rbuf = o;
@@ -1483,7 +1483,7 @@ struct SplitLayout {
         loff = o;  o += up16((size_t)(p.n_levels + 1) * 4);
         thr = o;   o += thr_bytes(p, IndexRule(p.Lmax).row_words());
         acc = o;   o += acc_bytes(p);
-        red = o;   o += 32 * 3 * 8;
+        red = o;   o += 16;  // the sweep's three sums
         ctl = o;   o += 32;
         xch = o;   o += 64;  // written by the peer: [sweep parity][dE, dM, flips, abort], final abort
         rbuf = o;
