@@ -1058,6 +1058,12 @@ void ptq::fill_instance(BatchInstance& I, const Prepared& p, unsigned char* base
     I.mail = (Mailbox*)(base + p.off_mbox);
 }
 
+// Every rung's threshold row in shared memory when the rows take at most 48 KB and the chains still
+// fit; resident chains come first.
+static int rows_resident(const BatchInstance& I) {
+    return (size_t)I.R * up16((size_t)IndexRule(I.Lmax).row_words() * 4) <= 49152 ? 1 : 0;
+}
+
 static void groups_of_form(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen) {
     // threads per chain: about one 4-copy unit per thread in an average level, at least two
     // warps, and no more groups than a CTA has chains; chains stay resident when they fit.
@@ -1079,10 +1085,7 @@ static void groups_of_form(BatchInstance& I, int cluster, int threads, size_t sm
     for (int w = 0; w < -widen && g > 32; ++w) g >>= 1;  // down to one warp per chain
     while (up_ok(g) && threads / g > C) g <<= 1;         // still no more groups than chains
     while (g > 32 && up_ok(g) && threads / g > 15) g <<= 1;  // named barriers 1..15 (0: the CTA's)
-    // every rung's threshold row in shared memory when the rows take at most 48 KB and the
-    // chains still fit; resident chains come first
-    const int thr_words = (int)(up16((size_t)IndexRule(I.Lmax).row_words() * 4) / 4);
-    const int thr_ok = (size_t)I.R * thr_words * 4 <= 49152 ? 1 : 0;
+    const int thr_ok = rows_resident(I);
     for (bool ok = false; !ok;) {
         // resident chains come first, then threshold rows, then the swap mailboxes; with chains
         // streamed through one buffer a group, a few groups less than the CTA's warps could
@@ -1102,6 +1105,24 @@ static void groups_of_form(BatchInstance& I, int cluster, int threads, size_t sm
         g <<= 1;
         while (up_ok(g) && threads / g > 15) g <<= 1;
     }
+}
+
+bool ptq::resident_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int group_threads, int least) {
+    BatchInstance T = I;
+    T.group_threads = group_threads;
+    T.resident = 1;
+    for (int n = threads / group_threads; n >= std::max(1, least); --n) {
+        T.n_groups = n;
+        for (int k = 0; k < 4; ++k) {
+            T.thr_resident = (k & 2) ? 0 : rows_resident(I);
+            T.mail_smem = (k & 1) ? 0 : 1;
+            if (batch_smem_bytes(T, cluster, threads) <= smem_cap) {
+                I = T;
+                return true;
+            }
+        }
+    }
+    return false;
 }
 
 void ptq::choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen) {

@@ -418,17 +418,12 @@ static bool chains_plan(const DevProblem& p, int dclass, int cluster, int widen,
     const size_t cap = batch_smem_cap();
     choose_groups(I, cluster, 512, cap, widen);
     if (force_group > 0) {
-        // the given width, with every rung's threshold row resident if that still fits
-        I.group_threads = force_group;
-        I.n_groups = 512 / force_group;
-        I.resident = 1;
-        I.thr_resident = 1;
-        I.mail_smem = 1;
-        if (batch_smem_bytes(I, cluster, 512) > cap) I.mail_smem = 0;
-        if (batch_smem_bytes(I, cluster, 512) > cap || (size_t)I.R * ((IndexRule(I.Lmax).row_words() * 4 + 15) / 16 * 16) > 49152)
-            I.thr_resident = 0;
+        if (!resident_groups(I, cluster, 512, cap, force_group, 1)) return false;
+    } else if (!I.resident) {
+        // a few groups less may hold every chain (each has a threshold row of its own)
+        const int most = 512 / I.group_threads;
+        if (!resident_groups(I, cluster, 512, cap, I.group_threads, (5 * most + 7) / 8)) return false;
     }
-    if (!I.resident) return false;
     const size_t smem = batch_smem_bytes(I, cluster, 512);
     if (smem > cap) return false;
     int ncl = 0;

@@ -313,6 +313,10 @@ constexpr int kGroupWidenDefault = -4;
 // with (the layout choose_groups picked for that cluster).
 double request_cycles(const BatchInstance& I, int cluster);
 void choose_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int widen = kGroupWidenDefault);
+// Every chain resident, swept by groups of the given width: as many groups as fit, at least `least`,
+// with every rung's threshold row and the swap mailboxes in shared memory where those fit too.
+// False (I unchanged) when the chains don't fit.
+bool resident_groups(BatchInstance& I, int cluster, int threads, size_t smem_cap, int group_threads, int least);
 
 // Batched launchers (pt_batch.cu).
 size_t batch_smem_bytes(const BatchInstance& I, int cluster, int threads);
