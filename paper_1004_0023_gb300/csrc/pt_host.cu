@@ -787,6 +787,15 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
                            c->plan.smem_bytes, max_smem);
     }
+    // enough threads for the average level (units = items * padded groups per parity)
+    auto level_threads = [&] {
+        int G = path == kPathBits && p.nibble ? P / 32 : ((P / 2) + 3) / 4, Gp = 1;
+        while (Gp < G) Gp <<= 1;
+        const long long units = (long long)items.size() * Gp;
+        long long avg = (units + p.n_levels - 1) / p.n_levels;
+        avg = ((avg + 31) / 32) * 32;
+        return (int)std::min<long long>(512, std::max<long long>(128, avg));
+    };
     if (opt && opt->threads_per_block > 0) {
         const int tmax =
             (path == kPathGeneric || path == kPathSplit || path == kPathSplitInline || path == kPathPeer) ? 512 : 1024;
@@ -804,13 +813,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     } else if (path == kPathGeneric && c->plan.copy) {
         c->plan.threads = copy_threads(&copy_producers);
     } else {
-        // enough threads for the average level (units = items * padded groups per parity)
-        int G = path == kPathBits && p.nibble ? P / 32 : ((P / 2) + 3) / 4, Gp = 1;
-        while (Gp < G) Gp <<= 1;
-        const long long units = (long long)items.size() * Gp;
-        long long avg = (units + p.n_levels - 1) / p.n_levels;
-        avg = ((avg + 31) / 32) * 32;
-        c->plan.threads = (int)std::min<long long>(512, std::max<long long>(128, avg));
+        c->plan.threads = level_threads();
     }
     c->plan.n_consumer = c->plan.threads;
     if (c->plan.copy) c->plan.n_consumer -= copy_producers;
@@ -838,7 +841,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     // the levels, rebalanced for the items this plan's kernel takes per round: consumer
     // threads over word columns per item (a power of two for the one-CTA kernels, W + 1 for
     // the split one); the level count and the dependencies stay the same
-    {
+    auto balance = [&] {
         int cols = 1;
         if (path == kPathSplit || path == kPathSplitInline) {
             cols = P / 16 + 1;
@@ -859,15 +862,77 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         c->plan.pieces = p.n_chunks;
         // the level offsets live in shared memory: size it for this schedule's level count
         c->plan.smem_bytes = plan_smem();
-        if ((long long)c->plan.smem_bytes > (long long)max_smem) {
-            free_ctx(c);
-            return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
-                               c->plan.smem_bytes, max_smem);
+    };
+    balance();
+    if ((long long)c->plan.smem_bytes > (long long)max_smem) {
+        free_ctx(c);
+        return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
+                           c->plan.smem_bytes, max_smem);
+    }
+    if (records_for(path, c->plan.copy)) {
+        p.records = 1;
+        if (plan_smem() > (size_t)max_smem) p.records = 0;
+        c->plan.smem_bytes = plan_smem();
+    }
+
+    // Swap passes inside one launch need every chain resident at once. The word-wise, one-copy and
+    // nibble kernels, and those that hold level 0's units in registers, take more registers or
+    // shared memory a CTA than the simplest kernel for the same chains; where those alone keep some
+    // chain out (ladders of several CTAs an SM: N=8, P=10, R=700 is resident with the byte-wise
+    // kernel's 80 registers, not with 117), the simplest kernel runs: byte-wise, one bit a copy,
+    // without held units (`lean`), with the threshold rows in global memory.
+    const int mode = opt ? opt->swap_mode : 0;
+    int coop_ok = 0;
+    cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, c->device);
+    auto all_resident = [&] {
+        long long res = 0;
+        const bool ok = prepare_sweep_kernel(c->plan) == cudaSuccess &&
+                        sweep_resident_chains(p, c->plan, &res) == cudaSuccess && res >= R;
+        if (!ok) (void)cudaGetLastError();
+        return ok;
+    };
+    const bool one_launch = coop_ok && mode != 2 && R > 1;
+    const bool pairs = path == kPathPeer || path == kPathSplit || path == kPathSplitInline;  // always resident
+    if ((pairs || (one_launch && R > n_sm)) && !want_chains && path != kPathClassical && path != kPathCluster &&
+        !all_resident()) {
+        const bool simpler = (path == kPathGeneric && c->plan.rows) || (path == kPathBits && p.nibble);
+        // 512 threads and more fill the registers of an SM's CTA either way
+        const bool lean = c->plan.threads < 512 && (path == kPathPacked || path == kPathPackedInline ||
+                                                    path == kPathBits || path == kPathPeer ||
+                                                    path == kPathSplitInline);
+        const DevProblem p0 = p;
+        const LaunchPlan plan0 = c->plan;
+        const std::vector<uint32_t> items0 = items;
+        const std::vector<int32_t> off0 = level_off;
+        bool ok = false;
+        for (int k = 1; k < 8 && !ok; ++k) {
+            const bool simple_k = (k & 1) != 0, lean_k = (k & 2) != 0, rows_out_k = (k & 4) != 0;
+            if ((simple_k && !simpler) || (lean_k && !lean)) continue;
+            p = p0;
+            c->plan = plan0;
+            items = items0;
+            level_off = off0;
+            p.records = 0;
+            if (simple_k) {
+                p.slots = p.nibble = 0;
+                c->plan.rows = c->plan.copy = c->plan.nibble = 0;
+                p.acc_in_smem = (size_t)R * kAccCount * 8 <= 16384 ? 1 : 0;
+                p.tables_in_smem = (size_t)R * p.nL3 * 4 <= 49152 ? 1 : 0;
+                if (plan_smem() > (size_t)max_smem) p.tables_in_smem = 0;
+                if (plan_smem() > (size_t)max_smem) p.acc_in_smem = 0;
+                c->plan.threads = want_threads > 0 ? want_threads : level_threads();
+                c->plan.n_consumer = c->plan.threads;
+            }
+            c->plan.lean = lean_k && !p.nibble ? 1 : 0;
+            if (rows_out_k) p.tables_in_smem = p.acc_in_smem = 0;
+            balance();
+            ok = c->plan.smem_bytes <= (size_t)max_smem && all_resident();
         }
-        if (records_for(path, c->plan.copy)) {
-            p.records = 1;
-            if (plan_smem() > (size_t)max_smem) p.records = 0;
-            c->plan.smem_bytes = plan_smem();
+        if (!ok) {
+            p = p0;
+            c->plan = plan0;
+            items = items0;
+            level_off = off0;
         }
     }
 
@@ -968,10 +1033,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
 
     // cooperative launch (swaps inside one launch) needs every chain resident at once
     long long resident = 0;
-    int coop_ok = 0;
-    cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, c->device);
     if (sweep_resident_chains(p, c->plan, &resident) != cudaSuccess) resident = 0;
-    const int mode = opt ? opt->swap_mode : 0;
     c->cooperative = coop_ok && resident >= R && mode != 2;
     if (mode == 1 && !c->cooperative) {
         free_ctx(c);

@@ -1299,8 +1299,9 @@ __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n
 // Path 8: R clusters of two CTAs; rank 0 sweeps chain (cluster index) with every thread,
 // rank 1 produces its random words. The cluster shape is compiled in, and checked on entry
 // (both CTAs return before any barrier or remote access if it is not 2).
-template <int DC, bool PIECES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
+// MAXT = 1024: the lean instance, without the held level-0 units (as sweep_packed_kernel).
+template <int DC, bool PIECES, int MAXT = 512>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MAXT, 1)
     sweep_peer_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                       long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1315,11 +1316,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     cluster_arrive_relaxed();
     if (cluster.block_rank() == 0) {
         if (IndexRule(p.Lmax).wide)
-            sweep_packed_body<DC, true, true, false, true, true, false, 0, false, PIECES>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
-                                                                 timeout_ns, blockDim.x, smem);
+            sweep_packed_body<DC, true, true, false, (MAXT <= 512), true, false, 0, false, PIECES>(
+                p, slot, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, blockDim.x, smem);
         else
-            sweep_packed_body<DC, true, false, false, true, true, false, 0, false, PIECES>(p, slot, t0, q0, n_sweeps, sweeps_per_swap,
-                                                                  timeout_ns, blockDim.x, smem);
+            sweep_packed_body<DC, true, false, false, (MAXT <= 512), true, false, 0, false, PIECES>(
+                p, slot, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, blockDim.x, smem);
     } else
         peer_producer<DC, PIECES>(p, slot, t0, n_sweeps, smem);
 }
@@ -1791,8 +1792,11 @@ __device__ __forceinline__ void split_body(const DevProblem& p, long long t0, lo
     }
 }
 
-template <int DC, bool PRE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
+// MAXT = 640: the lean instance. Its 96 registers a thread (98 otherwise) let one more CTA of a small
+// block be resident (160 threads: 4 an SM instead of 3); with that limit on every launch the kernels
+// took 5 to 20 % longer (N=200, degree 7, P=64, R=70: 6.83 -> 8.19 us per sweep).
+template <int DC, bool PRE, int MAXT = 512>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MAXT, 1)
     sweep_split_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                        long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1951,6 +1955,9 @@ static const void* sweep_fn(const LaunchPlan& plan) {
     if (plan.path == kPathPeer) {
         if (plan.pieces > 1)
             return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, true> : (const void*)sweep_peer_kernel<8, true>;
+        if (plan.lean)
+            return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, false, 1024>
+                                    : (const void*)sweep_peer_kernel<8, false, 1024>;
         return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, false> : (const void*)sweep_peer_kernel<8, false>;
     }
     if (plan.path == kPathCluster) {
@@ -1961,6 +1968,8 @@ static const void* sweep_fn(const LaunchPlan& plan) {
     }
     if (plan.path == kPathSplit)
         return plan.dclass == 4 ? (const void*)sweep_split_kernel<4, true> : (const void*)sweep_split_kernel<8, true>;
+    if (plan.path == kPathSplitInline && plan.dclass == 4 && plan.lean)
+        return (const void*)sweep_split_kernel<4, false, 640>;
     if (plan.path == kPathSplitInline)
         return plan.dclass == 4 ? (const void*)sweep_split_kernel<4, false> : (const void*)sweep_split_kernel<8, false>;
     if (plan.path == kPathBits && plan.nibble) {
@@ -1968,14 +1977,14 @@ static const void* sweep_fn(const LaunchPlan& plan) {
         return plan.nibble == 6 ? (const void*)sweep_nibble_kernel<8, 6> : (const void*)sweep_nibble_kernel<8, 7>;
     }
     if (plan.path == kPathBits) {
-        if (plan.threads > 512)
+        if (plan.threads > 512 || plan.lean)
             return plan.dclass == 4 ? (const void*)sweep_packed_kernel<4, false, 1024, true>
                                     : (const void*)sweep_packed_kernel<8, false, 1024, true>;
         return plan.dclass == 4 ? (const void*)sweep_packed_kernel<4, false, 512, true>
                                 : (const void*)sweep_packed_kernel<8, false, 512, true>;
     }
     const bool pre = plan.path == kPathPacked;
-    if (plan.threads > 512) {
+    if (plan.threads > 512 || plan.lean) {
         if (plan.dclass == 4)
             return pre ? (const void*)sweep_packed_kernel<4, true, 1024> : (const void*)sweep_packed_kernel<4, false, 1024>;
         return pre ? (const void*)sweep_packed_kernel<8, true, 1024> : (const void*)sweep_packed_kernel<8, false, 1024>;

@@ -141,11 +141,23 @@ extern "C" int pt_run_noalloc(const pt_device_problem* q, int64_t n_sweeps, int3
     }
     plan.n_consumer = plan.threads;
     if (prepare_sweep_kernel(plan) != cudaSuccess) return fail(PT_ECUDA, "cudaFuncSetAttribute failed");
-    if (swaps) {
+    auto all_resident = [&] {
         int per_sm = 0;
-        if (sweep_kernel_occupancy(p, plan, &per_sm) != cudaSuccess || !coop || (long long)per_sm * n_sm < q->R)
+        return sweep_kernel_occupancy(p, plan, &per_sm) == cudaSuccess && (long long)per_sm * n_sm >= q->R;
+    };
+    if (swaps && plan.rows && !all_resident()) {
+        // the byte-wise kernel takes less registers and shared memory a chain
+        p.slots = plan.rows = 0;
+        p.acc_in_smem = (size_t)q->R * kAccCount * 8 <= 16384 ? 1 : 0;
+        p.tables_in_smem = (size_t)q->R * p.nL3 * 4 <= 49152 ? 1 : 0;
+        if (sweep_smem_bytes(p, kPathGeneric, plan.dclass) > (size_t)max_smem) p.tables_in_smem = 0;
+        if (sweep_smem_bytes(p, kPathGeneric, plan.dclass) > (size_t)max_smem) p.acc_in_smem = 0;
+        plan.smem_bytes = sweep_smem_bytes(p, kPathGeneric, plan.dclass);
+        if (plan.smem_bytes > (size_t)max_smem || prepare_sweep_kernel(plan) != cudaSuccess)
             return fail(PT_EINVAL, "all chains must be resident at once for swaps inside the launch");
     }
+    if (swaps && (!coop || !all_resident()))
+        return fail(PT_EINVAL, "all chains must be resident at once for swaps inside the launch");
 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const long long timeout_ns = (long long)(wait_timeout_ms > 0 ? wait_timeout_ms : 5000) * 1000000ll;

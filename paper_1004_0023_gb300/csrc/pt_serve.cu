@@ -526,8 +526,16 @@ static int launch_streamed(pt_server* s, ServeReq* q) {
     const int sps = q->inst.sweeps_per_swap;
     const bool swaps = sps > 0 && pr.R > 1;
     int per_sm = 0;
-    const bool coop = swaps && sweep_kernel_occupancy(p, plan, &per_sm) == cudaSuccess &&
-                      (long long)per_sm * s->n_sm >= pr.R;
+    auto all_resident = [&] {
+        return sweep_kernel_occupancy(p, plan, &per_sm) == cudaSuccess && (long long)per_sm * s->n_sm >= pr.R;
+    };
+    bool coop = swaps && all_resident();
+    if (swaps && !coop && plan.threads < 512) {
+        // the instance with less registers a thread, where that makes every chain resident
+        plan.lean = 1;
+        coop = prepare_sweep_kernel(plan) == cudaSuccess && all_resident();
+        if (!coop) plan.lean = 0;
+    }
     long long t = q->inst.t0, qq = q->inst.q0;
     long long left = q->remaining;
     const long long timeout = 5000000000ll;

@@ -9,6 +9,7 @@ from native_build import compile_host
 from oracle import Oracle
 from paper_1004_0023_gb300 import pt
 from test_gpu_units import _problem
+from test_zz_no_alloc import _device_problem, _state_of
 
 
 def test_no_layout_asks_for_more_than_its_data_and_800_bytes(libpt, tmp_path):
@@ -45,3 +46,42 @@ def test_fewer_groups_than_the_cta_has_match_the_oracle(libpt, n, P, R, lmax, gr
         g.run(sweeps, sps)
         o.run(sweeps, sps)
         assert np.array_equal(g.read_state(), o.read_state())
+
+
+# ladders of several CTAs an SM that the simplest kernel of the path holds at once: one copy a thread,
+# the automatic plan's, held level-0 units, nibble words at the widest block, words from a second CTA,
+# split chains
+LADDERS = [
+    (8, 3, 10, 700, dict(kernel_path=1)), (8, 3, 12, 700, dict()), (9, 5, 20, 800, dict(kernel_path=1)),
+    (8, 3, 16, 700, dict(kernel_path=2, threads_per_block=128)), (8, 3, 16, 700, dict(kernel_path=3, threads_per_block=128)),
+    (8, 3, 32, 250, dict(kernel_path=4, threads_per_block=512)), (8, 5, 16, 250, dict(kernel_path=4, threads_per_block=448)),
+    (8, 3, 16, 100, dict(kernel_path=8, threads_per_block=320)), (8, 3, 16, 250, dict(kernel_path=6, threads_per_block=160)),
+]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,degree,P,R,kw", LADDERS)
+def test_long_ladders_stay_resident(libpt, n, degree, P, R, kw):
+    prob = _problem(n, degree, P, R, 9, n + R)
+    g = pt.PT.from_problem(prob, swap_mode=1, **kw)
+    assert g.info.cooperative == 1
+    o = Oracle.from_problem(prob)
+    for sweeps, sps in ((3, 1), (2, 0), (6, 2)):
+        g.run(sweeps, sps)
+        o.run(sweeps, sps)
+        assert np.array_equal(g.read_state(), o.read_state())
+    og, oo = g.obs(), o.obs()
+    for k in oo:
+        assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
+
+
+@pytest.mark.gpu
+def test_long_ladders_stay_resident_on_callers_memory(libpt):
+    torch = pytest.importorskip("torch")
+    prob = _problem(8, 3, 32, 700, 9, 5)
+    ref, o = pt.PT.from_problem(prob), Oracle.from_problem(prob)
+    dp, bufs = _device_problem(torch, prob, ref, None)
+    pt.run_noalloc(dp, 6, 2, 0, None)
+    o.run(6, 2)
+    got = _state_of(torch, bufs, prob)
+    assert got["status"] == 0 and np.array_equal(got["state"], o.read_state())
