@@ -70,9 +70,11 @@ struct BatchLayout {
 
 // Shared memory of the persistent kernel that outlives a problem.
 struct BatchShared {
-    unsigned long long next;      // next task of this CTA
     unsigned long long mbar[16];  // per group: arrival of a streamed chain
-    uint32_t phase[16];           // its parity of the next arrival
+    long long limit_ns;           // the time limit of every wait ...
+    int* status;                  // ... and the word that says PT_ETIMEDOUT when one ran out
+    uint32_t phase[16];           // per group: parity of the next arrival
+    unsigned next;                // next task of this CTA (TaskCursor)
     int abort;                    // a wait gave up
     int job;
 };
@@ -122,27 +124,22 @@ __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t 
 __device__ __forceinline__ void bulk_stores_done() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
-// The time limit of every wait inside the kernel, and the word that says PT_ETIMEDOUT when one ran out.
-struct WaitLimit {
-    long long ns;
-    int* status;
-};
-
 // Polls ready() until it holds, with a time limit (then the status and sh.abort say so) and back-off;
 // false when some wait of this CTA gave up. The whole warp, converged.
 template <typename Ready>
-__device__ __forceinline__ bool wait_for(BatchShared& sh, const WaitLimit& limit, Ready ready) {
-    const unsigned long long start = globaltimer_ns();
+__device__ __forceinline__ bool wait_for(BatchShared& sh, Ready ready) {
+    unsigned long long start = 0;
     unsigned int nap = 0;
     for (int polls = 0;; ++polls) {
         if (__all_sync(0xFFFFFFFFu, ready())) return true;
-        if (polls >= 32) {
+        if (polls >= 32) {  // (the clock is read only once the first polls have failed)
+            if (polls == 32) start = globaltimer_ns();
             nap = nap ? min(2u * nap, 256u) : 16u;
             __nanosleep(nap);
             if (*(volatile int*)&sh.abort) return false;
-            if ((long long)(globaltimer_ns() - start) > limit.ns) {
+            if ((long long)(globaltimer_ns() - start) > sh.limit_ns) {
                 if ((threadIdx.x & 31) == 0) {
-                    atomicCAS(limit.status, 0, PT_ETIMEDOUT);
+                    atomicCAS(sh.status, 0, PT_ETIMEDOUT);
                     *(volatile int*)&sh.abort = 1;
                 }
                 return false;
@@ -269,7 +266,7 @@ __device__ void store_chain(const BatchInstance& I, int8_t* dst, const int8_t* b
 }
 
 __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchShared& sh, cg::cluster_group& cluster,
-                            int rank, int K, const WaitLimit& limit) {
+                            int rank, int K) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const BatchLayout L(I, K, nt);
     uint32_t* s_sdesc = reinterpret_cast<uint32_t*>(smem + L.sdesc);
@@ -322,7 +319,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
             for (int lc = 0; lc < c_count; ++lc)
                 load_chain(I, reinterpret_cast<int8_t*>(s_chains + (size_t)lc * L.chain_stride),
                            I.spins + (size_t)(c_begin + lc) * I.slot_stride, tid, nt);
-        if (tid == 0) sh.next = 0ull;
+        if (tid == 0) sh.next = (unsigned)ngroups;
     }
     __syncthreads();
     if (K > 1) cluster_barrier();  // every mailbox is clear before anyone publishes
@@ -337,47 +334,56 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
     const bool keep = share.keep;
     const uint32_t qmod0 = (uint32_t)(I.q0 % kTagPeriod);
     uint32_t phase = grp < 16 ? sh.phase[grp] : 0u;
-    bool stored = false;  // lead: a bulk store of chain `stored_lc` is in flight
-    int stored_lc = 0, stored_seq = 0;
-    int kept_s = 0;
-    TaskCursor at;
+    bool stored = false;  // lead: a bulk store of the last task's chain (ctl_g) is in flight
+    TaskCursor at(grp);   // lead; a group that keeps its chain steps the sweep alone
+
+    auto next_task = [&] {  // lead
+        if (keep) {
+            ++at.s;
+        } else {
+            unsigned next = 0;
+            if (lane == 0) next = atomicAdd(&sh.next, 1u);
+            at.move_to(__shfl_sync(0xFFFFFFFFu, next, 0), c_count);
+        }
+    };
 
     for (;;) {
-        // ---- the next task, its chain's last sweep and that sweep's swap decision
+        // ---- the task, its chain's last sweep and that sweep's swap decision
         int s = 0, lc = grp, rung = 0, stop = 0;
+        int publish = -1;  // lead: the pass that follows this sweep
         if (grp >= ngroups || c_count == 0 || (keep && grp >= c_count)) break;
         if (lead) {
-            if (keep) {
-                s = kept_s++;
-                stop = s > I.n_sweeps;
-            } else {
+            s = at.s;
+            lc = at.lc;
+            stop = s > I.n_sweeps;
+            if (!keep) {
                 if (stored) {
                     // the chain is back in global memory before its next task may load it
                     if (lane == 0) {
                         bulk_stores_done();
                         fence_async();
                         __threadfence_block();
-                        *(volatile int*)&s_seq[stored_lc] = stored_seq;
+                        *(volatile int*)&s_seq[ctl_g[1]] = ctl_g[0] + 1;
                     }
                     stored = false;
                 }
-                unsigned long long task = 0;
-                if (lane == 0) task = atomicAdd(&sh.next, 1ull);
-                at.move_to(__shfl_sync(0xFFFFFFFFu, task, 0), c_count);
-                s = at.s;
-                lc = at.lc;
-                stop = s > I.n_sweeps;
                 if (!stop && s > 0) {
                     volatile int* seq = s_seq + lc;
-                    stop = !wait_for(sh, limit, [&] { return *seq >= s; });
+                    stop = !wait_for(sh, [&] { return *seq >= s; });
                     __threadfence_block();
                 }
             }
+            int passes = 0, since_pass = 1;  // s = passes * sps + since_pass
+            if (sps > 0) {
+                passes = s / sps;
+                since_pass = s - passes * sps;
+                if (since_pass + 1 == sps) publish = passes;
+            }
             if (!stop) {
                 rung = s_rung[lc];
-                if (s > 0 && sps > 0 && s % sps == 0) {
+                if (passes > 0 && since_pass == 0) {
                     // the pass after sweep s - 1
-                    const int pass = s / sps - 1;
+                    const int pass = passes - 1;
                     const long long q = I.q0 + pass;
                     const int rl = (rung & 1) == (int)(q & 1) ? rung : rung - 1;
                     const bool lower = rl == rung;
@@ -387,7 +393,8 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                         const unsigned long long* mb =
                             mail + ((size_t)(pass & (kClusterMailPasses - 1)) * R + partner) * 2;
                         unsigned long long wa = 0, wb = 0;
-                        stop = !wait_for(sh, limit, [&] {
+                        const double ca = I.coef[rl], cc = I.coef[(R - 1) + rl];  // (not after the wait)
+                        stop = !wait_for(sh, [&] {
                             if (I.mail_smem) {
                                 wa = ld_cluster_local_u64(mb);
                                 wb = ld_cluster_local_u64(mb + 1);
@@ -400,8 +407,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                         const long long E = s_E[lc], M = s_M[lc];
                         const long long pE = (long long)wa >> 24, pM = (long long)(int32_t)(uint32_t)(wb >> 32);
                         const bool acc = swap_accept_fast(lower ? E : pE, lower ? pE : E, lower ? M : pM,
-                                                          lower ? pM : M, I.coef[rl], I.coef[(R - 1) + rl],
-                                                          (uint32_t)q, (uint32_t)rl,
+                                                          lower ? pM : M, ca, cc, (uint32_t)q, (uint32_t)rl,
                                                           philox_schedule(I.key0, I.key1), false);
                         if (!stop) {
                             if (lower && lane < (acc ? 2 : 1)) atomicAdd(I.swap_stats + 2 * rl + lane, 1ull);
@@ -430,6 +436,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
         }
         if (stop) break;
         if (s == I.n_sweeps) {  // only the last pass's decision was left
+            if (lead) next_task();
             if (!one_warp) group_sync(bar, gsize);  // everyone has read the group's control words
             continue;
         }
@@ -455,10 +462,11 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                 for (int c = 0; c < 3; ++c) thr_g[c * index.S + l] = I.thr[(size_t)rung * I.nL3 + 3 * l + c];
         if (bulk_in) {
             // (the copy completes by itself; the limit only bounds the wait)
-            const unsigned long long start = globaltimer_ns();
+            unsigned long long start = 0;
             while (!mbar_try_wait(&sh.mbar[grp], phase)) {
-                if ((long long)(globaltimer_ns() - start) > limit.ns) {
-                    atomicCAS(limit.status, 0, PT_ETIMEDOUT);
+                if (start == 0) start = globaltimer_ns();
+                if ((long long)(globaltimer_ns() - start) > sh.limit_ns) {
+                    atomicCAS(sh.status, 0, PT_ETIMEDOUT);
                     *(volatile int*)&sh.abort = 1;
                     break;
                 }
@@ -502,8 +510,10 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
             if (!in_place && !last) {
                 if (lane == 0) bulk_store(g_chain, buf, (uint32_t)L.chain_stride);
                 stored = true;
-                stored_lc = lc;
-                stored_seq = s + 1;
+                if (one_warp && lane == 0) {
+                    ctl_g[0] = s;
+                    ctl_g[1] = lc;
+                }
             }
             if (!one_warp) {
                 dE = dM = nf = 0;
@@ -519,8 +529,8 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                 s_E[lc] = E;
                 s_M[lc] = M;
             }
-            if (sps > 0 && (s + 1) % sps == 0 && rung + 1 != I.withhold) {
-                const int pass = (s + 1) / sps - 1;
+            if (publish >= 0 && rung + 1 != I.withhold) {
+                const int pass = publish;
                 const unsigned long long tag = mbox_tag(qmod0, pass);
                 const unsigned long long wa = ((unsigned long long)E << 24) | tag;
                 const unsigned long long wb = ((unsigned long long)(uint32_t)(int32_t)M << 32) | tag;
@@ -541,6 +551,7 @@ __device__ void run_problem(const BatchInstance& I, unsigned char* smem, BatchSh
                 atomicAdd(I.acc + (size_t)rung * kAccCount + lane, v);
             }
             __syncwarp();
+            next_task();  // before the chain is marked (TaskCursor)
             if (!keep && !stored && lane == 0) {  // (a chain being stored is marked when it has arrived)
                 __threadfence_block();
                 *(volatile int*)&s_seq[lc] = s + 1;
@@ -571,17 +582,20 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
         mbar_init(&sh.mbar[threadIdx.x]);
         sh.phase[threadIdx.x] = 0u;
     }
-    if (threadIdx.x == 0) sh.abort = 0;
+    if (threadIdx.x == 0) {
+        sh.abort = 0;
+        sh.limit_ns = bp.timeout_ns;
+        sh.status = bp.status;
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async();
     __syncthreads();
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int K = (int)cluster.num_blocks();
-    const WaitLimit limit = {bp.timeout_ns, bp.status};
     if (bp.single) {
         // one problem on this one cluster; the host keeps its counters
-        run_problem(bp.one, smem, sh, cluster, rank, K, limit);
+        run_problem(bp.one, smem, sh, cluster, rank, K);
         if (K > 1) cluster.sync();  // peers are done reading this CTA's published (E, M)
         return;
     }
@@ -592,7 +606,7 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(BatchParams bp) {
         cluster.sync();  // every CTA has read the job before rank 0 may reuse or release sh.job
         if (job >= bp.count) break;
         const BatchInstance I = bp.inst[bp.order[job]];
-        run_problem(I, smem, sh, cluster, rank, K, limit);
+        run_problem(I, smem, sh, cluster, rank, K);
         cluster.sync();  // peers are done reading this CTA's published (E, M)
         if (rank == 0 && threadIdx.x == 0) {
             // a finished problem's counters advance on the device, so the same launch can be

@@ -220,23 +220,21 @@ struct CtaShare {
 };
 
 // A group's place in its CTA's sequence of tasks: task number s * count + lc is sweep s of chain
-// lc. The number needs 64 bits (2^30 sweeps of 1024 chains), but a group's next task is close to
-// its last one, so a 32-bit division of the step finds it.
+// lc. Group g begins with task g (there are more chains than groups); the others are numbered by a
+// counter from the groups' number on. The number can pass 2^32 (2^30 sweeps of 1024 chains), but the
+// counter only has to tell a group's next task from its last one: a group takes the next while the
+// chain of its last is still to be marked done, and until then each sweep of that chain holds up one
+// other group, so fewer than (groups + 1) x chains tasks lie between the two.
 struct TaskCursor {
-    unsigned long long task = 0;
-    int s = 0, lc = 0;
-    __host__ __device__ void move_to(unsigned long long next, int count) {
-        const unsigned long long step = next - task;
+    unsigned task;
+    int s, lc;
+    __host__ __device__ explicit TaskCursor(int group) : task((unsigned)group), s(0), lc(group) {}
+    __host__ __device__ void move_to(unsigned next, int count) {
+        const unsigned x = (unsigned)lc + (next - task);
+        const unsigned sweeps = x / (unsigned)count;
         task = next;
-        if (step < 0x40000000ull) {
-            const unsigned x = (unsigned)lc + (unsigned)step;
-            const unsigned sweeps = x / (unsigned)count;
-            s += (int)sweeps;
-            lc = (int)(x - sweeps * (unsigned)count);
-        } else {
-            s = (int)(next / (unsigned)count);
-            lc = (int)(next - (unsigned long long)s * (unsigned)count);
-        }
+        s += (int)sweeps;
+        lc = (int)(x - sweeps * (unsigned)count);
     }
 };
 

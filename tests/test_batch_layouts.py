@@ -91,14 +91,15 @@ def test_a_cta_that_keeps_its_chains_does_not_stream_them(layouts):
 
 @pytest.mark.parametrize("chains,first", [
     (1024, 0), (1024, 2 ** 21 - 3), (1024, 2 ** 22 - 3), (1024, 2 ** 30 - 40), (32, 2 ** 26 - 40), (32, 2 ** 30 - 40),
-    (17, 2 ** 31 // 17 - 5), (1, 2 ** 30 - 40),
+    (17, 2 ** 31 // 17 - 5), (17, 2 ** 30 - 40),
 ])
 def test_tasks_of_the_longest_runs_stay_in_range(native, chains, first):
     """2^30 sweeps of 1024 chains: the task number passes 2^31, 2^32 and ends at 2^40."""
-    r = subprocess.run([native("batch_tasks"), str(chains), str(2 ** 30), str(first), "60000"], capture_output=True,
-                       text=True)
+    groups = 16
+    r = subprocess.run([native("batch_tasks"), str(chains), str(2 ** 30), str(first), "60000", str(groups)],
+                       capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
-    assert int(r.stdout) == min(60000, (2 ** 30 + 1 - first) * chains)
+    assert int(r.stdout) == min(60000, (2 ** 30 + 1 - first) * chains - groups)
 
 
 @pytest.mark.gpu
