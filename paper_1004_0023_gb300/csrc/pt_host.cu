@@ -654,9 +654,10 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         *producers = std::min(128, std::max(32, (int)(copies / 3 + 31) / 32 * 32));
         return consumers + *producers <= 512 ? consumers + *producers : 0;
     };
-    // records in shared memory where the rest leaves room, and every chain has an SM to itself
-    auto records_for = [&](int pth, int copy) {
-        return R <= n_sm && (copy || pth == kPathPacked || pth == kPathPackedInline || pth == kPathPeer ||
+    // records in shared memory where the rest leaves room, every chain has an SM to itself and every
+    // word column a thread (a copy's always has: copy_threads)
+    auto records_for = [&](int pth, int copy, int consumers) {
+        return R <= n_sm && (copy || consumers >= P / 8) && (copy || pth == kPathPacked || pth == kPathPackedInline || pth == kPathPeer ||
                              pth == kPathCluster);
     };
     // a layout fits if it does with the threshold rows and / or the statistics moved out
@@ -869,7 +870,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         return create_fail(PT_EINVAL, "one chain needs %zu bytes of shared memory; the device allows %d",
                            c->plan.smem_bytes, max_smem);
     }
-    if (records_for(path, c->plan.copy)) {
+    if (records_for(path, c->plan.copy, c->plan.n_consumer)) {
         p.records = 1;
         if (plan_smem() > (size_t)max_smem) p.records = 0;
         c->plan.smem_bytes = plan_smem();
@@ -1138,7 +1139,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                 pc.n_levels = (int)off_c.size() - 1;
                 if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.tables_in_smem = 0;
                 if (copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.acc_in_smem = 0;
-                pc.records = records_for(cd.path, 1);
+                pc.records = records_for(cd.path, 1, pl.n_consumer);
                 if (pc.records && copy_smem_bytes(pc, cl) > (size_t)max_smem) pc.records = 0;
                 pl.smem_bytes = copy_smem_bytes(pc, cl);
                 return pl.smem_bytes <= (size_t)max_smem;
@@ -1179,7 +1180,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                     pl.pieces = pc.n_chunks;
                     return pl.smem_bytes <= (size_t)max_smem;
                 };
-                pc.records = records_for(cd.path, 0);
+                pc.records = records_for(cd.path, 0, pl.n_consumer);
                 if (table_bytes > 49152 && table_bytes <= 98304)
                     for (int pieces = 1; pieces <= (P >= 128 ? 1 : 2); ++pieces)
                         if (fits_in(pieces, 98304)) return true;
@@ -1188,7 +1189,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
                         if (fits_in(pieces, 49152)) return true;
                 return false;
             }
-            pc.records = records_for(cd.path, 0);
+            pc.records = records_for(cd.path, 0, pl.n_consumer);
             if (pc.records && sweep_smem_bytes(pc, cd.path, pl.dclass, cpre) > (size_t)max_smem) pc.records = 0;
             pl.smem_bytes = sweep_smem_bytes(pc, cd.path, pl.dclass, cpre);  // sized for this schedule
             return pl.smem_bytes <= (size_t)max_smem;

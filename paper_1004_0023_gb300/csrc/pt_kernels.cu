@@ -1022,7 +1022,12 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                     }
                     const int lev0 = piece > 0 ? p.chunk_level[piece] : spec_done ? 1 : 0;
                     const int lev_end = PIECES ? p.chunk_level[piece + 1] : p.n_levels;
-                    if (rec && g_fixed) {
+                    // Records only with a thread for every column, so the loop after this one has
+                    // descriptors alone: with a choice between the two in its units it took 15 to 20 %
+                    // longer (path 2, N=2048, P=32, R=48: 17.1 us per sweep against 14.8; 16.3 before
+                    // there were records). The path-8 kernel has the choice: its loop over records
+                    // is 1 % faster that way, and it seldom runs the other.
+                    if (rec && (!PEER || g_fixed)) {
                         // this thread's column never changes: its row offsets are loop invariants. Each
                         // level's first record is loaded before the barrier that ends the level before.
                         int end = s_loff[min(lev0 + 1, lev_end)], q = s_loff[lev0] + q_lane;
@@ -1053,7 +1058,8 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                                     packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot,
                                                                key, smem, rule, thr_c, sums);
                                 } else {
-                                    const Eval e = rec ? eval_rec(load_rec(q), q, g, c, rb, t) : eval_desc(q, g, c, rb, t);
+                                    const Eval e = PEER && rec ? eval_rec(load_rec(q), q, g, c, rb, t)
+                                                               : eval_desc(q, g, c, rb, t);
                                     commit(e, flips(e, c, thr_c));
                                 }
                             };
