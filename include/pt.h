@@ -81,9 +81,9 @@ typedef struct {
                                    inline or produced random words; byte-wise for P = 1 and
                                    where the words' layout does not fit), 2 = packed with inline random
                                    words, 3 = packed with random words produced one sweep
-                                   ahead by dedicated warps, 4 = packed with four bits
-                                   (P % 32 == 0, Lmax <= 31, if it fits) or one bit per copy
-                                   in shared memory (paths 2-6 need P % 8 == 0 and
+                                   ahead by dedicated warps, 4 = packed with two bits
+                                   (P % 32 == 0, Lmax <= 31, levels of many updates, if it
+                                   fits) or one bit per copy in shared memory (paths 2-6 need P % 8 == 0 and
                                    degree <= 7), 5 = path 3 with each chain split over a
                                    cluster of two CTAs, one half of the Trotter copies each
                                    (needs P % 16 == 0 and all R chains resident at once;

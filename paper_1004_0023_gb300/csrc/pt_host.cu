@@ -736,11 +736,18 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     }
     if (path == kPathBits) {
         // the nibble form (twice the shared memory of one bit a copy) when it holds whole words,
-        // its sums fit, and its layout does (with the tables in global memory if need be)
+        // its sums fit, its layout does (with the tables in global memory if need be), and a level
+        // has work for it: its unit of 16 copies takes 0.43 to 0.49 us a level whatever their number
+        // up to four warps, the one-bit unit of 4 copies 0.29 to 0.36 up to five and 0.5 from nine on.
+        // Seven warps of one-bit units in an average level (nibbles / one bit, us per sweep without
+        // swaps): 960 / 595 on a path of 2048 sites (P = 128, 32 units a level), 4.34 / 3.51 on 72
+        // cells' sites (P = 64, 165 units), 6.24 / 6.78 on 200 (291 units), 38.4 / 59.7 on N=2048,
+        // degree 3, P = 128 (6554 units).
+        const long long bit_units = (long long)items.size() * (P / 8) / p.n_levels;
         DevProblem q = p;
         q.nibble = 1;
         q.tables_in_smem = q.acc_in_smem = 0;
-        p.nibble = P % 32 == 0 && Lmax <= kWordBitsLmax && want_threads <= 512 &&
+        p.nibble = P % 32 == 0 && Lmax <= kWordBitsLmax && want_threads <= 512 && bit_units >= 224 &&
                    sweep_smem_bytes(q, kPathBits, packed_dc) <= (size_t)max_smem;
         c->plan.nibble = !p.nibble ? 0 : (packed_dc == 4 ? 3 : (dmax <= 6 ? 6 : 7));
     }

@@ -233,3 +233,22 @@ def test_partner_that_never_publishes_times_out_with_words_in_pieces(pieces):
     h.run(20, 1)
     o.run(20, 1)
     assert np.array_equal(h.read_state(), o.read_state())
+
+
+@pytest.mark.parametrize("n,degree,P,lmax,threads", [
+    (400, 3, 32, 31, 0), (400, 3, 32, 13, 96), (250, 3, 96, 31, 0), (700, 6, 32, 31, 0), (300, 6, 96, 30, 0),
+    (800, 7, 32, 31, 0), (300, 7, 128, 29, 512), (120, 2, 192, 5, 0),
+])
+def test_nibble_words_on_large_levels_match_the_oracle(n, degree, P, lmax, threads):
+    """Path 4 on levels of at least 224 one-bit units, which take 16 copies a unit: the largest Lmax
+    of the form, every number of neighbour slots, rows of several words."""
+    prob = _problem(n, degree, P, 3, lmax, n + P)
+    g, o = pt.PT.from_problem(prob, kernel_path=4, threads_per_block=threads), Oracle.from_problem(prob, threads=THREADS)
+    assert 2 * n * (P // 8) // g.info.n_levels >= 224
+    for sweeps, sps in ((1, 1), (2, 1), (6, 0), (10, 3)):
+        g.run(sweeps, sps)
+        o.run(sweeps, sps)
+        assert np.array_equal(g.read_state(), o.read_state()), (sweeps, sps)
+    og, oo = g.obs(), o.obs()
+    for k in oo:
+        assert np.array_equal(np.asarray(og[k]), np.asarray(oo[k])), k
