@@ -68,8 +68,7 @@ __device__ __forceinline__ double det_exp(double x) {
 }
 
 // The uniform word of swap pass q for the pair (rl, rl + 1).
-template <typename Key = PhiloxKey>
-__device__ __forceinline__ uint32_t swap_word(uint32_t q, uint32_t rl, const Key& key) {
+__device__ __forceinline__ uint32_t swap_word(uint32_t q, uint32_t rl, const PhiloxKey& key) {
     return philox(make_uint4(q, rl, 0u, kTagSwap << 28), key).x;
 }
 
@@ -121,10 +120,9 @@ __device__ __forceinline__ bool swap_accept_fast_by(long long EX, long long EY, 
 }
 
 // The two rules with the word drawn from (q, rl) under `key` when needed.
-template <typename Key = PhiloxKey>
 __device__ __forceinline__ bool swap_accept_fast(long long EX, long long EY, long long MX, long long MY,
                                                  double a, double c, uint32_t q, uint32_t rl,
-                                                 const Key& key, bool exact_only) {
+                                                 const PhiloxKey& key, bool exact_only) {
     return swap_accept_fast_by(EX, EY, MX, MY, a, c, [&] { return swap_word(q, rl, key); }, exact_only);
 }
 
@@ -562,9 +560,9 @@ __device__ __forceinline__ void trotter_differences(const uint32_t* V, const uin
 
 // Random words of a unit: read from rbq[0 .. W-1] (PRE), else word w of philox((t, i, slot,
 // par<<24 | gg + x)) for word x, gg the unit's first 8-copy chunk in the whole chain.
-template <int W, bool PRE, typename Key>
+template <int W, bool PRE>
 __device__ __forceinline__ void unit_words(uint32_t* u, uint32_t item, const uint4* rbq, uint32_t t, uint32_t slot,
-                                           uint32_t gg, const Key& key) {
+                                           uint32_t gg, const PhiloxKey& key) {
 #pragma unroll
     for (int x = 0; x < W; ++x) {
         const uint4 r =
@@ -598,10 +596,10 @@ __device__ __forceinline__ void unit_eval_site(UnitEval<W>& e, int8_t* sp, const
     }
 }
 
-template <int DC, int W, bool PRE, bool WIDE, typename Key = PhiloxKey>
+template <int DC, int W, bool PRE, bool WIDE>
 __device__ __forceinline__ UnitEval<W> unit_eval(int8_t* sp, const uint32_t* s_sdesc, uint32_t item,
                                                  const UnitOffsets& o, const uint4* rbq, uint32_t t, uint32_t slot,
-                                                 uint32_t gg, const UnitRule<WIDE>& rule, const Key& key) {
+                                                 uint32_t gg, const UnitRule<WIDE>& rule, const PhiloxKey& key) {
     UnitEval<W> e;
     const SiteTerms<DC> s = load_site<DC>(s_sdesc + (item >> 1) * SiteDesc<DC>::DW);
     unit_words<W, PRE>(e.u, item, rbq, t, slot, gg, key);
