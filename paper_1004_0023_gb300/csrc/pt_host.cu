@@ -888,7 +888,8 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     // shared memory a CTA than the simplest kernel for the same chains; where those alone keep some
     // chain out (ladders of several CTAs an SM: N=8, P=10, R=700 is resident with the byte-wise
     // kernel's 80 registers, not with 117), the simplest kernel runs: byte-wise, one bit a copy,
-    // without held units (`lean`), with the threshold rows in global memory.
+    // without held units (`lean`), with the threshold rows in global memory. (Path 7 with swap_mode 1
+    // is held to the residency of the plan it is set up on.)
     const int mode = opt ? opt->swap_mode : 0;
     int coop_ok = 0;
     cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, c->device);
@@ -901,8 +902,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     };
     const bool one_launch = coop_ok && mode != 2 && R > 1;
     const bool pairs = path == kPathPeer || path == kPathSplit || path == kPathSplitInline;  // always resident
-    if ((pairs || (one_launch && R > n_sm)) && !want_chains && path != kPathClassical && path != kPathCluster &&
-        !all_resident()) {
+    if ((pairs || (one_launch && R > n_sm)) && path != kPathClassical && path != kPathCluster && !all_resident()) {
         const bool simpler = (path == kPathGeneric && c->plan.rows) || (path == kPathBits && p.nibble);
         // 512 threads and more fill the registers of an SM's CTA either way
         const bool lean = c->plan.threads < 512 && (path == kPathPacked || path == kPathPackedInline ||

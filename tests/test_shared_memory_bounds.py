@@ -55,6 +55,7 @@ LADDERS = [
     (8, 3, 10, 700, dict(kernel_path=1)), (8, 3, 12, 700, dict()), (9, 5, 20, 800, dict(kernel_path=1)),
     (8, 3, 16, 700, dict(kernel_path=2, threads_per_block=128)), (8, 3, 16, 700, dict(kernel_path=3, threads_per_block=128)),
     (8, 3, 32, 250, dict(kernel_path=4, threads_per_block=512)), (8, 5, 16, 250, dict(kernel_path=4, threads_per_block=448)),
+    (16, 3, 24, 700, dict(kernel_path=7, group_threads=512, cluster_size=4)),
     (8, 3, 16, 100, dict(kernel_path=8, threads_per_block=320)), (8, 3, 16, 250, dict(kernel_path=6, threads_per_block=160)),
 ]
 
