@@ -305,6 +305,34 @@ extern "C" int pt_server_create(const pt_server_options* opt, void* cuda_stream,
     return PT_OK;
 }
 
+// A request's chain as the streamed kernels hold it (int8 rows). Requests whose chains fit only as
+// bit words start in a batched launch, alone if need be.
+static bool fits_streamed(const pt_server* s, const Prepared& pr) {
+    DevProblem p;
+    memset(&p, 0, sizeof(p));
+    p.N = pr.N;
+    p.P = pr.P;
+    p.R = pr.R;
+    p.Lmax = pr.Lmax;
+    p.n_levels = pr.n_levels;
+    return sweep_smem_bytes(p, kPathPackedInline, pr.dc) <= s->smem_cap;
+}
+
+// The arena block of a batched launch of n requests: their records, the work order, then counter,
+// status and done flags.
+struct GroupLayout {
+    size_t order, counter, status, flags, bytes;
+};
+static GroupLayout group_layout(int n) {
+    GroupLayout l;
+    l.order = ((size_t)n * sizeof(BatchInstance) + 255) & ~(size_t)255;
+    l.counter = l.order + (((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255);
+    l.status = l.counter + 16;
+    l.flags = l.counter + 256;
+    l.bytes = l.flags + (((size_t)n * sizeof(int) + 255) & ~(size_t)255);
+    return l;
+}
+
 extern "C" int pt_server_submit(pt_server* s, const pt_request* r, int64_t* id) {
     if (!s || !r || !id) return PT_EINVAL;
     if (s->err) return s->err;
@@ -334,6 +362,11 @@ extern "C" int pt_server_submit(pt_server* s, const pt_request* r, int64_t* id) 
     q->req.ladder = nullptr;
     q->remaining = r->n_sweeps;
     q->id = s->next_id++;
+    if (!fits_streamed(s, q->prep) && q->block_bytes + group_layout(1).bytes > s->alloc->size()) {
+        delete q;
+        return sfail(s, PT_ENOMEM, "request needs %zu bytes and its launch %zu more, the arena holds %zu", q->block_bytes,
+                     group_layout(1).bytes, s->alloc->size());
+    }
     // the request's shared-memory plan must fit one CTA
     fill_instance(q->inst, q->prep, nullptr, q->req);
     choose_groups(q->inst, s->cluster, s->threads, s->smem_cap);
@@ -648,11 +681,11 @@ static int launch_group(pt_server* s, const std::vector<ServeReq*>& g) {
         if (s->ncl_by_log2[l] <= 0) K = s->cluster;
     }
     ServeGroup* grp = new ServeGroup();
-    const size_t order_off = ((size_t)n * sizeof(BatchInstance) + 255) & ~(size_t)255;
-    const size_t ctr_off = order_off + (((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255);
-    grp->status_off = ctr_off + 16;
-    grp->flags_off = ctr_off + 256;
-    grp->bytes = grp->flags_off + (((size_t)n * sizeof(int) + 255) & ~(size_t)255);
+    const GroupLayout block = group_layout(n);
+    const size_t order_off = block.order, ctr_off = block.counter;
+    grp->status_off = block.status;
+    grp->flags_off = block.flags;
+    grp->bytes = block.bytes;
     grp->n = n;
     grp->flags.assign(n, 0);
     if (!s->alloc->alloc(grp->bytes, &grp->off)) {
@@ -727,6 +760,14 @@ static int launch_group(pt_server* s, const std::vector<ServeReq*>& g) {
         grp->refs += 1;
     }
     return PT_OK;
+}
+
+// One request by itself. Returns 1 (nothing launched) when its launch finds no room in the arena.
+static int launch_alone(pt_server* s, ServeReq* q) {
+    if (!fits_streamed(s, q->prep)) return launch_group(s, std::vector<ServeReq*>(1, q));
+    const int rc = launch_streamed(s, q);
+    if (rc == 0) s->inflight_sms += q->prep.R;
+    return rc;
 }
 
 // Frees the block of a group whose launch has ended (false: still running).
@@ -813,10 +854,18 @@ static int step_streamed(pt_server* s) {
         if (!g.empty()) {
             const int rc = launch_group(s, g);
             if (rc > 0) {
-                for (ServeReq* q : g) {  // no room for the group's block: one launch each
-                    const int rc2 = launch_streamed(s, q);
-                    if (rc2) return rc2;
-                    s->inflight_sms += q->prep.R;
+                // no room for the group's block: one launch each
+                std::vector<ServeReq*> later;
+                for (ServeReq* q : g) {
+                    const int rc2 = launch_alone(s, q);
+                    if (rc2 > 0) later.push_back(q);
+                    else if (rc2) return rc2;
+                }
+                for (size_t k = later.size(); k-- > 0;) {  // back to the front of the queue, in order
+                    ServeReq* q = later[k];
+                    s->alloc->release(q->block_off, q->block_bytes);
+                    s->active.erase(std::find(s->active.begin(), s->active.end(), q->id));
+                    s->queued.push_front(q->id);
                 }
             } else if (rc) {
                 return rc;
@@ -829,11 +878,14 @@ static int step_streamed(pt_server* s) {
             size_t off = 0;
             if (!s->alloc->alloc(q->block_bytes, &off)) break;
             q->block_off = off;
+            const int rc = launch_alone(s, q);
+            if (rc > 0) {
+                s->alloc->release(q->block_off, q->block_bytes);
+                break;
+            }
             s->queued.pop_front();
-            const int rc = launch_streamed(s, q);
             if (rc) return rc;
             s->active.push_back(q->id);
-            s->inflight_sms += q->prep.R;
         }
     }
     s->steps += 1;

@@ -201,3 +201,39 @@ def test_backlog_on_device_memory_that_held_other_data():
             alone.run(p.n_sweeps, p.sweeps_per_swap)
             _same(results[k][0], results[k][1], alone.read_state(), alone.obs(), "round %d request %d" % (round_, k))
             alone.close()
+
+
+def test_requests_that_fit_only_as_bit_words_run_alone_and_among_others():
+    """N=1466, P=256: a chain is 375 KB as int8 and 47 KB as bit words, so its request starts in a
+    batched launch of its own; and an arena without room for that launch refuses it at submit."""
+    from test_gpu_units import _problem as problem_of
+
+    big = [problem_of(1466, 3, 256, 2 + k, 9, 5 + k) for k in range(2)]
+    small = [problem_of(20, 3, 32, 4, 9, 7 + k) for k in range(2)]
+    for k, p in enumerate(big + small):
+        p.n_sweeps, p.sweeps_per_swap = 4 + k, 1 + k % 2
+    srv = pt.Server(arena_bytes=1 << 27)
+    for batch in ([big[0]], [small[0], big[0], small[1], big[1]], small):
+        ids = [srv.submit(p) for p in batch]
+        done = set()
+        while len(done) < len(ids):
+            done |= set(srv.step())
+        for rid, p in zip(ids, batch):
+            o = Oracle.from_problem(p, threads=THREADS)
+            o.run(p.n_sweeps, p.sweeps_per_swap)
+            state, obs = srv.result(rid)
+            _same(state, obs, o.read_state(), o.obs(), "request %d" % rid)
+            srv.release(rid)
+    srv.submit(big[0])
+    while not srv.info().active:
+        srv.step()
+    used = srv.info().arena_used  # the request's block and its launch's
+    srv.close()
+    with pytest.raises(pt.PTError) as e:
+        pt.Server(arena_bytes=used - 256).submit(big[0])
+    assert e.value.code == pt.PT_ENOMEM
+    tight = pt.Server(arena_bytes=used)
+    rid = tight.submit(big[0])
+    while rid not in tight.step():
+        pass
+    tight.close()
