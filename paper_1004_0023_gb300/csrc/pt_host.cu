@@ -880,6 +880,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     if (records_for(path, c->plan.copy, c->plan.n_consumer)) {
         p.records = 1;
         if (plan_smem() > (size_t)max_smem) p.records = 0;
+        c->plan.records = p.records;
         c->plan.smem_bytes = plan_smem();
     }
 
@@ -920,7 +921,7 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             c->plan = plan0;
             items = items0;
             level_off = off0;
-            p.records = 0;
+            p.records = c->plan.records = 0;
             if (simple_k) {
                 p.slots = p.nibble = 0;
                 c->plan.rows = c->plan.copy = c->plan.nibble = 0;
@@ -1107,8 +1108,8 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
         const PlanKey key{N, P, R, packed_dc, p.n_levels, nE, p.slots, IndexRule(Lmax).wide ? 1 : 0,
                           table_bytes <= 49152 ? 0 : (table_bytes <= 98304 ? 1 : 2)};
         // a candidate's plan, shared-memory flags and level schedule
-        auto make = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
-                        std::vector<int32_t>& off_c) {
+        auto shape = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
+                         std::vector<int32_t>& off_c) {
             pc = p;
             pc.records = pc.n_chunks = 0;
             if (cd.path == kPathClassical) {
@@ -1200,6 +1201,12 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
             if (pc.records && sweep_smem_bytes(pc, cd.path, pl.dclass, cpre) > (size_t)max_smem) pc.records = 0;
             pl.smem_bytes = sweep_smem_bytes(pc, cd.path, pl.dclass, cpre);  // sized for this schedule
             return pl.smem_bytes <= (size_t)max_smem;
+        };
+        auto make = [&](const Cand& cd, LaunchPlan& pl, DevProblem& pc, std::vector<uint32_t>& it_c,
+                        std::vector<int32_t>& off_c) {
+            if (!shape(cd, pl, pc, it_c, off_c)) return false;
+            pl.records = pc.records;
+            return true;
         };
         // every chain of a made plan resident at once
         auto runs_here = [&](const LaunchPlan& pl, const DevProblem& pc) {

@@ -139,6 +139,7 @@ struct LaunchPlan {
     int copy = 0;           // paths 1, 3 and 9: one copy a thread (sweep_copy_kernel)
     int nibble = 0;         // path 4: neighbour slots of the nibble form, 0 = one bit a copy
     int rows = 0;           // path 1: the word-wise kernel (DevProblem::slots > 0)
+    int records = 0;        // the instance with records (DevProblem::records)
     int lean = 0;           // paths 2, 3, 4, 6 and 8: the instance with less registers a thread
     int chains_per_cta = 1; // path 10: chains packed on one CTA (cluster = ceil(R / chains_per_cta))
 };

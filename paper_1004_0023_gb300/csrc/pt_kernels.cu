@@ -721,8 +721,13 @@ __device__ __forceinline__ void produce_words(uint4* buf, uint32_t t, const uint
 // COPY (with DC = 0 and PRE): one copy a thread.
 // PIECES (with PEER): a sweep's random words come in p.n_chunks pieces (pt_internal.h).
 // NIB > 0: the nibble form of the bit-packed chain with NIB neighbour slots in use.
+// REC: records in place of descriptors (DevProblem::records, with a thread for every column). The
+// instances without records hold the loop over descriptors alone: beside the one over records it
+// took 15 to 20 % longer (path 2, N=2048, P=32, R=48: 17.1 us per sweep against 14.8). Those with
+// records keep both, and the run-time choice, although only one runs: the loop over records by
+// itself is compiled to 1 to 5 % slower code (path 9, N=16, P=32, R=16: 2.31 -> 2.40 us per sweep).
 template <int DC, bool PRE, bool WIDE, bool BITS = false, bool SPEC = true, bool PEER = false, bool CSWAP = false,
-          int NIB = 0, bool COPY = false, bool PIECES = false>
+          int NIB = 0, bool COPY = false, bool PIECES = false, bool REC = false>
 __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot, long long t0, long long q0,
                                                   int n_sweeps, int sweeps_per_swap, long long timeout_ns,
                                                   int n_consumer, unsigned char* smem) {
@@ -758,7 +763,8 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
     const int G = NIB ? P >> 5 : ((P >> 1) + 3) >> 2;
     const uint32_t half = 4u * (uint32_t)G;
     const int desc_words = ROWS ? rows_desc_words(p.slots) : SiteDesc<ROWS ? 4 : DC>::DW;
-    const bool rec = !BITS && (COPY || !ROWS) && p.records;  // records in place of descriptors
+    static_assert(!REC || (!BITS && (COPY || !ROWS)), "kernels that have records");
+    const bool rec = REC && p.records;
 
     // what no earlier kernel writes
     if constexpr (ROWS) {
@@ -1022,12 +1028,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                     }
                     const int lev0 = piece > 0 ? p.chunk_level[piece] : spec_done ? 1 : 0;
                     const int lev_end = PIECES ? p.chunk_level[piece + 1] : p.n_levels;
-                    // Records only with a thread for every column, so the loop after this one has
-                    // descriptors alone: with a choice between the two in its units it took 15 to 20 %
-                    // longer (path 2, N=2048, P=32, R=48: 17.1 us per sweep against 14.8; 16.3 before
-                    // there were records). The path-8 kernel has the choice: its loop over records
-                    // is 1 % faster that way, and it seldom runs the other.
-                    if (rec && (!PEER || g_fixed)) {
+                    if (rec && g_fixed) {
                         // this thread's column never changes: its row offsets are loop invariants. Each
                         // level's first record is loaded before the barrier that ends the level before.
                         int end = s_loff[min(lev0 + 1, lev_end)], q = s_loff[lev0] + q_lane;
@@ -1058,8 +1059,7 @@ __device__ __forceinline__ void sweep_packed_body(const DevProblem& p, int slot,
                                     packed_unit_bits<DC, WIDE>(bp, s_desc, s_items[q], g, G, s_lut, t, (uint32_t)slot,
                                                                key, smem, rule, thr_c, sums);
                                 } else {
-                                    const Eval e = PEER && rec ? eval_rec(load_rec(q), q, g, c, rb, t)
-                                                               : eval_desc(q, g, c, rb, t);
+                                    const Eval e = rec ? eval_rec(load_rec(q), q, g, c, rb, t) : eval_desc(q, g, c, rb, t);
                                     commit(e, flips(e, c, thr_c));
                                 }
                             };
@@ -1306,7 +1306,7 @@ __device__ void peer_producer(const DevProblem& p, int slot, long long t0, int n
 // rank 1 produces its random words. The cluster shape is compiled in, and checked on entry
 // (both CTAs return before any barrier or remote access if it is not 2).
 // MAXT = 1024: the lean instance, without the held level-0 units (as sweep_packed_kernel).
-template <int DC, bool PIECES, int MAXT = 512>
+template <int DC, bool PIECES, bool REC, int MAXT = 512>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MAXT, 1)
     sweep_peer_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                       long long timeout_ns, int n_consumer) {
@@ -1322,27 +1322,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MAXT, 1)
     cluster_arrive_relaxed();
     if (cluster.block_rank() == 0) {
         if (IndexRule(p.Lmax).wide)
-            sweep_packed_body<DC, true, true, false, (MAXT <= 512), true, false, 0, false, PIECES>(
+            sweep_packed_body<DC, true, true, false, (MAXT <= 512), true, false, 0, false, PIECES, REC>(
                 p, slot, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, blockDim.x, smem);
         else
-            sweep_packed_body<DC, true, false, false, (MAXT <= 512), true, false, 0, false, PIECES>(
+            sweep_packed_body<DC, true, false, false, (MAXT <= 512), true, false, 0, false, PIECES, REC>(
                 p, slot, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, blockDim.x, smem);
     } else
         peer_producer<DC, PIECES>(p, slot, t0, n_sweeps, smem);
 }
 
-template <int DC, bool PRE, int MAXT, bool BITS = false>
+template <int DC, bool PRE, int MAXT, bool BITS = false, bool REC = false>
 __global__ void __launch_bounds__(MAXT, 1)
 sweep_packed_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                     long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
     // the held level-0 units do not fit the 64 registers of a 1024-thread block
     if (IndexRule(p.Lmax).wide)
-        sweep_packed_body<DC, PRE, true, BITS, (MAXT <= 512)>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap,
-                                                              timeout_ns, n_consumer, smem);
+        sweep_packed_body<DC, PRE, true, BITS, (MAXT <= 512), false, false, 0, false, false, REC>(
+            p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem);
     else
-        sweep_packed_body<DC, PRE, false, BITS, (MAXT <= 512)>(p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap,
-                                                               timeout_ns, n_consumer, smem);
+        sweep_packed_body<DC, PRE, false, BITS, (MAXT <= 512), false, false, 0, false, false, REC>(
+            p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem);
 }
 
 // Path 4's nibble form (P % 32 == 0, Lmax <= kWordBitsLmax).
@@ -1357,14 +1357,15 @@ __global__ void __launch_bounds__(512, 1)
 
 // One copy a thread (DevProblem::slots > 0): a CTA per chain, or (path 9) all of them in one
 // cluster, checked on entry as sweep_cluster_kernel does.
+template <bool REC>
 __global__ void __launch_bounds__(512, 1)
     sweep_copy_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                       long long timeout_ns, int n_consumer) {
     extern __shared__ __align__(16) unsigned char smem[];
-    sweep_packed_body<0, true, false, false, true, false, false, 0, true>(p, blockIdx.x, t0, q0, n_sweeps,
-                                                                          sweeps_per_swap, timeout_ns, n_consumer,
-                                                                          smem);
+    sweep_packed_body<0, true, false, false, true, false, false, 0, true, false, REC>(
+        p, blockIdx.x, t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem);
 }
+template <bool REC>
 __global__ void __launch_bounds__(512, 1)
     sweep_copy_cluster_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                               long long timeout_ns, int n_consumer) {
@@ -1374,9 +1375,8 @@ __global__ void __launch_bounds__(512, 1)
         if (threadIdx.x == 0) atomicCAS(p.status, 0, PT_ECUDA);
         return;
     }
-    sweep_packed_body<0, true, false, false, true, false, true, 0, true>(p, (int)cluster.block_rank(), t0, q0,
-                                                                         n_sweeps, sweeps_per_swap, timeout_ns,
-                                                                         n_consumer, smem);
+    sweep_packed_body<0, true, false, false, true, false, true, 0, true, false, REC>(
+        p, (int)cluster.block_rank(), t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem);
 }
 
 // Path 1's word-wise kernel: any even P and any degree up to 32 whose descriptors fit.
@@ -1396,7 +1396,7 @@ __global__ void __launch_bounds__(512, 1)
 // with the swap mailboxes in shared memory. The cluster shape is set at launch and checked
 // on entry: if the cluster is not the whole grid, every CTA returns before any cluster
 // barrier or remote access.
-template <int DC, bool PRE>
+template <int DC, bool PRE, bool REC>
 __global__ void __launch_bounds__(384, 1)
     sweep_cluster_kernel(DevProblem p, long long t0, long long q0, int n_sweeps, int sweeps_per_swap,
                          long long timeout_ns, int n_consumer) {
@@ -1407,11 +1407,11 @@ __global__ void __launch_bounds__(384, 1)
         return;
     }
     if (IndexRule(p.Lmax).wide)
-        sweep_packed_body<DC, PRE, true, false, true, false, true>(p, (int)cluster.block_rank(), t0, q0, n_sweeps,
-                                                                   sweeps_per_swap, timeout_ns, n_consumer, smem);
+        sweep_packed_body<DC, PRE, true, false, true, false, true, 0, false, false, REC>(
+            p, (int)cluster.block_rank(), t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem);
     else
-        sweep_packed_body<DC, PRE, false, false, true, false, true>(p, (int)cluster.block_rank(), t0, q0, n_sweeps,
-                                                                    sweeps_per_swap, timeout_ns, n_consumer, smem);
+        sweep_packed_body<DC, PRE, false, false, true, false, true, 0, false, false, REC>(
+            p, (int)cluster.block_rank(), t0, q0, n_sweeps, sweeps_per_swap, timeout_ns, n_consumer, smem);
 }
 
 // Several problems in one cooperative launch (all chains resident at once): block b sweeps
@@ -1940,9 +1940,29 @@ __global__ void scatter_kernel(DevProblem p, const int8_t* in) {
 }
 
 // ------------------------------------------------------------------------- launchers
+// The instances of a neighbour class with (REC) and without records.
+template <int DC, bool REC>
+static const void* class_fn(const LaunchPlan& plan) {
+    if (plan.path == kPathPeer) {
+        if (plan.pieces > 1) return (const void*)sweep_peer_kernel<DC, true, REC>;
+        return (const void*)sweep_peer_kernel<DC, false, REC>;
+    }
+    if (plan.path == kPathCluster)
+        return plan.n_consumer < plan.threads ? (const void*)sweep_cluster_kernel<DC, true, REC>
+                                              : (const void*)sweep_cluster_kernel<DC, false, REC>;
+    const bool pre = plan.path == kPathPacked;
+    // (at 64 registers the descriptors' loop alone is no faster: one instance serves both)
+    if (plan.threads > 512 || plan.lean)
+        return pre ? (const void*)sweep_packed_kernel<DC, true, 1024, false, true>
+                   : (const void*)sweep_packed_kernel<DC, false, 1024, false, true>;
+    return pre ? (const void*)sweep_packed_kernel<DC, true, 512, false, REC>
+               : (const void*)sweep_packed_kernel<DC, false, 512, false, REC>;
+}
 static const void* sweep_fn(const LaunchPlan& plan) {
-    if (plan.copy)
-        return plan.path == kPathCluster ? (const void*)sweep_copy_cluster_kernel : (const void*)sweep_copy_kernel;
+    if (plan.copy && plan.path == kPathCluster)
+        return plan.records ? (const void*)sweep_copy_cluster_kernel<true>
+                            : (const void*)sweep_copy_cluster_kernel<false>;
+    if (plan.copy) return plan.records ? (const void*)sweep_copy_kernel<true> : (const void*)sweep_copy_kernel<false>;
     if (plan.path == kPathClassical) {
         switch (plan.dclass) {
             case 4: return (const void*)sweep_classical_kernel<4>;
@@ -1958,20 +1978,9 @@ static const void* sweep_fn(const LaunchPlan& plan) {
             default: return (const void*)sweep_kernel<32>;
         }
     }
-    if (plan.path == kPathPeer) {
-        if (plan.pieces > 1)
-            return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, true> : (const void*)sweep_peer_kernel<8, true>;
-        if (plan.lean)
-            return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, false, 1024>
-                                    : (const void*)sweep_peer_kernel<8, false, 1024>;
-        return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, false> : (const void*)sweep_peer_kernel<8, false>;
-    }
-    if (plan.path == kPathCluster) {
-        const bool pre = plan.n_consumer < plan.threads;
-        if (plan.dclass == 4)
-            return pre ? (const void*)sweep_cluster_kernel<4, true> : (const void*)sweep_cluster_kernel<4, false>;
-        return pre ? (const void*)sweep_cluster_kernel<8, true> : (const void*)sweep_cluster_kernel<8, false>;
-    }
+    if (plan.path == kPathPeer && plan.lean && plan.pieces <= 1)  // (without records)
+        return plan.dclass == 4 ? (const void*)sweep_peer_kernel<4, false, false, 1024>
+                                : (const void*)sweep_peer_kernel<8, false, false, 1024>;
     if (plan.path == kPathSplit)
         return plan.dclass == 4 ? (const void*)sweep_split_kernel<4, true> : (const void*)sweep_split_kernel<8, true>;
     if (plan.path == kPathSplitInline && plan.dclass == 4 && plan.lean)
@@ -1989,15 +1998,8 @@ static const void* sweep_fn(const LaunchPlan& plan) {
         return plan.dclass == 4 ? (const void*)sweep_packed_kernel<4, false, 512, true>
                                 : (const void*)sweep_packed_kernel<8, false, 512, true>;
     }
-    const bool pre = plan.path == kPathPacked;
-    if (plan.threads > 512 || plan.lean) {
-        if (plan.dclass == 4)
-            return pre ? (const void*)sweep_packed_kernel<4, true, 1024> : (const void*)sweep_packed_kernel<4, false, 1024>;
-        return pre ? (const void*)sweep_packed_kernel<8, true, 1024> : (const void*)sweep_packed_kernel<8, false, 1024>;
-    }
-    if (plan.dclass == 4)
-        return pre ? (const void*)sweep_packed_kernel<4, true, 512> : (const void*)sweep_packed_kernel<4, false, 512>;
-    return pre ? (const void*)sweep_packed_kernel<8, true, 512> : (const void*)sweep_packed_kernel<8, false, 512>;
+    if (plan.dclass == 4) return plan.records ? class_fn<4, true>(plan) : class_fn<4, false>(plan);
+    return plan.records ? class_fn<8, true>(plan) : class_fn<8, false>(plan);
 }
 
 // The dynamic shared-memory limit is a per-function attribute shared by every context, so
@@ -2099,6 +2101,7 @@ static unsigned overlap_attr(bool overlap, cudaStream_t s, cudaLaunchAttribute* 
 cudaError_t launch_sweeps(const DevProblem& p, const LaunchPlan& plan, long long t0, long long q0,
                           int n_sweeps, int sweeps_per_swap, long long timeout_ns, bool cooperative,
                           cudaStream_t s) {
+    if ((plan.records != 0) != (p.records != 0)) return cudaErrorInvalidValue;  // the kernel's layout
     DevProblem pp = p;
     // the last argument: consumer threads, or (path 10) chains per CTA
     int n_consumer = plan.path == kPathClassical ? plan.chains_per_cta : plan.n_consumer;
