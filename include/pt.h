@@ -119,8 +119,9 @@ typedef struct {
                                    batched launches: CTAs per thread-block cluster (1..16), or
                                    0 = autotune (pt_batch_create times a short run of each
                                    layout and keeps the fastest, remembered per batch shape --
-                                   every request's N, P, R, degree class, levels and sweeps --
-                                   for the process; results never depend on it) */
+                                   every request's N, P, R, degree class, levels, sweeps and
+                                   the chain form that Lmax allows -- for the process; results
+                                   never depend on it) */
     int32_t no_autotune;        /* 0: when kernel_path and threads_per_block are automatic and
                                    the chains are int8 in shared memory, pt_create times a
                                    short run of each candidate plan (paths 2, 3, 5, 6, 7, 8 and
@@ -323,7 +324,8 @@ const char* pt_batch_last_error(const pt_batch* b);
  * request's own R stay within the device's SM count, so that every admitted request is
  * resident at once (a request larger than that is admitted when nothing else runs). An
  * admitted request's state and counters live in the arena; all of its sweeps are launched
- * at once on the least-loaded stream of a pool (one CTA per chain), so requests that arrive
+ * at once on the least-loaded stream of a pool (one CTA per chain; a request whose chains fit
+ * a CTA only as bit words: in a batched launch of its own), so requests that arrive
  * while others run overlap with them on the device. When a backlog of 8 or more requests waits, they
  * start together in one persistent batched launch (as pt_batch_run) instead; each of them
  * is reported finished as soon as its own chains are written back, not when the whole
