@@ -887,10 +887,10 @@ extern "C" int pt_create(const pt_instance* inst, int32_t P, const pt_rung* ladd
     // Swap passes inside one launch need every chain resident at once. The word-wise, one-copy and
     // nibble kernels, and those that hold level 0's units in registers, take more registers or
     // shared memory a CTA than the simplest kernel for the same chains; where those alone keep some
-    // chain out (ladders of several CTAs an SM: N=8, P=10, R=700 is resident with the byte-wise
-    // kernel's 80 registers, not with 117), the simplest kernel runs: byte-wise, one bit a copy,
-    // without held units (`lean`), with the threshold rows in global memory. (Path 7 with swap_mode 1
-    // is held to the residency of the plan it is set up on.)
+    // chain out (ladders of several CTAs an SM: N=9, degree 5, P=20, R=800 is resident with the
+    // byte-wise kernel's 80 registers, not with the 117 of the word-wise one), the simplest kernel
+    // runs: byte-wise, one bit a copy, without held units (`lean`), with the threshold rows in global
+    // memory. (Path 7 with swap_mode 1 is held to the residency of the plan it is set up on.)
     const int mode = opt ? opt->swap_mode : 0;
     int coop_ok = 0;
     cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, c->device);
